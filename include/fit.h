@@ -142,10 +142,11 @@ int fit_init(fit_handle** h, const fit_config* cfg_r, const fit_config* cfg_z, i
  * update with hit l.  Track t of the concatenation reads in.par[k*in.ld + t],
  * hits.pos[(l*3 + k)*hits.ld + t], ... and writes out.par[k*out.ld + t], ...
  * nlayer must equal the configured nlayer of every mode used.
- * Consecutive events of the same mode run as one kernel launch.  A call with
- * events of both modes runs its p2z launches on the handle's second stream,
- * forked from `stream` before them and joined back after them, so that they
- * overlap the p2r launches; `stream` follows the whole call as before.  Calls
+ * The events of a mode run as one kernel launch (one for every 1024 runs of
+ * consecutive same-mode events), whatever their order.  A call with events of
+ * both modes runs its p2z launch on the handle's second stream, forked from
+ * `stream` before it and joined back after it, so that it overlaps the p2r
+ * launch; `stream` follows the whole call as before.  Calls
  * on one handle from several host threads take turns for that stream.
  * Errors: FIT_ERR_ARG (NULL pointer, misaligned pointer or ld, sizes out of
  * range, unconfigured mode), FIT_ERR_CUDA (launch failure).
@@ -222,8 +223,8 @@ int fit_propagate_update_noalloc(const fit_config* cfg_r, const fit_config* cfg_
 typedef struct {
   int threads_per_block; /* 32, 64, 128 or 256 (64, 128 or 256 with one track per thread) */
   int blocks_per_sm;     /* grid = blocks_per_sm x SM count; 0 = as many as fit */
-  int persistent;        /* 1: one persistent launch; 0: one launch per run of
-                            same-mode events (fit_propagate_update's form) */
+  int persistent;        /* 1: one persistent launch; 0: one launch per mode
+                            (fit_propagate_update's form) */
   int tracks_per_thread; /* 2 (or 0, a zeroed struct): two tracks per thread in
                             packed f32x2 instructions; 1: one track per thread
                             (persistent form only) */
@@ -267,7 +268,7 @@ int fit_plan_run(fit_plan* plan, const fit_tracks_in* in, const fit_tracks_out* 
  * worth ~30 %, registers per thread ~10 %).  Times every candidate launch
  * shape -- persistent with two tracks per thread and 32, 64, 128 or 256 threads
  * per block, or one track per thread and 64, 128 or 256 threads per block,
- * each at every resident-block count, and the per-segment form -- on these
+ * each at every resident-block count, and the one-launch-per-mode form -- on these
  * buffers (out must not alias in; it is written) and keeps the fastest.  The
  * buffers are in the plan's layout.  A plan created with FIT_LAYOUT_TUNE
  * passes SoA buffers and has every shape timed in both layouts (the AoSoA runs

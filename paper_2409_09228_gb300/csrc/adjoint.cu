@@ -35,16 +35,18 @@ struct AdjArgs {
   float* g_hpos;
   float* g_par0;
   float* g_cov0;
-  int64_t t0, t1;
+  int64_t t0;  // base of the run table
   int nlayer;
   Geo geo;
 };
 
 template <int MODE>
-__global__ void __launch_bounds__(kAdjBlock) fit_tape_kernel(const __grid_constant__ FitArgs a,
-                                                             float* tape, int32_t* ndone) {
-  const int64_t t = a.t0 + (int64_t)blockIdx.x * kAdjBlock + threadIdx.x;
-  if (t >= a.t1) return;
+__global__ void __launch_bounds__(kAdjBlock)
+    fit_tape_kernel(const __grid_constant__ FitArgs a, const __grid_constant__ TrackRuns runs,
+                    float* tape, int32_t* ndone) {
+  const unsigned i = blockIdx.x * kAdjBlock + threadIdx.x;
+  if (i >= runs.n) return;
+  const int64_t t = a.t0 + run_element(runs, i, 1);
   const int64_t ld = a.ld_out;
   State<float> s;
   load_state(a, t, s);
@@ -95,9 +97,11 @@ __global__ void __launch_bounds__(kAdjBlock) fit_tape_kernel(const __grid_consta
 }
 
 template <int MODE>
-__global__ void __launch_bounds__(kAdjBlock) fit_adjoint_kernel(const __grid_constant__ AdjArgs b) {
-  const int64_t t = b.t0 + (int64_t)blockIdx.x * kAdjBlock + threadIdx.x;
-  if (t >= b.t1) return;
+__global__ void __launch_bounds__(kAdjBlock)
+    fit_adjoint_kernel(const __grid_constant__ AdjArgs b, const __grid_constant__ TrackRuns runs) {
+  const unsigned i = blockIdx.x * kAdjBlock + threadIdx.x;
+  if (i >= runs.n) return;
+  const int64_t t = b.t0 + run_element(runs, i, 1);
   const int64_t ld = b.ld;
   const float wgt = b.grad_chi2[t];
   const int nl = b.ndone[t];
@@ -193,25 +197,17 @@ int fit_adjoint_forward(fit_handle* h, const fit_tracks_in* in, const fit_tracks
   FitArgs a = base_args(in, out, hits, nlayer, h->d_counters);
   float* tp = static_cast<float*>(tape);
   int32_t* ndone = reinterpret_cast<int32_t*>(tp + (size_t)kTapeRow * nlayer * out->ld);
-  int64_t t = 0;
-  int e = 0;
-  while (e < nevt) {
-    const int m = mode[e];
-    int64_t t1 = t;
-    while (e < nevt && mode[e] == m) t1 += ntrk[e++];
-    if (t1 > t) {
-      a.t0 = t;
-      a.t1 = t1;
-      a.geo = h->geo[m];
-      const unsigned nblk = (unsigned)((t1 - t + kAdjBlock - 1) / kAdjBlock);
+  for (int m : {FIT_MODE_R, FIT_MODE_Z}) {  // one launch per mode
+    a.geo = h->geo[m];
+    rc = launch_track_runs(nevt, ntrk, mode, m, "fit_adjoint_forward", [&](int64_t t0, const TrackRuns& r) {
+      a.t0 = t0;
+      const unsigned nblk = (r.n + kAdjBlock - 1) / kAdjBlock;
       if (m == FIT_MODE_Z)
-        fit_tape_kernel<FIT_MODE_Z><<<nblk, kAdjBlock, 0, s>>>(a, tp, ndone);
+        fit_tape_kernel<FIT_MODE_Z><<<nblk, kAdjBlock, 0, s>>>(a, r, tp, ndone);
       else
-        fit_tape_kernel<FIT_MODE_R><<<nblk, kAdjBlock, 0, s>>>(a, tp, ndone);
-      cudaError_t err = cudaGetLastError();
-      if (err != cudaSuccess) return cuda_fail(err, "fit_adjoint_forward: launch");
-    }
-    t = t1;
+        fit_tape_kernel<FIT_MODE_R><<<nblk, kAdjBlock, 0, s>>>(a, r, tp, ndone);
+    });
+    if (rc != FIT_OK) return rc;
   }
   h->tracks += (uint64_t)total;
   return FIT_OK;
@@ -253,25 +249,17 @@ int fit_adjoint_backward(fit_handle* h, const fit_hits* hits, int nevt, const in
   b.g_par0 = grad_par0;
   b.g_cov0 = grad_cov0;
   b.nlayer = nlayer;
-  int64_t t = 0;
-  int e = 0;
-  while (e < nevt) {
-    const int m = mode[e];
-    int64_t t1 = t;
-    while (e < nevt && mode[e] == m) t1 += ntrk[e++];
-    if (t1 > t) {
-      b.t0 = t;
-      b.t1 = t1;
-      b.geo = h->geo[m];
-      const unsigned nblk = (unsigned)((t1 - t + kAdjBlock - 1) / kAdjBlock);
+  for (int m : {FIT_MODE_R, FIT_MODE_Z}) {  // one launch per mode
+    b.geo = h->geo[m];
+    const int rc = launch_track_runs(nevt, ntrk, mode, m, kWho, [&](int64_t t0, const TrackRuns& r) {
+      b.t0 = t0;
+      const unsigned nblk = (r.n + kAdjBlock - 1) / kAdjBlock;
       if (m == FIT_MODE_Z)
-        fit_adjoint_kernel<FIT_MODE_Z><<<nblk, kAdjBlock, 0, s>>>(b);
+        fit_adjoint_kernel<FIT_MODE_Z><<<nblk, kAdjBlock, 0, s>>>(b, r);
       else
-        fit_adjoint_kernel<FIT_MODE_R><<<nblk, kAdjBlock, 0, s>>>(b);
-      cudaError_t err = cudaGetLastError();
-      if (err != cudaSuccess) return cuda_fail(err, std::string(kWho + std::string(": launch")).c_str());
-    }
-    t = t1;
+        fit_adjoint_kernel<FIT_MODE_R><<<nblk, kAdjBlock, 0, s>>>(b, r);
+    });
+    if (rc != FIT_OK) return rc;
   }
   return FIT_OK;
 }

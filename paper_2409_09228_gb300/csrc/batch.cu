@@ -110,20 +110,6 @@ __global__ void relayout_kernel(const uint32_t* __restrict__ src, int64_t src_ld
   }
 }
 
-// Same-mode runs of events, one launch each (the fit_propagate_update path),
-// kept as an autotuner candidate: for few, large events it can win.
-template <int MODE, int L>
-__global__ void __launch_bounds__(kBlock, MODE == FIT_MODE_Z ? 4 : 3)
-    fit_segment_kernel(const __grid_constant__ FitArgs a) {
-  const int64_t t = pair_track(a);
-  if (t >= a.t1) return;
-  unsigned st[2] = {0u, 0u}, iters[2] = {0u, 0u};
-  run_pair<MODE, L>(a, a.geo, a.t0, a.t1, t, st, iters);
-  if (st[0]) count_status(st[0], a.counters);
-  if (st[1]) count_status(st[1], a.counters);
-  if (MODE == FIT_MODE_R) count_iterations(iters[0] + iters[1], &a.counters[4]);
-}
-
 int tracks_per_thread(const fit_launch_config& c) { return c.tracks_per_thread == 1 ? 1 : 2; }
 
 // The batched kernel of a launch shape and its launcher, or NULL for a
@@ -312,36 +298,10 @@ int issue(fit_plan* p, const FitArgs& base, cudaStream_t s) {
     if (e != cudaSuccess) return cuda_fail(e, "fit_plan: launch");
     return FIT_OK;
   }
-  FitArgs a = base;
-  int64_t t = 0;
-  size_t e = 0;
-  const size_t nevt = p->ntrk.size();
-  while (e < nevt) {
-    const int m = p->mode[e];
-    int64_t t1 = t;
-    while (e < nevt && p->mode[e] == m) t1 += p->ntrk[e++];
-    if (t1 > t) {
-      a.t0 = t;
-      a.t1 = t1;
-      a.geo = p->h->geo[m];
-      const int64_t npairs = (t1 - (t & ~int64_t(1)) + 1) / 2;
-      const unsigned nblk = (unsigned)((npairs + kBlock - 1) / kBlock);
-      if (p->cfg.layout == FIT_LAYOUT_AOSOA32) {
-        if (m == FIT_MODE_Z)
-          fit_segment_kernel<FIT_MODE_Z, 1><<<nblk, kBlock, 0, s>>>(a);
-        else
-          fit_segment_kernel<FIT_MODE_R, 1><<<nblk, kBlock, 0, s>>>(a);
-      } else if (m == FIT_MODE_Z) {
-        fit_segment_kernel<FIT_MODE_Z, 0><<<nblk, kBlock, 0, s>>>(a);
-      } else {
-        fit_segment_kernel<FIT_MODE_R, 0><<<nblk, kBlock, 0, s>>>(a);
-      }
-      cudaError_t err = cudaGetLastError();
-      if (err != cudaSuccess) return cuda_fail(err, "fit_plan: launch");
-    }
-    t = t1;
-  }
-  return FIT_OK;
+  // fit_propagate_update's form, one launch per mode: kept as an autotuner
+  // candidate (for few, large events it can win)
+  return run_fit(p->h, base, p->cfg.layout, false, (int)p->ntrk.size(), p->ntrk.data(), p->mode.data(),
+                 "fit_plan", s, s);
 }
 
 void drop_graph(fit_plan* p) {

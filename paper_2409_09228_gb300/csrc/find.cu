@@ -39,7 +39,7 @@ struct FindArgs {
   int64_t ld_cand;
   int8_t* chosen;  // [nlayer][ld_out]
   T gate;
-  int64_t t0, t1;
+  int64_t t0;  // base of the run table
   int nlayer;
   T kB;
   unsigned long long* counters;
@@ -47,9 +47,11 @@ struct FindArgs {
 };
 
 template <int MODE, class T>
-__global__ void __launch_bounds__(kBlock) fit_find_kernel(const __grid_constant__ FindArgs<T> a) {
-  const int64_t t = a.t0 + (int64_t)blockIdx.x * kBlock + threadIdx.x;
-  if (t >= a.t1) return;
+__global__ void __launch_bounds__(kBlock)
+    fit_find_kernel(const __grid_constant__ FindArgs<T> a, const __grid_constant__ TrackRuns r) {
+  const unsigned i = blockIdx.x * kBlock + threadIdx.x;
+  if (i >= r.n) return;
+  const int64_t t = a.t0 + run_element(r, i, 1);
   // The covariance in the fused fit's loop form (fused.cuh, enter_loop_form):
   // p2z c with a zero z row, p2r the local form cl with the null direction
   // (bc, bs).
@@ -176,9 +178,9 @@ __global__ void __launch_bounds__(kBlock) fit_find_kernel(const __grid_constant_
     if (nc) st |= FIT_ST_NOT_CONVERGED;
     propagated = true;
   }
-  for (int r = l; r < a.nlayer; ++r) {  // layers not reached
-    a.chosen[(int64_t)r * a.ld_out + t] = -1;
-    if (a.chi2_layer) a.chi2_layer[(int64_t)r * a.ld_out + t] = T(0.f);
+  for (int k = l; k < a.nlayer; ++k) {  // layers not reached
+    a.chosen[(int64_t)k * a.ld_out + t] = -1;
+    if (a.chi2_layer) a.chi2_layer[(int64_t)k * a.ld_out + t] = T(0.f);
   }
   if (l == 0) {  // nothing applied: the input covariance
 #pragma unroll
@@ -257,27 +259,18 @@ int find_tracks(fit_handle* h, const In* in, const Out* out, const Cand* cand, d
   a.gate = (T)gate;
   a.nlayer = nlayer;
   a.counters = h->d_counters;
-  int64_t t = 0;
-  int e = 0;
-  while (e < nevt) {  // one launch per run of same-mode events
-    const int m = mode[e];
-    int64_t t1 = t;
-    while (e < nevt && mode[e] == m) t1 += ntrk[e++];
-    if (t1 > t) {
-      a.t0 = t;
-      a.t1 = t1;
-      a.geo = h->geo[m];
-      a.kB = sizeof(T) == 8 ? (T)(0.00299792458 * (double)h->B[m]) : (T)h->geo[m].kB;
-      const int64_t nblk = (t1 - t + kBlock - 1) / kBlock;
-      if (nblk > 0x7fffffff) return fail(FIT_ERR_ARG, w + ": too many tracks");
+  for (int m : {FIT_MODE_R, FIT_MODE_Z}) {  // one launch per mode
+    a.geo = h->geo[m];
+    a.kB = sizeof(T) == 8 ? (T)(0.00299792458 * (double)h->B[m]) : (T)h->geo[m].kB;
+    const int rc = launch_track_runs(nevt, ntrk, mode, m, w.c_str(), [&](int64_t t0, const TrackRuns& r) {
+      a.t0 = t0;
+      const unsigned nblk = (r.n + kBlock - 1) / kBlock;
       if (m == FIT_MODE_Z)
-        fit_find_kernel<FIT_MODE_Z, T><<<(unsigned)nblk, kBlock, 0, s>>>(a);
+        fit_find_kernel<FIT_MODE_Z, T><<<nblk, kBlock, 0, s>>>(a, r);
       else
-        fit_find_kernel<FIT_MODE_R, T><<<(unsigned)nblk, kBlock, 0, s>>>(a);
-      cudaError_t err = cudaGetLastError();
-      if (err != cudaSuccess) return cuda_fail(err, (w + ": launch").c_str());
-    }
-    t = t1;
+        fit_find_kernel<FIT_MODE_R, T><<<nblk, kBlock, 0, s>>>(a, r);
+    });
+    if (rc != FIT_OK) return rc;
   }
   h->tracks += (uint64_t)total;
   return FIT_OK;

@@ -29,37 +29,65 @@ int cuda_fail(cudaError_t e, const char* what) {
 
 namespace {
 
+// The thread's track t: its pair's first one, or a lone one.  The first
+// blocks take the lone tracks, so that their one-lane path runs beside the
+// pairs of other blocks (in a pair's warp it would run after them: a range
+// with odd edges took 38 us instead of 22 at 8191 tracks).
+enum class Part { kNone, kPair, kLone };
+template <int K>
+__device__ __forceinline__ Part thread_part(const FitArgs& a, const PairRuns<K>& r, int64_t& t) {
+  const unsigned lone_blocks = (r.nlone + kBlock - 1) / kBlock;
+  if (blockIdx.x < lone_blocks) {
+    const unsigned i = blockIdx.x * kBlock + threadIdx.x;
+    if (i >= r.nlone) return Part::kNone;
+    t = a.t0 + r.lone[i];
+    return Part::kLone;
+  }
+  const unsigned i = (blockIdx.x - lone_blocks) * kBlock + threadIdx.x;
+  if (i >= r.pairs.n) return Part::kNone;
+  t = a.t0 + run_element(r.pairs, i, 2);
+  return Part::kPair;
+}
+
 // 3 resident blocks per SM for p2r (156 registers, no spills; 2 blocks were
 // 17 % slower); p2z fits 4 (128 registers, no spills).
-template <int MODE, int L = 0>
+template <int MODE, int L, int K>
 __global__ void __launch_bounds__(kBlock, MODE == FIT_MODE_Z ? 4 : 3)
-    fit_fused_kernel(const __grid_constant__ FitArgs a) {
-  const int64_t t = pair_track(a);
-  if (t >= a.t1) return;
+    fit_fused_kernel(const __grid_constant__ FitArgs a, const __grid_constant__ PairRuns<K> r) {
+  int64_t t;
+  const Part part = thread_part(a, r, t);
+  if (part == Part::kNone) return;
   unsigned st[2] = {0u, 0u}, iters[2] = {0u, 0u};
-  run_pair<MODE, L, MODE == FIT_MODE_Z && L == 0>(a, a.geo, a.t0, a.t1, t, st, iters);
+  if (part == Part::kPair)
+    run_whole_pair<MODE, L, MODE == FIT_MODE_Z && L == 0>(a, a.geo, t, st, iters);
+  else
+    run_lone<MODE, L>(a, a.geo, t, st[0], iters[0]);
   if (st[0]) count_status(st[0], a.counters);
   if (st[1]) count_status(st[1], a.counters);
   if (MODE == FIT_MODE_R) count_iterations(iters[0] + iters[1], &a.counters[4]);
 }
 
-template <int MODE>
+template <int MODE, int K>
 __global__ void __launch_bounds__(kBlock, MODE == FIT_MODE_Z ? 4 : 3)
-    fit_fused_kernel_noalloc(const __grid_constant__ FitArgs a, const int64_t* __restrict__ evt_off,
-                             int e0, int e1) {
-  const int64_t t = pair_track(a);
-  if (t >= a.t1) return;
+    fit_fused_kernel_noalloc(const __grid_constant__ FitArgs a,
+                             const __grid_constant__ PairRuns<K> r,
+                             const int64_t* __restrict__ evt_off, int nevt) {
+  int64_t t;
+  const Part part = thread_part(a, r, t);
+  if (part == Part::kNone) return;
   unsigned st[2] = {0u, 0u}, iters[2] = {0u, 0u};
-  run_pair<MODE>(a, a.geo, a.t0, a.t1, t, st, iters);
+  if (part == Part::kPair)
+    run_whole_pair<MODE>(a, a.geo, t, st, iters);
+  else
+    run_lone<MODE>(a, a.geo, t, st[0], iters[0]);
 #pragma unroll
   for (int i = 0; i < 2; ++i) {
-    if (t + i < a.t0 || t + i >= a.t1) continue;
-    unsigned long long* cnt = a.counters + (int64_t)event_of(t + i, evt_off, e0, e1) * kEventSlots + 1;
+    if (i == 1 && part == Part::kLone) continue;
+    unsigned long long* cnt = a.counters + (int64_t)event_of(t + i, evt_off, 0, nevt) * kEventSlots + 1;
     if (st[i]) count_status(st[i], cnt);
     if (MODE == FIT_MODE_R && iters[i]) atomicAdd(&cnt[4], (unsigned long long)iters[i]);
   }
 }
-
 
 }  // namespace
 
@@ -146,47 +174,112 @@ FitArgs base_args(const fit_tracks_in* in, const fit_tracks_out* out, const fit_
   return a;
 }
 
-// Runs consecutive events of one mode as one launch each.  launch(a, m, nblk,
-// e0, e1) issues the kernel for tracks [a.t0, a.t1) = events [e0, e1).
+// Adds the tracks [t0, t1) (relative to the launch's even base) to r.
+void add_run(PairRuns<kMaxRuns>& r, uint32_t t0, uint32_t t1) {
+  const uint32_t p0 = (t0 + 1) & ~1u, p1 = t1 & ~1u;
+  if (t0 & 1) r.lone[r.nlone++] = t0;
+  if (p1 > p0) {
+    Runs<kMaxRuns>& p = r.pairs;
+    p.first[p.nrun] = p0;
+    p.before[p.nrun++] = p.n;
+    p.n += (p1 - p0) / 2;
+  }
+  if ((t1 & 1) && t1 > p0) r.lone[r.nlone++] = t1 - 1;
+}
+
+// The events' tracks as one launch per mode: the runs of consecutive
+// same-mode events gathered in a table, with a new launch where it is full
+// or its tracks span 2^31.  launch(a, m, r, nblk) issues the kernel for the
+// runs r of mode m (a.t0: their base; a.geo: the mode's geometry).
+// An uneven mixed batch (500 events, 1M tracks, ~250 runs) takes 0.228 ms in
+// two launches; with one launch per run it took 4.11 ms, a run's few blocks
+// leaving most SMs idle for the ~20 us of its layers.
 template <class Launch>
-int launch_segments(const fit_handle* h, FitArgs a, int nevt, const int64_t* ntrk,
-                    const int32_t* mode, const char* who, Launch launch) {
-  int64_t t = 0;
-  int e = 0;
-  while (e < nevt) {
-    const int m = mode[e];
-    const int e0 = e;
-    int64_t t1 = t;
-    while (e < nevt && mode[e] == m) t1 += ntrk[e++];
-    if (t1 > t) {
-      a.t0 = t;
-      a.t1 = t1;
-      a.geo = h->geo[m];
-      const int64_t npairs = (t1 - (t & ~int64_t(1)) + 1) / 2;  // two tracks per thread
-      const int64_t nblk = (npairs + kBlock - 1) / kBlock;
-      if (nblk > 0x7fffffff) return fail(FIT_ERR_ARG, std::string(who) + ": too many tracks");
-      launch(a, m, (unsigned)nblk, e0, e);
+int launch_runs(const fit_handle* h, FitArgs a, int nevt, const int64_t* ntrk, const int32_t* mode,
+                const char* who, Launch launch) {
+  for (int m : {FIT_MODE_R, FIT_MODE_Z}) {
+    PairRuns<kMaxRuns> r;
+    auto clear = [&r]() { r.pairs.nrun = 0, r.pairs.n = 0, r.nlone = 0; };
+    clear();
+    auto flush = [&]() {
+      const unsigned nblk = (r.nlone + kBlock - 1) / kBlock + (r.pairs.n + kBlock - 1) / kBlock;
+      if (!nblk) return FIT_OK;
+      launch(a, m, r, nblk);
+      clear();
       cudaError_t err = cudaGetLastError();
-      if (err != cudaSuccess) return cuda_fail(err, (std::string(who) + ": launch").c_str());
+      return err == cudaSuccess ? FIT_OK : cuda_fail(err, (std::string(who) + ": launch").c_str());
+    };
+    a.geo = h->geo[m];
+    a.t0 = 0;
+    constexpr int64_t kSpan = int64_t(1) << 31;
+    int64_t t = 0;
+    for (int e = 0; e < nevt;) {
+      if (mode[e] != m) {
+        t += ntrk[e++];
+        continue;
+      }
+      int64_t t1 = t;
+      while (e < nevt && mode[e] == m) t1 += ntrk[e++];
+      while (t < t1) {
+        if (!r.pairs.nrun && !r.nlone) a.t0 = t & ~int64_t(1);
+        const int64_t end = a.t0 + kSpan < t1 ? a.t0 + kSpan : t1;  // (even where it cuts a run)
+        if (r.pairs.nrun == kMaxRuns || r.nlone + 2 > 2 * kMaxRuns || end <= t) {
+          const int rc = flush();
+          if (rc != FIT_OK) return rc;
+          continue;
+        }
+        add_run(r, (uint32_t)(t - a.t0), (uint32_t)(end - a.t0));
+        t = end;
+      }
+      t = t1;
     }
-    t = t1;
+    const int rc = flush();
+    if (rc != FIT_OK) return rc;
   }
   return FIT_OK;
 }
 
-// The fused fit of events [0, nevt) on the tracks of a (a.t0, a.t1 set per
-// run of same-mode events): the p2r runs on stream s, the p2z runs on sz.
-int run_fit(const fit_handle* h, const FitArgs& a, int nevt, const int64_t* ntrk,
-            const int32_t* mode, const char* who, cudaStream_t s, cudaStream_t sz) {
-  return launch_segments(h, a, nevt, ntrk, mode, who,
-                         [s, sz, h](const FitArgs& a1, int m, unsigned nblk, int, int) {
-                           if (m == FIT_MODE_Z)
-                             fit_fused_kernel<FIT_MODE_Z><<<nblk, kBlock, 0, sz>>>(a1);
-                           else if (h->seeded)
-                             launch_seeded_fit(a1, h->d_mlp, s);
-                           else
-                             fit_fused_kernel<FIT_MODE_R><<<nblk, kBlock, 0, s>>>(a1);
-                         });
+// Calls f with r in the smallest compiled table that holds it.
+template <class F>
+void with_table(const PairRuns<kMaxRuns>& r, F f) {
+  if (r.pairs.nrun > 1 || r.nlone > 2) return f(r);
+  PairRuns<1> one;
+  one.pairs.nrun = r.pairs.nrun;
+  one.pairs.n = r.pairs.n;
+  one.pairs.first[0] = r.pairs.nrun ? r.pairs.first[0] : 0;
+  one.pairs.before[0] = 0;
+  one.nlone = r.nlone;
+  for (uint32_t i = 0; i < 2; ++i) one.lone[i] = i < r.nlone ? r.lone[i] : 0;
+  f(one);
+}
+
+template <int MODE, int L>
+void launch_fused(const FitArgs& a, const PairRuns<kMaxRuns>& r, unsigned nblk, cudaStream_t s) {
+  with_table(r, [&](const auto& tab) {
+    constexpr int K = sizeof(tab.lone) / sizeof(tab.lone[0]) / 2;
+    fit_fused_kernel<MODE, L, K><<<nblk, kBlock, 0, s>>>(a, tab);
+  });
+}
+
+// The fused fit of events [0, nevt) on the tracks of a: the p2r events on
+// stream s, the p2z events on sz.
+int run_fit(const fit_handle* h, const FitArgs& a, int layout, bool seeded, int nevt,
+            const int64_t* ntrk, const int32_t* mode, const char* who, cudaStream_t s,
+            cudaStream_t sz) {
+  if (seeded) {
+    const int rc = launch_seeded_fit(h, a, nevt, ntrk, mode, who, s);
+    if (rc != FIT_OK) return rc;
+  }
+  return launch_runs(h, a, nevt, ntrk, mode, who,
+                     [=](const FitArgs& a1, int m, const PairRuns<kMaxRuns>& r, unsigned nblk) {
+                       if (m == FIT_MODE_R && seeded) return;
+                       if (layout == FIT_LAYOUT_SOA)
+                         m == FIT_MODE_Z ? launch_fused<FIT_MODE_Z, 0>(a1, r, nblk, sz)
+                                         : launch_fused<FIT_MODE_R, 0>(a1, r, nblk, s);
+                       else
+                         m == FIT_MODE_Z ? launch_fused<FIT_MODE_Z, 1>(a1, r, nblk, sz)
+                                         : launch_fused<FIT_MODE_R, 1>(a1, r, nblk, s);
+                     });
 }
 
 // Scratch of fit_propagate_update_noalloc, in the library image instead of
@@ -280,7 +373,7 @@ int fit_propagate_update(fit_handle* h, const fit_tracks_in* in, const fit_track
   for (int e = 0; e < nevt; ++e)
     if (ntrk[e] > 0) used[mode[e] == FIT_MODE_Z] = true;
   if (!(used[0] && used[1])) {
-    rc = run_fit(h, a, nevt, ntrk, mode, kWho, s, s);
+    rc = run_fit(h, a, FIT_LAYOUT_SOA, h->seeded, nevt, ntrk, mode, kWho, s, s);
   } else {
     // The two modes' events are independent: the p2z launches go to the
     // handle's second stream, so that they overlap the p2r launches (their
@@ -291,7 +384,7 @@ int fit_propagate_update(fit_handle* h, const fit_tracks_in* in, const fit_track
     cudaError_t e = cudaEventRecord(h->fork, s);
     if (e == cudaSuccess) e = cudaStreamWaitEvent(h->side, h->fork, 0);
     if (e != cudaSuccess) return cuda_fail(e, "fit_propagate_update: fork to the second stream");
-    rc = run_fit(h, a, nevt, ntrk, mode, kWho, s, h->side);
+    rc = run_fit(h, a, FIT_LAYOUT_SOA, h->seeded, nevt, ntrk, mode, kWho, s, h->side);
     e = cudaEventRecord(h->join, h->side);
     if (e == cudaSuccess) e = cudaStreamWaitEvent(s, h->join, 0);
     if (e != cudaSuccess && rc == FIT_OK)
@@ -319,13 +412,8 @@ int fit_propagate_update_layout(fit_handle* h, const fit_tracks_in* in, const fi
   if (h->seeded) return fail(FIT_ERR_ARG, std::string(kWho) + ": no learned seed in AoSoA");
   DeviceGuard g(h->device);
   cudaStream_t s = static_cast<cudaStream_t>(stream);
-  rc = launch_segments(h, base_args(in, out, hits, nlayer, h->d_counters), nevt, ntrk, mode, kWho,
-                       [s](const FitArgs& a, int m, unsigned nblk, int, int) {
-                         if (m == FIT_MODE_Z)
-                           fit_fused_kernel<FIT_MODE_Z, 1><<<nblk, kBlock, 0, s>>>(a);
-                         else
-                           fit_fused_kernel<FIT_MODE_R, 1><<<nblk, kBlock, 0, s>>>(a);
-                       });
+  rc = run_fit(h, base_args(in, out, hits, nlayer, h->d_counters), layout, false, nevt, ntrk, mode,
+               kWho, s, s);
   if (rc != FIT_OK) return rc;
   h->tracks += (uint64_t)total;
   return FIT_OK;
@@ -367,15 +455,15 @@ int fit_propagate_update_noalloc(const fit_config* cfg_r, const fit_config* cfg_
     e = cudaMemcpyAsync(d_off, off, (size_t)(nevt + 1) * sizeof(int64_t), cudaMemcpyHostToDevice, s);
     if (e != cudaSuccess) return cuda_fail(e, "fit_propagate_update_noalloc: offset copy");
     if (total > 0) {
-      rc = launch_segments(&h, base_args(in, out, hits, nlayer, scratch), nevt, ntrk, mode, kWho,
-                           [s, d_off](const FitArgs& a, int m, unsigned nblk, int e0, int e1) {
-                             if (m == FIT_MODE_Z)
-                               fit_fused_kernel_noalloc<FIT_MODE_Z>
-                                   <<<nblk, kBlock, 0, s>>>(a, d_off, e0, e1);
-                             else
-                               fit_fused_kernel_noalloc<FIT_MODE_R>
-                                   <<<nblk, kBlock, 0, s>>>(a, d_off, e0, e1);
-                           });
+      rc = launch_runs(&h, base_args(in, out, hits, nlayer, scratch), nevt, ntrk, mode, kWho,
+                       [=](const FitArgs& a, int m, const PairRuns<kMaxRuns>& r, unsigned nblk) {
+                         if (m == FIT_MODE_Z)
+                           fit_fused_kernel_noalloc<FIT_MODE_Z, kMaxRuns>
+                               <<<nblk, kBlock, 0, s>>>(a, r, d_off, nevt);
+                         else
+                           fit_fused_kernel_noalloc<FIT_MODE_R, kMaxRuns>
+                               <<<nblk, kBlock, 0, s>>>(a, r, d_off, nevt);
+                       });
       if (rc != FIT_OK) return rc;
     }
   }

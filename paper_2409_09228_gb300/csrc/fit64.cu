@@ -31,7 +31,7 @@ struct Args64 {
   const double* hpos;
   const double* hcov;
   int64_t ld_hit;
-  int64_t t0, t1;
+  int64_t t0;  // base of the run table
   int nlayer;
   double kB;  // kA * B in double
   unsigned long long* counters;
@@ -43,9 +43,11 @@ struct Args64 {
 // (fused.cuh, enter_loop_form): p2z with its zero z row, p2r in the
 // cylinder's local coordinates.
 template <int MODE>
-__global__ void __launch_bounds__(kBlock) fit_f64_kernel(const __grid_constant__ Args64 a) {
-  const int64_t t = a.t0 + (int64_t)blockIdx.x * kBlock + threadIdx.x;
-  if (t >= a.t1) return;
+__global__ void __launch_bounds__(kBlock)
+    fit_f64_kernel(const __grid_constant__ Args64 a, const __grid_constant__ TrackRuns r) {
+  const unsigned i = blockIdx.x * kBlock + threadIdx.x;
+  if (i >= r.n) return;
+  const int64_t t = a.t0 + run_element(r, i, 1);
   double p[6], c[21], cl[15], bc = 0.0, bs = 0.0;
 #pragma unroll
   for (int k = 0; k < 6; ++k) fitk::ld(p[k], a.par_in + k * a.ld_in + t);
@@ -187,27 +189,18 @@ extern "C" int fit_propagate_update_f64(fit_handle* h, const fit_tracks_in_f64* 
   a.ld_hit = hits->ld;
   a.nlayer = nlayer;
   a.counters = h->d_counters;
-  int64_t t = 0;
-  int e = 0;
-  while (e < nevt) {  // one launch per run of same-mode events
-    const int m = mode[e];
-    int64_t t1 = t;
-    while (e < nevt && mode[e] == m) t1 += ntrk[e++];
-    if (t1 > t) {
-      a.t0 = t;
-      a.t1 = t1;
-      a.geo = h->geo[m];
-      a.kB = 0.00299792458 * (double)h->B[m];
-      const int64_t nblk = (t1 - t + kBlock - 1) / kBlock;
-      if (nblk > 0x7fffffff) return fail(FIT_ERR_ARG, w + ": too many tracks");
+  for (int m : {FIT_MODE_R, FIT_MODE_Z}) {  // one launch per mode
+    a.geo = h->geo[m];
+    a.kB = 0.00299792458 * (double)h->B[m];
+    const int rc = launch_track_runs(nevt, ntrk, mode, m, w.c_str(), [&](int64_t t0, const TrackRuns& r) {
+      a.t0 = t0;
+      const unsigned nblk = (r.n + kBlock - 1) / kBlock;
       if (m == FIT_MODE_Z)
-        fit_f64_kernel<FIT_MODE_Z><<<(unsigned)nblk, kBlock, 0, s>>>(a);
+        fit_f64_kernel<FIT_MODE_Z><<<nblk, kBlock, 0, s>>>(a, r);
       else
-        fit_f64_kernel<FIT_MODE_R><<<(unsigned)nblk, kBlock, 0, s>>>(a);
-      cudaError_t err = cudaGetLastError();
-      if (err != cudaSuccess) return cuda_fail(err, "fit_propagate_update_f64: launch");
-    }
-    t = t1;
+        fit_f64_kernel<FIT_MODE_R><<<nblk, kBlock, 0, s>>>(a, r);
+    });
+    if (rc != FIT_OK) return rc;
   }
   h->tracks += (uint64_t)total;
   return FIT_OK;

@@ -351,42 +351,69 @@ __device__ __forceinline__ void finish_one(const FitArgs& a, const Geo& geo, int
   iters = it1[0];
 }
 
-// Tracks t and t+1 of the range [t0, t1) (t even).  Both valid: the pair
-// shares packed instructions until a surface that one of them cannot reach
-// (or, for p2r, whose crossing needs the one-lane form of the closed-form
-// start), from where each finishes alone.  One valid (the range starts or ends at an
-// odd index): that one alone.
+// Tracks t and t+1 (t even): the pair shares packed instructions until a
+// surface that one of them cannot reach (or, for p2r, whose crossing needs
+// the one-lane form of the closed-form start), from where each finishes alone.
 template <int MODE, int L = 0, bool STAGE = false>
+__device__ __forceinline__ void run_whole_pair(const FitArgs& a, const Geo& geo, int64_t t,
+                                               unsigned (&st)[2], unsigned (&iters)[2]) {
+  State<F2> s;
+  begin_state<MODE, L>(a, geo, t, s);
+  fitk::M2 alive = {true, true};
+  const int l = run_layers<MODE, F2, L, STAGE>(a, geo, t, 0, s, st, iters, alive);
+  if (l == a.nlayer) {
+    finish_state<MODE, L>(a, t, l, s);
+    store_state<L>(a, t, s, st);
+    return;
+  }
+#pragma unroll 1
+  for (int i = 0; i < 2; ++i) {
+    State<float> one = lane_of<MODE>(s, i);
+    finish_one<MODE, L>(a, geo, t + i, l, one, st[i], iters[i], Lanes<F2>::get(alive, i));
+  }
+}
+
+// Track t alone, from its first layer.
+template <int MODE, int L = 0>
+__device__ __forceinline__ void run_lone(const FitArgs& a, const Geo& geo, int64_t t, unsigned& st,
+                                         unsigned& iters) {
+  State<float> one;
+  begin_state<MODE, L>(a, geo, t, one);
+  finish_one<MODE, L>(a, geo, t, 0, one, st, iters, true);
+}
+
+// Tracks t and t+1 of the range [t0, t1) (t even): the pair, or, where the
+// range starts or ends at an odd index, the valid one alone.
+template <int MODE, int L = 0>
 __device__ __forceinline__ void run_pair(const FitArgs& a, const Geo& geo, int64_t t0, int64_t t1,
                                          int64_t t, unsigned (&st)[2], unsigned (&iters)[2]) {
   const bool v0 = t >= t0, v1 = t + 1 < t1;
   if (v0 && v1) {
-    State<F2> s;
-    begin_state<MODE, L>(a, geo, t, s);
-    fitk::M2 alive = {true, true};
-    const int l = run_layers<MODE, F2, L, STAGE>(a, geo, t, 0, s, st, iters, alive);
-    if (l == a.nlayer) {
-      finish_state<MODE, L>(a, t, l, s);
-      store_state<L>(a, t, s, st);
-      return;
-    }
-#pragma unroll 1
-    for (int i = 0; i < 2; ++i) {
-      State<float> one = lane_of<MODE>(s, i);
-      finish_one<MODE, L>(a, geo, t + i, l, one, st[i], iters[i], Lanes<F2>::get(alive, i));
-    }
+    run_whole_pair<MODE, L>(a, geo, t, st, iters);
   } else {
     const int i = v0 ? 0 : 1;
-    State<float> one;
-    begin_state<MODE, L>(a, geo, t + i, one);
-    finish_one<MODE, L>(a, geo, t + i, 0, one, st[i], iters[i], true);
+    run_lone<MODE, L>(a, geo, t + i, st[i], iters[i]);
   }
 }
 
-// First track of the thread's pair: pairs start at even indices so that the
-// packed loads and stores are 8-byte aligned.
-__device__ __forceinline__ int64_t pair_track(const FitArgs& a) {
-  return (a.t0 & ~int64_t(1)) + 2 * ((int64_t)blockIdx.x * kBlock + threadIdx.x);
+// The run of element i of a run table (internal.h), by binary search: the
+// last one that starts at or before i.
+template <int K>
+__device__ __forceinline__ int64_t run_element(const Runs<K>& r, uint32_t i, uint32_t stride) {
+  int lo = 0;
+  if constexpr (K > 1) {
+    int hi = r.nrun - 1;
+    while (lo < hi) {
+      const int mid = (lo + hi + 1) >> 1;
+      if (r.before[mid] <= i)
+        lo = mid;
+      else
+        hi = mid - 1;
+    }
+  }
+  int64_t t = (int64_t)r.first[lo] + (int64_t)stride * (i - r.before[lo]);
+  asm("" : "+l"(t));  // one 64-bit index: kept as its parts it is re-added for every address
+  return t;
 }
 
 __device__ __forceinline__ void count_iterations(unsigned iters, unsigned long long* counter) {

@@ -49,11 +49,38 @@ struct FitArgs {
   const float* hpos;
   const float* hcov;
   int64_t ld_hit;
-  int64_t t0, t1;  // track range [t0, t1)
+  int64_t t0;  // the track that the launch's run table counts from
   int nlayer;
   unsigned long long* counters;
   Geo geo;
 };
+
+// The tracks of one launch: runs of same-mode events, which other events'
+// tracks separate, as one list of elements (tracks, or pairs of tracks).
+// Element i lies in the run r with the largest before[r] <= i, at track
+// first[r] + stride * (i - before[r]) counted from the launch's FitArgs::t0.
+// The tables travel as kernel parameters: no allocation, no copy to wait for,
+// nothing to keep alive, and a captured launch holds its own.
+template <int K>
+struct Runs {
+  int nrun;
+  uint32_t n;  // elements
+  uint32_t first[K];
+  uint32_t before[K];
+};
+
+// Runs as pairs of tracks (2 k, 2 k + 1) for the packed kernels, and the
+// tracks that a run's odd edges leave without a partner.
+template <int K>
+struct PairRuns {
+  Runs<K> pairs;
+  uint32_t nlone;
+  uint32_t lone[2 * K];
+};
+
+// Capacities compiled: the usual call has one run per mode; a call of uneven
+// mixed events has hundreds.  kMaxRuns pair runs take 16 KiB of parameters.
+constexpr int kMaxRuns = 1024;
 
 inline bool aligned16(const void* p) { return (reinterpret_cast<uintptr_t>(p) & 15u) == 0; }
 
@@ -102,14 +129,61 @@ int check_call(const fit_handle* h, const fit_tracks_in* in, const fit_tracks_ou
 FitArgs base_args(const fit_tracks_in* in, const fit_tracks_out* out, const fit_hits* hits,
                   int nlayer, unsigned long long* counters);
 
-// The p2r fit seeded by the learned path length (mlp.cu), one track per
-// thread over a.t0 .. a.t1; img is the handle's d_mlp.
-void launch_seeded_fit(const FitArgs& a, const void* img, cudaStream_t s);
+// The p2r events of a fit seeded by the learned path length (mlp.cu), one
+// track per thread.
+int launch_seeded_fit(const fit_handle* h, const FitArgs& a, int nevt, const int64_t* ntrk,
+                      const int32_t* mode, const char* who, cudaStream_t s);
 
-// The fused fit of events [0, nevt) (fit.cu): one launch per run of
-// same-mode events, the p2r runs on stream s and the p2z runs on sz.
-int run_fit(const fit_handle* h, const FitArgs& a, int nevt, const int64_t* ntrk,
-            const int32_t* mode, const char* who, cudaStream_t s, cudaStream_t sz);
+// The kernels with one track per thread: the tracks of mode m's events as
+// run tables of up to kTrackRuns runs (1 KiB of parameters, which costs a
+// launch nothing measurable), launch(base, r) for each; returns FIT_OK or the
+// first launch's error.
+constexpr int kTrackRuns = 128;
+using TrackRuns = Runs<kTrackRuns>;
+
+template <class Launch>
+int launch_track_runs(int nevt, const int64_t* ntrk, const int32_t* mode, int m, const char* who,
+                      Launch launch) {
+  TrackRuns r;
+  r.nrun = 0, r.n = 0;
+  int64_t base = 0, t = 0;
+  auto flush = [&]() {
+    if (!r.n) return FIT_OK;
+    launch(base, r);
+    r.nrun = 0, r.n = 0;
+    const cudaError_t e = cudaGetLastError();
+    return e == cudaSuccess ? FIT_OK : cuda_fail(e, (std::string(who) + ": launch").c_str());
+  };
+  constexpr int64_t kSpan = int64_t(1) << 31;
+  for (int e = 0; e < nevt; ++e) {
+    int64_t t1 = t + ntrk[e];
+    if (mode[e] == m) {
+      while (e + 1 < nevt && mode[e + 1] == m) t1 += ntrk[++e];
+      while (t < t1) {
+        if (!r.nrun) base = t;
+        const int64_t end = base + kSpan < t1 ? base + kSpan : t1;
+        if (r.nrun == kTrackRuns || end <= t) {
+          const int rc = flush();
+          if (rc != FIT_OK) return rc;
+          continue;
+        }
+        r.first[r.nrun] = (uint32_t)(t - base);
+        r.before[r.nrun++] = r.n;
+        r.n += (uint32_t)(end - t);
+        t = end;
+      }
+    }
+    t = t1;
+  }
+  return flush();
+}
+
+// The fused fit of events [0, nevt) (fit.cu) in the given layout: the p2r
+// events in one launch on stream s (kMaxRuns runs each), the p2z events in
+// one on sz.  seeded: the p2r events start from the handle's learned seed.
+int run_fit(const fit_handle* h, const FitArgs& a, int layout, bool seeded, int nevt,
+            const int64_t* ntrk, const int32_t* mode, const char* who, cudaStream_t s,
+            cudaStream_t sz);
 
 // Frees the staging of fit_propagate_update_host (host.cu).
 void destroy_host_stage(fit_handle* h);

@@ -474,14 +474,16 @@ __global__ void __launch_bounds__(kBlock)
 // the layer loop early; a track that stops (surface not reached, non-finite
 // update) only stops moving.  Outputs, status bits and counters as
 // fit_fused_kernel<FIT_MODE_R>.
-__global__ void __launch_bounds__(kBlock) fit_seeded_kernel(const __grid_constant__ FitArgs a,
-                                                            const Image* __restrict__ img) {
+__global__ void __launch_bounds__(kBlock)
+    fit_seeded_kernel(const __grid_constant__ FitArgs a, const __grid_constant__ TrackRuns runs,
+                      const Image* __restrict__ img) {
   __shared__ Image W;
   __shared__ uint4 stage[kBlock / 32][64];
   mlpk::copy_image(W, img);
   __syncthreads();
-  const int64_t t = a.t0 + (int64_t)blockIdx.x * kBlock + threadIdx.x;
-  const bool valid = t < a.t1;
+  const unsigned i = blockIdx.x * kBlock + threadIdx.x;
+  const bool valid = i < runs.n;
+  const int64_t t = valid ? a.t0 + run_element(runs, i, 1) : 0;
   State<float> s;
   if (valid) {
     load_state(a, t, s);
@@ -603,9 +605,15 @@ int launch_adam(fit_mlp* m, const float* grad, int nblk, float lr, float* curve,
 
 namespace fitimpl {
 
-void launch_seeded_fit(const FitArgs& a, const void* img, cudaStream_t s) {
-  const int64_t nblk = (a.t1 - a.t0 + kBlock - 1) / kBlock;
-  fit_seeded_kernel<<<(unsigned)nblk, kBlock, 0, s>>>(a, static_cast<const Image*>(img));
+int launch_seeded_fit(const fit_handle* h, const FitArgs& args, int nevt, const int64_t* ntrk,
+                      const int32_t* mode, const char* who, cudaStream_t s) {
+  FitArgs a = args;
+  a.geo = h->geo[FIT_MODE_R];
+  return launch_track_runs(nevt, ntrk, mode, FIT_MODE_R, who, [&](int64_t t0, const TrackRuns& r) {
+    a.t0 = t0;
+    fit_seeded_kernel<<<(r.n + kBlock - 1) / kBlock, kBlock, 0, s>>>(
+        a, r, static_cast<const Image*>(h->d_mlp));
+  });
 }
 
 size_t mlp_image_bytes() { return sizeof(Image); }

@@ -1,0 +1,148 @@
+"""A call's events gathered into one launch per mode (the run tables): more
+runs of same-mode events than one table holds, runs that begin and end at odd
+tracks, runs of a single track, empty events."""
+import numpy as np
+import pytest
+
+import oracle
+import parity
+from paper_2409_09228_gb300 import fit, inputs
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+if not torch.cuda.is_available():  # pragma: no cover - collected on CPU hosts too
+    pytest.skip("needs a CUDA device", allow_module_level=True)
+
+import gpu_util  # noqa: E402
+
+NLAYER = 20
+
+
+def _events(nevt, seed=61):
+    """nevt events, modes alternating, 0..5 tracks each (the first one odd)."""
+    nt = np.array([1, 2, 3, 1, 5, 0, 4, 1, 1, 2, 0])[np.arange(nevt) % 11]
+    return inputs.generate_events(nt, np.arange(nevt) % 2, seed=seed, nlayer=NLAYER)
+
+
+def _device(ev, ld, dtype=None):
+    d = [gpu_util.to_dev(a, ld) for a in (ev.par0, ev.cov0, ev.q, ev.hpos, ev.hcov)]
+    return d if dtype is None else [a.to(dtype) if k != 2 else a for k, a in enumerate(d)]
+
+
+def _fitter(ev):
+    return fit.Fitter(fit.Geometry(ev.B, ev.surf[0]), fit.Geometry(ev.B, ev.surf[1]))
+
+
+def _of_mode(ev, m):
+    return np.nonzero(np.repeat(ev.mode, ev.ntrk) == m)[0]
+
+
+def _check(ev, got, label):
+    for m in (0, 1):
+        idx = _of_mode(ev, m)
+        if not len(idx):
+            continue
+        ts = inputs.TrackSet(m, ev.B, ev.surf[m], *(np.ascontiguousarray(a[..., idx]) for a in
+                                                    (ev.par0, ev.cov0, ev.q, ev.hpos, ev.hcov)))
+        parity.check({k: v[..., idx] for k, v in got.items()}, oracle.fit_set(ts), f"{label} mode {m}")
+
+
+# 7 runs: every mode in one small table; 2303: two full tables of 1024 a mode
+@pytest.mark.parametrize("nevt", [1, 7, 2303])
+@pytest.mark.parametrize("entry", ["fit", "aosoa", "noalloc", "plan"])
+def test_pair_kernels_many_runs(entry, nevt):
+    ev = _events(nevt)
+    ld = (ev.n + 31) // 32 * 32
+    d = _device(ev, ld)
+    f = _fitter(ev)
+    out = f.outputs(ev.n, ld=ld)
+    for k in ("par", "cov", "chi2"):
+        out[k].fill_(float("nan"))
+    bufs = dict(par_out=out["par"], cov_out=out["cov"], q_out=out["q"], chi2=out["chi2"],
+                status=out["status"])
+    if entry == "fit":
+        f.run(*d, ev.ntrk, ev.mode, out=out)
+    elif entry == "plan":
+        plan = fit.fit_plan_create(f.h, ev.ntrk, ev.mode, NLAYER, persistent=False)
+        fit.fit_plan_run(plan, *d, **bufs)
+        torch.cuda.synchronize()
+        fit.fit_plan_destroy(plan)
+    elif entry == "noalloc":
+        geo = [fit.Geometry(ev.B, s) for s in ev.surf]
+        per_event = fit.fit_propagate_update_noalloc(geo[0], geo[1], *d, ev.ntrk, ev.mode, **bufs)
+        for c, n, m in zip(per_event, ev.ntrk, ev.mode):  # one step a layer, seldom two
+            assert n * NLAYER * (m == 0) <= c["iterations"] <= 2 * n * NLAYER * (m == 0)
+        assert [c["tracks"] for c in per_event] == [int(n) for n in ev.ntrk]
+    else:
+        tiles = [a if k == 2 else torch.from_numpy(inputs.to_aosoa32(a.cpu().numpy(), ld)).cuda()
+                 for k, a in enumerate(d)]
+        fit.fit_propagate_update_layout(f.h, *tiles, ev.ntrk, ev.mode, fit.FIT_LAYOUT_AOSOA32, ld,
+                                        out["par"], out["cov"], out["q"], out["chi2"],
+                                        status=out["status"])
+    if entry != "noalloc":
+        assert f.sync()["tracks"] == ev.n
+    got = {k: out[k].cpu().numpy() for k in ("par", "cov", "chi2", "q", "status")}
+    if entry == "aosoa":
+        for k in ("par", "cov"):
+            got[k] = inputs.from_aosoa32(got[k].reshape(-1), got[k].shape, ev.n)
+    f.close()
+    _check(ev, {k: v[..., :ev.n] for k, v in got.items()}, entry)
+
+
+# 303 runs: two tables of 128 a mode.  The kernels with one track per thread
+# treat every track alone, so their results in event order are bit for bit
+# those of the same tracks sorted by mode (two runs).
+@pytest.mark.parametrize("entry", ["f64", "find", "find64", "adjoint", "seeded"])
+def test_track_kernels_many_runs(entry):
+    ev = _events(303)
+    n, ld = ev.n, (ev.n + 3) // 4 * 4
+    order = np.concatenate([_of_mode(ev, 0), _of_mode(ev, 1)])
+    counts = [len(_of_mode(ev, 0)), len(_of_mode(ev, 1))]
+    f = _fitter(ev)
+    if entry == "seeded":
+        m = fit.fit_mlp_create(0, seed=3)
+        fit.fit_mlp_attach(f.h, m)
+        torch.cuda.synchronize()
+        fit.fit_mlp_destroy(m)
+    dtype = torch.float64 if entry in ("f64", "find64") else torch.float32
+
+    def run(nt, md, idx):
+        par, cov, q, hpos, hcov = _device(ev, ld, dtype)
+        if idx is not None:
+            par, cov, q, hpos, hcov = (gpu_util.to_dev(a.cpu().numpy()[..., idx], ld)
+                                       for a in (par, cov, q, hpos, hcov))
+        out = f.outputs(n, ld=ld)
+        o = {k: v.to(dtype) if v is not None and v.is_floating_point() else v for k, v in out.items()}
+        args = (o["par"], o["cov"], o["q"], o["chi2"])
+        res = [o["par"], o["cov"], o["q"], o["chi2"], o["status"]]
+        if entry == "f64":
+            fit.fit_propagate_update_f64(f.h, par, cov, q, hpos, hcov, nt, md, *args,
+                                         status=o["status"])
+        elif entry == "seeded":
+            f.run(par, cov, q, hpos, hcov, nt, md, out=o)
+        elif entry == "adjoint":
+            tape = torch.empty(fit.fit_tape_bytes(NLAYER, ld) // 4, device="cuda")
+            g = [torch.empty((NLAYER, 3, ld), device="cuda"), torch.empty((6, ld), device="cuda"),
+                 torch.empty((21, ld), device="cuda")]
+            fit.fit_adjoint_forward(f.h, par, cov, q, hpos, hcov, nt, md, tape, *args,
+                                    status=o["status"])
+            fit.fit_adjoint_backward(f.h, hpos, hcov, nt, md, tape, torch.ones(ld, device="cuda"), *g)
+            res += g
+        else:
+            chosen = torch.empty((NLAYER, ld), dtype=torch.int8, device="cuda")
+            fit.fit_find_tracks(f.h, par, cov, q, hpos[:, None].contiguous(),
+                                hcov[:, None].contiguous(), nt, md, 30.0, chosen, *args,
+                                status=o["status"])
+            res.append(chosen)
+        torch.cuda.synchronize()
+        assert f.sync()["tracks"] == n
+        return [r.cpu().numpy()[..., :n] for r in res]
+
+    got = run(ev.ntrk, ev.mode, None)
+    ref = run(counts, [0, 1], order)
+    f.close()
+    # the seeded handle's p2z tracks run in pairs, which the order changes
+    keep = slice(0, counts[0]) if entry == "seeded" else slice(0, n)
+    for a, b in zip(got, ref):
+        np.testing.assert_array_equal(a[..., order][..., keep], b[..., keep])
