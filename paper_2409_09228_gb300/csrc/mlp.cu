@@ -4,6 +4,7 @@
 // layer's iteration from the network.
 #include <cuda_runtime.h>
 
+#include <algorithm>
 #include <cmath>
 #include <cstdint>
 #include <string>
@@ -28,6 +29,7 @@ struct fit_mlp {
   int64_t partial_blocks = 0;
   float* d_curve = nullptr;  // loss per epoch
   int curve_cap = 0;
+  unsigned* d_sync = nullptr;  // the training kernel's grid barrier and error flag
   int64_t step = 0;  // Adam steps taken
   float beta1 = 0.9f, beta2 = 0.999f, eps = 1e-8f;
 };
@@ -149,7 +151,7 @@ struct GradSmem {
   uint4 dz2[kRows][8];
   uint4 a1[kRows][8];
   uint4 dz1[kRows][8];
-  float red[3 * 64 + 3];  // db1, db2, dW3, db3, sum of squared errors, count
+  float red[kBlock / 32][3 * 64 + 3];  // per warp: db1, db2, dW3, db3, squared errors, count
 };
 
 __device__ __forceinline__ uint32_t* swz(uint4 (*m)[8], int row, int chunk) {
@@ -174,28 +176,48 @@ __device__ __forceinline__ float sum_over_g(float v) {
   return v;
 }
 
-// Block b takes samples (off + 64 b + r) mod n, r < 64, of the first cnt of
-// the batch; each of the four warps a 16-sample tile.  Writes the block's
-// partial gradient of (1/cnt) sum (y - t)^2, its sum of squared errors and
-// its count of finite targets to partials[b].
-__global__ void __launch_bounds__(kBlock) mlp_grad_kernel(const TrainImage* __restrict__ img,
-                                                          const float* __restrict__ X,
-                                                          const float* __restrict__ T, int64_t n,
-                                                          int64_t off, int64_t cnt, float inv_cnt,
-                                                          float* __restrict__ partials) {
+// One sample's inputs and, for the lanes that need them, two targets.
+struct Sample {
+  float4 lo, hi;
+  float t0, t1;  // rows r0 and r0 + 8 (lanes with c = 0); NaN beyond the batch
+};
+
+// Loads what the thread needs of tile b: samples (off + 64 b + r) mod n,
+// r < 64, of the first cnt of the batch (off < n, cnt <= n).
+__device__ __forceinline__ Sample load_sample(const float* __restrict__ X,
+                                              const float* __restrict__ T, int64_t n, int64_t off,
+                                              int64_t cnt, int64_t b) {
+  const int tid = threadIdx.x, r0 = (tid >> 5) * 16 + ((tid & 31) >> 2);
+  const int64_t base = b * kRows;
+  auto at = [&](int r) {
+    const int64_t i = off + base + r;
+    return i < n ? i : i - n;
+  };
+  Sample s;
+  s.lo = s.hi = make_float4(0.f, 0.f, 0.f, 0.f);
+  s.t0 = s.t1 = __int_as_float(0x7fc00000);
+  if (tid < kRows && base + tid < cnt) {
+    const float4* xi = reinterpret_cast<const float4*>(X + at(tid) * mlpk::kIn);
+    s.lo = __ldg(xi), s.hi = __ldg(xi + 1);
+  }
+  if ((tid & 3) == 0) {
+    if (base + r0 < cnt) s.t0 = __ldg(T + at(r0));
+    if (base + r0 + 8 < cnt) s.t1 = __ldg(T + at(r0 + 8));
+  }
+  return s;
+}
+
+// The partial gradient of (1/cnt) sum (y - t)^2 over one tile of 64 samples
+// (each of the four warps a 16-sample tile), its sum of squared errors and
+// its count of finite targets, written to P[kPartial].  The whole block
+// calls it, with the image in S.W.
+__device__ __forceinline__ void grad_tile(GradSmem& S, const Sample& smp, float inv_cnt,
+                                          float* __restrict__ P) {
   using namespace mlpk;
-  __shared__ GradSmem S;
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, g = lane >> 2, c = lane & 3;
-  copy_image(S.W, img);
-  for (int i = tid; i < 3 * 64 + 3; i += kBlock) S.red[i] = 0.f;
-  const int64_t base = (int64_t)blockIdx.x * kRows;
   if (tid < kRows) {
-    float f[kIn] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
-    if (base + tid < cnt) {
-      const float4* xi = reinterpret_cast<const float4*>(X + ((off + base + tid) % n) * kIn);
-      const float4 u = __ldg(xi), v = __ldg(xi + 1);
-      f[0] = u.x, f[1] = u.y, f[2] = u.z, f[3] = u.w, f[4] = v.x, f[5] = v.y, f[6] = v.z, f[7] = v.w;
-    }
+    const float f[kIn] = {smp.lo.x, smp.lo.y, smp.lo.z, smp.lo.w,
+                          smp.hi.x, smp.hi.y, smp.hi.z, smp.hi.w};
     stage_inputs(f, &S.xs[0][tid], &S.xs[1][tid]);
   }
   __syncthreads();
@@ -220,15 +242,8 @@ __global__ void __launch_bounds__(kBlock) mlp_grad_kernel(const TrainImage* __re
   // output error (lanes c = 0 hold rows r0 and r0 + 8), broadcast over the quad
   float e0 = 0.f, e1 = 0.f, nval = 0.f;
   if (c == 0) {
-    const int64_t b0 = base + r0, b1 = base + r0 + 8;
-    if (b0 < cnt) {
-      const float t = __ldg(T + (off + b0) % n);
-      if (isfinite(t)) e0 = o[0] - t, nval += 1.f;
-    }
-    if (b1 < cnt) {
-      const float t = __ldg(T + (off + b1) % n);
-      if (isfinite(t)) e1 = o[2] - t, nval += 1.f;
-    }
+    if (isfinite(smp.t0)) e0 = o[0] - smp.t0, nval += 1.f;
+    if (isfinite(smp.t1)) e1 = o[2] - smp.t1, nval += 1.f;
   }
   float sse = e0 * e0 + e1 * e1;
   const float dy0 = __shfl_sync(0xffffffffu, 2.f * e0 * inv_cnt, lane & ~3);
@@ -298,9 +313,9 @@ __global__ void __launch_bounds__(kBlock) mlp_grad_kernel(const TrainImage* __re
       const float v1 = sum_over_g(gb1[nb][e]), v2 = sum_over_g(gb2[nb][e]),
                   v3 = sum_over_g(gw3[nb][e]);
       if (g == 0) {
-        atomicAdd(&S.red[nb * 8 + 2 * c + e], v1);
-        atomicAdd(&S.red[64 + nb * 8 + 2 * c + e], v2);
-        atomicAdd(&S.red[128 + nb * 8 + 2 * c + e], v3);
+        S.red[warp][nb * 8 + 2 * c + e] = v1;
+        S.red[warp][64 + nb * 8 + 2 * c + e] = v2;
+        S.red[warp][128 + nb * 8 + 2 * c + e] = v3;
       }
     }
   }
@@ -311,9 +326,9 @@ __global__ void __launch_bounds__(kBlock) mlp_grad_kernel(const TrainImage* __re
     nval += __shfl_xor_sync(0xffffffffu, nval, m);
   }
   if (lane == 0) {
-    atomicAdd(&S.red[192], db3);
-    atomicAdd(&S.red[193], sse);
-    atomicAdd(&S.red[194], nval);
+    S.red[warp][192] = db3;
+    S.red[warp][193] = sse;
+    S.red[warp][194] = nval;
   }
   __syncthreads();
 
@@ -346,7 +361,6 @@ __global__ void __launch_bounds__(kBlock) mlp_grad_kernel(const TrainImage* __re
     mma_acc(gw1[1], A1, Bx[2], Bx[3]);
   }
 
-  float* P = partials + (int64_t)blockIdx.x * kPartial;
   const int j0 = warp * 16 + g;
 #pragma unroll
   for (int nb = 0; nb < 8; ++nb) {
@@ -359,16 +373,27 @@ __global__ void __launch_bounds__(kBlock) mlp_grad_kernel(const TrainImage* __re
   P[kOffW1 + j0 * 8 + 2 * c + 1] = gw1[0][1] + gw1[1][1];
   P[kOffW1 + (j0 + 8) * 8 + 2 * c] = gw1[0][2] + gw1[1][2];
   P[kOffW1 + (j0 + 8) * 8 + 2 * c + 1] = gw1[0][3] + gw1[1][3];
-  for (int i = tid; i < 64; i += kBlock) {
-    P[kOffB1 + i] = S.red[i];
-    P[kOffB2 + i] = S.red[64 + i];
-    P[kOffW3 + i] = S.red[128 + i];
+  // the warps' sums in a fixed order
+  for (int i = tid; i < 3 * 64 + 3; i += kBlock) {
+    float v = S.red[0][i];
+#pragma unroll
+    for (int w = 1; w < kBlock / 32; ++w) v += S.red[w][i];
+    const int at = i < 64 ? kOffB1 + i : i < 128 ? kOffB2 + i - 64 : i < 192 ? kOffW3 + i - 128
+                 : i == 192 ? kOffB3 : i == 193 ? kSse : kCount;
+    P[at] = v;
   }
-  if (tid == 0) {
-    P[kOffB3] = S.red[192];
-    P[kSse] = S.red[193];
-    P[kCount] = S.red[194];
-  }
+}
+
+// Block b: the partial gradient of tile b of the batch.
+__global__ void __launch_bounds__(kBlock) mlp_grad_kernel(const TrainImage* __restrict__ img,
+                                                          const float* __restrict__ X,
+                                                          const float* __restrict__ T, int64_t n,
+                                                          int64_t off, int64_t cnt, float inv_cnt,
+                                                          float* __restrict__ partials) {
+  __shared__ GradSmem S;
+  mlpk::copy_image(S.W, img);
+  const Sample smp = load_sample(X, T, n, off, cnt, blockIdx.x);
+  grad_tile(S, smp, inv_cnt, partials + (int64_t)blockIdx.x * kPartial);
 }
 
 // Sum of the per-block partials (fixed order): gradient and mean loss.
@@ -388,39 +413,205 @@ __global__ void __launch_bounds__(256)
   }
 }
 
-// One Adam step (Kingma and Ba, 2015, Algorithm 1) with the gradient grad, or
-// the sum of nblk partials when grad is NULL; bc1 = 1 - beta1^t and
-// bc2 = 1 - beta2^t; one parameter per thread over the grid.  Block 0 adds
-// curve_scale times the partials' squared errors to *curve.  The BF16 image
-// is rebuilt from the new parameters by mlp_image_kernel afterwards.
-constexpr int kAdamThreads = 256;
+// ---- Adam ------------------------------------------------------------------------
+
+// Thread u < kParams owns one parameter.  Four consecutive threads own a 2x2
+// block of W2 (the image packs pairs along both of its directions), the
+// others follow in the parameter vector's order; a pair that shares a word
+// of the image always sits in neighbouring lanes.
+__device__ __forceinline__ int owned_param(int u) {
+  using namespace mlpk;
+  if (u < kHid * kHid) {
+    const int q = u >> 2, e = u & 3;
+    return kOffW2 + (2 * (q >> 5) + (e >> 1)) * kHid + 2 * (q & 31) + (e & 1);
+  }
+  const int v = u - kHid * kHid;  // W1 and b1, then b2, W3 and b3
+  return v < kOffW2 ? v : kOffB2 + (v - kOffW2);
+}
+
+// Writes the image's words of thread u's parameter, whose value is p (the
+// inverse of build_image's indexing).  Whole warps call it; u >= kParams has
+// no parameter.
+__device__ __forceinline__ void write_image(TrainImage* img, int u, float p) {
+  using namespace mlpk;
+  const float right = __shfl_xor_sync(0xffffffffu, p, 1);  // the next column (or row of W3)
+  const float below = __shfl_xor_sync(0xffffffffu, p, 2);  // the next row of W2
+  // word of columns k, k + 1 (k even) of row n in the order of w2 and w2t
+  auto w2_word = [](int n, int k) {
+    const int nb = n >> 3, lane = (n & 7) * 4 + ((k & 7) >> 1);
+    return (((k >> 4) * 4 + (nb >> 1)) * 32 + lane) * 4 + ((nb & 1) << 1) + ((k >> 3) & 1);
+  };
+  if (u < kHid * kHid) {
+    const int i = owned_param(u) - kOffW2, n = i / kHid, k = i % kHid;
+    if (!(u & 1)) (&img->fwd.w2[0][0][0].x)[w2_word(n, k)] = pack_bf16(p, right);
+    if (!(u & 2)) (&img->w2t[0][0][0].x)[w2_word(k, n)] = pack_bf16(p, below);
+  } else if (u < kParams) {
+    const int i = owned_param(u);
+    if (i < kOffB1) {
+      const int n = i / kIn, nb = n >> 3, lane = (n & 7) * 4 + ((i & 7) >> 1);
+      if (!(i & 1)) (&img->fwd.w1[0][0].x)[((nb >> 2) * 32 + lane) * 4 + (nb & 3)] = pack_bf16(p, right);
+    } else if (i < kOffW2) {
+      img->fwd.b1[i - kOffB1] = p;
+    } else if (i < kOffW3) {
+      img->fwd.b2[i - kOffB2] = p;
+    } else if (i < kOffB3) {
+      const int k = i - kOffW3;
+      img->w3f[k] = bf16_round(p);
+      if (!(k & 1))
+        (&img->fwd.w3[0][0].x)[((k >> 5) * 32 + ((k & 7) >> 1)) * 4 + (((k >> 4) & 1) << 1) +
+                               ((k >> 3) & 1)] = pack_bf16(p, right);
+    } else {
+      img->fwd.b3 = p;
+    }
+  }
+}
+
+// What one Adam step needs beside the gradient: bc1 = 1 - beta1^t and
+// bc2 = 1 - beta2^t.
+struct AdamRate {
+  float lr, bc1, bc2;
+};
+struct AdamBetas {
+  float beta1, beta2, eps;
+};
+
+// One Adam step of one parameter (Kingma and Ba, 2015, Algorithm 1).
+__device__ __forceinline__ void adam(float& p, float& m, float& v, float gi, AdamRate r,
+                                     AdamBetas b) {
+  m = fmaf(b.beta1, m, (1.f - b.beta1) * gi);
+  v = fmaf(b.beta2, v, (1.f - b.beta2) * gi * gi);
+  p -= r.lr * (m / r.bc1) / (sqrtf(v / r.bc2) + b.eps);
+}
+
+// Sum of entry i of the nblk partials, in order (the partials are the same
+// kernel's in training: __ldcg, past the L1).
+__device__ __forceinline__ float sum_partials(const float* partials, int nblk, int i) {
+  float s = 0.f;
+#pragma unroll 32
+  for (int b = 0; b < nblk; ++b) s += __ldcg(partials + (int64_t)b * kPartial + i);
+  return s;
+}
+
+// One Adam step with the gradient grad, or the sum of nblk partials when grad
+// is NULL, and the image's words of the new parameters.  Block 0 adds
+// curve_scale times the partials' squared errors to *curve.
+constexpr int kAdamThreads = 128;
 constexpr int kAdamBlocks = (mlpk::kParams + kAdamThreads - 1) / kAdamThreads;
 
 __global__ void __launch_bounds__(kAdamThreads)
     mlp_adam_kernel(float* __restrict__ P, float* __restrict__ M, float* __restrict__ V,
-                    const float* __restrict__ grad, const float* __restrict__ partials, int nblk,
-                    float lr, float beta1, float beta2, float eps, float bc1, float bc2,
+                    TrainImage* img, const float* __restrict__ grad,
+                    const float* __restrict__ partials, int nblk, AdamRate rate, AdamBetas betas,
                     float* curve, float curve_scale) {
-  const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i < mlpk::kParams) {
-    float gi;
-    if (grad) {
-      gi = grad[i];
-    } else {
-      gi = 0.f;
-      for (int b = 0; b < nblk; ++b) gi += partials[(int64_t)b * kPartial + i];
+  const int u = blockIdx.x * kAdamThreads + threadIdx.x;
+  float p = 0.f;
+  if (u < mlpk::kParams) {
+    const int i = owned_param(u);
+    p = P[i];
+    float m = M[i], v = V[i];
+    adam(p, m, v, grad ? grad[i] : sum_partials(partials, nblk, i), rate, betas);
+    P[i] = p, M[i] = m, V[i] = v;
+  }
+  write_image(img, u, p);
+  if (curve && u == 0) *curve += sum_partials(partials, nblk, kSse) * curve_scale;
+}
+
+// ---- training: many steps in one launch --------------------------------------------
+
+// The steps of one launch, as kernel parameters.
+constexpr int kTrainSteps = 512;
+struct TrainSteps {
+  int count, first_epoch;
+  int steps_per_epoch, first_step;  // place of the launch's first step in its epoch
+  AdamRate rate[kTrainSteps];
+  int64_t off[kTrainSteps];  // first sample of the step's batch
+};
+
+// How often a block looks at the grid barrier before it gives up (seconds;
+// a step takes microseconds).
+constexpr unsigned kBarrierLooks = 1u << 22;
+
+// Barrier over the grid (cooperative launch): sync[0] counts arrivals, round
+// is the barrier's number from 1.  Returns true if a block gave up waiting,
+// which sync[1] then tells the others and the host.
+__device__ __forceinline__ bool grid_barrier(unsigned* sync, unsigned round) {
+  bool gave_up = false;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    __threadfence();
+    asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(sync) : "memory");
+    const unsigned target = round * gridDim.x;
+    for (unsigned looks = 0;; ++looks) {
+      unsigned seen;
+      asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(seen) : "l"(sync) : "memory");
+      if (seen >= target) break;
+      if (looks >= kBarrierLooks) {
+        atomicExch(sync + 1, 1u);
+        gave_up = true;
+        break;
+      }
     }
-    const float m = fmaf(beta1, M[i], (1.f - beta1) * gi);
-    const float v = fmaf(beta2, V[i], (1.f - beta2) * gi * gi);
-    M[i] = m;
-    V[i] = v;
-    P[i] -= lr * (m / bc1) / (sqrtf(v / bc2) + eps);
+    __threadfence();
   }
-  if (curve && i == 0) {
-    float s = 0.f;
-    for (int b = 0; b < nblk; ++b) s += partials[(int64_t)b * kPartial + kSse];
-    *curve += s * curve_scale;
+  return __syncthreads_or(gave_up);
+}
+
+// Adam steps back to back: in every step the blocks form the partial
+// gradients of the batch's tiles, meet, sum them for the one parameter each
+// thread owns (held with its moments in registers across the steps), apply
+// the step and write the BF16 image's words, meet again and reload the image.
+// The same sums in the same order as mlp_grad_kernel and mlp_adam_kernel.
+// A step is a chain of latencies, not of work (0.1 GFLOP, 1.2 MB of partials
+// in the L2), so what counts is the number of launches and meetings: a batch
+// of 4096 takes TIME_NOW us a step, with three launches (gradient, Adam on 19
+// blocks, image on one) it took 23.5.  The next step's samples are loaded
+// before the barrier, whose wait hides them.
+__global__ void __launch_bounds__(kBlock)
+    mlp_train_kernel(const __grid_constant__ TrainSteps steps, TrainImage* img,
+                     const float* __restrict__ X, const float* __restrict__ T, int64_t n,
+                     int batch, float inv_cnt, float* partials, float* P, float* M, float* V,
+                     AdamBetas betas, float* curve, float curve_scale, unsigned* sync) {
+  __shared__ GradSmem S;
+  const int nblk = (batch + kRows - 1) / kRows;
+  const int u = blockIdx.x * kBlock + threadIdx.x;
+  const int own = u < mlpk::kParams ? owned_param(u) : u == mlpk::kParams ? kSse : -1;
+  float p = 0.f, m = 0.f, v = 0.f;
+  if (u < mlpk::kParams) p = P[own], m = M[own], v = V[own];
+  int epoch = steps.first_epoch, in_epoch = steps.first_step;
+  float loss = u == mlpk::kParams ? curve[epoch] : 0.f;
+  Sample smp;
+  if ((int)blockIdx.x < nblk) smp = load_sample(X, T, n, steps.off[0], batch, blockIdx.x);
+  unsigned round = 0;
+  for (int k = 0; k < steps.count; ++k) {
+    if ((int)blockIdx.x < nblk) {
+      const uint4* src = reinterpret_cast<const uint4*>(img);
+      uint4* dst = reinterpret_cast<uint4*>(&S.W);
+      constexpr int kWords = sizeof(TrainImage) / 16;
+      for (int i = threadIdx.x; i < kWords; i += kBlock) dst[i] = __ldcg(src + i);
+      for (int b = blockIdx.x; b < nblk; b += gridDim.x) {
+        if (b != (int)blockIdx.x) {
+          __syncthreads();  // the tile before is done with the staging
+          smp = load_sample(X, T, n, steps.off[k], batch, b);
+        }
+        grad_tile(S, smp, inv_cnt, partials + (int64_t)b * kPartial);
+      }
+      if (k + 1 < steps.count) smp = load_sample(X, T, n, steps.off[k + 1], batch, blockIdx.x);
+    }
+    if (grid_barrier(sync, ++round)) return;
+    if (own >= 0) {
+      const float gi = sum_partials(partials, nblk, own);
+      if (own != kSse) {
+        adam(p, m, v, gi, steps.rate[k], betas);
+      } else {
+        loss += gi * curve_scale;
+        if (++in_epoch == steps.steps_per_epoch || k + 1 == steps.count) curve[epoch] = loss;
+        if (in_epoch == steps.steps_per_epoch) ++epoch, in_epoch = 0, loss = 0.f;
+      }
+    }
+    write_image(img, u, p);
+    if (grid_barrier(sync, ++round)) return;
   }
+  if (u < mlpk::kParams) P[own] = p, M[own] = m, V[own] = v;
 }
 
 // ---- the p2r path-length iteration alone ---------------------------------------
@@ -588,17 +779,31 @@ int upload_params(fit_mlp* m, const float* host) {
   return FIT_OK;
 }
 
-int launch_adam(fit_mlp* m, const float* grad, int nblk, float lr, float* curve, float scale,
-                cudaStream_t s) {
+// The rate of the network's next Adam step.
+AdamRate next_rate(fit_mlp* m, float lr) {
   m->step += 1;
   const double bc1 = 1.0 - std::pow((double)m->beta1, (double)m->step);
   const double bc2 = 1.0 - std::pow((double)m->beta2, (double)m->step);
-  mlp_adam_kernel<<<kAdamBlocks, kAdamThreads, 0, s>>>(m->d_params, m->d_m, m->d_v, grad,
-                                                        m->d_partials, nblk, lr, m->beta1, m->beta2,
-                                                        m->eps, (float)bc1, (float)bc2, curve, scale);
-  mlp_image_kernel<<<1, 1024, 0, s>>>(m->d_params, m->d_img);
+  return {lr, (float)bc1, (float)bc2};
+}
+
+int launch_adam(fit_mlp* m, const float* grad, int nblk, AdamRate rate, float* curve, float scale,
+                cudaStream_t s) {
+  mlp_adam_kernel<<<kAdamBlocks, kAdamThreads, 0, s>>>(m->d_params, m->d_m, m->d_v, m->d_img, grad,
+                                                        m->d_partials, nblk, rate,
+                                                        {m->beta1, m->beta2, m->eps}, curve, scale);
   cudaError_t e = cudaGetLastError();
   return e == cudaSuccess ? FIT_OK : cuda_fail(e, "fit_mlp: Adam launch");
+}
+
+// Blocks of mlp_train_kernel that fit on the device together.
+int train_blocks(int device) {
+  int per_sm = 0, sms = 0;
+  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, mlp_train_kernel, kBlock, 0) !=
+          cudaSuccess ||
+      cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, device) != cudaSuccess)
+    return 0;
+  return per_sm * sms;
 }
 
 }  // namespace
@@ -636,7 +841,8 @@ int fit_mlp_create(fit_mlp** out, int device, uint64_t seed) {
   const size_t pb = mlpk::kParams * sizeof(float);
   if (cudaMalloc(&m->d_params, pb) != cudaSuccess || cudaMalloc(&m->d_m, pb) != cudaSuccess ||
       cudaMalloc(&m->d_v, pb) != cudaSuccess ||
-      cudaMalloc(&m->d_img, sizeof(TrainImage)) != cudaSuccess) {
+      cudaMalloc(&m->d_img, sizeof(TrainImage)) != cudaSuccess ||
+      cudaMalloc(&m->d_sync, 2 * sizeof(unsigned)) != cudaSuccess) {
     fit_mlp_destroy(m);
     return fail(FIT_ERR_NOMEM, "fit_mlp_create: cudaMalloc");
   }
@@ -670,6 +876,7 @@ void fit_mlp_destroy(fit_mlp* m) {
     cudaFree(m->d_img);
     cudaFree(m->d_partials);
     cudaFree(m->d_curve);
+    cudaFree(m->d_sync);
   }
   delete m;
 }
@@ -751,7 +958,8 @@ int fit_mlp_adam_step(fit_mlp* m, const float* grad, float lr, void* stream) {
   if (!m || !grad) return fail(FIT_ERR_ARG, "fit_mlp_adam_step: NULL argument");
   if (!(lr >= 0.f)) return fail(FIT_ERR_ARG, "fit_mlp_adam_step: lr must be >= 0");
   DeviceGuard guard(m->device);
-  return launch_adam(m, grad, 0, lr, nullptr, 0.f, static_cast<cudaStream_t>(stream));
+  return launch_adam(m, grad, 0, next_rate(m, lr), nullptr, 0.f,
+                     static_cast<cudaStream_t>(stream));
 }
 
 int fit_mlp_train(fit_mlp* m, const float* x, const float* target, int64_t n,
@@ -779,6 +987,7 @@ int fit_mlp_train(fit_mlp* m, const float* x, const float* target, int64_t n,
   }
   cudaStream_t s = static_cast<cudaStream_t>(stream);
   cudaError_t e = cudaMemsetAsync(m->d_curve, 0, cfg->epochs * sizeof(float), s);
+  if (e == cudaSuccess) e = cudaMemsetAsync(m->d_sync, 0, 2 * sizeof(unsigned), s);
   if (e != cudaSuccess) return cuda_fail(e, "fit_mlp_train: memset");
   m->beta1 = cfg->beta1;
   m->beta2 = cfg->beta2;
@@ -787,6 +996,14 @@ int fit_mlp_train(fit_mlp* m, const float* x, const float* target, int64_t n,
   const int64_t total = steps * cfg->epochs;
   const float scale = 1.f / (float)((double)cfg->batch * (double)steps);
   uint64_t rs = cfg->seed;
+  // One cooperative launch for every kTrainSteps steps.  Its blocks must hold
+  // a parameter per thread and run together; a device partition too small
+  // for that takes the steps as two launches each.
+  const int together = train_blocks(m->device);
+  const bool one_launch = together > kAdamBlocks;
+  const unsigned grid = (unsigned)std::min(std::max(nblk, kAdamBlocks), std::max(together, 1));
+  TrainSteps ts;
+  ts.count = 0;
   int64_t t = 0;
   for (int ep = 0; ep < cfg->epochs; ++ep) {
     const int64_t start = (int64_t)(splitmix64(rs) % (uint64_t)n);
@@ -794,14 +1011,46 @@ int fit_mlp_train(fit_mlp* m, const float* x, const float* target, int64_t n,
       const double frac = total > 1 ? (double)t / (double)(total - 1) : 0.0;
       const float lr = (float)(cfg->lr_final + 0.5 * (cfg->lr - cfg->lr_final) *
                                                    (1.0 + std::cos(3.14159265358979323846 * frac)));
-      mlp_grad_kernel<<<nblk, kBlock, 0, s>>>(m->d_img, x, target, n, (start + k * cfg->batch) % n,
-                                              cfg->batch, 1.f / (float)cfg->batch, m->d_partials);
-      rc = launch_adam(m, nullptr, nblk, lr, m->d_curve + ep, scale, s);
-      if (rc != FIT_OK) return rc;
+      const int64_t off = (start + k * cfg->batch) % n;
+      const float inv = 1.f / (float)cfg->batch;
+      if (!one_launch) {
+        mlp_grad_kernel<<<nblk, kBlock, 0, s>>>(m->d_img, x, target, n, off, cfg->batch, inv,
+                                                m->d_partials);
+        rc = launch_adam(m, nullptr, nblk, next_rate(m, lr), m->d_curve + ep, scale, s);
+        if (rc != FIT_OK) return rc;
+        continue;
+      }
+      if (!ts.count) {
+        ts.first_epoch = ep;
+        ts.steps_per_epoch = (int)steps;
+        ts.first_step = (int)k;
+      }
+      ts.rate[ts.count] = next_rate(m, lr);
+      ts.off[ts.count++] = off;
+      if (ts.count < kTrainSteps && t + 1 < total) continue;
+      e = cudaMemsetAsync(m->d_sync, 0, sizeof(unsigned), s);
+      AdamBetas betas{m->beta1, m->beta2, m->eps};
+      int batch = cfg->batch;
+      int64_t nsamp = n;
+      float cnt_inv = inv, cscale = scale;
+      void* args[] = {&ts,      &m->d_img, &x,     &target,     &nsamp,  &batch,    &cnt_inv,
+                      &m->d_partials, &m->d_params, &m->d_m, &m->d_v, &betas, &m->d_curve,
+                      &cscale,  &m->d_sync};
+      if (e == cudaSuccess)
+        e = cudaLaunchCooperativeKernel((const void*)mlp_train_kernel, dim3(grid), dim3(kBlock),
+                                        args, 0, s);
+      if (e != cudaSuccess) return cuda_fail(e, "fit_mlp_train: launch");
+      ts.count = 0;
     }
+  }
+  unsigned gave_up = 0;
+  if (one_launch) {
+    e = cudaMemcpyAsync(&gave_up, m->d_sync + 1, sizeof(unsigned), cudaMemcpyDeviceToHost, s);
+    if (e != cudaSuccess) return cuda_fail(e, "fit_mlp_train: barrier status");
   }
   e = cudaStreamSynchronize(s);
   if (e != cudaSuccess) return cuda_fail(e, "fit_mlp_train: synchronize");
+  if (gave_up) return fail(FIT_ERR_TIMEOUT, "fit_mlp_train: the training kernel's barrier timed out");
   if (loss_per_epoch) {
     e = cudaMemcpy(loss_per_epoch, m->d_curve, cfg->epochs * sizeof(float), cudaMemcpyDeviceToHost);
     if (e != cudaSuccess) return cuda_fail(e, "fit_mlp_train: copy losses");

@@ -374,3 +374,53 @@ def test_full_size_seeded_fit_sampled(trained):
                      "full-size seeded fit")
     finally:
         f.close()
+
+
+def _splitmix64(x):
+    mask = (1 << 64) - 1
+    x = (x + 0x9e3779b97f4a7c15) & mask
+    z = ((x ^ (x >> 30)) * 0xbf58476d1ce4e5b9) & mask
+    z = ((z ^ (z >> 27)) * 0x94d049bb133111eb) & mask
+    return x, z ^ (z >> 31)
+
+
+# A ragged tile, one tile, a usual batch, more tiles than blocks run together,
+# and more steps (1100) than one launch holds (512), ending within an epoch.
+@pytest.mark.parametrize("batch,n,epochs", [(100, 1030, 3), (64, 64, 5), (4096, 9000, 2),
+                                            (65536, 70000, 2), (64, 64 * 550 + 7, 2)])
+def test_training_is_its_steps(batch, n, epochs):
+    """fit_mlp_train, whose steps share a launch, gives bit for bit the
+    parameters of the same steps taken by fit_mlp_gradient and
+    fit_mlp_adam_step, and the loss of each epoch."""
+    g = torch.Generator("cuda").manual_seed(batch)
+    x = torch.randn((n, 8), generator=g, device="cuda")
+    t = torch.randn(n, generator=g, device="cuda")
+    t[::17] = float("nan")  # samples without a target
+    lr, lr_final, seed = 2e-3, 1e-4, 11
+    one, two = fit.fit_mlp_create(0, seed=5), fit.fit_mlp_create(0, seed=5)
+    curve = fit.fit_mlp_train(one, x, t, epochs=epochs, batch=batch, lr=lr, lr_final=lr_final, seed=seed)
+    grad, loss = torch.empty(fit.FIT_MLP_PARAMS, device="cuda"), torch.empty(1, device="cuda")
+    steps, rs, k = n // batch, seed, 0
+    lr32, fin32 = float(np.float32(lr)), float(np.float32(lr_final))
+    for ep in range(epochs):
+        rs, r = _splitmix64(rs)
+        losses = []
+        for i in range(steps):
+            frac = k / (steps * epochs - 1) if steps * epochs > 1 else 0.0
+            rate = fin32 + 0.5 * float(np.float32(np.float32(lr) - np.float32(lr_final))) * (
+                1.0 + np.cos(3.14159265358979323846 * frac))
+            off = (r % n + i * batch) % n
+            xb, tb = torch.roll(x, -off, 0)[:batch].contiguous(), torch.roll(t, -off)[:batch].contiguous()
+            fit.fit_mlp_gradient(two, xb, tb, grad, loss)
+            fit.fit_mlp_adam_step(two, grad, rate)
+            losses.append(float(loss))
+            k += 1
+        # (losses sum in another order: a float per step)
+        assert abs(curve[ep] - np.mean(losses)) <= 1e-5 * np.mean(losses)
+    np.testing.assert_array_equal(fit.fit_mlp_get_params(one), fit.fit_mlp_get_params(two))
+    y1, y2 = torch.empty(n, device="cuda"), torch.empty(n, device="cuda")
+    fit.fit_mlp_forward(one, x, y1)  # the BF16 images agree too
+    fit.fit_mlp_forward(two, x, y2)
+    assert torch.equal(y1, y2)
+    fit.fit_mlp_destroy(one)
+    fit.fit_mlp_destroy(two)
