@@ -42,49 +42,6 @@ constexpr int kSse = 4801;       // squared errors, count of finite targets
 constexpr int kCount = 4802;
 constexpr int kMaxGradSamples = 65536;
 
-// ---- the BF16 fragment image of the parameters ------------------------------
-
-__device__ void build_image(const float* __restrict__ P, TrainImage* img, int tid, int nthr) {
-  using namespace mlpk;
-  uint32_t* w1 = &img->fwd.w1[0][0].x;
-  for (int i = tid; i < 2 * 32 * 4; i += nthr) {
-    const int e = i & 3, lane = (i >> 2) & 31, j = i >> 7;
-    const int g = lane >> 2, c = lane & 3;
-    const int row = (4 * j + e) * 8 + g;
-    w1[i] = pack_bf16(P[kOffW1 + row * 8 + 2 * c], P[kOffW1 + row * 8 + 2 * c + 1]);
-  }
-  uint32_t* w2 = &img->fwd.w2[0][0][0].x;
-  uint32_t* w2t = &img->w2t[0][0][0].x;
-  for (int i = tid; i < 4 * 4 * 32 * 4; i += nthr) {
-    const int e = i & 3, lane = (i >> 2) & 31, j = (i >> 7) & 3, kb = i >> 9;
-    const int g = lane >> 2, c = lane & 3;
-    const int nb = 2 * j + (e >> 1), k0 = kb * 16 + (e & 1) * 8 + 2 * c, n = nb * 8 + g;
-    w2[i] = pack_bf16(P[kOffW2 + n * 64 + k0], P[kOffW2 + n * 64 + k0 + 1]);
-    w2t[i] = pack_bf16(P[kOffW2 + k0 * 64 + n], P[kOffW2 + (k0 + 1) * 64 + n]);
-  }
-  uint32_t* w3 = &img->fwd.w3[0][0].x;
-  for (int i = tid; i < 2 * 32 * 4; i += nthr) {
-    const int e = i & 3, lane = (i >> 2) & 31, j = i >> 7;
-    const int g = lane >> 2, c = lane & 3;
-    const int k0 = (2 * j + (e >> 1)) * 16 + (e & 1) * 8 + 2 * c;
-    w3[i] = g == 0 ? pack_bf16(P[kOffW3 + k0], P[kOffW3 + k0 + 1]) : 0u;
-  }
-  for (int i = tid; i < kHid; i += nthr) {
-    img->fwd.b1[i] = P[kOffB1 + i];
-    img->fwd.b2[i] = P[kOffB2 + i];
-    img->w3f[i] = bf16_round(P[kOffW3 + i]);
-  }
-  if (tid == 0) {
-    img->fwd.b3 = P[kOffB3];
-    img->fwd.pad[0] = img->fwd.pad[1] = img->fwd.pad[2] = 0.f;
-  }
-}
-
-__global__ void __launch_bounds__(1024) mlp_image_kernel(const float* __restrict__ P,
-                                                         TrainImage* img) {
-  build_image(P, img, threadIdx.x, blockDim.x);
-}
-
 // ---- inputs and targets -------------------------------------------------------
 
 __global__ void __launch_bounds__(256)
@@ -168,12 +125,19 @@ __device__ __forceinline__ void stage_a(uint4 (*m)[8], int r0, int kb, int c,
   swz(m, r0 + 8, 2 * kb + 1)[c] = a[3];
 }
 
-// Sum over the eight lanes with the same c (lane bits 2..4).
-__device__ __forceinline__ float sum_over_g(float v) {
-  v += __shfl_xor_sync(0xffffffffu, v, 4);
-  v += __shfl_xor_sync(0xffffffffu, v, 8);
-  v += __shfl_xor_sync(0xffffffffu, v, 16);
-  return v;
+// One halving of a sum over lanes: of N values each lane keeps the half that
+// its bit `mask` selects, with the partner's added.  Three of them sum 48
+// values over the eight lanes with the same c in 42 shuffles, and leave six
+// finished sums in each lane (a butterfly for each value takes 144 shuffles
+// for the same additions).
+template <int N>
+__device__ __forceinline__ void halve(const float (&v)[N], float (&out)[N / 2], int mask) {
+  const bool up = threadIdx.x & mask;
+#pragma unroll
+  for (int k = 0; k < N / 2; ++k) {
+    const float keep = up ? v[k + N / 2] : v[k], send = up ? v[k] : v[k + N / 2];
+    out[k] = keep + __shfl_xor_sync(0xffffffffu, send, mask);
+  }
 }
 
 // One sample's inputs and, for the lanes that need them, two targets.
@@ -305,18 +269,25 @@ __device__ __forceinline__ void grad_tile(GradSmem& S, const Sample& smp, float 
     stage_a(S.dz1, r0, kb, c, d);
   }
 
-  // bias and dW3 sums over the block's rows
+  // bias and dW3 sums over the warp's rows
+  {
+    float v[48], h1[24], h2[12], h3[6];
 #pragma unroll
-  for (int nb = 0; nb < 8; ++nb) {
+    for (int nb = 0; nb < 8; ++nb)
 #pragma unroll
-    for (int e = 0; e < 2; ++e) {
-      const float v1 = sum_over_g(gb1[nb][e]), v2 = sum_over_g(gb2[nb][e]),
-                  v3 = sum_over_g(gw3[nb][e]);
-      if (g == 0) {
-        S.red[warp][nb * 8 + 2 * c + e] = v1;
-        S.red[warp][64 + nb * 8 + 2 * c + e] = v2;
-        S.red[warp][128 + nb * 8 + 2 * c + e] = v3;
+      for (int e = 0; e < 2; ++e) {
+        v[2 * nb + e] = gb1[nb][e];
+        v[16 + 2 * nb + e] = gb2[nb][e];
+        v[32 + 2 * nb + e] = gw3[nb][e];
       }
+    halve(v, h1, 4);
+    halve(h1, h2, 8);
+    halve(h2, h3, 16);
+    const int first = (lane & 4 ? 24 : 0) + (lane & 8 ? 12 : 0) + (lane & 16 ? 6 : 0);
+#pragma unroll
+    for (int k = 0; k < 6; ++k) {
+      const int i = first + k, j = i & 15;
+      S.red[warp][(i >> 4) * 64 + (j >> 1) * 8 + 2 * c + (j & 1)] = h3[k];
     }
   }
 #pragma unroll
@@ -429,9 +400,9 @@ __device__ __forceinline__ int owned_param(int u) {
   return v < kOffW2 ? v : kOffB2 + (v - kOffW2);
 }
 
-// Writes the image's words of thread u's parameter, whose value is p (the
-// inverse of build_image's indexing).  Whole warps call it; u >= kParams has
-// no parameter.
+// Writes the words of the BF16 fragment image (mlp.cuh) that hold thread u's
+// parameter, whose value is p; the words of w3 with no column stay zero from
+// fit_mlp_create.  Whole warps call it; u >= kParams has no parameter.
 __device__ __forceinline__ void write_image(TrainImage* img, int u, float p) {
   using namespace mlpk;
   const float right = __shfl_xor_sync(0xffffffffu, p, 1);  // the next column (or row of W3)
@@ -486,9 +457,16 @@ __device__ __forceinline__ void adam(float& p, float& m, float& v, float gi, Ada
 // Sum of entry i of the nblk partials, in order (the partials are the same
 // kernel's in training: __ldcg, past the L1).
 __device__ __forceinline__ float sum_partials(const float* partials, int nblk, int i) {
+  constexpr int N = 64;  // loads in flight
+  const float* q = partials + i;
   float s = 0.f;
-#pragma unroll 32
-  for (int b = 0; b < nblk; ++b) s += __ldcg(partials + (int64_t)b * kPartial + i);
+  for (int b = 0; b < nblk; b += N, q += (int64_t)N * kPartial) {
+    float t[N];
+#pragma unroll
+    for (int j = 0; j < N; ++j) t[j] = b + j < nblk ? __ldcg(q + j * kPartial) : 0.f;
+#pragma unroll
+    for (int j = 0; j < N; ++j) s += t[j];
+  }
   return s;
 }
 
@@ -516,6 +494,20 @@ __global__ void __launch_bounds__(kAdamThreads)
   if (curve && u == 0) *curve += sum_partials(partials, nblk, kSse) * curve_scale;
 }
 
+// New parameters (already in P): the moments cleared, the image written.
+__global__ void __launch_bounds__(kAdamThreads)
+    mlp_load_kernel(const float* __restrict__ P, float* __restrict__ M, float* __restrict__ V,
+                    TrainImage* img) {
+  const int u = blockIdx.x * kAdamThreads + threadIdx.x;
+  float p = 0.f;
+  if (u < mlpk::kParams) {
+    const int i = owned_param(u);
+    p = P[i];
+    M[i] = V[i] = 0.f;
+  }
+  write_image(img, u, p);
+}
+
 // ---- training: many steps in one launch --------------------------------------------
 
 // The steps of one launch, as kernel parameters.
@@ -538,7 +530,6 @@ __device__ __forceinline__ bool grid_barrier(unsigned* sync, unsigned round) {
   bool gave_up = false;
   __syncthreads();
   if (threadIdx.x == 0) {
-    __threadfence();
     asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(sync) : "memory");
     const unsigned target = round * gridDim.x;
     for (unsigned looks = 0;; ++looks) {
@@ -551,7 +542,6 @@ __device__ __forceinline__ bool grid_barrier(unsigned* sync, unsigned round) {
         break;
       }
     }
-    __threadfence();
   }
   return __syncthreads_or(gave_up);
 }
@@ -563,7 +553,7 @@ __device__ __forceinline__ bool grid_barrier(unsigned* sync, unsigned round) {
 // The same sums in the same order as mlp_grad_kernel and mlp_adam_kernel.
 // A step is a chain of latencies, not of work (0.1 GFLOP, 1.2 MB of partials
 // in the L2), so what counts is the number of launches and meetings: a batch
-// of 4096 takes TIME_NOW us a step, with three launches (gradient, Adam on 19
+// of 4096 takes 8.8 us a step, with three launches (gradient, Adam on 19
 // blocks, image on one) it took 23.5.  The next step's samples are loaded
 // before the barrier, whose wait hides them.
 __global__ void __launch_bounds__(kBlock)
@@ -586,8 +576,14 @@ __global__ void __launch_bounds__(kBlock)
     if ((int)blockIdx.x < nblk) {
       const uint4* src = reinterpret_cast<const uint4*>(img);
       uint4* dst = reinterpret_cast<uint4*>(&S.W);
-      constexpr int kWords = sizeof(TrainImage) / 16;
-      for (int i = threadIdx.x; i < kWords; i += kBlock) dst[i] = __ldcg(src + i);
+      constexpr int kWords = sizeof(TrainImage) / 16, kPer = (kWords + kBlock - 1) / kBlock;
+      uint4 w[kPer];  // all loads in flight at once
+#pragma unroll
+      for (int i = 0; i < kPer; ++i)
+        if (i * kBlock + (int)threadIdx.x < kWords) w[i] = __ldcg(src + i * kBlock + threadIdx.x);
+#pragma unroll
+      for (int i = 0; i < kPer; ++i)
+        if (i * kBlock + (int)threadIdx.x < kWords) dst[i * kBlock + threadIdx.x] = w[i];
       for (int b = blockIdx.x; b < nblk; b += gridDim.x) {
         if (b != (int)blockIdx.x) {
           __syncthreads();  // the tile before is done with the staging
@@ -768,11 +764,9 @@ int ensure_partials(fit_mlp* m, int64_t nblk) {
 int upload_params(fit_mlp* m, const float* host) {
   cudaError_t e = cudaMemcpy(m->d_params, host, mlpk::kParams * sizeof(float),
                              cudaMemcpyHostToDevice);
-  if (e == cudaSuccess) e = cudaMemset(m->d_m, 0, mlpk::kParams * sizeof(float));
-  if (e == cudaSuccess) e = cudaMemset(m->d_v, 0, mlpk::kParams * sizeof(float));
   if (e != cudaSuccess) return cuda_fail(e, "fit_mlp: upload");
   m->step = 0;
-  mlp_image_kernel<<<1, 1024>>>(m->d_params, m->d_img);
+  mlp_load_kernel<<<kAdamBlocks, kAdamThreads>>>(m->d_params, m->d_m, m->d_v, m->d_img);
   e = cudaGetLastError();
   if (e == cudaSuccess) e = cudaDeviceSynchronize();
   if (e != cudaSuccess) return cuda_fail(e, "fit_mlp: image");
@@ -842,6 +836,7 @@ int fit_mlp_create(fit_mlp** out, int device, uint64_t seed) {
   if (cudaMalloc(&m->d_params, pb) != cudaSuccess || cudaMalloc(&m->d_m, pb) != cudaSuccess ||
       cudaMalloc(&m->d_v, pb) != cudaSuccess ||
       cudaMalloc(&m->d_img, sizeof(TrainImage)) != cudaSuccess ||
+      cudaMemset(m->d_img, 0, sizeof(TrainImage)) != cudaSuccess ||
       cudaMalloc(&m->d_sync, 2 * sizeof(unsigned)) != cudaSuccess) {
     fit_mlp_destroy(m);
     return fail(FIT_ERR_NOMEM, "fit_mlp_create: cudaMalloc");
@@ -1028,7 +1023,7 @@ int fit_mlp_train(fit_mlp* m, const float* x, const float* target, int64_t n,
       ts.rate[ts.count] = next_rate(m, lr);
       ts.off[ts.count++] = off;
       if (ts.count < kTrainSteps && t + 1 < total) continue;
-      e = cudaMemsetAsync(m->d_sync, 0, sizeof(unsigned), s);
+      if (t >= kTrainSteps) e = cudaMemsetAsync(m->d_sync, 0, sizeof(unsigned), s);
       AdamBetas betas{m->beta1, m->beta2, m->eps};
       int batch = cfg->batch;
       int64_t nsamp = n;
