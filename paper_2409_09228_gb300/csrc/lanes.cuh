@@ -1,6 +1,6 @@
 // Lane types for the fused kernel: float (one track per thread), F2 (two
 // tracks per thread, held in the two halves of a float2), and double (the
-// FP64 variant, one track per thread, IEEE operations throughout).
+// FP64 variant, one track per thread).
 //
 // The per-track math is written once as templates over the lane type.  With
 // F2 every add, multiply and fused multiply-add is one packed sm_100+
@@ -101,12 +101,55 @@ __device__ __forceinline__ F2 sel(M2 m, F2 a, F2 b) {
   return F2(m.x ? a.v.x : b.v.x, m.y ? a.v.y : b.v.y);
 }
 
-// ---- double (the FP64 variant, one track per thread): IEEE operations ------
+// ---- double (the FP64 variant, one track per thread) -----------------------
+// A warp's FP64 operation holds its SM's FP64 pipe for 16 cycles, so the FP64
+// kernels are bound by the count of these alone (the pipe is 89 % busy).  Reciprocal and
+// reciprocal square root take a coarse start from the MUFU (rcp.approx.ftz.f64,
+// rsqrt.approx.ftz.f64: about 2^-19) and one correction of third order
+// (Householder, "The Numerical Treatment of a Single Nonlinear Equation",
+// 1970): with e = 1 - x y, 1/x = y / (1 - e) = y (1 + e + e^2 + ...), and with
+// e = 1 - x y^2, x^(-1/2) = y (1 - e)^(-1/2) = y (1 + e/2 + 3 e^2/8 + ...).
+// What is dropped is below 2^-55, so the results stay within an ulp of the
+// IEEE functions', in 3 and 5 operations.  A zero, subnormal, huge, negative
+// (rsqrt) or non-finite argument goes to those.
 __device__ __forceinline__ double fma(double a, double b, double c) { return ::fma(a, b, c); }
-__device__ __forceinline__ double fdiv(double a, double b) { return a / b; }
-__device__ __forceinline__ double frcp(double x) { return 1.0 / x; }
-__device__ __forceinline__ double fsqrt(double x) { return ::sqrt(x); }  // NaN for x < 0, as in FP32
-__device__ __forceinline__ double frsqrt(double x) { return 1.0 / ::sqrt(x); }
+// 2^-500 <= |x| < 2^500, on the integer pipe; positive: also x > 0
+__device__ __forceinline__ bool mid_range(double x, bool positive) {
+  const int hi = positive ? __double2hiint(x) : __double2hiint(x) & 0x7fffffff;
+  return (unsigned)(hi - 0x20b00000) < 0x3e800000u;
+}
+static __device__ __noinline__ double ieee_rcp(double x) { return 1.0 / x; }
+static __device__ __noinline__ double ieee_div(double a, double b) { return a / b; }
+static __device__ __noinline__ double ieee_sqrt(double x) { return ::sqrt(x); }
+__device__ __forceinline__ double frcp(double x) {
+  if (!mid_range(x, false)) return ieee_rcp(x);
+  double y;
+  asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
+  const double e = ::fma(-x, y, 1.0);
+  return ::fma(::fma(e, e, e), y, y);
+}
+// a (1/b), with the quotient's remainder folded back
+__device__ __forceinline__ double fdiv(double a, double b) {
+  if (!mid_range(b, false)) return ieee_div(a, b);
+  const double y = frcp(b), q = a * y;
+  return ::fma(::fma(-b, q, a), y, q);
+}
+__device__ __forceinline__ double frsqrt(double x) {
+  if (!mid_range(x, true)) return ieee_rcp(ieee_sqrt(x));
+  double y;
+  asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
+  const double e = ::fma(-(x * y), y, 1.0);
+  return ::fma(::fma(e, 0.375, 0.5), e * y, y);
+}
+__device__ __forceinline__ double fsqrt(double x) {  // NaN for x < 0, as in FP32
+  if (!mid_range(x, true)) return ieee_sqrt(x);
+  const double y = frsqrt(x), s = x * y;
+  return ::fma(::fma(-s, s, x), 0.5 * y, s);
+}
+// |x| < the double whose upper word is hi (a positive one), on the integer pipe
+__device__ __forceinline__ bool below_hi(double x, int hi) {
+  return (__double2hiint(x) & 0x7fffffff) < hi;
+}
 __device__ __forceinline__ double fabs_(double x) { return ::fabs(x); }
 __device__ __forceinline__ double floor_(double x) { return ::floor(x); }
 __device__ __forceinline__ double fmax_(double a, double b) { return ::fmax(a, b); }

@@ -553,7 +553,7 @@ __device__ __forceinline__ bool grid_barrier(unsigned* sync, unsigned round) {
 // The same sums in the same order as mlp_grad_kernel and mlp_adam_kernel.
 // A step is a chain of latencies, not of work (0.1 GFLOP, 1.2 MB of partials
 // in the L2), so what counts is the number of launches and meetings: a batch
-// of 4096 takes 8.8 us a step, with three launches (gradient, Adam on 19
+// of 4096 takes 6.7 us a step, with three launches (gradient, Adam on 19
 // blocks, image on one) it took 23.5.  The next step's samples are loaded
 // before the barrier, whose wait hides them.
 __global__ void __launch_bounds__(kBlock)

@@ -28,6 +28,7 @@
 #pragma once
 
 #include <cstdint>
+#include <type_traits>
 
 #include "fit.h"
 #include "lanes.cuh"
@@ -200,39 +201,50 @@ __device__ __forceinline__ void turn_by(T& c, T& s, T d) {
   }
 }
 
-// FP64 variant: sin and cos from the CUDA math library; sin(u)/u and its
-// derivative by their Taylor series (to u^8 and u^7, remainders below 1e-19
-// relative for |u| < 1e-2) only where sin(u)/u and (cos u - sin(u)/u)/u
-// would cancel.
+// FP64 variant.  The angles of a layer are small, so their functions are
+// Taylor series, cut where the next term is below 2^-56 of the result at the
+// end of the range: sin(u)/u, cos u and (sin(u)/u)' to u^12, u^14 and u^13 for
+// |u| < 1/4 (a third of the operations of sincos and two divisions), sin d
+// and cos d to d^11 and d^10 for |d| < 1/16.  Beyond, sin and cos come from
+// the CUDA math library.
 __device__ __forceinline__ void sincos_cw(double x, double& s, double& c) { ::sincos(x, &s, &c); }
-__device__ __forceinline__ void sinc_c(double u, double& s, double& cu) {
-  double sn;
-  ::sincos(u, &sn, &cu);
-  if (::fabs(u) < 1e-2) {
-    const double u2 = u * u;
-    s = fma(u2, fma(u2, fma(u2, fma(u2, 1.0 / 362880.0, -1.0 / 5040.0), 1.0 / 120.0), -1.0 / 6.0),
-            1.0);
+__device__ __forceinline__ void sinc_cs(double u, double& s, double& cu, double& sp) {
+  if (below_hi(u, 0x3fd00000)) {
+    const double v = -(u * u);
+    s = fma(v, fma(v, fma(v, fma(v, fma(v, fma(v, 1.0 / 6227020800.0, 1.0 / 39916800.0),
+                                        1.0 / 362880.0), 1.0 / 5040.0), 1.0 / 120.0), 1.0 / 6.0), 1.0);
+    cu = fma(v, fma(v, fma(v, fma(v, fma(v, fma(v, fma(v, 1.0 / 87178291200.0, 1.0 / 479001600.0),
+                                                1.0 / 3628800.0), 1.0 / 40320.0), 1.0 / 720.0),
+                           1.0 / 24.0), 0.5), 1.0);
+    // 2 k / (2 k + 1)!
+    sp = -u * fma(v, fma(v, fma(v, fma(v, fma(v, fma(v, 14.0 / 1307674368000.0, 12.0 / 6227020800.0),
+                                              10.0 / 39916800.0), 8.0 / 362880.0), 6.0 / 5040.0),
+                         4.0 / 120.0), 2.0 / 6.0);
   } else {
+    double sn;
+    ::sincos(u, &sn, &cu);
     s = sn / u;
+    sp = (cu - s) / u;
   }
 }
-__device__ __forceinline__ double sinc_deriv(double u, double s, double cu) {
-  if (::fabs(u) < 1e-2) {
-    const double u2 = u * u;
-    return u * fma(u2, fma(u2, fma(u2, 1.0 / 45360.0, -1.0 / 840.0), 1.0 / 30.0), -1.0 / 3.0);
-  }
-  return (cu - s) / u;
+__device__ __forceinline__ void sinc_c(double u, double& s, double& cu) {
+  double sp;
+  sinc_cs(u, s, cu, sp);
 }
 __device__ __forceinline__ void turn_by(double& c, double& s, double d) {
   double sd, cd;
-  ::sincos(d, &sd, &cd);
+  if (below_hi(d, 0x3fb00000)) {
+    const double v = -(d * d);
+    sd = d * fma(v, fma(v, fma(v, fma(v, fma(v, 1.0 / 39916800.0, 1.0 / 362880.0), 1.0 / 5040.0),
+                               1.0 / 120.0), 1.0 / 6.0), 1.0);
+    cd = fma(v, fma(v, fma(v, fma(v, fma(v, 1.0 / 3628800.0, 1.0 / 40320.0), 1.0 / 720.0),
+                           1.0 / 24.0), 0.5), 1.0);
+  } else {
+    ::sincos(d, &sd, &cd);
+  }
   turn(c, s, cd, sd);
 }
 __device__ __forceinline__ void turn_small(double& c, double& s, double d) { turn_by(c, s, d); }
-__device__ __forceinline__ void sinc_cs(double u, double& s, double& cu, double& sp) {
-  sinc_c(u, s, cu);
-  sp = sinc_deriv(u, s, cu);
-}
 
 // Two turns by small angles (as turn_by) with one range test.
 template <class T>
@@ -590,7 +602,14 @@ __device__ __forceinline__ typename Lanes<T>::M prop_z(T (&p)[6], T (&c)[21], Tr
                                                        float Z, const Overlap& ov = Overlap()) {
   ov();  // the caller's independent work, beside the path length's reciprocal
   const T dz = T(Z) - p[2];
-  const T tanth = fdiv(g.sth, g.cth);
+  // double: one reciprocal for tan(theta) and dh/dtheta
+  T icth, tanth;
+  if constexpr (std::is_same_v<T, double>) {
+    icth = frcp(g.cth);
+    tanth = g.sth * icth;
+  } else {
+    tanth = fdiv(g.sth, g.cth);
+  }
   const T h = dz * tanth;
   const auto fail = not_(lt(T(0.f), h));
   if (any(fail)) return fail;
@@ -606,7 +625,11 @@ __device__ __forceinline__ typename Lanes<T>::M prop_z(T (&p)[6], T (&c)[21], Tr
   T c1 = cm, s1 = sm;
   turn(c1, s1, cu, su);  // phi + 2u = phi'
   const T hh = T(0.5f) * h * h * dkdw;
-  const T hth = fdiv(dz, g.cth * g.cth);  // dh/dtheta
+  T hth;  // dh/dtheta
+  if constexpr (std::is_same_v<T, double>)
+    hth = dz * icth * icth;
+  else
+    hth = fdiv(dz, g.cth * g.cth);
   // grad h = (0, 0, -tan(theta), 0, 0, dh/dtheta); d p'/d h = (cos phi',
   // sin phi', 0 on the plane, 0, kappa, 0)
   const T gr[6] = {T(0.f), T(0.f), -tanth, T(0.f), T(0.f), hth};
@@ -623,7 +646,7 @@ __device__ __forceinline__ typename Lanes<T>::M prop_z(T (&p)[6], T (&c)[21], Tr
 }
 
 // atan(t) / t: its Taylor series to t^12 (remainder below 2.5e-10 for
-// |t| <= 1/4, the range crossing_start admits); in double atan itself.
+// |t| <= 1/4, the range crossing_start admits).
 template <class T>
 __device__ __forceinline__ T atan_ratio(T t) {
   const T t2 = t * t;
@@ -631,7 +654,14 @@ __device__ __forceinline__ T atan_ratio(T t) {
                                              T(1.f / 9.f)), T(-1.f / 7.f)), T(1.f / 5.f)),
                       T(-1.f / 3.f)), T(1.f));
 }
-__device__ __forceinline__ double atan_ratio(double t) { return t != 0.0 ? ::atan(t) / t : 1.0; }
+// In double to t^20 (remainder below 3e-15): where the iteration starts, not
+// what it converges to.
+__device__ __forceinline__ double atan_ratio(double t) {
+  const double v = -(t * t);
+  return fma(v, fma(v, fma(v, fma(v, fma(v, fma(v, fma(v, fma(v, fma(v, fma(v, 1.0 / 21.0, 1.0 / 19.0),
+             1.0 / 17.0), 1.0 / 15.0), 1.0 / 13.0), 1.0 / 11.0), 1.0 / 9.0), 1.0 / 7.0), 1.0 / 5.0),
+             1.0 / 3.0), 1.0);
+}
 
 // Where the helix of the propagation crosses the cylinder r = R, in closed
 // form.  With b0 and t0 the start's components along and across the
@@ -1097,8 +1127,12 @@ __device__ __forceinline__ typename Lanes<T>::M normalise(T (&p)[6], T (&c)[NC],
                                                           T lag = T(0.f)) {
   constexpr int D = NC == 21 ? 6 : 5, W = NC == 21 ? 3 : 2;
   turn_by2(g.cphi, g.sphi, (p[4] - phi_before) + lag, g.cth, g.sth, p[5] - th_before);
-  const T k = floor_((pi_<T>() - p[4]) * inv_two_pi_<T>());
-  p[4] = fma(k, two_pi_<T>(), p[4]);
+  bool inside = false;  // double: |phi| < 3.14 needs no FP64 operation
+  if constexpr (std::is_same_v<T, double>) inside = below_hi(p[4], 0x40091eb8);
+  if (!inside) {
+    const T k = floor_((pi_<T>() - p[4]) * inv_two_pi_<T>());
+    p[4] = fma(k, two_pi_<T>(), p[4]);
+  }
   const auto flip = lt(p[3], T(0.f));
   if (any(flip)) {
     const T sgn = sel(flip, T(-1.f), T(1.f));
