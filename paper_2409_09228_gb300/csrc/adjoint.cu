@@ -193,11 +193,14 @@ int fit_adjoint_forward(fit_handle* h, const fit_tracks_in* in, const fit_tracks
   if (out->ld != hits->ld)
     return fail(FIT_ERR_ARG, "fit_adjoint_forward: outputs and hits must share ld");
   DeviceGuard g(h->device);
-  cudaStream_t s = static_cast<cudaStream_t>(stream);
   FitArgs a = base_args(in, out, hits, nlayer, h->d_counters);
   float* tp = static_cast<float*>(tape);
   int32_t* ndone = reinterpret_cast<int32_t*>(tp + (size_t)kTapeRow * nlayer * out->ld);
+  ModeStreams ms(h, static_cast<cudaStream_t>(stream), "fit_adjoint_forward");
+  rc = ms.begin(nevt, ntrk, mode);
+  if (rc != FIT_OK) return rc;
   for (int m : {FIT_MODE_R, FIT_MODE_Z}) {  // one launch per mode
+    const cudaStream_t s = ms.of(m);
     a.geo = h->geo[m];
     rc = launch_track_runs(nevt, ntrk, mode, m, "fit_adjoint_forward", [&](int64_t t0, const TrackRuns& r) {
       a.t0 = t0;
@@ -207,8 +210,10 @@ int fit_adjoint_forward(fit_handle* h, const fit_tracks_in* in, const fit_tracks
       else
         fit_tape_kernel<FIT_MODE_R><<<nblk, kAdjBlock, 0, s>>>(a, r, tp, ndone);
     });
-    if (rc != FIT_OK) return rc;
+    if (rc != FIT_OK) break;
   }
+  rc = ms.end(rc);
+  if (rc != FIT_OK) return rc;
   h->tracks += (uint64_t)total;
   return FIT_OK;
 }
@@ -237,7 +242,6 @@ int fit_adjoint_backward(fit_handle* h, const fit_hits* hits, int nevt, const in
   if (grad_cov0 && !aligned16(grad_cov0))
     return fail(FIT_ERR_ARG, std::string(kWho) + ": grad_cov0 misaligned");
   DeviceGuard g(h->device);
-  cudaStream_t s = static_cast<cudaStream_t>(stream);
   AdjArgs b{};
   b.hpos = hits->pos;
   b.hcov = hits->cov;
@@ -249,9 +253,13 @@ int fit_adjoint_backward(fit_handle* h, const fit_hits* hits, int nevt, const in
   b.g_par0 = grad_par0;
   b.g_cov0 = grad_cov0;
   b.nlayer = nlayer;
+  ModeStreams ms(h, static_cast<cudaStream_t>(stream), kWho);
+  int rc = ms.begin(nevt, ntrk, mode);
+  if (rc != FIT_OK) return rc;
   for (int m : {FIT_MODE_R, FIT_MODE_Z}) {  // one launch per mode
+    const cudaStream_t s = ms.of(m);
     b.geo = h->geo[m];
-    const int rc = launch_track_runs(nevt, ntrk, mode, m, kWho, [&](int64_t t0, const TrackRuns& r) {
+    rc = launch_track_runs(nevt, ntrk, mode, m, kWho, [&](int64_t t0, const TrackRuns& r) {
       b.t0 = t0;
       const unsigned nblk = (r.n + kAdjBlock - 1) / kAdjBlock;
       if (m == FIT_MODE_Z)
@@ -259,9 +267,9 @@ int fit_adjoint_backward(fit_handle* h, const fit_hits* hits, int nevt, const in
       else
         fit_adjoint_kernel<FIT_MODE_R><<<nblk, kAdjBlock, 0, s>>>(b, r);
     });
-    if (rc != FIT_OK) return rc;
+    if (rc != FIT_OK) break;
   }
-  return FIT_OK;
+  return ms.end(rc);
 }
 
 }  // extern "C"

@@ -282,6 +282,29 @@ int run_fit(const fit_handle* h, const FitArgs& a, int layout, bool seeded, int 
                      });
 }
 
+int ModeStreams::begin(int nevt, const int64_t* ntrk, const int32_t* mode) {
+  bool used[2] = {false, false};
+  for (int e = 0; e < nevt; ++e)
+    if (ntrk[e] > 0) used[mode[e] == FIT_MODE_Z] = true;
+  if (!(used[0] && used[1])) return FIT_OK;
+  lock_ = std::unique_lock<std::mutex>(h_->side_mu);
+  cudaError_t e = cudaEventRecord(h_->fork, s_);
+  if (e == cudaSuccess) e = cudaStreamWaitEvent(h_->side, h_->fork, 0);
+  if (e != cudaSuccess)
+    return cuda_fail(e, (std::string(who_) + ": fork to the second stream").c_str());
+  forked_ = true;
+  return FIT_OK;
+}
+
+int ModeStreams::end(int rc) {
+  if (!forked_) return rc;
+  cudaError_t e = cudaEventRecord(h_->join, h_->side);
+  if (e == cudaSuccess) e = cudaStreamWaitEvent(s_, h_->join, 0);
+  if (e != cudaSuccess && rc == FIT_OK)
+    return cuda_fail(e, (std::string(who_) + ": join from the second stream").c_str());
+  return rc;
+}
+
 // Scratch of fit_propagate_update_noalloc, in the library image instead of
 // allocated memory: per-event counters [FIT_NOALLOC_MAX_EVENTS][kEventSlots]
 // followed by the event offsets [FIT_NOALLOC_MAX_EVENTS + 1] (int64).  Every
@@ -336,6 +359,11 @@ int fit_init(fit_handle** out, const fit_config* cfg_r, const fit_config* cfg_z,
     return rc;
   }
   DeviceGuard g(device);
+  e = cudaDeviceGetAttribute(&h->sms, cudaDevAttrMultiProcessorCount, device);
+  if (e != cudaSuccess) {
+    delete h;
+    return cuda_fail(e, "fit_init: cudaDeviceGetAttribute");
+  }
   e = cudaMalloc(&h->d_counters, kCounters * sizeof(unsigned long long));
   if (e != cudaSuccess) {
     delete h;
@@ -367,29 +395,11 @@ int fit_propagate_update(fit_handle* h, const fit_tracks_in* in, const fit_track
   if (rc != FIT_OK || total == 0) return rc;
   DeviceGuard g(h->device);
   static const char* kWho = "fit_propagate_update";
-  const cudaStream_t s = static_cast<cudaStream_t>(stream);
-  const FitArgs a = base_args(in, out, hits, nlayer, h->d_counters);
-  bool used[2] = {false, false};
-  for (int e = 0; e < nevt; ++e)
-    if (ntrk[e] > 0) used[mode[e] == FIT_MODE_Z] = true;
-  if (!(used[0] && used[1])) {
-    rc = run_fit(h, a, FIT_LAYOUT_SOA, h->seeded, nevt, ntrk, mode, kWho, s, s);
-  } else {
-    // The two modes' events are independent: the p2z launches go to the
-    // handle's second stream, so that they overlap the p2r launches (their
-    // blocks fill the SMs a launch's last wave leaves idle).  The join is
-    // recorded even after a failed launch, so that the caller's stream
-    // still follows everything that was queued.
-    std::lock_guard<std::mutex> lock(h->side_mu);
-    cudaError_t e = cudaEventRecord(h->fork, s);
-    if (e == cudaSuccess) e = cudaStreamWaitEvent(h->side, h->fork, 0);
-    if (e != cudaSuccess) return cuda_fail(e, "fit_propagate_update: fork to the second stream");
-    rc = run_fit(h, a, FIT_LAYOUT_SOA, h->seeded, nevt, ntrk, mode, kWho, s, h->side);
-    e = cudaEventRecord(h->join, h->side);
-    if (e == cudaSuccess) e = cudaStreamWaitEvent(s, h->join, 0);
-    if (e != cudaSuccess && rc == FIT_OK)
-      return cuda_fail(e, "fit_propagate_update: join from the second stream");
-  }
+  ModeStreams ms(h, static_cast<cudaStream_t>(stream), kWho);
+  rc = ms.begin(nevt, ntrk, mode);
+  if (rc != FIT_OK) return rc;
+  rc = ms.end(run_fit(h, base_args(in, out, hits, nlayer, h->d_counters), FIT_LAYOUT_SOA,
+                      h->seeded, nevt, ntrk, mode, kWho, ms.of(FIT_MODE_R), ms.of(FIT_MODE_Z)));
   if (rc != FIT_OK) return rc;
   h->tracks += (uint64_t)total;
   return FIT_OK;
@@ -411,9 +421,11 @@ int fit_propagate_update_layout(fit_handle* h, const fit_tracks_in* in, const fi
     return fail(FIT_ERR_ARG, std::string(kWho) + ": AoSoA slots (ld) must be a multiple of 32");
   if (h->seeded) return fail(FIT_ERR_ARG, std::string(kWho) + ": no learned seed in AoSoA");
   DeviceGuard g(h->device);
-  cudaStream_t s = static_cast<cudaStream_t>(stream);
-  rc = run_fit(h, base_args(in, out, hits, nlayer, h->d_counters), layout, false, nevt, ntrk, mode,
-               kWho, s, s);
+  ModeStreams ms(h, static_cast<cudaStream_t>(stream), kWho);
+  rc = ms.begin(nevt, ntrk, mode);
+  if (rc != FIT_OK) return rc;
+  rc = ms.end(run_fit(h, base_args(in, out, hits, nlayer, h->d_counters), layout, false, nevt,
+                      ntrk, mode, kWho, ms.of(FIT_MODE_R), ms.of(FIT_MODE_Z)));
   if (rc != FIT_OK) return rc;
   h->tracks += (uint64_t)total;
   return FIT_OK;

@@ -102,6 +102,7 @@ class DeviceGuard {
 
 struct fit_handle {
   int device = 0;
+  int sms = 0;  // streaming multiprocessors of the device
   bool has[2] = {false, false};
   int nlayer[2] = {0, 0};
   fitimpl::Geo geo[2];
@@ -111,9 +112,9 @@ struct fit_handle {
   bool seeded = false;    // p2r seeds from d_mlp
   void* host_stage = nullptr;  // staging of fit_propagate_update_host (host.cu)
   float B[2] = {0.f, 0.f};     // field of each mode's configuration
-  // A call of fit_propagate_update with events of both modes runs its p2z
-  // launches on `side`, forked from the caller's stream by `fork` and joined
-  // back by `join`; side_mu keeps concurrent calls from interleaving them.
+  // A call with events of both modes runs its p2z launches on `side`, forked
+  // from the caller's stream by `fork` and joined back by `join`; side_mu
+  // keeps concurrent calls from interleaving them (ModeStreams).
   cudaStream_t side = nullptr;
   cudaEvent_t fork = nullptr, join = nullptr;
   std::mutex side_mu;
@@ -184,6 +185,28 @@ int launch_track_runs(int nevt, const int64_t* ntrk, const int32_t* mode, int m,
 int run_fit(const fit_handle* h, const FitArgs& a, int layout, bool seeded, int nevt,
             const int64_t* ntrk, const int32_t* mode, const char* who, cudaStream_t s,
             cudaStream_t sz);
+
+// The two modes' events of a call are independent: with both present, the
+// p2z launches go to the handle's second stream, so that they overlap the p2r
+// launches (their blocks fill the SMs a launch's last wave leaves idle).
+// begin() forks it from the caller's stream s, end(rc) joins it back (even
+// after a failed launch, so that s still follows everything that was queued)
+// and returns rc or the join's error.  A mutex keeps calls from several host
+// threads from interleaving their fork and join.
+class ModeStreams {
+ public:
+  ModeStreams(fit_handle* h, cudaStream_t s, const char* who) : h_(h), s_(s), who_(who) {}
+  int begin(int nevt, const int64_t* ntrk, const int32_t* mode);
+  int end(int rc);
+  cudaStream_t of(int m) const { return m == FIT_MODE_Z && forked_ ? h_->side : s_; }
+
+ private:
+  fit_handle* h_;
+  cudaStream_t s_;
+  const char* who_;
+  bool forked_ = false;
+  std::unique_lock<std::mutex> lock_;
+};
 
 // Frees the staging of fit_propagate_update_host (host.cu).
 void destroy_host_stage(fit_handle* h);
