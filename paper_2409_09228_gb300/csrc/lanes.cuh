@@ -84,6 +84,13 @@ __device__ __forceinline__ bool le(float a, float b) { return a <= b; }
 __device__ __forceinline__ M2 le(F2 a, F2 b) { return {a.v.x <= b.v.x, a.v.y <= b.v.y}; }
 __device__ __forceinline__ bool lt(float a, float b) { return a < b; }
 __device__ __forceinline__ M2 lt(F2 a, F2 b) { return {a.v.x < b.v.x, a.v.y < b.v.y}; }
+// x > 0, x < 0 and x <= 0 (in double on the integer pipe, see below)
+__device__ __forceinline__ bool pos(float x) { return 0.f < x; }
+__device__ __forceinline__ M2 pos(F2 x) { return {0.f < x.v.x, 0.f < x.v.y}; }
+__device__ __forceinline__ bool neg(float x) { return x < 0.f; }
+__device__ __forceinline__ M2 neg(F2 x) { return {x.v.x < 0.f, x.v.y < 0.f}; }
+__device__ __forceinline__ bool nonpos(float x) { return x <= 0.f; }
+__device__ __forceinline__ M2 nonpos(F2 x) { return {x.v.x <= 0.f, x.v.y <= 0.f}; }
 __device__ __forceinline__ bool finite_(float a) { return isfinite(a); }
 __device__ __forceinline__ M2 finite_(F2 a) { return {(bool)isfinite(a.v.x), (bool)isfinite(a.v.y)}; }
 __device__ __forceinline__ bool all(bool m) { return m; }
@@ -121,6 +128,13 @@ __device__ __forceinline__ bool mid_range(double x, bool positive) {
 static __device__ __noinline__ double ieee_rcp(double x) { return 1.0 / x; }
 static __device__ __noinline__ double ieee_div(double a, double b) { return a / b; }
 static __device__ __noinline__ double ieee_sqrt(double x) { return ::sqrt(x); }
+// Comparisons with zero by the upper word (a subnormal counts as zero; a NaN
+// as neither sign, but as x <= 0, whose callers test another value too).
+__device__ __forceinline__ bool pos(double x) { return (unsigned)(__double2hiint(x) - 1) < 0x7ff00000u; }
+__device__ __forceinline__ bool neg(double x) {
+  return (unsigned)__double2hiint(x) - 0x80000001u < 0x7ff00000u;
+}
+__device__ __forceinline__ bool nonpos(double x) { return !pos(x); }
 __device__ __forceinline__ double frcp(double x) {
   if (!mid_range(x, false)) return ieee_rcp(x);
   double y;
@@ -143,8 +157,7 @@ __device__ __forceinline__ double frsqrt(double x) {
 }
 __device__ __forceinline__ double fsqrt(double x) {  // NaN for x < 0, as in FP32
   if (!mid_range(x, true)) return ieee_sqrt(x);
-  const double y = frsqrt(x), s = x * y;
-  return ::fma(::fma(-s, s, x), 0.5 * y, s);
+  return x * frsqrt(x);
 }
 // |x| < the double whose upper word is hi (a positive one), on the integer pipe
 __device__ __forceinline__ bool below_hi(double x, int hi) {
@@ -156,7 +169,9 @@ __device__ __forceinline__ double fmax_(double a, double b) { return ::fmax(a, b
 __device__ __forceinline__ double copysign_(double a, double b) { return ::copysign(a, b); }
 __device__ __forceinline__ bool le(double a, double b) { return a <= b; }
 __device__ __forceinline__ bool lt(double a, double b) { return a < b; }
-__device__ __forceinline__ bool finite_(double a) { return isfinite(a); }
+__device__ __forceinline__ bool finite_(double a) {
+  return (__double2hiint(a) & 0x7ff00000) != 0x7ff00000;
+}
 __device__ __forceinline__ double sel(bool m, double a, double b) { return m ? a : b; }
 
 // ---- lanes ---------------------------------------------------------------

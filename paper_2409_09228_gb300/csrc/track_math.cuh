@@ -203,14 +203,20 @@ __device__ __forceinline__ void turn_by(T& c, T& s, T d) {
 
 // FP64 variant.  The angles of a layer are small, so their functions are
 // Taylor series, cut where the next term is below 2^-56 of the result at the
-// end of the range: sin(u)/u, cos u and (sin(u)/u)' to u^12, u^14 and u^13 for
-// |u| < 1/4 (a third of the operations of sincos and two divisions), sin d
-// and cos d to d^11 and d^10 for |d| < 1/16.  Beyond, sin and cos come from
+// end of the range: sin(u)/u, cos u and (sin(u)/u)' to u^8, u^8 and u^9 for
+// |u| < 1/16 (nearly every layer of 20) and to u^12, u^14 and u^13 for
+// |u| < 1/4, sin d and cos d to d^7 and d^6 for |d| < 1/64 (nearly every
+// update) and to d^11 and d^10 for |d| < 1/16.  Beyond, sin and cos come from
 // the CUDA math library.
 __device__ __forceinline__ void sincos_cw(double x, double& s, double& c) { ::sincos(x, &s, &c); }
 __device__ __forceinline__ void sinc_cs(double u, double& s, double& cu, double& sp) {
-  if (below_hi(u, 0x3fd00000)) {
-    const double v = -(u * u);
+  const double v = -(u * u);
+  if (below_hi(u, 0x3fb00000)) {
+    s = fma(v, fma(v, fma(v, fma(v, 1.0 / 362880.0, 1.0 / 5040.0), 1.0 / 120.0), 1.0 / 6.0), 1.0);
+    cu = fma(v, fma(v, fma(v, fma(v, 1.0 / 40320.0, 1.0 / 720.0), 1.0 / 24.0), 0.5), 1.0);
+    sp = -u * fma(v, fma(v, fma(v, fma(v, 10.0 / 39916800.0, 8.0 / 362880.0), 6.0 / 5040.0),
+                         4.0 / 120.0), 2.0 / 6.0);
+  } else if (below_hi(u, 0x3fd00000)) {
     s = fma(v, fma(v, fma(v, fma(v, fma(v, fma(v, 1.0 / 6227020800.0, 1.0 / 39916800.0),
                                         1.0 / 362880.0), 1.0 / 5040.0), 1.0 / 120.0), 1.0 / 6.0), 1.0);
     cu = fma(v, fma(v, fma(v, fma(v, fma(v, fma(v, fma(v, 1.0 / 87178291200.0, 1.0 / 479001600.0),
@@ -233,8 +239,11 @@ __device__ __forceinline__ void sinc_c(double u, double& s, double& cu) {
 }
 __device__ __forceinline__ void turn_by(double& c, double& s, double d) {
   double sd, cd;
-  if (below_hi(d, 0x3fb00000)) {
-    const double v = -(d * d);
+  const double v = -(d * d);
+  if (below_hi(d, 0x3f900000)) {
+    sd = d * fma(v, fma(v, fma(v, 1.0 / 5040.0, 1.0 / 120.0), 1.0 / 6.0), 1.0);
+    cd = fma(v, fma(v, fma(v, 1.0 / 720.0, 1.0 / 24.0), 0.5), 1.0);
+  } else if (below_hi(d, 0x3fb00000)) {
     sd = d * fma(v, fma(v, fma(v, fma(v, fma(v, 1.0 / 39916800.0, 1.0 / 362880.0), 1.0 / 5040.0),
                                1.0 / 120.0), 1.0 / 6.0), 1.0);
     cd = fma(v, fma(v, fma(v, fma(v, fma(v, 1.0 / 3628800.0, 1.0 / 40320.0), 1.0 / 720.0),
@@ -611,7 +620,7 @@ __device__ __forceinline__ typename Lanes<T>::M prop_z(T (&p)[6], T (&c)[21], Tr
     tanth = fdiv(g.sth, g.cth);
   }
   const T h = dz * tanth;
-  const auto fail = not_(lt(T(0.f), h));
+  const auto fail = not_(pos(h));
   if (any(fail)) return fail;
   const T kappa = dkdw * p[3];
   const T u = T(0.5f) * kappa * h;
@@ -654,10 +663,13 @@ __device__ __forceinline__ T atan_ratio(T t) {
                                              T(1.f / 9.f)), T(-1.f / 7.f)), T(1.f / 5.f)),
                       T(-1.f / 3.f)), T(1.f));
 }
-// In double to t^20 (remainder below 3e-15): where the iteration starts, not
-// what it converges to.
+// In double to t^20, or to t^10 for |t| < 1/16 (remainders below 3e-15): where
+// the iteration starts, not what it converges to.
 __device__ __forceinline__ double atan_ratio(double t) {
   const double v = -(t * t);
+  if (below_hi(t, 0x3fb00000))
+    return fma(v, fma(v, fma(v, fma(v, fma(v, 1.0 / 11.0, 1.0 / 9.0), 1.0 / 7.0), 1.0 / 5.0),
+                      1.0 / 3.0), 1.0);
   return fma(v, fma(v, fma(v, fma(v, fma(v, fma(v, fma(v, fma(v, fma(v, fma(v, 1.0 / 21.0, 1.0 / 19.0),
              1.0 / 17.0), 1.0 / 15.0), 1.0 / 13.0), 1.0 / 11.0), 1.0 / 9.0), 1.0 / 7.0), 1.0 / 5.0),
              1.0 / 3.0), 1.0);
@@ -722,6 +734,11 @@ __device__ __noinline__ S crossing_exact(S x, S y, S cph, S sph, S kappa, S R) {
 // failing and its caller reruns the surface for it (the fused kernel
 // propagates each track of the pair alone from there; a call inside the
 // packed loop cost it registers on every layer).
+// |t| <= 1/4 (in double < 1/4, on the integer pipe)
+template <class T>
+__device__ __forceinline__ typename Lanes<T>::M quarter(T t) { return le(fabs_(t), T(0.25f)); }
+__device__ __forceinline__ bool quarter(double t) { return below_hi(t, 0x3fd00000); }
+
 template <class T, bool EXACT>
 __device__ __forceinline__ typename Lanes<T>::M crossing_start(T x, T y, T cph, T sph, T kappa,
                                                                float R, T b0, T c0, T& h) {
@@ -733,7 +750,7 @@ __device__ __forceinline__ typename Lanes<T>::M crossing_start(T x, T y, T cph, 
   const T hl = fdiv(-c0, den);
   const T t = T(0.5f) * kappa * hl;
   // X < 0 (the circle misses the cylinder) makes den NaN, which fails den > 0
-  const M ok = and_(le(c0, T(0.f)), and_(lt(T(0.f), den), le(fabs_(t), T(0.25f))));
+  const M ok = and_(nonpos(c0), and_(pos(den), quarter(t)));
   h = hl * atan_ratio(t);
   if constexpr (Lanes<T>::n > 1 || !EXACT) {
     return not_(ok);
@@ -751,6 +768,18 @@ __device__ __forceinline__ typename Lanes<T>::M crossing_start(T x, T y, T cph, 
 // crossing_exact outside its hot loop (a call or the exact form's code inside
 // that loop slowed the memory-bound finder by 20 %).  kGiven: h_given.
 enum class Start { kAuto, kFast, kGiven };
+
+// Whether every lane's c2 is within 1e-4 b^2, where path_r's step takes the
+// first-order root; in double by the exponents alone: |c2| < 2^-16 b^2 if
+// e(c2) + 1 + 16 <= 2 e(b), and otherwise the general root, which is as good.
+template <class T>
+__device__ __forceinline__ bool near_circle(T c2, T b) {
+  return all(le(fabs_(c2), T(1e-4f) * (b * b)));
+}
+__device__ __forceinline__ bool near_circle(double c2, double b) {
+  const int ec = (__double2hiint(c2) >> 20) & 0x7ff, eb = (__double2hiint(b) >> 20) & 0x7ff;
+  return ec - 1023 + 17 <= 2 * (eb - 1023);
+}
 
 // The helix quantities of path_r's last evaluation.
 template <class T>
@@ -856,7 +885,7 @@ __device__ __forceinline__ typename Lanes<T>::M path_r(const T (&p)[6], const Tr
     const T b = fma(px, c1, py * s1);
     const T c2 = fma(px, px, fma(py, py, -R2));
     ib = frcp(b);
-    if (all(le(fabs_(c2), T(1e-4f) * (b * b)))) {
+    if (near_circle(c2, b)) {
       // Close to the circle the root is -c2 / (2 b) (1 + c2 / (4 b^2) + ...):
       // the dropped factor is below 2.5e-5 relative, on a step below
       // 5e-5 |b|; on a converged step (|d| <= tol) it moves h by less than
@@ -1133,7 +1162,7 @@ __device__ __forceinline__ typename Lanes<T>::M normalise(T (&p)[6], T (&c)[NC],
     const T k = floor_((pi_<T>() - p[4]) * inv_two_pi_<T>());
     p[4] = fma(k, two_pi_<T>(), p[4]);
   }
-  const auto flip = lt(p[3], T(0.f));
+  const auto flip = neg(p[3]);
   if (any(flip)) {
     const T sgn = sel(flip, T(-1.f), T(1.f));
     p[3] = p[3] * sgn;
