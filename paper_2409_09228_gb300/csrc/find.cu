@@ -53,16 +53,17 @@ struct FindArgs {
 // update takes its candidate from registers.  Loaded one at a time and the
 // chosen one again, the p2r kernel waited on loads 8.2 cycles an instruction
 // (now 0.9): 240k tracks, 4 candidates, 20 layers 217 -> 175 us, and both
-// modes of that size 383 -> 271 us with p2z on the second stream.  Four slots
-// fit 128 registers (4 blocks of 128 an SM); in double, bound by the FP64 pipe,
-// one slot is enough.
+// modes of that size 383 -> 260 us with p2z on the second stream.  Four slots
+// and 4 (p2r) and 5 (p2z) blocks of 128 an SM: 4 and 4 take 271 us, 5 and 6
+// 268, two slots with 6 and 7 265, three with 5 and 6 288.  In double, bound by
+// the FP64 pipe, one slot is enough.
 template <class T>
 constexpr int kSlots = sizeof(T) == 4 ? 4 : 1;
-template <class T>
-constexpr int kFindMinBlocks = sizeof(T) == 4 ? 4 : 1;
+template <int MODE, class T>
+constexpr int kFindMinBlocks = sizeof(T) == 8 ? 1 : MODE == FIT_MODE_Z ? 5 : 4;
 
 template <int MODE, class T>
-__global__ void __launch_bounds__(kBlock, kFindMinBlocks<T>)
+__global__ void __launch_bounds__(kBlock, kFindMinBlocks<MODE, T>)
     fit_find_kernel(const __grid_constant__ FindArgs<T> a, const __grid_constant__ TrackRuns r) {
   const unsigned i = blockIdx.x * kBlock + threadIdx.x;
   if (i >= r.n) return;
