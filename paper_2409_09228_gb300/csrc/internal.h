@@ -86,14 +86,16 @@ inline bool aligned16(const void* p) { return (reinterpret_cast<uintptr_t>(p) & 
 
 class DeviceGuard {
  public:
-  explicit DeviceGuard(int dev) {
+  explicit DeviceGuard(int dev) : dev_(dev) {
     cudaGetDevice(&prev_);
-    if (prev_ != dev) cudaSetDevice(dev);
+    if (prev_ != dev_) cudaSetDevice(dev_);
   }
-  ~DeviceGuard() { cudaSetDevice(prev_); }
+  ~DeviceGuard() {
+    if (prev_ != dev_) cudaSetDevice(prev_);
+  }
 
  private:
-  int prev_ = 0;
+  int dev_, prev_ = 0;
 };
 
 

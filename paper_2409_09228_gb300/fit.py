@@ -13,6 +13,7 @@ from __future__ import annotations
 
 import ctypes
 import os
+import struct
 from dataclasses import dataclass
 from typing import Optional, Sequence
 
@@ -92,6 +93,8 @@ class fit_mlp_train_config(ctypes.Structure):
                 ("eps", ctypes.c_float), ("seed", ctypes.c_uint64)]
 
 
+_STATUS_KEYS = tuple(k for k, _ in fit_status._fields_)
+
 EXPORTS = ("fit_init", "fit_propagate_update", "fit_sync", "fit_destroy", "fit_last_error",
            "fit_propagate_update_noalloc", "fit_plan_create", "fit_plan_run", "fit_plan_tune",
            "fit_plan_get_info", "fit_plan_destroy", "fit_tape_bytes", "fit_adjoint_forward",
@@ -128,69 +131,51 @@ def load(build_if_missing: bool = True):
         raise RuntimeError(f"libfit.so not found at {path}; run __graft_entry__.build()")
     L = ctypes.CDLL(path)
     vp, i64 = ctypes.c_void_p, ctypes.c_int64
+    # pointers to structs and event arrays as void*: the calls pass packed bytes
+    ci = ctypes.c_int
     L.fit_init.argtypes = [ctypes.POINTER(vp), ctypes.POINTER(fit_config),
-                           ctypes.POINTER(fit_config), ctypes.c_int]
-    L.fit_init.restype = ctypes.c_int
-    L.fit_propagate_update.argtypes = [vp, ctypes.POINTER(fit_tracks_in),
-                                       ctypes.POINTER(fit_tracks_out), ctypes.POINTER(fit_hits),
-                                       ctypes.c_int, ctypes.POINTER(i64), ctypes.c_int,
-                                       ctypes.POINTER(ctypes.c_int32), vp]
-    L.fit_propagate_update.restype = ctypes.c_int
+                           ctypes.POINTER(fit_config), ci]
+    L.fit_init.restype = ci
+    L.fit_propagate_update.argtypes = [vp, vp, vp, vp, ci, vp, ci, vp, vp]
+    L.fit_propagate_update.restype = ci
     L.fit_sync.argtypes = [vp, vp, ctypes.c_double, ctypes.POINTER(fit_status)]
-    L.fit_sync.restype = ctypes.c_int
+    L.fit_sync.restype = ci
     L.fit_destroy.argtypes = [vp]
     L.fit_destroy.restype = None
     L.fit_last_error.argtypes = []
     L.fit_last_error.restype = ctypes.c_char_p
     L.fit_propagate_update_noalloc.argtypes = [
-        ctypes.POINTER(fit_config), ctypes.POINTER(fit_config), ctypes.POINTER(fit_tracks_in),
-        ctypes.POINTER(fit_tracks_out), ctypes.POINTER(fit_hits), ctypes.c_int,
-        ctypes.POINTER(i64), ctypes.c_int, ctypes.POINTER(ctypes.c_int32), vp,
-        ctypes.POINTER(fit_status)]
-    L.fit_propagate_update_noalloc.restype = ctypes.c_int
-    L.fit_plan_create.argtypes = [vp, ctypes.c_int, ctypes.POINTER(i64),
-                                  ctypes.POINTER(ctypes.c_int32), ctypes.c_int,
-                                  ctypes.POINTER(fit_launch_config), ctypes.POINTER(vp)]
-    L.fit_plan_create.restype = ctypes.c_int
-    L.fit_plan_run.argtypes = [vp, ctypes.POINTER(fit_tracks_in), ctypes.POINTER(fit_tracks_out),
-                               ctypes.POINTER(fit_hits), vp]
-    L.fit_plan_run.restype = ctypes.c_int
-    L.fit_plan_tune.argtypes = [vp, ctypes.POINTER(fit_tracks_in), ctypes.POINTER(fit_tracks_out),
-                                ctypes.POINTER(fit_hits), vp, ctypes.c_char_p]
-    L.fit_plan_tune.restype = ctypes.c_int
+        ctypes.POINTER(fit_config), ctypes.POINTER(fit_config), vp, vp, vp, ci, vp, ci, vp, vp, vp]
+    L.fit_propagate_update_noalloc.restype = ci
+    L.fit_plan_create.argtypes = [vp, ci, vp, vp, ci, ctypes.POINTER(fit_launch_config),
+                                  ctypes.POINTER(vp)]
+    L.fit_plan_create.restype = ci
+    L.fit_plan_run.argtypes = [vp, vp, vp, vp, vp]
+    L.fit_plan_run.restype = ci
+    L.fit_plan_tune.argtypes = [vp, vp, vp, vp, vp, ctypes.c_char_p]
+    L.fit_plan_tune.restype = ci
     L.fit_plan_get_info.argtypes = [vp, ctypes.POINTER(fit_plan_info)]
-    L.fit_plan_get_info.restype = ctypes.c_int
+    L.fit_plan_get_info.restype = ci
     L.fit_plan_destroy.argtypes = [vp]
     L.fit_plan_destroy.restype = None
-    L.fit_tape_bytes.argtypes = [ctypes.c_int, i64]
+    L.fit_tape_bytes.argtypes = [ci, i64]
     L.fit_tape_bytes.restype = ctypes.c_size_t
-    L.fit_adjoint_forward.argtypes = [vp, ctypes.POINTER(fit_tracks_in),
-                                      ctypes.POINTER(fit_tracks_out), ctypes.POINTER(fit_hits),
-                                      ctypes.c_int, ctypes.POINTER(i64), ctypes.c_int,
-                                      ctypes.POINTER(ctypes.c_int32), vp, vp]
-    L.fit_adjoint_forward.restype = ctypes.c_int
-    L.fit_adjoint_backward.argtypes = [vp, ctypes.POINTER(fit_hits), ctypes.c_int,
-                                       ctypes.POINTER(i64), ctypes.c_int,
-                                       ctypes.POINTER(ctypes.c_int32), vp, vp, vp, vp, vp, vp]
-    L.fit_adjoint_backward.restype = ctypes.c_int
-    L.fit_find_tracks.argtypes = [vp, ctypes.POINTER(fit_tracks_in), ctypes.POINTER(fit_tracks_out),
-                                  ctypes.POINTER(fit_candidates), ctypes.c_float, vp, ctypes.c_int,
-                                  ctypes.POINTER(i64), ctypes.c_int, ctypes.POINTER(ctypes.c_int32),
-                                  vp]
-    L.fit_find_tracks.restype = ctypes.c_int
-    L.fit_find_tracks_f64.argtypes = [vp, ctypes.POINTER(fit_tracks_in),
-                                      ctypes.POINTER(fit_tracks_out), ctypes.POINTER(fit_candidates),
-                                      ctypes.c_double, vp, ctypes.c_int, ctypes.POINTER(i64),
-                                      ctypes.c_int, ctypes.POINTER(ctypes.c_int32), vp]
-    L.fit_find_tracks_f64.restype = ctypes.c_int
-    L.fit_propagate_update_layout.argtypes = L.fit_propagate_update.argtypes[:-1] + [ctypes.c_int, vp]
-    L.fit_propagate_update_layout.restype = ctypes.c_int
+    L.fit_adjoint_forward.argtypes = [vp, vp, vp, vp, ci, vp, ci, vp, vp, vp]
+    L.fit_adjoint_forward.restype = ci
+    L.fit_adjoint_backward.argtypes = [vp, vp, ci, vp, ci, vp, vp, vp, vp, vp, vp, vp]
+    L.fit_adjoint_backward.restype = ci
+    L.fit_find_tracks.argtypes = [vp, vp, vp, vp, ctypes.c_float, vp, ci, vp, ci, vp, vp]
+    L.fit_find_tracks.restype = ci
+    L.fit_find_tracks_f64.argtypes = [vp, vp, vp, vp, ctypes.c_double, vp, ci, vp, ci, vp, vp]
+    L.fit_find_tracks_f64.restype = ci
+    L.fit_propagate_update_layout.argtypes = L.fit_propagate_update.argtypes[:-1] + [ci, vp]
+    L.fit_propagate_update_layout.restype = ci
     L.fit_propagate_update_f64.argtypes = L.fit_propagate_update.argtypes
-    L.fit_propagate_update_f64.restype = ctypes.c_int
+    L.fit_propagate_update_f64.restype = ci
     L.fit_propagate_update_host.argtypes = L.fit_propagate_update.argtypes
-    L.fit_propagate_update_host.restype = ctypes.c_int
+    L.fit_propagate_update_host.restype = ci
     L.fit_propagate_update_mapped.argtypes = L.fit_propagate_update.argtypes
-    L.fit_propagate_update_mapped.restype = ctypes.c_int
+    L.fit_propagate_update_mapped.restype = ci
     i32p = ctypes.POINTER(ctypes.c_int32)
     L.fit_mlp_create.argtypes = [ctypes.POINTER(vp), ctypes.c_int, ctypes.c_uint64]
     L.fit_mlp_create.restype = ctypes.c_int
@@ -232,9 +217,31 @@ def _ptr(t) -> Optional[int]:
     return None if t is None else t.data_ptr()
 
 
+# The structs of fit.h as packed bytes and the event arrays as their bytes:
+# ctypes passes a bytes object by its address, and building ctypes structures
+# and typed numpy pointers instead cost ~20 us of a call (47 us with a 22 us
+# kernel) on the Grace host.
+_TRACKS_IN = struct.Struct("=QQQq").pack
+_TRACKS_OUT = struct.Struct("=QQQQQQq").pack
+_HITS = struct.Struct("=QQq").pack
+_CANDIDATES = struct.Struct("=QQi4xq").pack
+
+
+def _addr(t) -> int:
+    return 0 if t is None else t.data_ptr()
+
+
+def _event_bytes(ntrk, mode):
+    """(number of events, ntrk as int64 bytes, mode as int32 bytes)."""
+    nt = np.asarray(ntrk, dtype=np.int64)
+    return nt.size, nt.tobytes(), np.asarray(mode, dtype=np.int32).tobytes()
+
+
 def _stream_handle(stream) -> Optional[int]:
     if stream is None:
         import torch
+        if torch.cuda.is_initialized():  # the current stream's handle, without a Stream object
+            return torch._C._cuda_getCurrentRawStream(torch._C._cuda_getDevice()) or None
         stream = torch.cuda.current_stream()
     return getattr(stream, "cuda_stream", stream) or None
 
@@ -271,21 +278,11 @@ def fit_propagate_update(h: int, par_in, cov_in, q_in, hpos, hcov, ntrk: Sequenc
                          mode: Sequence[int], par_out=None, cov_out=None, q_out=None, chi2=None,
                          chi2_layer=None, status=None, stream=None) -> None:
     """The fused fit on device tensors; outputs default to the inputs (in place)."""
-    L = load()
-    par_out = par_in if par_out is None else par_out
-    cov_out = cov_in if cov_out is None else cov_out
-    q_out = q_in if q_out is None else q_out
-    nlayer = hpos.shape[0]
-    tin = fit_tracks_in(_ptr(par_in), _ptr(cov_in), _ptr(q_in), par_in.shape[-1])
-    tout = fit_tracks_out(_ptr(par_out), _ptr(cov_out), _ptr(q_out), _ptr(chi2),
-                          _ptr(chi2_layer), _ptr(status), par_out.shape[-1])
-    hits = fit_hits(_ptr(hpos), _ptr(hcov), hpos.shape[-1])
-    nt = np.ascontiguousarray(ntrk, dtype=np.int64)
-    md = np.ascontiguousarray(mode, dtype=np.int32)
-    _check(L.fit_propagate_update(
-        ctypes.c_void_p(h), ctypes.byref(tin), ctypes.byref(tout), ctypes.byref(hits), len(nt),
-        nt.ctypes.data_as(ctypes.POINTER(ctypes.c_int64)), nlayer,
-        md.ctypes.data_as(ctypes.POINTER(ctypes.c_int32)), _stream_handle(stream)))
+    tin, tout, hits = _buffers(par_in, cov_in, q_in, hpos, hcov, par_out, cov_out, q_out, chi2,
+                               chi2_layer, status)
+    nevt, nt, md = _event_bytes(ntrk, mode)
+    _check(load().fit_propagate_update(h, tin, tout, hits, nevt, nt, hpos.shape[0], md,
+                                       _stream_handle(stream)))
 
 
 def fit_propagate_update_layout(h: int, par_in, cov_in, q_in, hpos, hcov, ntrk: Sequence[int],
@@ -293,18 +290,13 @@ def fit_propagate_update_layout(h: int, par_in, cov_in, q_in, hpos, hcov, ntrk: 
                                 chi2, chi2_layer=None, status=None, stream=None) -> None:
     """The fused fit on arrays in `layout` (see fit.h); ld = track slots (for
     FIT_LAYOUT_AOSOA32 a multiple of 32).  Tensors are passed by pointer."""
-    L = load()
-    tin = fit_tracks_in(_ptr(par_in), _ptr(cov_in), _ptr(q_in), ld)
-    tout = fit_tracks_out(_ptr(par_out), _ptr(cov_out), _ptr(q_out), _ptr(chi2),
-                          _ptr(chi2_layer), _ptr(status), ld)
-    hits = fit_hits(_ptr(hpos), _ptr(hcov), ld)
-    nt = np.ascontiguousarray(ntrk, dtype=np.int64)
-    md = np.ascontiguousarray(mode, dtype=np.int32)
-    nlayer = hpos.numel() // (3 * ld)
-    _check(L.fit_propagate_update_layout(
-        ctypes.c_void_p(h), ctypes.byref(tin), ctypes.byref(tout), ctypes.byref(hits), len(nt),
-        nt.ctypes.data_as(ctypes.POINTER(ctypes.c_int64)), nlayer,
-        md.ctypes.data_as(ctypes.POINTER(ctypes.c_int32)), int(layout), _stream_handle(stream)))
+    tin = _TRACKS_IN(_addr(par_in), _addr(cov_in), _addr(q_in), ld)
+    tout = _TRACKS_OUT(_addr(par_out), _addr(cov_out), _addr(q_out), _addr(chi2),
+                       _addr(chi2_layer), _addr(status), ld)
+    nevt, nt, md = _event_bytes(ntrk, mode)
+    _check(load().fit_propagate_update_layout(
+        h, tin, tout, _HITS(_addr(hpos), _addr(hcov), ld), nevt, nt, hpos.numel() // (3 * ld), md,
+        int(layout), _stream_handle(stream)))
 
 
 def fit_propagate_update_f64(h: int, par_in, cov_in, q_in, hpos, hcov, ntrk: Sequence[int],
@@ -315,17 +307,11 @@ def fit_propagate_update_f64(h: int, par_in, cov_in, q_in, hpos, hcov, ntrk: Seq
     for t in (par_in, cov_in, hpos, hcov, par_out, cov_out, chi2):
         if t.dtype != torch.float64:
             raise ValueError("fit_propagate_update_f64 takes float64 tensors")
-    L = load()
-    tin = fit_tracks_in(_ptr(par_in), _ptr(cov_in), _ptr(q_in), par_in.shape[-1])
-    tout = fit_tracks_out(_ptr(par_out), _ptr(cov_out), _ptr(q_out), _ptr(chi2),
-                          _ptr(chi2_layer), _ptr(status), par_out.shape[-1])
-    hits = fit_hits(_ptr(hpos), _ptr(hcov), hpos.shape[-1])
-    nt = np.ascontiguousarray(ntrk, dtype=np.int64)
-    md = np.ascontiguousarray(mode, dtype=np.int32)
-    _check(L.fit_propagate_update_f64(
-        ctypes.c_void_p(h), ctypes.byref(tin), ctypes.byref(tout), ctypes.byref(hits), len(nt),
-        nt.ctypes.data_as(ctypes.POINTER(ctypes.c_int64)), hpos.shape[0],
-        md.ctypes.data_as(ctypes.POINTER(ctypes.c_int32)), _stream_handle(stream)))
+    tin, tout, hits = _buffers(par_in, cov_in, q_in, hpos, hcov, par_out, cov_out, q_out, chi2,
+                               chi2_layer, status)
+    nevt, nt, md = _event_bytes(ntrk, mode)
+    _check(load().fit_propagate_update_f64(h, tin, tout, hits, nevt, nt, hpos.shape[0], md,
+                                           _stream_handle(stream)))
 
 
 def fit_find_tracks(h: int, par_in, cov_in, q_in, cpos, ccov, ntrk: Sequence[int],
@@ -337,17 +323,13 @@ def fit_find_tracks(h: int, par_in, cov_in, q_in, cpos, ccov, ntrk: Sequence[int
     import torch
     f64 = par_in.dtype == torch.float64
     L = load()
-    tin = fit_tracks_in(_ptr(par_in), _ptr(cov_in), _ptr(q_in), par_in.shape[-1])
-    tout = fit_tracks_out(_ptr(par_out), _ptr(cov_out), _ptr(q_out), _ptr(chi2),
-                          _ptr(chi2_layer), _ptr(status), par_out.shape[-1])
-    cand = fit_candidates(_ptr(cpos), _ptr(ccov), cpos.shape[1], cpos.shape[-1])
-    nt = np.ascontiguousarray(ntrk, dtype=np.int64)
-    md = np.ascontiguousarray(mode, dtype=np.int32)
+    tin, tout, _ = _buffers(par_in, cov_in, q_in, cpos, ccov, par_out, cov_out, q_out, chi2,
+                            chi2_layer, status)
+    cand = _CANDIDATES(_addr(cpos), _addr(ccov), cpos.shape[1], cpos.shape[-1])
+    nevt, nt, md = _event_bytes(ntrk, mode)
     fn = L.fit_find_tracks_f64 if f64 else L.fit_find_tracks
-    _check(fn(ctypes.c_void_p(h), ctypes.byref(tin), ctypes.byref(tout), ctypes.byref(cand),
-              float(chi2_gate), _ptr(chosen), len(nt),
-              nt.ctypes.data_as(ctypes.POINTER(ctypes.c_int64)), cpos.shape[0],
-              md.ctypes.data_as(ctypes.POINTER(ctypes.c_int32)), _stream_handle(stream)))
+    _check(fn(h, tin, tout, cand, float(chi2_gate), _ptr(chosen), nevt, nt, cpos.shape[0], md,
+              _stream_handle(stream)))
 
 
 def fit_find_tracks_f64(h: int, par_in, cov_in, q_in, cpos, ccov, ntrk, mode, chi2_gate, chosen,
@@ -361,10 +343,10 @@ def fit_find_tracks_f64(h: int, par_in, cov_in, q_in, cpos, ccov, ntrk, mode, ch
                     cov_out, q_out, chi2, chi2_layer, status, stream)
 
 
-def _hptr(a) -> Optional[int]:
+def _haddr(a) -> int:
     """Address of a host array: a (pinned) torch CPU tensor or a numpy array."""
     if a is None:
-        return None
+        return 0
     if hasattr(a, "data_ptr"):
         if a.is_cuda:
             raise ValueError("the host entry points take host arrays")
@@ -378,20 +360,16 @@ def fit_propagate_update_host(h: int, par_in, cov_in, q_in, hpos, hcov, ntrk: Se
     """The fused fit on HOST arrays (page-locked torch tensors for overlap, or
     numpy arrays), copied through the library's device staging in chunks; the
     arrays must stay alive until the stream passes the call (fit_sync)."""
-    L = load()
     par_out = par_in if par_out is None else par_out
     cov_out = cov_in if cov_out is None else cov_out
     q_out = q_in if q_out is None else q_out
-    tin = fit_tracks_in(_hptr(par_in), _hptr(cov_in), _hptr(q_in), par_in.shape[-1])
-    tout = fit_tracks_out(_hptr(par_out), _hptr(cov_out), _hptr(q_out), _hptr(chi2),
-                          _hptr(chi2_layer), _hptr(status), par_out.shape[-1])
-    hits = fit_hits(_hptr(hpos), _hptr(hcov), hpos.shape[-1])
-    nt = np.ascontiguousarray(ntrk, dtype=np.int64)
-    md = np.ascontiguousarray(mode, dtype=np.int32)
-    _check(L.fit_propagate_update_host(
-        ctypes.c_void_p(h), ctypes.byref(tin), ctypes.byref(tout), ctypes.byref(hits), len(nt),
-        nt.ctypes.data_as(ctypes.POINTER(ctypes.c_int64)), hpos.shape[0],
-        md.ctypes.data_as(ctypes.POINTER(ctypes.c_int32)), _stream_handle(stream)))
+    tin = _TRACKS_IN(_haddr(par_in), _haddr(cov_in), _haddr(q_in), par_in.shape[-1])
+    tout = _TRACKS_OUT(_haddr(par_out), _haddr(cov_out), _haddr(q_out), _haddr(chi2),
+                       _haddr(chi2_layer), _haddr(status), par_out.shape[-1])
+    nevt, nt, md = _event_bytes(ntrk, mode)
+    _check(load().fit_propagate_update_host(h, tin, tout, _HITS(_haddr(hpos), _haddr(hcov),
+                                                                hpos.shape[-1]),
+                                            nevt, nt, hpos.shape[0], md, _stream_handle(stream)))
 
 
 def fit_propagate_update_mapped(h: int, par_in, cov_in, q_in, hpos, hcov, ntrk: Sequence[int],
@@ -400,20 +378,16 @@ def fit_propagate_update_mapped(h: int, par_in, cov_in, q_in, hpos, hcov, ntrk: 
     """The fused fit reading and writing page-locked HOST tensors in place
     (zero-copy over the host link); the tensors must stay alive, and the
     outputs unread, until the stream passes the call (fit_sync)."""
-    L = load()
     par_out = par_in if par_out is None else par_out
     cov_out = cov_in if cov_out is None else cov_out
     q_out = q_in if q_out is None else q_out
-    tin = fit_tracks_in(_hptr(par_in), _hptr(cov_in), _hptr(q_in), par_in.shape[-1])
-    tout = fit_tracks_out(_hptr(par_out), _hptr(cov_out), _hptr(q_out), _hptr(chi2),
-                          _hptr(chi2_layer), _hptr(status), par_out.shape[-1])
-    hits = fit_hits(_hptr(hpos), _hptr(hcov), hpos.shape[-1])
-    nt = np.ascontiguousarray(ntrk, dtype=np.int64)
-    md = np.ascontiguousarray(mode, dtype=np.int32)
-    _check(L.fit_propagate_update_mapped(
-        ctypes.c_void_p(h), ctypes.byref(tin), ctypes.byref(tout), ctypes.byref(hits), len(nt),
-        nt.ctypes.data_as(ctypes.POINTER(ctypes.c_int64)), hpos.shape[0],
-        md.ctypes.data_as(ctypes.POINTER(ctypes.c_int32)), _stream_handle(stream)))
+    tin = _TRACKS_IN(_haddr(par_in), _haddr(cov_in), _haddr(q_in), par_in.shape[-1])
+    tout = _TRACKS_OUT(_haddr(par_out), _haddr(cov_out), _haddr(q_out), _haddr(chi2),
+                       _haddr(chi2_layer), _haddr(status), par_out.shape[-1])
+    nevt, nt, md = _event_bytes(ntrk, mode)
+    _check(load().fit_propagate_update_mapped(h, tin, tout, _HITS(_haddr(hpos), _haddr(hcov),
+                                                                hpos.shape[-1]),
+                                            nevt, nt, hpos.shape[0], md, _stream_handle(stream)))
 
 
 def fit_propagate_update_noalloc(geom_r: Optional[Geometry], geom_z: Optional[Geometry], par_in,
@@ -427,37 +401,29 @@ def fit_propagate_update_noalloc(geom_r: Optional[Geometry], geom_z: Optional[Ge
     fit.h).  Returns a list with one counter dict per event when per_event is
     true (the call then waits for its work), else None.
     """
-    L = load()
-    par_out = par_in if par_out is None else par_out
-    cov_out = cov_in if cov_out is None else cov_out
-    q_out = q_in if q_out is None else q_out
+    tin, tout, hits = _buffers(par_in, cov_in, q_in, hpos, hcov, par_out, cov_out, q_out, chi2,
+                               chi2_layer, status)
     cr, _keep_r = _config(geom_r)
     cz, _keep_z = _config(geom_z)
-    tin = fit_tracks_in(_ptr(par_in), _ptr(cov_in), _ptr(q_in), par_in.shape[-1])
-    tout = fit_tracks_out(_ptr(par_out), _ptr(cov_out), _ptr(q_out), _ptr(chi2),
-                          _ptr(chi2_layer), _ptr(status), par_out.shape[-1])
-    hits = fit_hits(_ptr(hpos), _ptr(hcov), hpos.shape[-1])
-    nt = np.ascontiguousarray(ntrk, dtype=np.int64)
-    md = np.ascontiguousarray(mode, dtype=np.int32)
-    st = (fit_status * max(1, len(nt)))() if per_event else None
-    _check(L.fit_propagate_update_noalloc(
-        ctypes.byref(cr) if cr else None, ctypes.byref(cz) if cz else None, ctypes.byref(tin),
-        ctypes.byref(tout), ctypes.byref(hits), len(nt),
-        nt.ctypes.data_as(ctypes.POINTER(ctypes.c_int64)), hpos.shape[0],
-        md.ctypes.data_as(ctypes.POINTER(ctypes.c_int32)), _stream_handle(stream), st))
+    nevt, nt, md = _event_bytes(ntrk, mode)
+    st = (fit_status * max(1, nevt))() if per_event else None
+    _check(load().fit_propagate_update_noalloc(
+        ctypes.byref(cr) if cr else None, ctypes.byref(cz) if cz else None, tin, tout, hits, nevt,
+        nt, hpos.shape[0], md, _stream_handle(stream), st))
     if not per_event:
         return None
-    return [{k: int(getattr(st[e], k)) for k, _ in fit_status._fields_} for e in range(len(nt))]
+    rows = np.frombuffer(st, dtype=np.uint64).reshape(-1, len(_STATUS_KEYS)).tolist()
+    return [dict(zip(_STATUS_KEYS, row)) for row in rows[:nevt]]
 
 
 def _buffers(par_in, cov_in, q_in, hpos, hcov, par_out, cov_out, q_out, chi2, chi2_layer, status):
+    """fit_tracks_in, fit_tracks_out and fit_hits as bytes; outputs default to the inputs."""
     par_out = par_in if par_out is None else par_out
-    cov_out = cov_in if cov_out is None else cov_out
-    q_out = q_in if q_out is None else q_out
-    tin = fit_tracks_in(_ptr(par_in), _ptr(cov_in), _ptr(q_in), par_in.shape[-1])
-    tout = fit_tracks_out(_ptr(par_out), _ptr(cov_out), _ptr(q_out), _ptr(chi2),
-                          _ptr(chi2_layer), _ptr(status), par_out.shape[-1])
-    return tin, tout, fit_hits(_ptr(hpos), _ptr(hcov), hpos.shape[-1])
+    return (_TRACKS_IN(_addr(par_in), _addr(cov_in), _addr(q_in), par_in.shape[-1]),
+            _TRACKS_OUT(_addr(par_out), _addr(cov_in if cov_out is None else cov_out),
+                        _addr(q_in if q_out is None else q_out), _addr(chi2), _addr(chi2_layer),
+                        _addr(status), par_out.shape[-1]),
+            _HITS(_addr(hpos), _addr(hcov), hpos.shape[-1]))
 
 
 def fit_plan_create(h: int, ntrk: Sequence[int], mode: Sequence[int], nlayer: int,
@@ -465,15 +431,11 @@ def fit_plan_create(h: int, ntrk: Sequence[int], mode: Sequence[int], nlayer: in
                     persistent: bool = True, tracks_per_thread: int = 2,
                     layout: int = FIT_LAYOUT_SOA) -> int:
     """A plan for the batched persistent form (see fit.h)."""
-    nt = np.ascontiguousarray(ntrk, dtype=np.int64)
-    md = np.ascontiguousarray(mode, dtype=np.int32)
+    nevt, nt, md = _event_bytes(ntrk, mode)
     cfg = fit_launch_config(threads_per_block, blocks_per_sm, int(persistent),
                             int(tracks_per_thread), int(layout))
     p = ctypes.c_void_p()
-    _check(load().fit_plan_create(ctypes.c_void_p(h), len(nt),
-                                  nt.ctypes.data_as(ctypes.POINTER(ctypes.c_int64)),
-                                  md.ctypes.data_as(ctypes.POINTER(ctypes.c_int32)), nlayer,
-                                  ctypes.byref(cfg), ctypes.byref(p)))
+    _check(load().fit_plan_create(h, nevt, nt, md, nlayer, ctypes.byref(cfg), ctypes.byref(p)))
     return p.value
 
 
@@ -481,16 +443,14 @@ def fit_plan_run(plan: int, par_in, cov_in, q_in, hpos, hcov, par_out=None, cov_
                  q_out=None, chi2=None, chi2_layer=None, status=None, stream=None) -> None:
     tin, tout, hits = _buffers(par_in, cov_in, q_in, hpos, hcov, par_out, cov_out, q_out, chi2,
                                chi2_layer, status)
-    _check(load().fit_plan_run(ctypes.c_void_p(plan), ctypes.byref(tin), ctypes.byref(tout),
-                               ctypes.byref(hits), _stream_handle(stream)))
+    _check(load().fit_plan_run(plan, tin, tout, hits, _stream_handle(stream)))
 
 
 def fit_plan_tune(plan: int, par_in, cov_in, q_in, hpos, hcov, par_out, cov_out, q_out, chi2,
                   chi2_layer=None, status=None, stream=None, cache_path: Optional[str] = None) -> dict:
     tin, tout, hits = _buffers(par_in, cov_in, q_in, hpos, hcov, par_out, cov_out, q_out, chi2,
                                chi2_layer, status)
-    _check(load().fit_plan_tune(ctypes.c_void_p(plan), ctypes.byref(tin), ctypes.byref(tout),
-                                ctypes.byref(hits), _stream_handle(stream),
+    _check(load().fit_plan_tune(plan, tin, tout, hits, _stream_handle(stream),
                                 cache_path.encode() if cache_path else None))
     return fit_plan_get_info(plan)
 
@@ -527,33 +487,24 @@ def fit_tape_bytes(nlayer: int, ld: int) -> int:
     return int(load().fit_tape_bytes(nlayer, ld))
 
 
-def _events(ntrk, mode):
-    nt = np.ascontiguousarray(ntrk, dtype=np.int64)
-    md = np.ascontiguousarray(mode, dtype=np.int32)
-    return (len(nt), nt.ctypes.data_as(ctypes.POINTER(ctypes.c_int64)),
-            md.ctypes.data_as(ctypes.POINTER(ctypes.c_int32)), nt, md)
-
-
 def fit_adjoint_forward(h: int, par_in, cov_in, q_in, hpos, hcov, ntrk, mode, tape, par_out,
                         cov_out, q_out, chi2, chi2_layer=None, status=None, stream=None) -> None:
     """The fused fit that also records the per-layer checkpoints in `tape`."""
     tin, tout, hits = _buffers(par_in, cov_in, q_in, hpos, hcov, par_out, cov_out, q_out, chi2,
                                chi2_layer, status)
-    nevt, pn, pm, _k1, _k2 = _events(ntrk, mode)
-    _check(load().fit_adjoint_forward(ctypes.c_void_p(h), ctypes.byref(tin), ctypes.byref(tout),
-                                      ctypes.byref(hits), nevt, pn, hpos.shape[0], pm,
-                                      _ptr(tape), _stream_handle(stream)))
+    nevt, nt, md = _event_bytes(ntrk, mode)
+    _check(load().fit_adjoint_forward(h, tin, tout, hits, nevt, nt, hpos.shape[0], md, _ptr(tape),
+                                      _stream_handle(stream)))
 
 
 def fit_adjoint_backward(h: int, hpos, hcov, ntrk, mode, tape, grad_chi2, grad_hpos, grad_par0,
                          grad_cov0=None, stream=None) -> None:
     """Reverse sweep: gradients of grad_chi2-weighted summed chi2 (see fit.h)."""
-    hits = fit_hits(_ptr(hpos), _ptr(hcov), hpos.shape[-1])
-    nevt, pn, pm, _k1, _k2 = _events(ntrk, mode)
-    _check(load().fit_adjoint_backward(ctypes.c_void_p(h), ctypes.byref(hits), nevt, pn,
-                                       hpos.shape[0], pm, _ptr(tape), _ptr(grad_chi2),
-                                       _ptr(grad_hpos), _ptr(grad_par0), _ptr(grad_cov0),
-                                       _stream_handle(stream)))
+    hits = _HITS(_addr(hpos), _addr(hcov), hpos.shape[-1])
+    nevt, nt, md = _event_bytes(ntrk, mode)
+    _check(load().fit_adjoint_backward(h, hits, nevt, nt, hpos.shape[0], md, _ptr(tape),
+                                       _ptr(grad_chi2), _ptr(grad_hpos), _ptr(grad_par0),
+                                       _ptr(grad_cov0), _stream_handle(stream)))
 
 
 def _chi2_function():
@@ -573,12 +524,16 @@ def _chi2_function():
                                 out["par"], out["cov"], out["q"], out["chi2"],
                                 status=out["status"])
             ctx.save_for_backward(hpos, hcov, tape)
-            ctx.fitter, ctx.ntrk, ctx.mode = fitter, list(ntrk), list(mode)
+            ctx.fitter = fitter
+            ctx.ntrk, ctx.mode = np.array(ntrk, np.int64), np.array(mode, np.int32)
             ctx.mark_non_differentiable(out["par"], out["cov"])
+            ctx.set_materialize_grads(False)  # no zeros for the gradients of par and cov
             return out["chi2"], out["par"], out["cov"]
 
         @staticmethod
         def backward(ctx, grad_chi2, _gpar, _gcov):
+            if grad_chi2 is None:
+                return None, None, None, None, None, None, None, None
             hpos, hcov, tape = ctx.saved_tensors
             ld = hpos.shape[-1]
             g_hpos = torch.empty_like(hpos)
@@ -742,8 +697,8 @@ class Fitter:
         return out
 
     def run(self, par, cov, q, hpos, hcov, ntrk, mode, out=None, layers=False, stream=None):
-        n = int(np.sum(ntrk))
-        out = out or self.outputs(n, ld=par.shape[-1], layers=layers)
+        if not out:
+            out = self.outputs(int(np.sum(ntrk)), ld=par.shape[-1], layers=layers)
         fit_propagate_update(self.h, par, cov, q, hpos, hcov, ntrk, mode, par_out=out["par"],
                              cov_out=out["cov"], q_out=out["q"], chi2=out["chi2"],
                              chi2_layer=out["chi2_layer"], status=out["status"], stream=stream)
