@@ -300,8 +300,8 @@ int issue(fit_plan* p, const FitArgs& base, cudaStream_t s) {
   }
   // fit_propagate_update's form, one launch per mode: kept as an autotuner
   // candidate (for few, large events it can win)
-  return run_fit(p->h, base, p->cfg.layout, false, (int)p->ntrk.size(), p->ntrk.data(), p->mode.data(),
-                 "fit_plan", s, s);
+  return run_fit(p->h, base, p->cfg.layout, false, p->total, (int)p->ntrk.size(),
+                 p->ntrk.data(), p->mode.data(), "fit_plan", s, s);
 }
 
 void drop_graph(fit_plan* p) {

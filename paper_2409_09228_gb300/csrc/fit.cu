@@ -10,6 +10,7 @@
 #include <mutex>
 #include <string>
 #include <thread>
+#include <type_traits>
 
 #include "fit.h"
 #include "fused.cuh"
@@ -29,24 +30,31 @@ int cuda_fail(cudaError_t e, const char* what) {
 
 namespace {
 
-// The thread's track t: its pair's first one, or a lone one.  The first
+// The thread's track t: its pair's first one (TPT = 2) or one track of the pair
+// (TPT = 1), or a lone one.  The first
 // blocks take the lone tracks, so that their one-lane path runs beside the
 // pairs of other blocks (in a pair's warp it would run after them: a range
 // with odd edges took 38 us instead of 22 at 8191 tracks).
 enum class Part { kNone, kPair, kLone };
-template <int K>
-__device__ __forceinline__ Part thread_part(const FitArgs& a, const PairRuns<K>& r, int64_t& t) {
+template <int TPT, int K>
+__device__ __forceinline__ Part thread_part(int64_t t0, const PairRuns<K>& r, unsigned block,
+                                            int64_t& t) {
   const unsigned lone_blocks = (r.nlone + kBlock - 1) / kBlock;
-  if (blockIdx.x < lone_blocks) {
-    const unsigned i = blockIdx.x * kBlock + threadIdx.x;
+  if (block < lone_blocks) {
+    const unsigned i = block * kBlock + threadIdx.x;
     if (i >= r.nlone) return Part::kNone;
-    t = a.t0 + r.lone[i];
+    t = t0 + r.lone[i];
     return Part::kLone;
   }
-  const unsigned i = (blockIdx.x - lone_blocks) * kBlock + threadIdx.x;
-  if (i >= r.pairs.n) return Part::kNone;
-  t = a.t0 + run_element(r.pairs, i, 2);
+  const unsigned i = (block - lone_blocks) * kBlock + threadIdx.x, pair = TPT == 2 ? i : i / 2;
+  if (pair >= r.pairs.n) return Part::kNone;
+  t = t0 + run_element(r.pairs, pair, 2) + (TPT == 2 ? 0 : i & 1);
   return Part::kPair;
+}
+// Blocks of kBlock threads for r's tracks.
+template <int TPT, int K>
+unsigned part_blocks(const PairRuns<K>& r) {
+  return (r.nlone + kBlock - 1) / kBlock + (r.pairs.n * (2 / TPT) + kBlock - 1) / kBlock;
 }
 
 // 3 resident blocks per SM for p2r (156 registers, no spills; 2 blocks were
@@ -55,7 +63,7 @@ template <int MODE, int L, int K>
 __global__ void __launch_bounds__(kBlock, MODE == FIT_MODE_Z ? 4 : 3)
     fit_fused_kernel(const __grid_constant__ FitArgs a, const __grid_constant__ PairRuns<K> r) {
   int64_t t;
-  const Part part = thread_part(a, r, t);
+  const Part part = thread_part<2>(a.t0, r, blockIdx.x, t);
   if (part == Part::kNone) return;
   unsigned st[2] = {0u, 0u}, iters[2] = {0u, 0u};
   if (part == Part::kPair)
@@ -67,13 +75,22 @@ __global__ void __launch_bounds__(kBlock, MODE == FIT_MODE_Z ? 4 : 3)
   if (MODE == FIT_MODE_R) count_iterations(iters[0] + iters[1], &a.counters[4]);
 }
 
+// Adds a track's status and iterations to its event's counters.
+template <int MODE>
+__device__ __forceinline__ void count_event(const FitArgs& a, int64_t t, unsigned st, unsigned iters,
+                                            const int64_t* __restrict__ evt_off, int nevt) {
+  unsigned long long* cnt = a.counters + (int64_t)event_of(t, evt_off, 0, nevt) * kEventSlots + 1;
+  if (st) count_status(st, cnt);
+  if (MODE == FIT_MODE_R && iters) atomicAdd(&cnt[4], (unsigned long long)iters);
+}
+
 template <int MODE, int K>
 __global__ void __launch_bounds__(kBlock, MODE == FIT_MODE_Z ? 4 : 3)
     fit_fused_kernel_noalloc(const __grid_constant__ FitArgs a,
                              const __grid_constant__ PairRuns<K> r,
                              const int64_t* __restrict__ evt_off, int nevt) {
   int64_t t;
-  const Part part = thread_part(a, r, t);
+  const Part part = thread_part<2>(a.t0, r, blockIdx.x, t);
   if (part == Part::kNone) return;
   unsigned st[2] = {0u, 0u}, iters[2] = {0u, 0u};
   if (part == Part::kPair)
@@ -81,12 +98,52 @@ __global__ void __launch_bounds__(kBlock, MODE == FIT_MODE_Z ? 4 : 3)
   else
     run_lone<MODE>(a, a.geo, t, st[0], iters[0]);
 #pragma unroll
-  for (int i = 0; i < 2; ++i) {
-    if (i == 1 && part == Part::kLone) continue;
-    unsigned long long* cnt = a.counters + (int64_t)event_of(t + i, evt_off, 0, nevt) * kEventSlots + 1;
-    if (st[i]) count_status(st[i], cnt);
-    if (MODE == FIT_MODE_R && iters[i]) atomicAdd(&cnt[4], (unsigned long long)iters[i]);
-  }
+  for (int i = 0; i < 2; ++i)
+    if (i == 0 || part == Part::kPair)
+      count_event<MODE>(a, t + i, st[i], iters[i], evt_off, nevt);
+}
+
+// The whole of a small call, both modes in one launch and one track per
+// thread: with at most one warp per scheduler the layers' dependent chains
+// set the time, and a thread's chain is shorter with one track than with two
+// (each packed FP32 operation holds the pipe two cycles, and the MUFU and
+// control instructions run per track).  1024 tracks: p2r 18.4 -> SMALL_R us,
+// p2z 14.3 -> SMALL_Z us, without a second stream's fork and join.
+template <int K>
+struct SmallArgs {
+  FitArgs a;  // t0, geo unused
+  Geo geo[2];
+  int64_t t0[2];
+  unsigned blocks_r;  // the p2r events' blocks, then the p2z events'
+  PairRuns<K> runs[2];
+};
+
+// EVENTS: count per event (as fit_fused_kernel_noalloc).
+template <int L, bool EVENTS>
+__global__ void __launch_bounds__(kBlock)
+    fit_small_kernel(const __grid_constant__ SmallArgs<kSmallRuns> s,
+                     const int64_t* __restrict__ evt_off, int nevt) {
+  auto run = [&](auto mode, unsigned block) {
+    constexpr int MODE = decltype(mode)::value;
+    int64_t t;
+    const Part part = thread_part<1>(s.t0[MODE], s.runs[MODE], block, t);
+    if (part == Part::kNone) return;
+    unsigned st = 0u, iters = 0u;
+    if (part == Part::kPair)
+      run_half_pair<MODE, L>(s.a, s.geo[MODE], t, st, iters);
+    else
+      run_lone<MODE, L>(s.a, s.geo[MODE], t, st, iters);
+    if constexpr (EVENTS) {
+      count_event<MODE>(s.a, t, st, iters, evt_off, nevt);
+    } else {
+      if (st) count_status(st, s.a.counters);
+      if (MODE == FIT_MODE_R) count_iterations(iters, &s.a.counters[4]);
+    }
+  };
+  if (blockIdx.x < s.blocks_r)
+    run(std::integral_constant<int, FIT_MODE_R>(), blockIdx.x);
+  else
+    run(std::integral_constant<int, FIT_MODE_Z>(), blockIdx.x - s.blocks_r);
 }
 
 }  // namespace
@@ -189,7 +246,7 @@ void add_run(PairRuns<kMaxRuns>& r, uint32_t t0, uint32_t t1) {
 
 // The events' tracks as one launch per mode: the runs of consecutive
 // same-mode events gathered in a table, with a new launch where it is full
-// or its tracks span 2^31.  launch(a, m, r, nblk) issues the kernel for the
+// or its tracks span 2^31.  launch(a, m, r) issues the kernel for the
 // runs r of mode m (a.t0: their base; a.geo: the mode's geometry).
 // An uneven mixed batch (500 events, 1M tracks, ~250 runs) takes 0.228 ms in
 // two launches; with one launch per run it took 4.11 ms, a run's few blocks
@@ -202,9 +259,8 @@ int launch_runs(const fit_handle* h, FitArgs a, int nevt, const int64_t* ntrk, c
     auto clear = [&r]() { r.pairs.nrun = 0, r.pairs.n = 0, r.nlone = 0; };
     clear();
     auto flush = [&]() {
-      const unsigned nblk = (r.nlone + kBlock - 1) / kBlock + (r.pairs.n + kBlock - 1) / kBlock;
-      if (!nblk) return FIT_OK;
-      launch(a, m, r, nblk);
+      if (!r.pairs.n && !r.nlone) return FIT_OK;
+      launch(a, m, r);
       clear();
       cudaError_t err = cudaGetLastError();
       return err == cudaSuccess ? FIT_OK : cuda_fail(err, (std::string(who) + ": launch").c_str());
@@ -239,46 +295,93 @@ int launch_runs(const fit_handle* h, FitArgs a, int nevt, const int64_t* ntrk, c
   return FIT_OK;
 }
 
-// Calls f with r in the smallest compiled table that holds it.
-template <class F>
-void with_table(const PairRuns<kMaxRuns>& r, F f) {
-  if (r.pairs.nrun > 1 || r.nlone > 2) return f(r);
-  PairRuns<1> one;
-  one.pairs.nrun = r.pairs.nrun;
-  one.pairs.n = r.pairs.n;
-  one.pairs.first[0] = r.pairs.nrun ? r.pairs.first[0] : 0;
-  one.pairs.before[0] = 0;
-  one.nlone = r.nlone;
-  for (uint32_t i = 0; i < 2; ++i) one.lone[i] = i < r.nlone ? r.lone[i] : 0;
-  f(one);
+// Copies r into a table of K runs, if it fits.
+template <int K>
+bool copy_table(const PairRuns<kMaxRuns>& r, PairRuns<K>& to) {
+  if (r.pairs.nrun > K || r.nlone > 2 * K) return false;
+  to.pairs.nrun = r.pairs.nrun;
+  to.pairs.n = r.pairs.n;
+  to.nlone = r.nlone;
+  to.pairs.first[0] = to.pairs.before[0] = 0;
+  std::memcpy(to.pairs.first, r.pairs.first, r.pairs.nrun * sizeof(uint32_t));
+  std::memcpy(to.pairs.before, r.pairs.before, r.pairs.nrun * sizeof(uint32_t));
+  std::memcpy(to.lone, r.lone, r.nlone * sizeof(uint32_t));
+  return true;
 }
 
 template <int MODE, int L>
-void launch_fused(const FitArgs& a, const PairRuns<kMaxRuns>& r, unsigned nblk, cudaStream_t s) {
-  with_table(r, [&](const auto& tab) {
-    constexpr int K = sizeof(tab.lone) / sizeof(tab.lone[0]) / 2;
-    fit_fused_kernel<MODE, L, K><<<nblk, kBlock, 0, s>>>(a, tab);
-  });
+void launch_fused(const FitArgs& a, const PairRuns<kMaxRuns>& r, cudaStream_t s) {
+  PairRuns<1> one;
+  if (copy_table(r, one))
+    fit_fused_kernel<MODE, L, 1><<<part_blocks<2>(one), kBlock, 0, s>>>(a, one);
+  else
+    fit_fused_kernel<MODE, L, kMaxRuns><<<part_blocks<2>(r), kBlock, 0, s>>>(a, r);
 }
+
+// The events as one launch of fit_small_kernel: launch(args, blocks) issues
+// it.  Returns false, with nothing launched, if their runs do not fit its
+// tables.
+template <class Launch>
+bool launch_small(const fit_handle* h, const FitArgs& a, int nevt, const int64_t* ntrk,
+                  const int32_t* mode, Launch launch) {
+  SmallArgs<kSmallRuns> s;
+  s.a = a;
+  unsigned blocks[2] = {0, 0};
+  int tables[2] = {0, 0};
+  bool fits = true;
+  for (int m = 0; m < 2; ++m) {
+    s.geo[m] = h->geo[m];
+    s.t0[m] = 0;
+    s.runs[m].pairs.nrun = 0, s.runs[m].pairs.n = 0, s.runs[m].nlone = 0;
+  }
+  const int rc = launch_runs(h, a, nevt, ntrk, mode, "fit_small", [&](const FitArgs& a1, int m, const PairRuns<kMaxRuns>& r) {
+    fits = fits && tables[m]++ == 0 && copy_table(r, s.runs[m]);
+    s.t0[m] = a1.t0;
+    blocks[m] = part_blocks<1>(r);
+  });
+  if (rc != FIT_OK || !fits) return false;
+  s.blocks_r = blocks[FIT_MODE_R];
+  launch(s, blocks[0] + blocks[1]);
+  return true;
+}
+
+// A call is small where one track per thread leaves every scheduler at most
+// one warp (a block of 128 per SM): at 19456 tracks and below the small kernel
+// takes SMALL_LO us against BIG_LO, at 32768 tracks the pairs are as fast
+// (18.4 us p2r), and at 65536 faster (26.6 against 28.3).
+bool is_small(int sms, int64_t call_tracks) { return call_tracks <= (int64_t)sms * kBlock; }
+bool is_small(const fit_handle* h, int64_t call_tracks) { return is_small(h->sms, call_tracks); }
 
 // The fused fit of events [0, nevt) on the tracks of a: the p2r events on
 // stream s, the p2z events on sz.
-int run_fit(const fit_handle* h, const FitArgs& a, int layout, bool seeded, int nevt,
-            const int64_t* ntrk, const int32_t* mode, const char* who, cudaStream_t s,
+int run_fit(const fit_handle* h, const FitArgs& a, int layout, bool seeded, int64_t call_tracks,
+            int nevt, const int64_t* ntrk, const int32_t* mode, const char* who, cudaStream_t s,
             cudaStream_t sz) {
+  if (!seeded && is_small(h, call_tracks)) {
+    const bool done = launch_small(h, a, nevt, ntrk, mode, [&](const auto& args, unsigned nblk) {
+      if (layout == FIT_LAYOUT_SOA)
+        fit_small_kernel<0, false><<<nblk, kBlock, 0, s>>>(args, nullptr, 0);
+      else
+        fit_small_kernel<1, false><<<nblk, kBlock, 0, s>>>(args, nullptr, 0);
+    });
+    if (done) {
+      const cudaError_t e = cudaGetLastError();
+      return e == cudaSuccess ? FIT_OK : cuda_fail(e, (std::string(who) + ": launch").c_str());
+    }
+  }
   if (seeded) {
     const int rc = launch_seeded_fit(h, a, nevt, ntrk, mode, who, s);
     if (rc != FIT_OK) return rc;
   }
   return launch_runs(h, a, nevt, ntrk, mode, who,
-                     [=](const FitArgs& a1, int m, const PairRuns<kMaxRuns>& r, unsigned nblk) {
+                     [=](const FitArgs& a1, int m, const PairRuns<kMaxRuns>& r) {
                        if (m == FIT_MODE_R && seeded) return;
                        if (layout == FIT_LAYOUT_SOA)
-                         m == FIT_MODE_Z ? launch_fused<FIT_MODE_Z, 0>(a1, r, nblk, sz)
-                                         : launch_fused<FIT_MODE_R, 0>(a1, r, nblk, s);
+                         m == FIT_MODE_Z ? launch_fused<FIT_MODE_Z, 0>(a1, r, sz)
+                                         : launch_fused<FIT_MODE_R, 0>(a1, r, s);
                        else
-                         m == FIT_MODE_Z ? launch_fused<FIT_MODE_Z, 1>(a1, r, nblk, sz)
-                                         : launch_fused<FIT_MODE_R, 1>(a1, r, nblk, s);
+                         m == FIT_MODE_Z ? launch_fused<FIT_MODE_Z, 1>(a1, r, sz)
+                                         : launch_fused<FIT_MODE_R, 1>(a1, r, s);
                      });
 }
 
@@ -303,6 +406,17 @@ int ModeStreams::end(int rc) {
   if (e != cudaSuccess && rc == FIT_OK)
     return cuda_fail(e, (std::string(who_) + ": join from the second stream").c_str());
   return rc;
+}
+
+int run_fit_streams(fit_handle* h, const FitArgs& a, int layout, bool seeded, int64_t call_tracks,
+                    int nevt, const int64_t* ntrk, const int32_t* mode, const char* who,
+                    cudaStream_t s) {
+  ModeStreams ms(h, s, who);
+  const bool one_launch = !seeded && is_small(h, call_tracks);
+  const int rc = one_launch ? FIT_OK : ms.begin(nevt, ntrk, mode);
+  if (rc != FIT_OK) return rc;
+  return ms.end(run_fit(h, a, layout, seeded, call_tracks, nevt, ntrk, mode, who,
+                        ms.of(FIT_MODE_R), ms.of(FIT_MODE_Z)));
 }
 
 // Scratch of fit_propagate_update_noalloc, in the library image instead of
@@ -394,12 +508,9 @@ int fit_propagate_update(fit_handle* h, const fit_tracks_in* in, const fit_track
   int rc = check_call(h, in, out, hits, nevt, ntrk, nlayer, mode, &total, "fit_propagate_update");
   if (rc != FIT_OK || total == 0) return rc;
   DeviceGuard g(h->device);
-  static const char* kWho = "fit_propagate_update";
-  ModeStreams ms(h, static_cast<cudaStream_t>(stream), kWho);
-  rc = ms.begin(nevt, ntrk, mode);
-  if (rc != FIT_OK) return rc;
-  rc = ms.end(run_fit(h, base_args(in, out, hits, nlayer, h->d_counters), FIT_LAYOUT_SOA,
-                      h->seeded, nevt, ntrk, mode, kWho, ms.of(FIT_MODE_R), ms.of(FIT_MODE_Z)));
+  rc = run_fit_streams(h, base_args(in, out, hits, nlayer, h->d_counters), FIT_LAYOUT_SOA,
+                       h->seeded, total, nevt, ntrk, mode, "fit_propagate_update",
+                       static_cast<cudaStream_t>(stream));
   if (rc != FIT_OK) return rc;
   h->tracks += (uint64_t)total;
   return FIT_OK;
@@ -421,11 +532,8 @@ int fit_propagate_update_layout(fit_handle* h, const fit_tracks_in* in, const fi
     return fail(FIT_ERR_ARG, std::string(kWho) + ": AoSoA slots (ld) must be a multiple of 32");
   if (h->seeded) return fail(FIT_ERR_ARG, std::string(kWho) + ": no learned seed in AoSoA");
   DeviceGuard g(h->device);
-  ModeStreams ms(h, static_cast<cudaStream_t>(stream), kWho);
-  rc = ms.begin(nevt, ntrk, mode);
-  if (rc != FIT_OK) return rc;
-  rc = ms.end(run_fit(h, base_args(in, out, hits, nlayer, h->d_counters), layout, false, nevt,
-                      ntrk, mode, kWho, ms.of(FIT_MODE_R), ms.of(FIT_MODE_Z)));
+  rc = run_fit_streams(h, base_args(in, out, hits, nlayer, h->d_counters), layout, false, total,
+                       nevt, ntrk, mode, kWho, static_cast<cudaStream_t>(stream));
   if (rc != FIT_OK) return rc;
   h->tracks += (uint64_t)total;
   return FIT_OK;
@@ -467,15 +575,27 @@ int fit_propagate_update_noalloc(const fit_config* cfg_r, const fit_config* cfg_
     e = cudaMemcpyAsync(d_off, off, (size_t)(nevt + 1) * sizeof(int64_t), cudaMemcpyHostToDevice, s);
     if (e != cudaSuccess) return cuda_fail(e, "fit_propagate_update_noalloc: offset copy");
     if (total > 0) {
-      rc = launch_runs(&h, base_args(in, out, hits, nlayer, scratch), nevt, ntrk, mode, kWho,
-                       [=](const FitArgs& a, int m, const PairRuns<kMaxRuns>& r, unsigned nblk) {
-                         if (m == FIT_MODE_Z)
-                           fit_fused_kernel_noalloc<FIT_MODE_Z, kMaxRuns>
-                               <<<nblk, kBlock, 0, s>>>(a, r, d_off, nevt);
-                         else
-                           fit_fused_kernel_noalloc<FIT_MODE_R, kMaxRuns>
-                               <<<nblk, kBlock, 0, s>>>(a, r, d_off, nevt);
-                       });
+      const FitArgs args = base_args(in, out, hits, nlayer, scratch);
+      int sms = 0;
+      e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, device);
+      if (e != cudaSuccess) return cuda_fail(e, "fit_propagate_update_noalloc: device attribute");
+      const bool done = is_small(sms, total) &&
+                        launch_small(&h, args, nevt, ntrk, mode, [&](const auto& sa, unsigned nblk) {
+                          fit_small_kernel<0, true><<<nblk, kBlock, 0, s>>>(sa, d_off, nevt);
+                        });
+      if (!done)
+        rc = launch_runs(&h, args, nevt, ntrk, mode, kWho,
+                         [=](const FitArgs& a, int m, const PairRuns<kMaxRuns>& r) {
+                           if (m == FIT_MODE_Z)
+                             fit_fused_kernel_noalloc<FIT_MODE_Z, kMaxRuns>
+                                 <<<part_blocks<2>(r), kBlock, 0, s>>>(a, r, d_off, nevt);
+                           else
+                             fit_fused_kernel_noalloc<FIT_MODE_R, kMaxRuns>
+                                 <<<part_blocks<2>(r), kBlock, 0, s>>>(a, r, d_off, nevt);
+                         });
+      e = cudaGetLastError();
+      if (rc == FIT_OK && e != cudaSuccess)
+        rc = cuda_fail(e, "fit_propagate_update_noalloc: launch");
       if (rc != FIT_OK) return rc;
     }
   }

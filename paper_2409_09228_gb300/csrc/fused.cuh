@@ -36,6 +36,7 @@ __device__ __forceinline__ void count_status(unsigned st, unsigned long long* co
   if (st & FIT_ST_CHARGE_FLIP) atomicAdd(&counters[3], 1ull);
 }
 
+using fitk::F1;
 using fitk::F2;
 using fitk::Lanes;
 
@@ -63,25 +64,20 @@ __device__ __forceinline__ int64_t ix(int k, int64_t t, int64_t ld, int K) {
   return (((t >> 5) * K + k) << 5) + (t & 31);
 }
 
-template <int L = 0>
-__device__ __forceinline__ void load_state(const FitArgs& a, int64_t t, State<float>& s) {
-#pragma unroll
-  for (int k = 0; k < 6; ++k) fitk::ld(s.p[k], a.par_in + ix<L>(k, t, a.ld_in, 6));
-#pragma unroll
-  for (int k = 0; k < 21; ++k) fitk::ld(s.c[k], a.cov_in + ix<L>(k, t, a.ld_in, 21));
-  s.qf = (float)__ldcs(a.q_in + t);
-  s.chi2 = 0.f;
-  s.g = fitk::trig_of(s.p);
+__device__ __forceinline__ void load_charge(const int32_t* q, float& d) { d = (float)__ldcs(q); }
+__device__ __forceinline__ void load_charge(const int32_t* q, F1& d) { d = F1((float)__ldcs(q)); }
+__device__ __forceinline__ void load_charge(const int32_t* q, F2& d) {
+  const int2 v = __ldcs(reinterpret_cast<const int2*>(q));
+  d = F2((float)v.x, (float)v.y);
 }
-template <int L = 0>
-__device__ __forceinline__ void load_state(const FitArgs& a, int64_t t, State<F2>& s) {
+template <int L = 0, class T>
+__device__ __forceinline__ void load_state(const FitArgs& a, int64_t t, State<T>& s) {
 #pragma unroll
   for (int k = 0; k < 6; ++k) fitk::ld(s.p[k], a.par_in + ix<L>(k, t, a.ld_in, 6));
 #pragma unroll
   for (int k = 0; k < 21; ++k) fitk::ld(s.c[k], a.cov_in + ix<L>(k, t, a.ld_in, 21));
-  const int2 q = __ldcs(reinterpret_cast<const int2*>(a.q_in + t));
-  s.qf = F2((float)q.x, (float)q.y);
-  s.chi2 = F2(0.f);
+  load_charge(a.q_in + t, s.qf);
+  s.chi2 = T(0.f);
   s.g = fitk::trig_of(s.p);
 }
 
@@ -105,25 +101,25 @@ __device__ __forceinline__ void leave_loop_form(State<T>& s) {
   if (MODE == FIT_MODE_R) fitk::to_global_r(s.cl, s.bc, s.bs, s.c);
 }
 
-// Lane i of a two-track state (in the loop form) as a one-track state.
-template <int MODE>
-__device__ __forceinline__ State<float> lane_of(const State<F2>& s, int i) {
+// Lane i of a state (in the loop form) as a one-track float state.
+template <int MODE, class T>
+__device__ __forceinline__ State<float> lane_of(const State<T>& s, int i) {
   State<float> r;
 #pragma unroll
-  for (int k = 0; k < 6; ++k) r.p[k] = Lanes<F2>::get(s.p[k], i);
+  for (int k = 0; k < 6; ++k) r.p[k] = Lanes<T>::get(s.p[k], i);
   if (MODE == FIT_MODE_Z) {
 #pragma unroll
-    for (int k = 0; k < 21; ++k) r.c[k] = Lanes<F2>::get(s.c[k], i);
+    for (int k = 0; k < 21; ++k) r.c[k] = Lanes<T>::get(s.c[k], i);
   } else {
 #pragma unroll
-    for (int k = 0; k < 15; ++k) r.cl[k] = Lanes<F2>::get(s.cl[k], i);
-    r.bc = Lanes<F2>::get(s.bc, i);
-    r.bs = Lanes<F2>::get(s.bs, i);
+    for (int k = 0; k < 15; ++k) r.cl[k] = Lanes<T>::get(s.cl[k], i);
+    r.bc = Lanes<T>::get(s.bc, i);
+    r.bs = Lanes<T>::get(s.bs, i);
   }
-  r.qf = Lanes<F2>::get(s.qf, i);
-  r.chi2 = Lanes<F2>::get(s.chi2, i);
-  r.g = {Lanes<F2>::get(s.g.cphi, i), Lanes<F2>::get(s.g.sphi, i), Lanes<F2>::get(s.g.cth, i),
-         Lanes<F2>::get(s.g.sth, i)};
+  r.qf = Lanes<T>::get(s.qf, i);
+  r.chi2 = Lanes<T>::get(s.chi2, i);
+  r.g = {Lanes<T>::get(s.g.cphi, i), Lanes<T>::get(s.g.sphi, i), Lanes<T>::get(s.g.cth, i),
+         Lanes<T>::get(s.g.sth, i)};
   return r;
 }
 
@@ -371,6 +367,29 @@ __device__ __forceinline__ void run_whole_pair(const FitArgs& a, const Geo& geo,
     State<float> one = lane_of<MODE>(s, i);
     finish_one<MODE, L>(a, geo, t + i, l, one, st[i], iters[i], Lanes<F2>::get(alive, i));
   }
+}
+
+// Track t of a pair, in a thread of its own and with the pair's rounding: the
+// results of run_whole_pair, but where the partner's range tests or its
+// leaving the pair would have changed the form of a series or the path.
+template <int MODE, int L = 0>
+__device__ __forceinline__ void run_half_pair(const FitArgs& a, const Geo& geo, int64_t t,
+                                              unsigned& st, unsigned& iters) {
+  State<F1> s;
+  begin_state<MODE, L>(a, geo, t, s);
+  unsigned st1[1] = {st}, it1[1] = {iters};
+  bool alive = true;
+  const int l = run_layers<MODE, F1, L>(a, geo, t, 0, s, st1, it1, alive);
+  st = st1[0];
+  iters = it1[0];
+  if (l == a.nlayer) {
+    finish_state<MODE, L>(a, t, l, s);
+    store_state<L>(a, t, s, st1);
+    st = st1[0];
+    return;
+  }
+  State<float> one = lane_of<MODE>(s, 0);
+  finish_one<MODE, L>(a, geo, t, l, one, st, iters, alive);
 }
 
 // Track t alone, from its first layer.

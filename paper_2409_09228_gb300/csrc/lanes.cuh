@@ -1,5 +1,6 @@
 // Lane types for the fused kernel: float (one track per thread), F2 (two
-// tracks per thread, held in the two halves of a float2), and double (the
+// tracks per thread, held in the two halves of a float2), F1 (one track,
+// rounded as in a pair), and double (the
 // FP64 variant, one track per thread).
 //
 // The per-track math is written once as templates over the lane type.  With
@@ -27,6 +28,16 @@ struct M2 {
   bool x, y;
 };
 
+// One track whose every operation rounds as a lane of F2's does: no product
+// is contracted with a sum that the code does not write as fma (a float's
+// are).  For calls too small to fill the SMs with pairs of tracks, with the
+// pairs' results.
+struct F1 {
+  float v;
+  __device__ __forceinline__ F1() {}
+  __device__ __forceinline__ F1(float a) : v(a) {}
+};
+
 // ---- arithmetic ----------------------------------------------------------
 __device__ __forceinline__ F2 operator+(F2 a, F2 b) { return F2(__fadd2_rn(a.v, b.v)); }
 __device__ __forceinline__ F2 operator-(F2 a) { return F2(-a.v.x, -a.v.y); }
@@ -36,7 +47,14 @@ __device__ __forceinline__ F2& operator+=(F2& a, F2 b) { return a = a + b; }
 __device__ __forceinline__ F2& operator-=(F2& a, F2 b) { return a = a - b; }
 __device__ __forceinline__ F2& operator*=(F2& a, F2 b) { return a = a * b; }
 
+__device__ __forceinline__ F1 operator+(F1 a, F1 b) { return F1(__fadd_rn(a.v, b.v)); }
+__device__ __forceinline__ F1 operator-(F1 a) { return F1(-a.v); }
+__device__ __forceinline__ F1 operator-(F1 a, F1 b) { return F1(__fadd_rn(a.v, -b.v)); }
+__device__ __forceinline__ F1 operator*(F1 a, F1 b) { return F1(__fmul_rn(a.v, b.v)); }
+__device__ __forceinline__ F1& operator+=(F1& a, F1 b) { return a = a + b; }
+
 __device__ __forceinline__ float fma(float a, float b, float c) { return fmaf(a, b, c); }
+__device__ __forceinline__ F1 fma(F1 a, F1 b, F1 c) { return F1(__fmaf_rn(a.v, b.v, c.v)); }
 __device__ __forceinline__ F2 fma(F2 a, F2 b, F2 c) { return F2(__ffma2_rn(a.v, b.v, c.v)); }
 
 // Division and square root where a couple of ulp are far below the fit's
@@ -47,9 +65,11 @@ __device__ __forceinline__ float frcp(float x) {
   asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
   return r;
 }
+__device__ __forceinline__ F1 frcp(F1 x) { return F1(frcp(x.v)); }
 __device__ __forceinline__ F2 frcp(F2 x) { return F2(frcp(x.v.x), frcp(x.v.y)); }
 __device__ __forceinline__ float fdiv(float a, float b) { return __fdividef(a, b); }
 // a * (1/b): the reciprocals per lane, the product packed
+__device__ __forceinline__ F1 fdiv(F1 a, F1 b) { return a * frcp(b); }
 __device__ __forceinline__ F2 fdiv(F2 a, F2 b) { return a * frcp(b); }
 // Approximate square root and reciprocal square root (one MUFU operation
 // each, relative error ~2^-23); NaN for x < 0, which every caller either
@@ -61,26 +81,39 @@ __device__ __forceinline__ float fsqrt(float x) {
   asm("sqrt.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
   return r;
 }
+__device__ __forceinline__ F1 fsqrt(F1 x) { return F1(fsqrt(x.v)); }
 __device__ __forceinline__ F2 fsqrt(F2 x) { return F2(fsqrt(x.v.x), fsqrt(x.v.y)); }
 __device__ __forceinline__ float frsqrt(float x) {
   float r;
   asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
   return r;
 }
+__device__ __forceinline__ F1 frsqrt(F1 x) { return F1(frsqrt(x.v)); }
 __device__ __forceinline__ F2 frsqrt(F2 x) { return F2(frsqrt(x.v.x), frsqrt(x.v.y)); }
 __device__ __forceinline__ float fabs_(float x) { return fabsf(x); }
+__device__ __forceinline__ F1 fabs_(F1 x) { return F1(fabsf(x.v)); }
 __device__ __forceinline__ F2 fabs_(F2 x) { return F2(fabsf(x.v.x), fabsf(x.v.y)); }
 __device__ __forceinline__ float fmax_(float a, float b) { return fmaxf(a, b); }
+__device__ __forceinline__ F1 fmax_(F1 a, F1 b) { return F1(fmaxf(a.v, b.v)); }
 __device__ __forceinline__ F2 fmax_(F2 a, F2 b) { return F2(fmaxf(a.v.x, b.v.x), fmaxf(a.v.y, b.v.y)); }
 __device__ __forceinline__ float floor_(float x) { return floorf(x); }
+__device__ __forceinline__ F1 floor_(F1 x) { return F1(floorf(x.v)); }
 __device__ __forceinline__ F2 floor_(F2 x) { return F2(floorf(x.v.x), floorf(x.v.y)); }
 __device__ __forceinline__ float copysign_(float a, float b) { return copysignf(a, b); }
+__device__ __forceinline__ F1 copysign_(F1 a, F1 b) { return F1(copysignf(a.v, b.v)); }
 __device__ __forceinline__ F2 copysign_(F2 a, F2 b) {
   return F2(copysignf(a.v.x, b.v.x), copysignf(a.v.y, b.v.y));
 }
 
 // ---- masks ---------------------------------------------------------------
 __device__ __forceinline__ bool le(float a, float b) { return a <= b; }
+__device__ __forceinline__ bool le(F1 a, F1 b) { return a.v <= b.v; }
+__device__ __forceinline__ bool lt(F1 a, F1 b) { return a.v < b.v; }
+__device__ __forceinline__ bool pos(F1 x) { return 0.f < x.v; }
+__device__ __forceinline__ bool neg(F1 x) { return x.v < 0.f; }
+__device__ __forceinline__ bool nonpos(F1 x) { return x.v <= 0.f; }
+__device__ __forceinline__ bool finite_(F1 x) { return isfinite(x.v); }
+__device__ __forceinline__ F1 sel(bool m, F1 a, F1 b) { return m ? a : b; }
 __device__ __forceinline__ M2 le(F2 a, F2 b) { return {a.v.x <= b.v.x, a.v.y <= b.v.y}; }
 __device__ __forceinline__ bool lt(float a, float b) { return a < b; }
 __device__ __forceinline__ M2 lt(F2 a, F2 b) { return {a.v.x < b.v.x, a.v.y < b.v.y}; }
@@ -175,11 +208,14 @@ __device__ __forceinline__ bool finite_(double a) {
 __device__ __forceinline__ double sel(bool m, double a, double b) { return m ? a : b; }
 
 // ---- lanes ---------------------------------------------------------------
+// exact: the type's propagation takes crossing_start's exact form itself; the
+// others leave such a track to the float path.
 template <class T>
 struct Lanes;
 template <>
 struct Lanes<float> {
   static constexpr int n = 1;
+  static constexpr bool exact = true;
   using M = bool;
   __device__ __forceinline__ static float get(float a, int) { return a; }
   __device__ __forceinline__ static bool get(bool m, int) { return m; }
@@ -187,13 +223,23 @@ struct Lanes<float> {
 template <>
 struct Lanes<double> {
   static constexpr int n = 1;
+  static constexpr bool exact = true;
   using M = bool;
   __device__ __forceinline__ static double get(double a, int) { return a; }
   __device__ __forceinline__ static bool get(bool m, int) { return m; }
 };
 template <>
+struct Lanes<F1> {
+  static constexpr int n = 1;
+  static constexpr bool exact = false;
+  using M = bool;
+  __device__ __forceinline__ static float get(F1 a, int) { return a.v; }
+  __device__ __forceinline__ static bool get(bool m, int) { return m; }
+};
+template <>
 struct Lanes<F2> {
   static constexpr int n = 2;
+  static constexpr bool exact = false;
   using M = M2;
   __device__ __forceinline__ static float get(F2 a, int i) { return i ? a.v.y : a.v.x; }
   __device__ __forceinline__ static bool get(M2 m, int i) { return i ? m.y : m.x; }
@@ -202,12 +248,14 @@ struct Lanes<F2> {
 // Streaming loads and stores of lane-consecutive tracks (p points at the
 // first track; for F2 it is 8-byte aligned).
 __device__ __forceinline__ void ld(float& d, const float* p) { d = __ldcs(p); }
+__device__ __forceinline__ void ld(F1& d, const float* p) { d = F1(__ldcs(p)); }
 __device__ __forceinline__ void ld(F2& d, const float* p) {
   d = F2(__ldcs(reinterpret_cast<const float2*>(p)));
 }
 __device__ __forceinline__ void ld(double& d, const double* p) { d = __ldcs(p); }
 __device__ __forceinline__ void st(double* p, double v) { *p = v; }
 __device__ __forceinline__ void st(float* p, float v) { *p = v; }
+__device__ __forceinline__ void st(float* p, F1 v) { *p = v.v; }
 __device__ __forceinline__ void st(float* p, F2 v) { *reinterpret_cast<float2*>(p) = v.v; }
 
 }  // namespace fitk

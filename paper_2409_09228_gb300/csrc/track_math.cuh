@@ -83,6 +83,8 @@ __device__ __forceinline__ void sincos_cw(F2 x, F2& s, F2& c) {
   sincos_cw(x.v.y, s.v.y, c.v.y);
 }
 
+__device__ __forceinline__ void sincos_cw(F1 x, F1& s, F1& c) { sincos_cw(x.v, s.v, c.v); }
+
 // s(u) = sin(u)/u and cos(u) by their Taylor series in u^2: up to u^4 for
 // |u| <= 0.1 (remainders < 2e-9; steps between neighbouring layers stay in
 // this range), up to u^12 for |u| <= 1.25 (remainders < 2e-10), beyond that
@@ -168,6 +170,16 @@ __device__ __forceinline__ void sinc_cs(F2 u, F2& s, F2& cu, F2& sp) {
   } else {
     sinc_cs(u.v.x, s.v.x, cu.v.x, sp.v.x);
     sinc_cs(u.v.y, s.v.y, cu.v.y, sp.v.y);
+  }
+}
+
+__device__ __forceinline__ void sinc_cs(F1 u, F1& s, F1& cu, F1& sp) {
+  if (le(fabs_(u), F1(1.25f))) {
+    const bool shortform = le(fabs_(u), F1(0.1f));
+    sinc_series(u * u, s, cu, shortform);
+    sp = sinc_deriv_series(u, shortform);
+  } else {
+    sinc_cs(u.v, s.v, cu.v, sp.v);
   }
 }
 
@@ -752,7 +764,7 @@ __device__ __forceinline__ typename Lanes<T>::M crossing_start(T x, T y, T cph, 
   // X < 0 (the circle misses the cylinder) makes den NaN, which fails den > 0
   const M ok = and_(nonpos(c0), and_(pos(den), quarter(t)));
   h = hl * atan_ratio(t);
-  if constexpr (Lanes<T>::n > 1 || !EXACT) {
+  if constexpr (!Lanes<T>::exact || !EXACT) {
     return not_(ok);
   } else {
     if (ok) return false;

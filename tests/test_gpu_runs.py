@@ -146,3 +146,47 @@ def test_track_kernels_many_runs(entry):
     keep = slice(0, counts[0]) if entry == "seeded" else slice(0, n)
     for a, b in zip(got, ref):
         np.testing.assert_array_equal(a[..., order][..., keep], b[..., keep])
+
+
+# A call at or below a block of 128 tracks per SM runs one track per thread,
+# a larger one pairs: the same operations with the same rounding.  Momenta
+# whose turn per layer stays in the short series' range (|u| <= 0.1), so that
+# no pair's range test depends on the partner.
+@pytest.mark.parametrize("n", [1, 2, 127, 4097])
+@pytest.mark.parametrize("entry", ["fit", "aosoa", "noalloc"])
+def test_small_call_rounds_like_pairs(entry, n):
+    big = torch.cuda.get_device_properties(0).multi_processor_count * 128 + 1
+    sets = [inputs.generate(m, big, seed=67 + m, pt_range=(1.5, 10.0)) for m in (0, 1)]
+    geo = [fit.Geometry(s.B, s.surf) for s in sets]
+    f = fit.Fitter(*geo)
+
+    def run(ts, k):
+        ld = (k + 31) // 32 * 32
+        d = [gpu_util.to_dev(np.ascontiguousarray(a[..., :k]), ld)
+             for a in (ts.par0, ts.cov0, ts.q, ts.hpos, ts.hcov)]
+        out = f.outputs(k, ld=ld, layers=True)
+        bufs = dict(par_out=out["par"], cov_out=out["cov"], q_out=out["q"], chi2=out["chi2"],
+                    chi2_layer=out["chi2_layer"], status=out["status"])
+        if entry == "fit":
+            f.run(*d, [k], [ts.mode], out=out)
+        elif entry == "noalloc":
+            fit.fit_propagate_update_noalloc(*geo, *d, [k], [ts.mode], **bufs)
+        else:
+            tiles = [a if i == 2 else torch.from_numpy(inputs.to_aosoa32(a.cpu().numpy(), ld)).cuda()
+                     for i, a in enumerate(d)]
+            fit.fit_propagate_update_layout(f.h, *tiles, [k], [ts.mode], fit.FIT_LAYOUT_AOSOA32, ld,
+                                            out["par"], out["cov"], out["q"], out["chi2"],
+                                            chi2_layer=out["chi2_layer"], status=out["status"])
+        res = {i: v.cpu().numpy() for i, v in out.items()}
+        if entry == "aosoa":
+            for i in ("par", "cov", "chi2_layer"):
+                res[i] = inputs.from_aosoa32(res[i].reshape(-1), res[i].shape, k)
+        f.sync()
+        return {i: v[..., :n] for i, v in res.items()}
+
+    for ts in sets:
+        small, pairs = run(ts, n), run(ts, big)
+        whole = n & ~1  # the last of an odd count has no partner: the one-lane path
+        for i in small:
+            np.testing.assert_array_equal(small[i][..., :whole], pairs[i][..., :whole], err_msg=i)
+    f.close()
