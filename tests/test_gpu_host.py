@@ -145,3 +145,33 @@ def test_mapped_path_is_bit_identical_and_checks_its_pointers():
         assert torch.equal(before, hout["chi2"])
     finally:
         f.close()
+
+
+@pytest.mark.parametrize("pageable", ["all", "hits", "status"])
+def test_staged_chunks_are_bit_identical_to_device_path(pageable):
+    """Any pageable buffer sends the call through the staging sets: two whole
+    chunks and a small last one, events of both modes straddling their edges."""
+    nt = np.array([200001, 130000, 150003, 50000])
+    md = np.array([0, 1, 0, 1], np.int32)
+    ev = inputs.generate_events(nt, md, seed=113, nlayer=4)
+    n, ld = ev.n, gpu_util.pad_ld(ev.n)
+    assert 2 * fit.FIT_HOST_CHUNK < n < 3 * fit.FIT_HOST_CHUNK
+    f = fit.Fitter(fit.Geometry(ev.B, ev.surf[0]), fit.Geometry(ev.B, ev.surf[1]))
+    try:
+        d = [gpu_util.to_dev(a, ld) for a in (ev.par0, ev.cov0, ev.q, ev.hpos, ev.hcov)]
+        dev = f.run(*d, ev.ntrk, ev.mode, layers=True)
+        st_dev = f.sync()
+        hin, hout = _host(ev, ld, pageable != "all"), _host_out(n, ld, 4, pageable != "all")
+        if pageable == "hits":
+            hin[3] = hin[3].numpy().copy()
+        elif pageable == "status":
+            hout["status"] = hout["status"].numpy().copy()
+        fit.fit_propagate_update_host(f.h, *hin, ev.ntrk, ev.mode, par_out=hout["par"],
+                                      cov_out=hout["cov"], q_out=hout["q"], chi2=hout["chi2"],
+                                      chi2_layer=hout["chi2_layer"], status=hout["status"])
+        assert f.sync() == st_dev
+        for k in ("par", "cov", "q", "chi2", "chi2_layer", "status"):
+            a, b = dev[k].cpu().numpy()[..., :n], _np(hout[k], n)
+            assert np.array_equal(a.view(np.uint8), b.view(np.uint8)), k
+    finally:
+        f.close()
