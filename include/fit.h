@@ -210,19 +210,24 @@ int fit_propagate_update_noalloc(const fit_config* cfg_r, const fit_config* cfg_
                                  const int32_t* mode, void* stream, fit_status* per_event);
 
 /*
- * Batched form (many events of uneven size and mixed modes in one launch).
+ * Batched form (many events of uneven size and mixed modes).
  *
- * A plan fixes the event structure (ntrk[], mode[], nlayer) once.  Its work is
- * cut into items -- tiles of one event, 2 x threads_per_block tracks -- that a
- * persistent kernel's blocks pull from a counter until none is left, so the
- * uneven events and the two surface types share one launch.  fit_plan_run
- * captures that launch (and the counter reset) in a CUDA graph the first time
- * it sees a set of buffers and replays the graph afterwards.  The results are
- * those of fit_propagate_update on the same events.
+ * A plan fixes the event structure (ntrk[], mode[], nlayer) once.  Left at the
+ * default shape it runs fit_propagate_update's kernels, one launch per mode
+ * side by side.  In the persistent form its work is cut into items -- tiles of
+ * one event, 2 x threads_per_block tracks -- that a persistent kernel's blocks
+ * pull from a counter until none is left, so the uneven events and the two
+ * surface types share one launch.  fit_plan_run captures the launches (and the
+ * counter reset) in a CUDA graph the first time it sees a set of buffers and
+ * replays the graph afterwards.  The results are those of fit_propagate_update
+ * on the same events.
  */
 typedef struct {
   int threads_per_block; /* 32, 64, 128 or 256 (64, 128 or 256 with one track per thread) */
-  int blocks_per_sm;     /* grid = blocks_per_sm x SM count; 0 = as many as fit */
+  int blocks_per_sm;     /* grid = blocks_per_sm x SM count; 0 = as many as fit, or,
+                            with 128 threads and two tracks per thread, one
+                            launch per mode until the plan is tuned (faster
+                            than any persistent shape measured) */
   int persistent;        /* 1: one persistent launch; 0: one launch per mode
                             (fit_propagate_update's form) */
   int tracks_per_thread; /* 2 (or 0, a zeroed struct): two tracks per thread in
@@ -249,8 +254,8 @@ typedef struct fit_plan fit_plan;
 /*
  * fit_plan_create: a plan for nevt events (ntrk, mode: HOST arrays, copied).
  * cfg may be NULL (persistent, 128 threads per block, two tracks per thread,
- * as many blocks per SM as fit).  The plan allocates its work-item table and a counter on the
- * handle's device.  Errors: FIT_ERR_ARG, FIT_ERR_NOMEM, FIT_ERR_CUDA.
+ * blocks_per_sm 0).  The plan allocates a counter and, for the persistent
+ * form, its work-item table on the handle's device.  Errors: FIT_ERR_ARG, FIT_ERR_NOMEM, FIT_ERR_CUDA.
  */
 int fit_plan_create(fit_handle* h, int nevt, const int64_t* ntrk, const int32_t* mode, int nlayer,
                     const fit_launch_config* cfg, fit_plan** plan);

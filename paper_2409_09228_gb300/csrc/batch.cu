@@ -225,13 +225,21 @@ struct fit_plan {
   int64_t total = 0;
   fit_launch_config cfg{128, 0, 1, 2, FIT_LAYOUT_SOA};
   bool layout_free = false;  // created with FIT_LAYOUT_TUNE and not tuned yet
+  // Created with the default shape and blocks_per_sm 0, and not tuned: the
+  // plan runs the fused kernels on its events (same pairs as the persistent
+  // form), one launch per mode.  Each mode then has its own registers (127
+  // and 156 instead of 168), p2z its staged hits, and no block waits for the
+  // work counter: 2000 uneven mixed events,
+  // 4M tracks, 1045 -> 853 us.
+  bool free_form = false;
   int sms = 0;
   WorkItem* d_items = nullptr;
   int nitems = 0;
   int items_tile = 0;  // tracks per work item of the current table
   int items_tpt = 0;
   unsigned* d_work = nullptr;
-  cudaStream_t cap = nullptr;
+  cudaStream_t cap = nullptr, cap_z = nullptr;  // capture streams
+  cudaEvent_t fork = nullptr, join = nullptr;
   cudaGraphExec_t exec = nullptr;
   const void* key_ptrs[12] = {};
   unsigned long long* d_tune_counters = nullptr;  // counters of the tuning runs
@@ -276,9 +284,31 @@ int build_items(fit_plan* p, int tpb, int tpt) {
   return FIT_OK;
 }
 
+// The fused kernels on the plan's events: the p2z launch on the plan's second
+// capture stream, a branch of the graph beside the p2r launch.
+int issue_per_mode(fit_plan* p, const FitArgs& base, bool by_event, cudaStream_t s) {
+  const bool one_launch = is_small(p->h, p->total);
+  cudaError_t e = cudaSuccess;
+  if (!one_launch) {
+    e = cudaEventRecord(p->fork, s);
+    if (e == cudaSuccess) e = cudaStreamWaitEvent(p->cap_z, p->fork, 0);
+    if (e != cudaSuccess) return cuda_fail(e, "fit_plan: fork");
+  }
+  const int rc = run_fit(p->h, base, {p->cfg.layout, false, by_event, p->total},
+                         (int)p->ntrk.size(), p->ntrk.data(), p->mode.data(), "fit_plan", s,
+                         p->cap_z);
+  if (!one_launch) {
+    e = cudaEventRecord(p->join, p->cap_z);
+    if (e == cudaSuccess) e = cudaStreamWaitEvent(s, p->join, 0);
+    if (e != cudaSuccess && rc == FIT_OK) return cuda_fail(e, "fit_plan: join");
+  }
+  return rc;
+}
+
 // Issues the plan's work for one shape on stream s (captured into a graph).
 int issue(fit_plan* p, const FitArgs& base, cudaStream_t s) {
   if (p->total == 0) return FIT_OK;
+  if (p->free_form) return issue_per_mode(p, base, true, s);
   if (p->cfg.persistent) {
     BatchArgs b{};
     b.a = base;
@@ -298,10 +328,8 @@ int issue(fit_plan* p, const FitArgs& base, cudaStream_t s) {
     if (e != cudaSuccess) return cuda_fail(e, "fit_plan: launch");
     return FIT_OK;
   }
-  // fit_propagate_update's form, one launch per mode: kept as an autotuner
-  // candidate (for few, large events it can win)
-  return run_fit(p->h, base, p->cfg.layout, false, p->total, (int)p->ntrk.size(),
-                 p->ntrk.data(), p->mode.data(), "fit_plan", s, s);
+  // fit_propagate_update's form, one launch per mode: an autotuner candidate
+  return issue_per_mode(p, base, false, s);
 }
 
 void drop_graph(fit_plan* p) {
@@ -322,7 +350,9 @@ int run_graph(fit_plan* p, const fit_tracks_in* in, const fit_tracks_out* out,
                     std::memcmp(lds, p->key_ld, sizeof(lds)) == 0;
   if (!same) {
     drop_graph(p);
-    int rc = build_items(p, p->cfg.threads_per_block, tracks_per_thread(p->cfg));
+    int rc = FIT_OK;
+    if (p->cfg.persistent && !p->free_form)
+      rc = build_items(p, p->cfg.threads_per_block, tracks_per_thread(p->cfg));
     if (rc != FIT_OK) return rc;
     cudaGraph_t graph = nullptr;
     cudaError_t e = cudaStreamBeginCapture(p->cap, cudaStreamCaptureModeThreadLocal);
@@ -419,6 +449,8 @@ int fit_plan_create(fit_handle* h, int nevt, const int64_t* ntrk, const int32_t*
   p->layout_free = p->cfg.layout == FIT_LAYOUT_TUNE;
   p->cfg.layout = run_layout;
   p->cfg.tracks_per_thread = tracks_per_thread(p->cfg);
+  p->free_form = p->cfg.persistent && p->cfg.blocks_per_sm == 0 &&
+                 p->cfg.threads_per_block == 128 && p->cfg.tracks_per_thread == 2;
   if (p->cfg.blocks_per_sm == 0)
     p->cfg.blocks_per_sm =
         max_blocks_per_sm(p->cfg.threads_per_block, p->cfg.tracks_per_thread, p->cfg.layout);
@@ -426,11 +458,16 @@ int fit_plan_create(fit_handle* h, int nevt, const int64_t* ntrk, const int32_t*
   e = cudaMalloc(&p->d_work, sizeof(unsigned));
   if (e == cudaSuccess) e = cudaMalloc(&p->d_tune_counters, kCounters * sizeof(unsigned long long));
   if (e == cudaSuccess) e = cudaStreamCreateWithFlags(&p->cap, cudaStreamNonBlocking);
+  if (e == cudaSuccess) e = cudaStreamCreateWithFlags(&p->cap_z, cudaStreamNonBlocking);
+  if (e == cudaSuccess) e = cudaEventCreateWithFlags(&p->fork, cudaEventDisableTiming);
+  if (e == cudaSuccess) e = cudaEventCreateWithFlags(&p->join, cudaEventDisableTiming);
   if (e != cudaSuccess) {
     fit_plan_destroy(p);
     return fail(FIT_ERR_NOMEM, std::string("fit_plan_create: ") + cudaGetErrorString(e));
   }
-  int rc = build_items(p, p->cfg.threads_per_block, p->cfg.tracks_per_thread);
+  const int rc = p->free_form || !p->cfg.persistent
+                     ? FIT_OK
+                     : build_items(p, p->cfg.threads_per_block, p->cfg.tracks_per_thread);
   if (rc != FIT_OK) {
     fit_plan_destroy(p);
     return rc;
@@ -480,7 +517,7 @@ int fit_plan_tune(fit_plan* p, const fit_tracks_in* in, const fit_tracks_out* ou
   if (have && batched_kernel(found.threads_per_block, tracks_per_thread(found), found.layout)) {
     drop_graph(p);
     p->cfg = found;
-    p->layout_free = false;
+    p->layout_free = p->free_form = false;
     p->tuned = 2;
     p->best_ms = 0.f;
     return FIT_OK;
@@ -546,6 +583,8 @@ int fit_plan_tune(fit_plan* p, const fit_tracks_in* in, const fit_tracks_out* ou
   }
   float best = 1e30f;
   fit_launch_config best_cfg = p->cfg;
+  const bool was_free = p->free_form;
+  p->free_form = false;
   for (const fit_launch_config& c : cands) {
     const bool own = c.layout == in_layout;
     const fit_tracks_in* ci = own ? in : &in2;
@@ -578,7 +617,10 @@ int fit_plan_tune(fit_plan* p, const fit_tracks_in* in, const fit_tracks_out* ou
     cudaStreamSynchronize(s);
     cudaFree(scratch);
   }
-  if (rc != FIT_OK) return rc;
+  if (rc != FIT_OK) {
+    p->free_form = was_free;
+    return rc;
+  }
   p->cfg = best_cfg;
   p->layout_free = false;
   p->tuned = 1;
@@ -636,6 +678,9 @@ void fit_plan_destroy(fit_plan* p) {
     if (p->d_items) cudaFree(p->d_items);
     if (p->d_work) cudaFree(p->d_work);
     if (p->d_tune_counters) cudaFree(p->d_tune_counters);
+    if (p->join) cudaEventDestroy(p->join);
+    if (p->fork) cudaEventDestroy(p->fork);
+    if (p->cap_z) cudaStreamDestroy(p->cap_z);
     if (p->cap) cudaStreamDestroy(p->cap);
   }
   delete p;

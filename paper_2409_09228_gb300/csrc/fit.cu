@@ -268,9 +268,10 @@ void add_run(PairRuns<kMaxRuns>& r, uint32_t t0, uint32_t t1) {
 // An uneven mixed batch (500 events, 1M tracks, ~250 runs) takes 0.228 ms in
 // two launches; with one launch per run it took 4.11 ms, a run's few blocks
 // leaving most SMs idle for the ~20 us of its layers.
+// by_event: every event is a run of its own.
 template <class Launch>
-int launch_runs(const fit_handle* h, FitArgs a, int nevt, const int64_t* ntrk, const int32_t* mode,
-                const char* who, Launch launch) {
+int launch_runs(const fit_handle* h, FitArgs a, bool by_event, int nevt, const int64_t* ntrk,
+                const int32_t* mode, const char* who, Launch launch) {
   for (int m : {FIT_MODE_R, FIT_MODE_Z}) {
     PairRuns<kMaxRuns> r;
     auto clear = [&r]() { r.pairs.nrun = 0, r.pairs.n = 0, r.nlone = 0; };
@@ -291,8 +292,8 @@ int launch_runs(const fit_handle* h, FitArgs a, int nevt, const int64_t* ntrk, c
         t += ntrk[e++];
         continue;
       }
-      int64_t t1 = t;
-      while (e < nevt && mode[e] == m) t1 += ntrk[e++];
+      int64_t t1 = t + ntrk[e++];
+      while (!by_event && e < nevt && mode[e] == m) t1 += ntrk[e++];
       while (t < t1) {
         if (!r.pairs.nrun && !r.nlone) a.t0 = t & ~int64_t(1);
         const int64_t end = a.t0 + kSpan < t1 ? a.t0 + kSpan : t1;  // (even where it cuts a run)
@@ -339,8 +340,8 @@ void launch_fused(const FitArgs& a, const PairRuns<kMaxRuns>& r, cudaStream_t s)
 // it.  Returns false, with nothing launched, if their runs do not fit its
 // tables.
 template <class Launch>
-bool launch_small(const fit_handle* h, const FitArgs& a, int nevt, const int64_t* ntrk,
-                  const int32_t* mode, Launch launch) {
+bool launch_small(const fit_handle* h, const FitArgs& a, bool by_event, int nevt,
+                  const int64_t* ntrk, const int32_t* mode, Launch launch) {
   SmallArgs<kSmallRuns> s;
   s.a = a;
   unsigned blocks[2] = {0, 0};
@@ -351,11 +352,12 @@ bool launch_small(const fit_handle* h, const FitArgs& a, int nevt, const int64_t
     s.t0[m] = 0;
     s.runs[m].pairs.nrun = 0, s.runs[m].pairs.n = 0, s.runs[m].nlone = 0;
   }
-  const int rc = launch_runs(h, a, nevt, ntrk, mode, "fit_small", [&](const FitArgs& a1, int m, const PairRuns<kMaxRuns>& r) {
-    fits = fits && tables[m]++ == 0 && copy_table(r, s.runs[m]);
-    s.t0[m] = a1.t0;
-    blocks[m] = part_blocks<1>(r);
-  });
+  const int rc = launch_runs(h, a, by_event, nevt, ntrk, mode, "fit_small",
+                             [&](const FitArgs& a1, int m, const PairRuns<kMaxRuns>& r) {
+                               fits = fits && tables[m]++ == 0 && copy_table(r, s.runs[m]);
+                               s.t0[m] = a1.t0;
+                               blocks[m] = part_blocks<1>(r);
+                             });
   if (rc != FIT_OK || !fits) return false;
   s.blocks_r = blocks[FIT_MODE_R];
   launch(s, blocks[0] + blocks[1]);
@@ -371,29 +373,31 @@ bool is_small(const fit_handle* h, int64_t call_tracks) { return is_small(h->sms
 
 // The fused fit of events [0, nevt) on the tracks of a: the p2r events on
 // stream s, the p2z events on sz.
-int run_fit(const fit_handle* h, const FitArgs& a, int layout, bool seeded, int64_t call_tracks,
-            int nevt, const int64_t* ntrk, const int32_t* mode, const char* who, cudaStream_t s,
+int run_fit(const fit_handle* h, const FitArgs& a, const RunOptions& o, int nevt,
+            const int64_t* ntrk, const int32_t* mode, const char* who, cudaStream_t s,
             cudaStream_t sz) {
-  if (!seeded && is_small(h, call_tracks)) {
-    const bool done = launch_small(h, a, nevt, ntrk, mode, [&](const auto& args, unsigned nblk) {
-      if (layout == FIT_LAYOUT_SOA)
-        fit_small_kernel<0, false><<<nblk, kBlock, 0, s>>>(args, nullptr, 0);
-      else
-        fit_small_kernel<1, false><<<nblk, kBlock, 0, s>>>(args, nullptr, 0);
-    });
+  const bool soa = o.layout == FIT_LAYOUT_SOA;
+  if (!o.seeded && is_small(h, o.call_tracks)) {
+    const bool done = launch_small(h, a, o.by_event, nevt, ntrk, mode,
+                                   [&](const auto& args, unsigned nblk) {
+                                     if (soa)
+                                       fit_small_kernel<0, false><<<nblk, kBlock, 0, s>>>(args, nullptr, 0);
+                                     else
+                                       fit_small_kernel<1, false><<<nblk, kBlock, 0, s>>>(args, nullptr, 0);
+                                   });
     if (done) {
       const cudaError_t e = cudaGetLastError();
       return e == cudaSuccess ? FIT_OK : cuda_fail(e, (std::string(who) + ": launch").c_str());
     }
   }
-  if (seeded) {
+  if (o.seeded) {
     const int rc = launch_seeded_fit(h, a, nevt, ntrk, mode, who, s);
     if (rc != FIT_OK) return rc;
   }
-  return launch_runs(h, a, nevt, ntrk, mode, who,
-                     [=](const FitArgs& a1, int m, const PairRuns<kMaxRuns>& r) {
-                       if (m == FIT_MODE_R && seeded) return;
-                       if (layout == FIT_LAYOUT_SOA)
+  return launch_runs(h, a, o.by_event, nevt, ntrk, mode, who,
+                     [&](const FitArgs& a1, int m, const PairRuns<kMaxRuns>& r) {
+                       if (m == FIT_MODE_R && o.seeded) return;
+                       if (soa)
                          m == FIT_MODE_Z ? launch_fused<FIT_MODE_Z, 0>(a1, r, sz)
                                          : launch_fused<FIT_MODE_R, 0>(a1, r, s);
                        else
@@ -425,15 +429,13 @@ int ModeStreams::end(int rc) {
   return rc;
 }
 
-int run_fit_streams(fit_handle* h, const FitArgs& a, int layout, bool seeded, int64_t call_tracks,
-                    int nevt, const int64_t* ntrk, const int32_t* mode, const char* who,
-                    cudaStream_t s) {
+int run_fit_streams(fit_handle* h, const FitArgs& a, const RunOptions& o, int nevt,
+                    const int64_t* ntrk, const int32_t* mode, const char* who, cudaStream_t s) {
   ModeStreams ms(h, s, who);
-  const bool one_launch = !seeded && is_small(h, call_tracks);
+  const bool one_launch = !o.seeded && is_small(h, o.call_tracks);
   const int rc = one_launch ? FIT_OK : ms.begin(nevt, ntrk, mode);
   if (rc != FIT_OK) return rc;
-  return ms.end(run_fit(h, a, layout, seeded, call_tracks, nevt, ntrk, mode, who,
-                        ms.of(FIT_MODE_R), ms.of(FIT_MODE_Z)));
+  return ms.end(run_fit(h, a, o, nevt, ntrk, mode, who, ms.of(FIT_MODE_R), ms.of(FIT_MODE_Z)));
 }
 
 // Scratch of fit_propagate_update_noalloc, in the library image instead of
@@ -525,9 +527,9 @@ int fit_propagate_update(fit_handle* h, const fit_tracks_in* in, const fit_track
   int rc = check_call(h, in, out, hits, nevt, ntrk, nlayer, mode, &total, "fit_propagate_update");
   if (rc != FIT_OK || total == 0) return rc;
   DeviceGuard g(h->device);
-  rc = run_fit_streams(h, base_args(in, out, hits, nlayer, h->d_counters), FIT_LAYOUT_SOA,
-                       h->seeded, total, nevt, ntrk, mode, "fit_propagate_update",
-                       static_cast<cudaStream_t>(stream));
+  rc = run_fit_streams(h, base_args(in, out, hits, nlayer, h->d_counters),
+                       {FIT_LAYOUT_SOA, h->seeded, false, total}, nevt, ntrk, mode,
+                       "fit_propagate_update", static_cast<cudaStream_t>(stream));
   if (rc != FIT_OK) return rc;
   h->tracks += (uint64_t)total;
   return FIT_OK;
@@ -549,8 +551,9 @@ int fit_propagate_update_layout(fit_handle* h, const fit_tracks_in* in, const fi
     return fail(FIT_ERR_ARG, std::string(kWho) + ": AoSoA slots (ld) must be a multiple of 32");
   if (h->seeded) return fail(FIT_ERR_ARG, std::string(kWho) + ": no learned seed in AoSoA");
   DeviceGuard g(h->device);
-  rc = run_fit_streams(h, base_args(in, out, hits, nlayer, h->d_counters), layout, false, total,
-                       nevt, ntrk, mode, kWho, static_cast<cudaStream_t>(stream));
+  rc = run_fit_streams(h, base_args(in, out, hits, nlayer, h->d_counters),
+                       {layout, false, false, total}, nevt, ntrk, mode, kWho,
+                       static_cast<cudaStream_t>(stream));
   if (rc != FIT_OK) return rc;
   h->tracks += (uint64_t)total;
   return FIT_OK;
@@ -597,11 +600,11 @@ int fit_propagate_update_noalloc(const fit_config* cfg_r, const fit_config* cfg_
       e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, device);
       if (e != cudaSuccess) return cuda_fail(e, "fit_propagate_update_noalloc: device attribute");
       const bool done = is_small(sms, total) &&
-                        launch_small(&h, args, nevt, ntrk, mode, [&](const auto& sa, unsigned nblk) {
+                        launch_small(&h, args, false, nevt, ntrk, mode, [&](const auto& sa, unsigned nblk) {
                           fit_small_kernel<0, true><<<nblk, kBlock, 0, s>>>(sa, d_off, nevt);
                         });
       if (!done)
-        rc = launch_runs(&h, args, nevt, ntrk, mode, kWho,
+        rc = launch_runs(&h, args, false, nevt, ntrk, mode, kWho,
                          [=](const FitArgs& a, int m, const PairRuns<kMaxRuns>& r) {
                            if (m == FIT_MODE_Z)
                              fit_fused_kernel_noalloc<FIT_MODE_Z, kMaxRuns>

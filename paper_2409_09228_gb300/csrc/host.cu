@@ -174,8 +174,8 @@ extern "C" int fit_propagate_update_host(fit_handle* h, const fit_tracks_in* in,
   // 520 -> 334 us, 1.92M 8.1-20.8 -> 6.3 ms.
   // Pageable buffers go through the staging sets.
   if (mapped_call(in, out, hits, total, nlayer)) {
-    rc = run_fit_streams(h, base_args(in, out, hits, nlayer, h->d_counters), FIT_LAYOUT_SOA,
-                         h->seeded, total, nevt, ntrk, mode, kWho,
+    rc = run_fit_streams(h, base_args(in, out, hits, nlayer, h->d_counters),
+                         {FIT_LAYOUT_SOA, h->seeded, false, total}, nevt, ntrk, mode, kWho,
                          static_cast<cudaStream_t>(stream));
     if (rc == FIT_OK) h->tracks += (uint64_t)total;
     return rc;
@@ -227,8 +227,9 @@ extern "C" int fit_propagate_update_host(fit_handle* h, const fit_tracks_in* in,
     fit_tracks_out sout{S.par, S.cov, S.q, S.chi2, out->chi2_layer ? S.chi2_layer : nullptr,
                         out->status ? S.status : nullptr, hs->cap};
     fit_hits shit{S.hpos, S.hcov, hs->cap};
-    rc = run_fit(h, base_args(&sin, &sout, &shit, nlayer, h->d_counters), FIT_LAYOUT_SOA, h->seeded,
-                 total, (int)nt_local.size(), nt_local.data(), md_local.data(), kWho, s, s);
+    rc = run_fit(h, base_args(&sin, &sout, &shit, nlayer, h->d_counters),
+                 {FIT_LAYOUT_SOA, h->seeded, false, total}, (int)nt_local.size(), nt_local.data(),
+                 md_local.data(), kWho, s, s);
     if (rc != FIT_OK) return rc;
     e = copy_rows(out->par + c0, pout, S.par, P, w, 6, cudaMemcpyDeviceToHost, s);
     if (e == cudaSuccess) e = copy_rows(out->cov + c0, pout, S.cov, P, w, 21, cudaMemcpyDeviceToHost, s);
@@ -268,8 +269,9 @@ extern "C" int fit_propagate_update_mapped(fit_handle* h, const fit_tracks_in* i
       return fail(FIT_ERR_ARG, std::string(kWho) +
                                    ": a buffer is not page-locked host memory mapped into the "
                                    "device's address space");
-  rc = run_fit_streams(h, base_args(in, out, hits, nlayer, h->d_counters), FIT_LAYOUT_SOA,
-                       h->seeded, total, nevt, ntrk, mode, kWho, static_cast<cudaStream_t>(stream));
+  rc = run_fit_streams(h, base_args(in, out, hits, nlayer, h->d_counters),
+                       {FIT_LAYOUT_SOA, h->seeded, false, total}, nevt, ntrk, mode, kWho,
+                       static_cast<cudaStream_t>(stream));
   if (rc != FIT_OK) return rc;
   h->tracks += (uint64_t)total;
   return FIT_OK;

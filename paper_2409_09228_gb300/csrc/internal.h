@@ -81,7 +81,7 @@ struct PairRuns {
 // Capacities compiled: the usual call has one run per mode; a call of uneven
 // mixed events has hundreds.  kMaxRuns pair runs take 16 KiB of parameters.
 constexpr int kMaxRuns = 1024;
-constexpr int kSmallRuns = 128;  // of each mode, in a small call's one launch
+constexpr int kSmallRuns = 256;  // of each mode, in a small call's one launch
 
 inline bool aligned16(const void* p) { return (reinterpret_cast<uintptr_t>(p) & 15u) == 0; }
 
@@ -182,14 +182,21 @@ int launch_track_runs(int nevt, const int64_t* ntrk, const int32_t* mode, int m,
   return flush();
 }
 
-// The fused fit of events [0, nevt) (fit.cu) in the given layout: the p2r
-// events in one launch on stream s (kMaxRuns runs each), the p2z events in
-// one on sz.  seeded: the p2r events start from the handle's learned seed.
-// call_tracks: the tracks of the whole call (more than these events' where it
-// is cut into chunks); is_small(h, call_tracks) calls take one launch on s.
+// How run_fit takes a call's events.
+struct RunOptions {
+  int layout = FIT_LAYOUT_SOA;
+  bool seeded = false;      // the p2r events start from the handle's learned seed
+  bool by_event = false;    // pairs never cross an event (else: a run of same-mode events)
+  int64_t call_tracks = 0;  // tracks of the whole call, which may be cut into chunks
+};
+
+// Whether a call of that many tracks takes one launch for both modes (fit.cu).
 bool is_small(const fit_handle* h, int64_t call_tracks);
-int run_fit(const fit_handle* h, const FitArgs& a, int layout, bool seeded, int64_t call_tracks,
-            int nevt,
+
+// The fused fit of events [0, nevt) (fit.cu): the p2r events in one launch on
+// stream s (kMaxRuns runs each), the p2z events in one on sz; a small call in
+// one launch on s.
+int run_fit(const fit_handle* h, const FitArgs& a, const RunOptions& o, int nevt,
             const int64_t* ntrk, const int32_t* mode, const char* who, cudaStream_t s,
             cudaStream_t sz);
 
@@ -216,9 +223,8 @@ class ModeStreams {
 };
 
 // run_fit with the second stream for p2z where both modes are present.
-int run_fit_streams(fit_handle* h, const FitArgs& a, int layout, bool seeded, int64_t call_tracks,
-                    int nevt, const int64_t* ntrk, const int32_t* mode, const char* who,
-                    cudaStream_t s);
+int run_fit_streams(fit_handle* h, const FitArgs& a, const RunOptions& o, int nevt,
+                    const int64_t* ntrk, const int32_t* mode, const char* who, cudaStream_t s);
 
 // Frees the staging of fit_propagate_update_host (host.cu).
 void destroy_host_stage(fit_handle* h);

@@ -190,3 +190,41 @@ def test_small_call_rounds_like_pairs(entry, n):
         for i in small:
             np.testing.assert_array_equal(small[i][..., :whole], pairs[i][..., :whole], err_msg=i)
     f.close()
+
+
+@pytest.mark.parametrize("layout", [fit.FIT_LAYOUT_SOA, fit.FIT_LAYOUT_AOSOA32])
+def test_default_plan_equals_the_persistent_form(layout):
+    """A plan left at its default shape runs one launch per mode over the same
+    pairs as the persistent form: bit for bit its results.  Odd event edges;
+    more tracks than a small call has."""
+    ev = inputs.generate_events(inputs.uneven_event_sizes(60, 83, median=600.0, hi=3000),
+                                inputs.uneven_event_modes(60, 83), seed=83)
+    assert ev.n > torch.cuda.get_device_properties(0).multi_processor_count * 128
+    ld = (ev.n + 31) // 32 * 32
+    d = _device(ev, ld)
+    if layout == fit.FIT_LAYOUT_AOSOA32:
+        d = [a if k == 2 else torch.from_numpy(inputs.to_aosoa32(a.cpu().numpy(), ld)).cuda().view(a.shape)
+             for k, a in enumerate(d)]
+    f = _fitter(ev)
+    got = []
+    for blocks_per_sm in (0, 3):
+        out = f.outputs(ev.n, ld=ld, layers=True)
+        plan = fit.fit_plan_create(f.h, ev.ntrk, ev.mode, NLAYER, blocks_per_sm=blocks_per_sm,
+                                   layout=layout)
+        for _ in range(2):  # captured, then replayed
+            for k in ("par", "cov", "chi2", "chi2_layer"):
+                out[k].fill_(float("nan"))
+            fit.fit_plan_run(plan, *d, par_out=out["par"], cov_out=out["cov"], q_out=out["q"],
+                             chi2=out["chi2"], chi2_layer=out["chi2_layer"], status=out["status"])
+            torch.cuda.synchronize()
+        fit.fit_plan_destroy(plan)
+        got.append({k: v.cpu().numpy() for k, v in out.items()} | {"counters": f.sync()})
+    f.close()
+    assert got[0].pop("counters") == got[1].pop("counters")
+    for k in got[0]:
+        a, b = got[0][k], got[1][k]
+        if a.ndim == 1:
+            a, b = a[:ev.n], b[:ev.n]
+        elif layout == fit.FIT_LAYOUT_SOA:
+            a, b = a[:, :ev.n], b[:, :ev.n]
+        np.testing.assert_array_equal(a, b, err_msg=k)
