@@ -187,10 +187,12 @@ int fit_sync(fit_handle* h, void* stream, double timeout_s, fit_status* st);
  *   per_event     HOST array of nevt fit_status, or NULL.  If given, the call
  *                 waits for its work on `stream` and fills entry e with the
  *                 counts of event e (tracks = ntrk[e]).  If NULL the call
- *                 does not wait for its kernels; but the event offsets are
- *                 copied to the device from a local (pageable) host array,
- *                 and for such a copy the CUDA driver may wait for the work
- *                 queued earlier on `stream` before the call returns.
+ *                 does not wait for its kernels; but the event offsets of
+ *                 a call that is not small (up to 256 events and 128 tracks
+ *                 per SM) are copied to the device from a local (pageable)
+ *                 host array, and for such a copy the CUDA driver may wait
+ *                 for the work queued earlier on `stream` before the call
+ *                 returns.
  * The work runs on the current CUDA device.  The first call on a device looks
  * up the device address of the fixed array (once per device).  That first
  * call may also be where CUDA loads the library's kernels onto the device

@@ -91,11 +91,12 @@ __global__ void __launch_bounds__(kBlock, MODE == FIT_MODE_Z ? 4 : 3)
   if (MODE == FIT_MODE_R) count_iterations(iters[0] + iters[1], &a.counters[4]);
 }
 
-// Adds a track's status and iterations to its event's counters.
-template <int MODE>
+// Adds a track's status and iterations to its event's counters; evt_first
+// holds the first track of each of the nevt events.
+template <int MODE, class Off>
 __device__ __forceinline__ void count_event(const FitArgs& a, int64_t t, unsigned st, unsigned iters,
-                                            const int64_t* __restrict__ evt_off, int nevt) {
-  unsigned long long* cnt = a.counters + (int64_t)event_of(t, evt_off, 0, nevt) * kEventSlots + 1;
+                                            const Off* __restrict__ evt_first, int nevt) {
+  unsigned long long* cnt = a.counters + (int64_t)event_of(t, evt_first, nevt) * kEventSlots + 1;
   if (st) count_status(st, cnt);
   if (MODE == FIT_MODE_R && iters) atomicAdd(&cnt[4], (unsigned long long)iters);
 }
@@ -135,11 +136,19 @@ struct SmallArgs {
   PairRuns<K> runs[2];
 };
 
-// EVENTS: count per event (as fit_fused_kernel_noalloc).
-template <int L, bool EVENTS>
+// The first track of each event of a small call, as a kernel parameter.
+template <int K>
+struct EventTable {
+  int n;
+  uint32_t first[K];
+};
+constexpr int kSmallEvents = 256;
+
+// E > 0: count per event (as fit_fused_kernel_noalloc).
+template <int L, int E>
 __global__ void __launch_bounds__(kBlock)
     fit_small_kernel(const __grid_constant__ SmallArgs<kSmallRuns> s,
-                     const int64_t* __restrict__ evt_off, int nevt) {
+                     const __grid_constant__ EventTable<(E > 0 ? E : 1)> ev) {
   auto run = [&](auto mode, unsigned block) {
     constexpr int MODE = decltype(mode)::value;
     int64_t t;
@@ -150,8 +159,8 @@ __global__ void __launch_bounds__(kBlock)
       run_half_pair<MODE, L>(s.a, s.geo[MODE], t, st, iters);
     else
       run_lone<MODE, L>(s.a, s.geo[MODE], t, st, iters);
-    if constexpr (EVENTS) {
-      count_event<MODE>(s.a, t, st, iters, evt_off, nevt);
+    if constexpr (E > 0) {
+      count_event<MODE>(s.a, t, st, iters, ev.first, ev.n);
     } else {
       if (st) count_status(st, s.a.counters);
       if (MODE == FIT_MODE_R) count_iterations(iters, &s.a.counters[4]);
@@ -381,9 +390,9 @@ int run_fit(const fit_handle* h, const FitArgs& a, const RunOptions& o, int nevt
     const bool done = launch_small(h, a, o.by_event, nevt, ntrk, mode,
                                    [&](const auto& args, unsigned nblk) {
                                      if (soa)
-                                       fit_small_kernel<0, false><<<nblk, kBlock, 0, s>>>(args, nullptr, 0);
+                                       fit_small_kernel<0, 0><<<nblk, kBlock, 0, s>>>(args, {});
                                      else
-                                       fit_small_kernel<1, false><<<nblk, kBlock, 0, s>>>(args, nullptr, 0);
+                                       fit_small_kernel<1, 0><<<nblk, kBlock, 0, s>>>(args, {});
                                    });
     if (done) {
       const cudaError_t e = cudaGetLastError();
@@ -584,40 +593,53 @@ int fit_propagate_update_noalloc(const fit_config* cfg_r, const fit_config* cfg_
   if (rc != FIT_OK) return rc;
   cudaStream_t s = static_cast<cudaStream_t>(stream);
   if (nevt > 0) {
-    // The counters of this call's events start at zero; the event offsets
-    // are staged from the stack.
-    int64_t off[FIT_NOALLOC_MAX_EVENTS + 1];
-    off[0] = 0;
-    for (int i = 0; i < nevt; ++i) off[i + 1] = off[i] + ntrk[i];
-    int64_t* d_off = reinterpret_cast<int64_t*>(scratch + kNoallocCounterWords);
+    // The counters of this call's events start at zero.
     e = cudaMemsetAsync(scratch, 0, (size_t)nevt * kEventSlots * sizeof(unsigned long long), s);
     if (e != cudaSuccess) return cuda_fail(e, "fit_propagate_update_noalloc: cudaMemsetAsync");
-    e = cudaMemcpyAsync(d_off, off, (size_t)(nevt + 1) * sizeof(int64_t), cudaMemcpyHostToDevice, s);
-    if (e != cudaSuccess) return cuda_fail(e, "fit_propagate_update_noalloc: offset copy");
-    if (total > 0) {
-      const FitArgs args = base_args(in, out, hits, nlayer, scratch);
-      int sms = 0;
-      e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, device);
-      if (e != cudaSuccess) return cuda_fail(e, "fit_propagate_update_noalloc: device attribute");
-      const bool done = is_small(sms, total) &&
-                        launch_small(&h, args, false, nevt, ntrk, mode, [&](const auto& sa, unsigned nblk) {
-                          fit_small_kernel<0, true><<<nblk, kBlock, 0, s>>>(sa, d_off, nevt);
-                        });
-      if (!done)
-        rc = launch_runs(&h, args, false, nevt, ntrk, mode, kWho,
-                         [=](const FitArgs& a, int m, const PairRuns<kMaxRuns>& r) {
-                           if (m == FIT_MODE_Z)
-                             fit_fused_kernel_noalloc<FIT_MODE_Z, kMaxRuns>
-                                 <<<part_blocks<2>(r), kBlock, 0, s>>>(a, r, d_off, nevt);
-                           else
-                             fit_fused_kernel_noalloc<FIT_MODE_R, kMaxRuns>
-                                 <<<part_blocks<2>(r), kBlock, 0, s>>>(a, r, d_off, nevt);
-                         });
-      e = cudaGetLastError();
-      if (rc == FIT_OK && e != cudaSuccess)
-        rc = cuda_fail(e, "fit_propagate_update_noalloc: launch");
-      if (rc != FIT_OK) return rc;
+  }
+  if (total > 0) {
+    const FitArgs args = base_args(in, out, hits, nlayer, scratch);
+    int sms = 0;
+    e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, device);
+    if (e != cudaSuccess) return cuda_fail(e, "fit_propagate_update_noalloc: device attribute");
+    bool done = false;
+    if (is_small(sms, total) && nevt <= kSmallEvents) {
+      EventTable<kSmallEvents> ev;
+      ev.n = nevt;
+      uint32_t t = 0;
+      for (int i = 0; i < nevt; ++i) {
+        ev.first[i] = t;
+        t += (uint32_t)ntrk[i];
+      }
+      done = launch_small(&h, args, false, nevt, ntrk, mode, [&](const auto& sa, unsigned nblk) {
+        fit_small_kernel<0, kSmallEvents><<<nblk, kBlock, 0, s>>>(sa, ev);
+      });
     }
+    if (!done) {
+      // the event offsets, staged from the stack
+      int64_t off[FIT_NOALLOC_MAX_EVENTS];
+      int64_t t = 0;
+      for (int i = 0; i < nevt; ++i) {
+        off[i] = t;
+        t += ntrk[i];
+      }
+      int64_t* d_off = reinterpret_cast<int64_t*>(scratch + kNoallocCounterWords);
+      e = cudaMemcpyAsync(d_off, off, (size_t)nevt * sizeof(int64_t), cudaMemcpyHostToDevice, s);
+      if (e != cudaSuccess) return cuda_fail(e, "fit_propagate_update_noalloc: offset copy");
+      rc = launch_runs(&h, args, false, nevt, ntrk, mode, kWho,
+                       [=](const FitArgs& a, int m, const PairRuns<kMaxRuns>& r) {
+                         if (m == FIT_MODE_Z)
+                           fit_fused_kernel_noalloc<FIT_MODE_Z, kMaxRuns>
+                               <<<part_blocks<2>(r), kBlock, 0, s>>>(a, r, d_off, nevt);
+                         else
+                           fit_fused_kernel_noalloc<FIT_MODE_R, kMaxRuns>
+                               <<<part_blocks<2>(r), kBlock, 0, s>>>(a, r, d_off, nevt);
+                       });
+    }
+    e = cudaGetLastError();
+    if (rc == FIT_OK && e != cudaSuccess)
+      rc = cuda_fail(e, "fit_propagate_update_noalloc: launch");
+    if (rc != FIT_OK) return rc;
   }
   if (per_event && nevt > 0) {
     static_assert(sizeof(fit_status) == kEventSlots * sizeof(unsigned long long),

@@ -441,19 +441,19 @@ __device__ __forceinline__ void count_iterations(unsigned iters, unsigned long l
   if ((int)(threadIdx.x & 31) == __ffs(mask) - 1) atomicAdd(counter, (unsigned long long)warp_iters);
 }
 
-// Variant for fit_propagate_update_noalloc: the same per-track work, with the
-// counters kept per event.  a.counters points at a [nevt][kEventSlots] table
-// (slot 0, the track count, is filled on the host); evt_off holds the first
-// track of events e0..e1 (and the end of e1 - 1), so a track finds its event
-// by binary search.
+// fit_propagate_update_noalloc keeps its counters per event: a.counters
+// points at a [nevt][kEventSlots] table (slot 0, the track count, is filled on
+// the host).  evt_first holds the first track of each event, and a track
+// finds its event by binary search: the last one that starts at or before it
+// (behind empty events, which start at the same track).
 constexpr int kEventSlots = 6;
 
-__device__ __forceinline__ int event_of(int64_t t, const int64_t* __restrict__ evt_off, int e0,
-                                        int e1) {
-  int lo = e0, hi = e1 - 1;
+template <class Off>
+__device__ __forceinline__ int event_of(int64_t t, const Off* __restrict__ evt_first, int nevt) {
+  int lo = 0, hi = nevt - 1;
   while (lo < hi) {
     const int mid = (lo + hi + 1) >> 1;
-    if (evt_off[mid] <= t)
+    if ((int64_t)evt_first[mid] <= t)
       lo = mid;
     else
       hi = mid - 1;

@@ -259,7 +259,11 @@ class Geometry:
 def _config(g: Optional[Geometry]):
     if g is None:
         return None, None
-    arr = (ctypes.c_float * len(g.surf))(*[float(s) for s in g.surf])
+    if isinstance(g.surf, (np.ndarray, list, tuple)):
+        surf = np.asarray(g.surf, dtype=np.float32)
+        arr = (ctypes.c_float * surf.size).from_buffer_copy(surf.tobytes())
+    else:
+        arr = (ctypes.c_float * len(g.surf))(*[float(s) for s in g.surf])
     return fit_config(float(g.B), len(g.surf), arr, int(g.max_iter), float(g.tol),
                       int(g.start)), arr
 
