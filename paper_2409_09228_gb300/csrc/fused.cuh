@@ -154,7 +154,7 @@ __device__ __forceinline__ void store_state(const FitArgs& a, int64_t t, const S
 // surface some live lane cannot reach (its propagation is not applied), the
 // layer after one where a packed lane turned non-finite, or nlayer.  A lane
 // whose update turns non-finite stops (alive false); its later per-layer
-// chi2 entries are 0.
+// chi2 entries are 0.  Every lane is alive on entry.
 //
 // STAGE (p2z, two tracks per thread, SoA, kBlock threads per block): the five
 // hit values the p2z update reads are copied one layer ahead into shared
@@ -188,11 +188,13 @@ __device__ __forceinline__ int run_layers(const FitArgs& a, const Geo& geo, int6
 #pragma unroll
     for (int k = 0; k < NU; ++k) pu0[k] = pu1[k] = T(0.f);
   };
-  auto done = [&](int r) {
+  // leaves the loop after `passed` surfaces, at layer r
+  auto done = [&](int r, int passed) {
     if constexpr (STAGE) cp_async_wait<0>();
     settle();
 #pragma unroll
     for (int i = 0; i < Lanes<T>::n; ++i) {
+      if (MODE == FIT_MODE_R) iters[i] += (unsigned)passed;  // the first iterations
       if (Lanes<T>::get(any_nc, i)) st[i] |= FIT_ST_NOT_CONVERGED;
       if (Lanes<T>::get(any_flip, i)) st[i] |= FIT_ST_CHARGE_FLIP;
       if (!Lanes<T>::get(alive, i)) st[i] |= FIT_ST_NONFINITE;
@@ -259,9 +261,10 @@ __device__ __forceinline__ int run_layers(const FitArgs& a, const Geo& geo, int6
     if (MODE == FIT_MODE_Z)
       fail = fitk::prop_z<true>(s.p, s.c, s.g, dkdw, sf, settle);
     else
-      fail = fitk::prop_r_local(s.p, s.cl, s.bc, s.bs, s.g, dkdw, sf, geo.max_iter,
-                                geo.tol * sf, geo.line_start, iters, nc, lag, T(0.f), settle);
-    if (fitk::any(fitk::and_(fail, alive))) return done(l);
+      fail = fitk::prop_r_local<T, fitk::Start::kAuto, false>(
+          s.p, s.cl, s.bc, s.bs, s.g, dkdw, sf, geo.max_iter, geo.tol * sf, geo.line_start, iters,
+          nc, lag, T(0.f), settle);
+    if (fitk::any(fail)) return done(l, l - l0);
     const T phi_pred = s.p[4], th_pred = s.p[5];
     T x2;
     M flip;
@@ -277,28 +280,28 @@ __device__ __forceinline__ int run_layers(const FitArgs& a, const Geo& geo, int6
       const T sgn = fitk::sel(flip, T(-1.f), T(1.f));
       pu0[W] = pu0[W] * sgn;
       pu1[W] = pu1[W] * sgn;
+      any_flip = fitk::or_(any_flip, flip);
     }
-    alive = fitk::and_(alive, fitk::finite_(x2));
-    any_nc = fitk::or_(any_nc, nc);
-    any_flip = fitk::or_(any_flip, flip);
+    if (fitk::any(nc)) any_nc = fitk::or_(any_nc, nc);
+    alive = fitk::finite_(x2);  // (every lane was, until here)
     x2 = fitk::sel(alive, x2, T(0.f));
     s.chi2 += x2;
     if (a.chi2_layer) fitk::st(a.chi2_layer + ix<L>(l, t, a.ld_out, a.nlayer), x2);
-    if (!fitk::any(alive)) {
-      if (a.chi2_layer)
-        for (int r = l + 1; r < a.nlayer; ++r)
-          fitk::st(a.chi2_layer + ix<L>(r, t, a.ld_out, a.nlayer), T(0.f));
-      return done(a.nlayer);
-    }
-    // A packed lane that turned non-finite would fail every later
-    // propagation, and a propagation that fails for any lane is applied to
-    // none: the pair splits at the next layer, where the live track goes on
-    // alone and the dead one is only stored.
-    if constexpr (Lanes<T>::n > 1) {
-      if (!fitk::all(alive)) return done(l + 1);
+    if (!fitk::all(alive)) {
+      if (!fitk::any(alive)) {
+        if (a.chi2_layer)
+          for (int r = l + 1; r < a.nlayer; ++r)
+            fitk::st(a.chi2_layer + ix<L>(r, t, a.ld_out, a.nlayer), T(0.f));
+        return done(a.nlayer, l + 1 - l0);
+      }
+      // A packed lane that turned non-finite would fail every later
+      // propagation, and a propagation that fails for any lane is applied to
+      // none: the pair splits at the next layer, where the live track goes
+      // on alone and the dead one is only stored.
+      return done(l + 1, l + 1 - l0);
     }
   }
-  return done(a.nlayer);
+  return done(a.nlayer, a.nlayer - l0);
 }
 
 // Outputs of a state that run_layers left at layer l: the loop form back to

@@ -820,7 +820,10 @@ struct PathR {
 // h_line when the start is inside the cylinder and that value is finite and
 // within h_line / 4 of h_line.  The iteration, its tolerance and its result
 // are otherwise unchanged.
-template <class T, bool SEEDED = false, Start START = Start::kAuto, class Overlap = NoOverlap>
+// FIRST = false: the first iteration is not counted (a caller's loop knows how
+// many surfaces it propagated to).
+template <class T, bool SEEDED = false, Start START = Start::kAuto, bool FIRST = true,
+          class Overlap = NoOverlap>
 __device__ __forceinline__ typename Lanes<T>::M path_r(const T (&p)[6], const Trig<T>& g, T kappa,
                                                        float R, int max_iter, float tol_abs,
                                                        bool line_start,
@@ -878,9 +881,11 @@ __device__ __forceinline__ typename Lanes<T>::M path_r(const T (&p)[6], const Tr
   M conv = lt(T(1.f), T(0.f));  // all false
   T u = T(0.f), s = T(1.f), cu = T(1.f), sp = T(0.f), sm = sph, cm = cph, px = x, py = y, c1 = cph,
     s1 = sph, d = T(0.f), ib = T(0.f);
-  auto step = [&]() {
+  auto step = [&](bool count) {
+    if (count) {
 #pragma unroll
-    for (int i = 0; i < Lanes<T>::n; ++i) iters[i] += Lanes<T>::get(conv, i) ? 0u : 1u;
+      for (int i = 0; i < Lanes<T>::n; ++i) iters[i] += Lanes<T>::get(conv, i) ? 0u : 1u;
+    }
     u = hk * h;
     sinc_cs(u, s, cu, sp);
     const T su = u * s;
@@ -912,8 +917,8 @@ __device__ __forceinline__ typename Lanes<T>::M path_r(const T (&p)[6], const Tr
     h += d;
     conv = or_(conv, le(fabs_(d), T(tol_abs)));
   };
-  step();
-  for (int it = 1; it < max_iter && !all(conv); ++it) step();
+  step(FIRST);
+  for (int it = 1; it < max_iter && !all(conv); ++it) step(true);
   notconv = not_(conv);
   w = {h, d, u, s, cu, sp, cm, sm, px, py, c1, s1, ib};
   return fail;
@@ -927,7 +932,7 @@ __device__ __forceinline__ typename Lanes<T>::M path_r(const T (&p)[6], const Tr
 // LOCAL also leaves the direction (g.cphi, g.sphi) at the angle of the last
 // evaluation, lag = kappa d short of p[4]: the caller turns it on with the
 // update's change of phi (normalise), one turn instead of two.
-template <class T, bool SEEDED, Start START, bool LOCAL, class Overlap = NoOverlap>
+template <class T, bool SEEDED, Start START, bool LOCAL, bool FIRST = true, class Overlap = NoOverlap>
 __device__ __forceinline__ typename Lanes<T>::M prop_r_impl(
     T (&p)[6], T (&c)[LOCAL ? 15 : 21], T& bc, T& bs, Trig<T>& g, T dkdw, float R, int max_iter,
     float tol_abs, bool line_start, unsigned (&iters)[Lanes<T>::n],
@@ -935,7 +940,7 @@ __device__ __forceinline__ typename Lanes<T>::M prop_r_impl(
   const T x = p[0], y = p[1];
   const T kappa = dkdw * p[3];
   PathR<T> w;
-  const auto fail = path_r<T, SEEDED, START>(p, g, kappa, R, max_iter, tol_abs, line_start,
+  const auto fail = path_r<T, SEEDED, START, FIRST>(p, g, kappa, R, max_iter, tol_abs, line_start,
                                              iters, notconv, w, gseed, h_given, ov);
   if (any(fail)) return fail;
   const T h = w.h, d = w.d, s = w.s, sp = w.sp, cm = w.cm, sm = w.sm;
@@ -1016,7 +1021,7 @@ __device__ __forceinline__ typename Lanes<T>::M prop_r(T (&p)[6], T (&c)[21], Tr
 // As prop_r, on the local form (cl, bc, bs) of the covariance; the direction
 // (g.cphi, g.sphi) is left lag short of p[4] (see prop_r_impl).  ov: work
 // independent of the path length, overlapped with its start (path_r).
-template <class T, Start START = Start::kAuto, class Overlap = NoOverlap>
+template <class T, Start START = Start::kAuto, bool FIRST = true, class Overlap = NoOverlap>
 __device__ __forceinline__ typename Lanes<T>::M prop_r_local(T (&p)[6], T (&cl)[15], T& bc, T& bs,
                                                              Trig<T>& g, T dkdw, float R,
                                                              int max_iter, float tol_abs,
@@ -1025,7 +1030,7 @@ __device__ __forceinline__ typename Lanes<T>::M prop_r_local(T (&p)[6], T (&cl)[
                                                              typename Lanes<T>::M& notconv,
                                                              T& lag, T h_given = T(0.f),
                                                              const Overlap& ov = Overlap()) {
-  return prop_r_impl<T, false, START, true>(p, cl, bc, bs, g, dkdw, R, max_iter, tol_abs,
+  return prop_r_impl<T, false, START, true, FIRST>(p, cl, bc, bs, g, dkdw, R, max_iter, tol_abs,
                                             line_start, iters, notconv, T(0.f), h_given, lag, ov);
 }
 
