@@ -9,6 +9,7 @@
 
 #include <cstdint>
 #include <string>
+#include <type_traits>
 
 #include "fit.h"
 #include "fused.cuh"
@@ -53,17 +54,20 @@ struct FindArgs {
 // update takes its candidate from registers.  Loaded one at a time and the
 // chosen one again, the p2r kernel waited on loads 8.2 cycles an instruction
 // (now 0.9): 240k tracks, 4 candidates, 20 layers 217 -> 175 us, and both
-// modes of that size 383 -> 260 us with p2z on the second stream.  Four slots
-// and 4 (p2r) and 5 (p2z) blocks of 128 an SM: 4 and 4 take 271 us, 5 and 6
-// 268, two slots with 6 and 7 265, three with 5 and 6 288.  In double, bound by
-// the FP64 pipe, one slot is enough.
+// modes of that size 383 -> 246 us with p2z on the second stream.  Four slots
+// and five blocks of 128 an SM (with addresses formed anew: 4 and 5 blocks
+// 260 us, 4 and 4 271, 5 and 6 268; two slots with 6 and 7 265, three with 5
+// and 6 288).  In double, bound by the FP64 pipe, one slot is enough.
 template <class T>
 constexpr int kSlots = sizeof(T) == 4 ? 4 : 1;
-template <int MODE, class T>
-constexpr int kFindMinBlocks = sizeof(T) == 8 ? 1 : MODE == FIT_MODE_Z ? 5 : 4;
+// In order: the slots are refilled in the order the candidates lie in memory,
+// which holds for up to S candidates and for multiples of S.  Then two running
+// pointers step through the rows; otherwise every candidate's address is
+// formed anew (the usual 4 candidates: 246 against 261 us).
+bool in_order(int ncand, int slots) { return ncand <= slots || ncand % slots == 0; }
 
-template <int MODE, class T>
-__global__ void __launch_bounds__(kBlock, kFindMinBlocks<MODE, T>)
+template <int MODE, class T, bool SEQ>
+__global__ void __launch_bounds__(kBlock, sizeof(T) == 8 ? 1 : 5)
     fit_find_kernel(const __grid_constant__ FindArgs<T> a, const __grid_constant__ TrackRuns r) {
   const unsigned i = blockIdx.x * kBlock + threadIdx.x;
   if (i >= r.n) return;
@@ -94,11 +98,15 @@ __global__ void __launch_bounds__(kBlock, kFindMinBlocks<MODE, T>)
   const int64_t ldc = a.ld_cand;
   constexpr int S = kSlots<T>;
   T sm[S][3], sv[S][6];
+  const T* qp = a.cpos + t;
+  const T* qc = a.ccov + t;
   // candidate k of layer l into slot j
   auto fill = [&](int j, int l, int k) {
-    const int64_t row = (int64_t)l * a.ncand + k;
-    const T* qp = a.cpos + 3 * row * ldc + t;
-    const T* qc = a.ccov + 6 * row * ldc + t;
+    if constexpr (!SEQ) {
+      const int64_t row = (int64_t)l * a.ncand + k;
+      qp = a.cpos + 3 * row * ldc + t;
+      qc = a.ccov + 6 * row * ldc + t;
+    }
 #pragma unroll
     for (int i = 0; i < 3; ++i, qp += ldc) fitk::ld(sm[j][i], qp);
 #pragma unroll
@@ -290,10 +298,17 @@ int find_tracks(fit_handle* h, const In* in, const Out* out, const Cand* cand, d
     rc = launch_track_runs(nevt, ntrk, mode, m, w.c_str(), [&](int64_t t0, const TrackRuns& r) {
       a.t0 = t0;
       const unsigned nblk = (r.n + kBlock - 1) / kBlock;
-      if (m == FIT_MODE_Z)
-        fit_find_kernel<FIT_MODE_Z, T><<<nblk, kBlock, 0, s>>>(a, r);
-      else
-        fit_find_kernel<FIT_MODE_R, T><<<nblk, kBlock, 0, s>>>(a, r);
+      auto launch = [&](auto seq) {
+        constexpr bool SEQ = decltype(seq)::value;
+        if (m == FIT_MODE_Z)
+          fit_find_kernel<FIT_MODE_Z, T, SEQ><<<nblk, kBlock, 0, s>>>(a, r);
+        else
+          fit_find_kernel<FIT_MODE_R, T, SEQ><<<nblk, kBlock, 0, s>>>(a, r);
+      };
+      if constexpr (kSlots<T> > 1) {
+        if (!in_order(a.ncand, kSlots<T>)) return launch(std::false_type());
+      }
+      launch(std::true_type());
     });
     if (rc != FIT_OK) break;
   }

@@ -228,3 +228,39 @@ def test_default_plan_equals_the_persistent_form(layout):
         elif layout == fit.FIT_LAYOUT_SOA:
             a, b = a[:, :ev.n], b[:, :ev.n]
         np.testing.assert_array_equal(a, b, err_msg=k)
+
+
+@pytest.mark.parametrize("ncand", [1, 2, 3, 4, 5, 7, 8, 13, 16])
+@pytest.mark.parametrize("dtype", [torch.float32, torch.float64])
+def test_finder_choice_does_not_depend_on_the_number_of_slots(ncand, dtype):
+    """Candidates pass through a few register slots, in one order or another by
+    their number.  Each layer's own hit in a random one of ncand places, the
+    others 1e3 cm away along z (p2r) or x (p2z), far beyond the gate: the
+    finder takes the own hit and fits what one candidate alone gives, bit for
+    bit."""
+    n, ld = 301, 304
+    g = torch.Generator().manual_seed(ncand)
+    for mode in (0, 1):
+        ts = inputs.generate(mode, n, seed=79)
+        par, cov, q, hpos, hcov = (gpu_util.to_dev(a, ld) if k == 2 else gpu_util.to_dev(a, ld).to(dtype)
+                                   for k, a in enumerate((ts.par0, ts.cov0, ts.q, ts.hpos, ts.hcov)))
+        slot = torch.randint(0, ncand, (NLAYER, ld), generator=g).cuda()
+        cpos, ccov = hpos[:, None].repeat(1, ncand, 1, 1), hcov[:, None].repeat(1, ncand, 1, 1)
+        far = torch.arange(ncand, device="cuda")[None, :, None] != slot[:, None]
+        cpos[:, :, 2 if mode == 0 else 0] += 1e3 * far
+        f = fit.Fitter(*[fit.Geometry(ts.B, ts.surf) if m == mode else None for m in (0, 1)])
+
+        def find(cp, cc):
+            o = f.outputs(n, ld=ld)
+            out = [o["par"].to(dtype), o["cov"].to(dtype), o["q"], o["chi2"].to(dtype)]
+            chosen = torch.empty((NLAYER, ld), dtype=torch.int8, device="cuda")
+            fit.fit_find_tracks(f.h, par, cov, q, cp, cc, [n], [mode], 1e4, chosen, *out)
+            f.sync()
+            return [r[..., :n] for r in out + [chosen]]
+
+        one = find(hpos[:, None].contiguous(), hcov[:, None].contiguous())
+        many = find(cpos, ccov)
+        f.close()
+        assert (one[4] == 0).all() and torch.equal(many[4].long(), slot[:, :n])
+        for a, b in zip(one[:4], many[:4]):
+            assert torch.equal(a, b)
