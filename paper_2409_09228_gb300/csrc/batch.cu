@@ -1,6 +1,7 @@
-// libfit: batched form of the fused fit -- many events of uneven size and
-// mixed surface types (p2r / p2z) in one persistent launch, replayed from a
-// CUDA graph, with a launch-shape autotuner (fit_plan_* in fit.h).
+// libfit: plans for many events of uneven size and mixed surface types (p2r /
+// p2z), replayed from a CUDA graph, with a launch-shape autotuner (fit_plan_*
+// in fit.h).  A plan runs the fused kernels of fit.cu, one launch per mode
+// (the default), or one persistent launch:
 //
 // Work items are tiles of one event: threads_per_block x tracks_per_thread
 // consecutive tracks (two per thread in packed f32x2 instructions, or one),
@@ -227,8 +228,8 @@ struct fit_plan {
   bool layout_free = false;  // created with FIT_LAYOUT_TUNE and not tuned yet
   // Created with the default shape and blocks_per_sm 0, and not tuned: the
   // plan runs the fused kernels on its events (same pairs as the persistent
-  // form), one launch per mode.  Each mode then has its own registers (127
-  // and 156 instead of 168), p2z its staged hits, and no block waits for the
+  // form), one launch per mode.  Each mode then has its own registers (p2z
+  // 127 instead of 168 for both) and p2z its staged hits, and no block waits for the
   // work counter: 2000 uneven mixed events,
   // 4M tracks, 1045 -> 853 us.
   bool free_form = false;
@@ -524,7 +525,7 @@ int fit_plan_tune(fit_plan* p, const fit_tracks_in* in, const fit_tracks_out* ou
   }
   // Candidates: persistent with two tracks per thread and 32, 64, 128 or 256
   // threads per block, or one track per thread and 64, 128 or 256, each at
-  // every resident-block count; and the one-launch-per-segment form.  With
+  // every resident-block count; and the one-launch-per-mode form.  With
   // the layout left to the tuner, each in both layouts: the other layout's
   // runs read a converted copy of the inputs (scratch, freed on return).
   std::vector<int> layouts = {in_layout};

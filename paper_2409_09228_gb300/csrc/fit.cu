@@ -73,8 +73,10 @@ unsigned part_blocks(const PairRuns<K>& r) {
   return (r.nlone + kBlock - 1) / kBlock + (r.pairs.n * (2 / TPT) + kBlock - 1) / kBlock;
 }
 
-// 3 resident blocks per SM for p2r (156 registers, no spills; 2 blocks were
-// 17 % slower); p2z fits 4 (128 registers, no spills).
+// 3 resident blocks per SM for p2r (168 registers, no spills; 2 blocks were
+// 17 % slower); p2z fits 4 (127 registers, no spills).  100 events of 9600
+// tracks: p2r 242.0 us, p2z 168.0 us, the dependent chains of a layer keeping
+// the FP32 pipe 59 and 63 % busy.
 template <int MODE, int L, int K>
 __global__ void __launch_bounds__(kBlock, MODE == FIT_MODE_Z ? 4 : 3)
     fit_fused_kernel(const __grid_constant__ FitArgs a, const __grid_constant__ PairRuns<K> r) {
