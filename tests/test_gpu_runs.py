@@ -264,3 +264,59 @@ def test_finder_choice_does_not_depend_on_the_number_of_slots(ncand, dtype):
         assert (one[4] == 0).all() and torch.equal(many[4].long(), slot[:, :n])
         for a, b in zip(one[:4], many[:4]):
             assert torch.equal(a, b)
+
+
+@pytest.mark.parametrize("entry", ["fit", "find", "f64", "adjoint"])
+@pytest.mark.parametrize("ntrk", [101, 13001])  # one launch or one for each mode, side by side
+def test_calls_replay_from_a_captured_graph(entry, ntrk):
+    """A call captured into a graph on the caller's stream holds its run tables
+    and both modes' launches: replayed on new inputs in the same buffers it
+    gives what the call gives."""
+    nt, md = np.array([ntrk, ntrk, 3]), np.array([0, 1, 0], np.int32)
+    evs = [inputs.generate_events(nt, md, seed=s, nlayer=NLAYER) for s in (101, 103)]
+    n, ld = evs[0].n, (evs[0].n + 31) // 32 * 32
+    dtype = torch.float64 if entry == "f64" else torch.float32
+    d = _device(evs[0], ld, dtype)
+    f = _fitter(evs[0])
+    out = f.outputs(n, ld=ld)
+    o = [out[k].to(dtype) if k != "q" else out[k] for k in ("par", "cov", "q", "chi2")]
+    chosen = torch.empty((NLAYER, ld), dtype=torch.int8, device="cuda")
+    tape = torch.empty(fit.fit_tape_bytes(NLAYER, ld) // 4, device="cuda")
+    grads = [torch.empty((NLAYER, 3, ld), device="cuda"), torch.empty((6, ld), device="cuda"),
+             torch.empty((21, ld), device="cuda")]
+    w = torch.ones(ld, device="cuda")
+    cand = [d[3][:, None].contiguous(), d[4][:, None].contiguous()]
+
+    def call():
+        if entry == "fit":
+            fit.fit_propagate_update(f.h, *d, nt, md, *o)
+        elif entry == "f64":
+            fit.fit_propagate_update_f64(f.h, *d, nt, md, *o)
+        elif entry == "find":
+            fit.fit_find_tracks(f.h, *d[:3], *cand, nt, md, 30.0, chosen, *o)
+        else:
+            fit.fit_adjoint_forward(f.h, *d, nt, md, tape, *o)
+            fit.fit_adjoint_backward(f.h, d[3], d[4], nt, md, tape, w, *grads)
+
+    call()
+    f.sync()
+    g = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(g):
+        call()
+    new = _device(evs[1], ld, dtype)
+    for a, b in zip(d, new):
+        a.copy_(b)
+    cand[0].copy_(d[3][:, None])
+    cand[1].copy_(d[4][:, None])
+    results = []
+    for run in (g.replay, call):
+        for t in o + grads:
+            t.fill_(7)
+        torch.cuda.synchronize()
+        run()
+        torch.cuda.synchronize()
+        results.append([t[..., :n].clone() for t in o + (grads if entry == "adjoint" else [])])
+    f.sync()
+    f.close()
+    for a, b in zip(*results):
+        assert torch.equal(a, b)
