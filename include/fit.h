@@ -219,10 +219,10 @@ int fit_propagate_update_noalloc(const fit_config* cfg_r, const fit_config* cfg_
  * side by side.  In the persistent form its work is cut into items -- tiles of
  * one event, 2 x threads_per_block tracks -- that a persistent kernel's blocks
  * pull from a counter until none is left, so the uneven events and the two
- * surface types share one launch.  fit_plan_run captures the launches (and the
- * counter reset) in a CUDA graph the first time it sees a set of buffers and
- * replays the graph afterwards.  The results are those of fit_propagate_update
- * on the same events.
+ * surface types share one launch.  With an explicit or tuned shape,
+ * fit_plan_run captures the launches (and the counter reset) in a CUDA graph
+ * the first time it sees a set of buffers and replays the graph afterwards.
+ * The results are those of fit_propagate_update on the same events.
  */
 typedef struct {
   int threads_per_block; /* 32, 64, 128 or 256 (64, 128 or 256 with one track per thread) */

@@ -1,7 +1,7 @@
 // libfit: plans for many events of uneven size and mixed surface types (p2r /
-// p2z), replayed from a CUDA graph, with a launch-shape autotuner (fit_plan_*
-// in fit.h).  A plan runs the fused kernels of fit.cu, one launch per mode
-// (the default), or one persistent launch:
+// p2z), explicit and tuned shapes replayed from a CUDA graph, with a
+// launch-shape autotuner (fit_plan_* in fit.h).  A plan runs the fused kernels of fit.cu, one launch per mode
+// (the default, launched directly), or one persistent launch:
 //
 // Work items are tiles of one event: threads_per_block x tracks_per_thread
 // consecutive tracks (two per thread in packed f32x2 instructions, or one),
@@ -229,9 +229,10 @@ struct fit_plan {
   // Created with the default shape and blocks_per_sm 0, and not tuned: the
   // plan runs the fused kernels on its events (same pairs as the persistent
   // form), one launch per mode.  Each mode then has its own registers (p2z
-  // 127 instead of 168 for both) and p2z its staged hits, and no block waits for the
-  // work counter: 2000 uneven mixed events,
-  // 4M tracks, 1045 -> 853 us.
+  // 127 instead of 168 for both) and p2z its staged hits, and no block waits
+  // for the work counter: 2000 uneven mixed events, 4M tracks, 1045 -> 841 us.
+  // Launched directly: two launches cost the host no more than a graph's, and
+  // new buffers no capture (the first pass on them 1132 -> 911 us; 961 captured).
   bool free_form = false;
   int sms = 0;
   WorkItem* d_items = nullptr;
@@ -285,9 +286,10 @@ int build_items(fit_plan* p, int tpb, int tpt) {
   return FIT_OK;
 }
 
-// The fused kernels on the plan's events: the p2z launch on the plan's second
-// capture stream, a branch of the graph beside the p2r launch.
-int issue_per_mode(fit_plan* p, const FitArgs& base, bool by_event, cudaStream_t s) {
+// fit_propagate_update's form on the plan's events, an autotuner candidate:
+// the p2z launch on the plan's second capture stream, a branch of the graph
+// beside the p2r launch.
+int issue_per_mode(fit_plan* p, const FitArgs& base, cudaStream_t s) {
   const bool one_launch = is_small(p->h, p->total);
   cudaError_t e = cudaSuccess;
   if (!one_launch) {
@@ -295,7 +297,7 @@ int issue_per_mode(fit_plan* p, const FitArgs& base, bool by_event, cudaStream_t
     if (e == cudaSuccess) e = cudaStreamWaitEvent(p->cap_z, p->fork, 0);
     if (e != cudaSuccess) return cuda_fail(e, "fit_plan: fork");
   }
-  const int rc = run_fit(p->h, base, {p->cfg.layout, false, by_event, p->total},
+  const int rc = run_fit(p->h, base, {p->cfg.layout, false, false, p->total},
                          (int)p->ntrk.size(), p->ntrk.data(), p->mode.data(), "fit_plan", s,
                          p->cap_z);
   if (!one_launch) {
@@ -309,7 +311,6 @@ int issue_per_mode(fit_plan* p, const FitArgs& base, bool by_event, cudaStream_t
 // Issues the plan's work for one shape on stream s (captured into a graph).
 int issue(fit_plan* p, const FitArgs& base, cudaStream_t s) {
   if (p->total == 0) return FIT_OK;
-  if (p->free_form) return issue_per_mode(p, base, true, s);
   if (p->cfg.persistent) {
     BatchArgs b{};
     b.a = base;
@@ -329,8 +330,7 @@ int issue(fit_plan* p, const FitArgs& base, cudaStream_t s) {
     if (e != cudaSuccess) return cuda_fail(e, "fit_plan: launch");
     return FIT_OK;
   }
-  // fit_propagate_update's form, one launch per mode: an autotuner candidate
-  return issue_per_mode(p, base, false, s);
+  return issue_per_mode(p, base, s);
 }
 
 void drop_graph(fit_plan* p) {
@@ -352,7 +352,7 @@ int run_graph(fit_plan* p, const fit_tracks_in* in, const fit_tracks_out* out,
   if (!same) {
     drop_graph(p);
     int rc = FIT_OK;
-    if (p->cfg.persistent && !p->free_form)
+    if (p->cfg.persistent)
       rc = build_items(p, p->cfg.threads_per_block, tracks_per_thread(p->cfg));
     if (rc != FIT_OK) return rc;
     cudaGraph_t graph = nullptr;
@@ -485,7 +485,13 @@ int fit_plan_run(fit_plan* p, const fit_tracks_in* in, const fit_tracks_out* out
   if (rc != FIT_OK) return rc;
   if (p->total == 0) return FIT_OK;
   DeviceGuard g(p->h->device);
-  rc = run_graph(p, in, out, hits, static_cast<cudaStream_t>(stream), p->h->d_counters);
+  const cudaStream_t s = static_cast<cudaStream_t>(stream);
+  if (p->free_form)
+    rc = run_fit_streams(p->h, base_args(in, out, hits, p->nlayer, p->h->d_counters),
+                         {p->cfg.layout, false, true, p->total}, (int)p->ntrk.size(),
+                         p->ntrk.data(), p->mode.data(), "fit_plan_run", s);
+  else
+    rc = run_graph(p, in, out, hits, s, p->h->d_counters);
   if (rc == FIT_OK) p->h->tracks += (uint64_t)p->total;
   return rc;
 }
