@@ -290,17 +290,20 @@ int build_items(fit_plan* p, int tpb, int tpt) {
 // the p2z launch on the plan's second capture stream, a branch of the graph
 // beside the p2r launch.
 int issue_per_mode(fit_plan* p, const FitArgs& base, cudaStream_t s) {
-  const bool one_launch = is_small(p->h, p->total);
+  // The second capture stream takes launches only once it is forked into the
+  // capture.  A small call is not: it is one launch, or, where its runs exceed
+  // that launch's tables, one launch per mode in order on s.
+  const bool fork = !is_small(p->h, p->total);
   cudaError_t e = cudaSuccess;
-  if (!one_launch) {
+  if (fork) {
     e = cudaEventRecord(p->fork, s);
     if (e == cudaSuccess) e = cudaStreamWaitEvent(p->cap_z, p->fork, 0);
     if (e != cudaSuccess) return cuda_fail(e, "fit_plan: fork");
   }
   const int rc = run_fit(p->h, base, {p->cfg.layout, false, false, p->total},
                          (int)p->ntrk.size(), p->ntrk.data(), p->mode.data(), "fit_plan", s,
-                         p->cap_z);
-  if (!one_launch) {
+                         fork ? p->cap_z : s);
+  if (fork) {
     e = cudaEventRecord(p->join, p->cap_z);
     if (e == cudaSuccess) e = cudaStreamWaitEvent(s, p->join, 0);
     if (e != cudaSuccess && rc == FIT_OK) return cuda_fail(e, "fit_plan: join");

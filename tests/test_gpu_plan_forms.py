@@ -1,0 +1,76 @@
+"""Plans whose events make more runs than a launch's tables hold, replayed on
+new inputs; calls that fill a run table and take another launch."""
+import numpy as np
+import pytest
+
+from paper_2409_09228_gb300 import fit, inputs
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+if not torch.cuda.is_available():  # pragma: no cover - collected on CPU hosts too
+    pytest.skip("needs a CUDA device", allow_module_level=True)
+
+import gpu_util  # noqa: E402
+
+NLAYER = 20
+SMALL_RUNS = 256  # pair runs of a mode that a small call's one launch holds (lone tracks: twice)
+
+
+def runs(nt, md, m):
+    """(pair runs, lone tracks) of mode m: its maximal runs of consecutive
+    events as pairs that start at even tracks, and what their odd edges leave."""
+    pairs = lone = 0
+    start = np.concatenate([[0], np.cumsum(nt)])
+    e = 0
+    while e < len(nt):
+        e0 = e
+        while e < len(nt) and md[e] == md[e0]:
+            e += 1
+        t0, t1 = int(start[e0]), int(start[e])
+        if md[e0] == m and t1 > t0:
+            p0, p1 = (t0 + 1) & ~1, t1 & ~1
+            pairs += p1 > p0
+            lone += (t0 & 1) + ((t1 & 1) and t1 > p0)
+    return pairs, lone
+
+
+def _device(ev, ld):
+    return [gpu_util.to_dev(a, ld) for a in (ev.par0, ev.cov0, ev.q, ev.hpos, ev.hcov)]
+
+
+def _fitter(ev):
+    return fit.Fitter(fit.Geometry(ev.B, ev.surf[0]), fit.Geometry(ev.B, ev.surf[1]))
+
+
+def test_small_per_mode_plan_with_many_runs_replays_both_modes():
+    """A plan of one launch per mode on few tracks in many runs: every run of
+    the captured graph fits both modes' tracks on what the buffers then hold,
+    bit for bit as one call does, and counts them."""
+    nt = np.full(1400, 3)
+    md = (np.arange(1400) % 2).astype(np.int32)
+    assert min(runs(nt, md, m)[0] for m in (0, 1)) > SMALL_RUNS
+    assert nt.sum() <= 128 * torch.cuda.get_device_properties(0).multi_processor_count
+    evs = [inputs.generate_events(nt, md, seed=s, nlayer=NLAYER) for s in (107, 109, 113)]
+    n = evs[0].n
+    ld = gpu_util.pad_ld(n)
+    f = _fitter(evs[0])
+    d = _device(evs[0], ld)
+    out = f.outputs(n, ld=ld, layers=True)
+    plan = fit.fit_plan_create(f.h, nt, md, NLAYER, persistent=False)
+    for ev in evs:  # captured by the first, replayed by the others
+        for a, b in zip(d, _device(ev, ld)):
+            a.copy_(b)
+        for k, v in out.items():
+            v.fill_(float("nan") if v.is_floating_point() else 77)
+        torch.cuda.synchronize()
+        fit.fit_plan_run(plan, *d, par_out=out["par"], cov_out=out["cov"], q_out=out["q"],
+                         chi2=out["chi2"], chi2_layer=out["chi2_layer"], status=out["status"])
+        got_counts = f.sync()
+        ref = f.run(*d, nt, md, layers=True)
+        ref_counts = f.sync()
+        assert got_counts == ref_counts and got_counts["tracks"] == n
+        for k in ref:
+            assert torch.equal(out[k][..., :n], ref[k][..., :n]), k
+    fit.fit_plan_destroy(plan)
+    f.close()
