@@ -156,7 +156,9 @@ int max_blocks_per_sm(int tpb, int tpt, int layout) {
 std::string cache_key(int device, int nlayer, const std::vector<int64_t>& ntrk,
                       const std::vector<int32_t>& mode, int layout) {
   // Device, geometry depth, and the event-size histogram (powers of two) per
-  // mode: plans with the same key have the same shape of work.
+  // mode: plans with the same key have the same shape of work.  v4: entries of
+  // v3 and before were timed when the per-mode form was one launch per run of
+  // events, or with p2z launches missing from its graph.
   cudaDeviceProp prop;
   std::string name = "gpu";
   if (cudaGetDeviceProperties(&prop, device) == cudaSuccess) name = prop.name;
@@ -170,7 +172,7 @@ std::string cache_key(int device, int nlayer, const std::vector<int64_t>& ntrk,
     hist[mode[e]][b]++;
     tracks[mode[e]] += ntrk[e];
   }
-  std::string k = name + ";v3;layout=" + std::to_string(layout) + ";nlayer=" +
+  std::string k = name + ";v4;layout=" + std::to_string(layout) + ";nlayer=" +
                   std::to_string(nlayer) + ";tracks=" +
                   std::to_string(tracks[0]) + "," + std::to_string(tracks[1]) + ";hist=";
   for (int m = 0; m < 2; ++m)

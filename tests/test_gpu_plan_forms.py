@@ -74,3 +74,29 @@ def test_small_per_mode_plan_with_many_runs_replays_both_modes():
             assert torch.equal(out[k][..., :n], ref[k][..., :n]), k
     fit.fit_plan_destroy(plan)
     f.close()
+
+
+def test_tuning_does_not_take_shapes_timed_on_older_kernels(tmp_path):
+    """A cache entry of the key's third version was timed on a per-mode form
+    that has changed since: it is measured anew, and the new entry is taken."""
+    cache = str(tmp_path / "tune.txt")
+    f = None
+    info = {}
+    for n in (1001, 1002):  # two keys that differ in the number of tracks alone
+        ev = inputs.generate_events([n], [0], seed=127, nlayer=NLAYER)
+        ld = gpu_util.pad_ld(n)
+        f = f or _fitter(ev)
+        out = f.outputs(n, ld=ld)
+        plan = fit.fit_plan_create(f.h, [n], [0], NLAYER)
+        info[n] = fit.fit_plan_tune(plan, *_device(ev, ld), out["par"], out["cov"], out["q"],
+                                    out["chi2"], status=out["status"], cache_path=cache)
+        fit.fit_plan_destroy(plan)
+        line = open(cache).read()
+        key, shape = line.split("\n")[-2].split("\t")
+        assert f"tracks={n},0;" in key
+        if n == 1001:
+            old = key.replace("tracks=1001,0;", "tracks=1002,0;").split(";")
+            old[1] = "v3"
+            open(cache, "a").write(";".join(old) + "\t" + shape + "\n")
+    f.close()
+    assert info[1001]["tuned"] == info[1002]["tuned"] == 1
