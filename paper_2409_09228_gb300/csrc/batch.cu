@@ -595,6 +595,7 @@ int fit_plan_tune(fit_plan* p, const fit_tracks_in* in, const fit_tracks_out* ou
   }
   float best = 1e30f;
   fit_launch_config best_cfg = p->cfg;
+  const fit_launch_config was_cfg = p->cfg;
   const bool was_free = p->free_form;
   p->free_form = false;
   for (const fit_launch_config& c : cands) {
@@ -629,7 +630,8 @@ int fit_plan_tune(fit_plan* p, const fit_tracks_in* in, const fit_tracks_out* ou
     cudaStreamSynchronize(s);
     cudaFree(scratch);
   }
-  if (rc != FIT_OK) {
+  if (rc != FIT_OK) {  // the plan as it was, in the layout of the caller's buffers
+    p->cfg = was_cfg;
     p->free_form = was_free;
     return rc;
   }

@@ -1,5 +1,7 @@
 """Plans whose events make more runs than a launch's tables hold, replayed on
 new inputs; calls that fill a run table and take another launch."""
+import ctypes
+
 import numpy as np
 import pytest
 
@@ -100,3 +102,39 @@ def test_tuning_does_not_take_shapes_timed_on_older_kernels(tmp_path):
             open(cache, "a").write(";".join(old) + "\t" + shape + "\n")
     f.close()
     assert info[1001]["tuned"] == info[1002]["tuned"] == 1
+
+
+def test_failed_tuning_leaves_the_plan_as_it_was():
+    """Tuning waits for its stream, which a stream under capture refuses: the
+    call fails in its first candidate, and the plan keeps its shape and layout
+    and runs as before."""
+    ev = inputs.generate_events([300, 301], [0, 1], seed=131, nlayer=NLAYER)
+    ld = (ev.n + 31) // 32 * 32
+    f = _fitter(ev)
+    d = _device(ev, ld)
+    out = f.outputs(ev.n, ld=ld)
+    bufs = dict(par_out=out["par"], cov_out=out["cov"], q_out=out["q"], chi2=out["chi2"],
+                status=out["status"])
+    plan = fit.fit_plan_create(f.h, ev.ntrk, ev.mode, NLAYER, threads_per_block=64, blocks_per_sm=2,
+                               layout=fit.FIT_LAYOUT_TUNE)
+    before = fit.fit_plan_get_info(plan)
+    rt = ctypes.CDLL("libcudart.so.13")
+    stream, graph = torch.cuda.Stream(), ctypes.c_void_p()
+    torch.cuda.synchronize()
+    assert rt.cudaStreamBeginCapture(ctypes.c_void_p(stream.cuda_stream), 2) == 0  # relaxed mode
+    try:
+        with pytest.raises(fit.FitError):
+            fit.fit_plan_tune(plan, *d, stream=stream, **bufs)
+    finally:  # whatever was captured is dropped unlaunched
+        rt.cudaStreamEndCapture(ctypes.c_void_p(stream.cuda_stream), ctypes.byref(graph))
+        if graph.value:
+            rt.cudaGraphDestroy(graph)
+        rt.cudaGetLastError()
+    assert fit.fit_plan_get_info(plan) == before
+    ref = f.run(*d, ev.ntrk, ev.mode)
+    fit.fit_plan_run(plan, *d, **bufs)
+    torch.cuda.synchronize()
+    fit.fit_plan_destroy(plan)
+    f.close()
+    np.testing.assert_allclose(out["par"][:, :ev.n].cpu().numpy(), ref["par"][:, :ev.n].cpu().numpy(),
+                               rtol=1e-4, atol=1e-4)
