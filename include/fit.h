@@ -243,9 +243,11 @@ typedef struct {
 } fit_launch_config;
 
 typedef struct {
-  fit_launch_config config; /* the launch shape the plan runs with */
+  fit_launch_config config; /* the launch shape the plan runs with; blocks_per_sm
+                               0: the default's one launch per mode */
   int64_t tracks;           /* tracks in the plan */
-  int32_t items;            /* work items of the persistent form */
+  int32_t items;            /* work items that the persistent form cuts its events
+                               into with this shape, whether it runs or not */
   int32_t tuned;            /* 0: default or given; 1: measured by fit_plan_tune;
                                2: taken from the tuning cache */
   float best_ms;            /* fit_plan_tune: time of the chosen shape, else 0 */

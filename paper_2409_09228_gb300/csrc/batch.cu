@@ -457,10 +457,12 @@ int fit_plan_create(fit_handle* h, int nevt, const int64_t* ntrk, const int32_t*
   p->cfg.tracks_per_thread = tracks_per_thread(p->cfg);
   p->free_form = p->cfg.persistent && p->cfg.blocks_per_sm == 0 &&
                  p->cfg.threads_per_block == 128 && p->cfg.tracks_per_thread == 2;
-  if (p->cfg.blocks_per_sm == 0)
-    p->cfg.blocks_per_sm =
-        max_blocks_per_sm(p->cfg.threads_per_block, p->cfg.tracks_per_thread, p->cfg.layout);
-  if (p->cfg.blocks_per_sm <= 0) p->cfg.blocks_per_sm = 1;
+  if (!p->free_form) {  // (whose blocks_per_sm stays 0: fit_plan_get_info says so)
+    if (p->cfg.blocks_per_sm == 0)
+      p->cfg.blocks_per_sm =
+          max_blocks_per_sm(p->cfg.threads_per_block, p->cfg.tracks_per_thread, p->cfg.layout);
+    if (p->cfg.blocks_per_sm <= 0) p->cfg.blocks_per_sm = 1;
+  }
   e = cudaMalloc(&p->d_work, sizeof(unsigned));
   if (e == cudaSuccess) e = cudaMalloc(&p->d_tune_counters, kCounters * sizeof(unsigned long long));
   if (e == cudaSuccess) e = cudaStreamCreateWithFlags(&p->cap, cudaStreamNonBlocking);

@@ -138,3 +138,20 @@ def test_failed_tuning_leaves_the_plan_as_it_was():
     f.close()
     np.testing.assert_allclose(out["par"][:, :ev.n].cpu().numpy(), ref["par"][:, :ev.n].cpu().numpy(),
                                rtol=1e-4, atol=1e-4)
+
+
+def test_info_tells_the_default_form_from_a_persistent_shape():
+    """A plan at its default shape runs one launch per mode and reports
+    blocks_per_sm 0, the value that asks for it; a persistent shape reports
+    the blocks per SM it launches."""
+    f = fit.Fitter(fit.Geometry(3.8, inputs.surfaces(0)), None)
+    blocks = {}
+    for name, kw in (("default", {}), ("given", dict(blocks_per_sm=2)),
+                     ("most", dict(threads_per_block=64))):
+        plan = fit.fit_plan_create(f.h, [5000], [0], NLAYER, **kw)
+        info = fit.fit_plan_get_info(plan)
+        blocks[name] = info["blocks_per_sm"]
+        assert info["persistent"] and info["items"] > 0 and info["tuned"] == 0
+        fit.fit_plan_destroy(plan)
+    f.close()
+    assert blocks["default"] == 0 and blocks["given"] == 2 and blocks["most"] > 2
