@@ -1,7 +1,7 @@
 /*
- * fit_probe.h -- measurement probes of libfit (C ABI).
+ * fit_probe.h -- measurement and test probes of libfit (C ABI).
  *
- * Not part of the fit.  The fused kernel's roofline is its FP32 rate against
+ * Not part of the fit.  fit_probe_fp32: the fused kernel's roofline is its FP32 rate against
  * the GPU's FP32 ceiling; the ceiling is derived from unit counts (SMs x 128
  * FP32 lanes x 2 flops x clock), and this probe measures it on the device the
  * fit runs on, with scalar and with packed (two-lane) fused multiply-adds, so
@@ -12,6 +12,8 @@
 #define FIT_PROBE_H
 
 #include <stdint.h>
+
+#include "fit.h"
 
 #ifdef __cplusplus
 extern "C" {
@@ -41,6 +43,14 @@ extern "C" {
  * if the launch fails (message in fit_last_error()).
  */
 int fit_probe_fp32(int packed, int blocks, int iters, float* out, void* stream, double* flops);
+
+/*
+ * fit_probe_host_in_place: whether fit_propagate_update_host would take these
+ * buffers of n tracks in place (1) or stage them (0) on the current device; a
+ * question to the driver, nothing runs.  FIT_ERR_ARG on a bad argument.
+ */
+int fit_probe_host_in_place(const fit_tracks_in* in, const fit_tracks_out* out,
+                            const fit_hits* hits, int64_t n, int nlayer);
 
 #ifdef __cplusplus
 }

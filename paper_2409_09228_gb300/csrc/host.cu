@@ -5,6 +5,7 @@
 // and copies of the others (paper Sec. 3.1: inputs are copied to the device
 // before the kernel and results back after it).  The caller's stream orders
 // the whole call.
+#include <cuda.h>
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -13,6 +14,7 @@
 #include <vector>
 
 #include "fit.h"
+#include "fit_probe.h"
 #include "internal.h"
 
 using namespace fitimpl;
@@ -125,12 +127,43 @@ bool mapped_host(const void* p) {
   return a.type == cudaMemoryTypeHost && a.devicePointer == p;
 }
 
-// The same for the first and last byte of rows x n elements of `size` bytes
-// with row stride ld.
+// The page-locked range (one allocation or registration) that holds p.  The
+// driver reports it, for both kinds of memory; the runtime does not.
+bool host_range(const void* p, uintptr_t* start, size_t* bytes) {
+  using Query = CUresult (*)(unsigned, CUpointer_attribute*, void**, CUdeviceptr);
+  static const Query query = [] {
+    void* f = nullptr;
+    cudaDriverEntryPointQueryResult found;
+    if (cudaGetDriverEntryPointByVersion("cuPointerGetAttributes", &f, 12000, cudaEnableDefault,
+                                         &found) != cudaSuccess ||
+        found != cudaDriverEntryPointSuccess) {
+      cudaGetLastError();
+      f = nullptr;
+    }
+    return reinterpret_cast<Query>(f);
+  }();
+  if (!query) return false;
+  CUdeviceptr first = 0;
+  CUpointer_attribute what[2] = {CU_POINTER_ATTRIBUTE_RANGE_START_ADDR,
+                                 CU_POINTER_ATTRIBUTE_RANGE_SIZE};
+  void* to[2] = {&first, bytes};
+  *bytes = 0;
+  if (query(2, what, to, reinterpret_cast<CUdeviceptr>(p)) != CUDA_SUCCESS || !first) return false;
+  *start = (uintptr_t)first;
+  return true;
+}
+
+// Whether the rows x n elements of `size` bytes at p, with row stride ld, lie
+// in one such range from the first byte to the last.  (Both ends in page-locked
+// memory are not enough: a caller may have locked an array's pieces, and what
+// lies between them may be pageable.)
 bool mapped_rows(const void* p, int64_t rows, int64_t ld, int64_t n, int64_t size) {
   if (!p || !rows) return true;
-  const char* c = static_cast<const char*>(p);
-  return mapped_host(c) && mapped_host(c + ((rows - 1) * ld + n) * size - 1);
+  uintptr_t start = 0;
+  size_t bytes = 0;
+  if (!mapped_host(p) || !host_range(p, &start, &bytes)) return false;
+  const uintptr_t before = reinterpret_cast<uintptr_t>(p) - start;
+  return before <= bytes && (size_t)(((rows - 1) * ld + n) * size) <= bytes - before;
 }
 
 // Whether every buffer of a call over n tracks is such memory throughout.
@@ -249,6 +282,14 @@ extern "C" int fit_propagate_update_host(fit_handle* h, const fit_tracks_in* in,
   if (e != cudaSuccess) return cuda_fail(e, "fit_propagate_update_host: stream order");
   h->tracks += (uint64_t)total;
   return FIT_OK;
+}
+
+extern "C" int fit_probe_host_in_place(const fit_tracks_in* in, const fit_tracks_out* out,
+                                       const fit_hits* hits, int64_t n, int nlayer) {
+  g_last_error.clear();
+  if (!in || !out || !hits || n < 1 || nlayer < 1)
+    return fail(FIT_ERR_ARG, "fit_probe_host_in_place: bad argument");
+  return mapped_call(in, out, hits, n, nlayer) ? 1 : 0;
 }
 
 extern "C" int fit_propagate_update_mapped(fit_handle* h, const fit_tracks_in* in,

@@ -103,7 +103,7 @@ EXPORTS = ("fit_init", "fit_propagate_update", "fit_sync", "fit_destroy", "fit_l
            "fit_mlp_adam_step", "fit_mlp_train", "fit_mlp_attach", "fit_path_lengths",
            "fit_propagate_update_host", "fit_propagate_update_mapped", "fit_propagate_update_f64",
            "fit_propagate_update_layout", "fit_find_tracks", "fit_find_tracks_f64",
-           "fit_relayout", "fit_probe_fp32")
+           "fit_relayout", "fit_probe_fp32", "fit_probe_host_in_place")
 FIT_LAYOUT_SOA = 0
 FIT_LAYOUT_AOSOA32 = 1
 FIT_LAYOUT_TUNE = 2
@@ -202,6 +202,8 @@ def load(build_if_missing: bool = True):
     L.fit_probe_fp32.argtypes = [ctypes.c_int, ctypes.c_int, ctypes.c_int, vp, vp,
                                  ctypes.POINTER(ctypes.c_double)]
     L.fit_probe_fp32.restype = ctypes.c_int
+    L.fit_probe_host_in_place.argtypes = [vp, vp, vp, i64, ci]
+    L.fit_probe_host_in_place.restype = ci
     L.fit_relayout.argtypes = [vp, i64, ctypes.c_int, vp, i64, ctypes.c_int, ctypes.c_int, i64, vp]
     L.fit_relayout.restype = ctypes.c_int
     _lib = L
@@ -655,6 +657,20 @@ def fit_last_error() -> str:
 
 
 FIT_PROBE_THREADS = 256
+
+
+def fit_probe_host_in_place(par_in, cov_in, q_in, hpos, hcov, n: int, par_out, cov_out, q_out,
+                            chi2, chi2_layer=None, status=None) -> bool:
+    """Whether fit_propagate_update_host takes these host arrays in place
+    (include/fit_probe.h)."""
+    tin = _TRACKS_IN(_haddr(par_in), _haddr(cov_in), _haddr(q_in), par_in.shape[-1])
+    tout = _TRACKS_OUT(_haddr(par_out), _haddr(cov_out), _haddr(q_out), _haddr(chi2),
+                       _haddr(chi2_layer), _haddr(status), par_out.shape[-1])
+    rc = load().fit_probe_host_in_place(tin, tout, _HITS(_haddr(hpos), _haddr(hcov), hpos.shape[-1]),
+                                        int(n), hpos.shape[0])
+    if rc < 0:
+        _check(rc)
+    return rc == 1
 
 
 def fit_probe_fp32(packed: bool, blocks: int, iters: int, out, stream=None) -> float:
