@@ -452,7 +452,8 @@ int fit_find_tracks_f64(fit_handle* h, const fit_tracks_in_f64* in, const fit_tr
  * structs, layouts and checks; every data pointer in in, out and hits is a
  * host pointer).  Where every buffer lies, from its first byte to its
  * last, in one page-locked range (one allocation or registration) that the
- * device reaches under the same address, the call is
+ * device reaches under the same address, and no output overlaps an input but
+ * par, cov or q of the same address and ld, the call is
  * fit_propagate_update_mapped: the kernels read and write the buffers in
  * place.  Otherwise the library
  * cuts the tracks into chunks of up to FIT_HOST_CHUNK and moves each through

@@ -153,30 +153,57 @@ bool host_range(const void* p, uintptr_t* start, size_t* bytes) {
   return true;
 }
 
-// Whether the rows x n elements of `size` bytes at p, with row stride ld, lie
-// in one such range from the first byte to the last.  (Both ends in page-locked
-// memory are not enough: a caller may have locked an array's pieces, and what
-// lies between them may be pageable.)
-bool mapped_rows(const void* p, int64_t rows, int64_t ld, int64_t n, int64_t size) {
-  if (!p || !rows) return true;
+// rows x n elements of `size` bytes, with row stride ld; p may be NULL.
+struct HostArray {
+  const void* p;
+  int64_t rows, ld, n, size;
+  size_t bytes() const { return p && rows ? (size_t)(((rows - 1) * ld + n) * size) : 0; }
+};
+
+// Whether an array lies in one such range from the first byte to the last.
+// (Both ends in page-locked memory are not enough: a caller may have locked an
+// array's pieces, and what lies between them may be pageable.)
+bool mapped_array(const HostArray& a) {
+  if (!a.bytes()) return true;
   uintptr_t start = 0;
   size_t bytes = 0;
-  if (!mapped_host(p) || !host_range(p, &start, &bytes)) return false;
-  const uintptr_t before = reinterpret_cast<uintptr_t>(p) - start;
-  return before <= bytes && (size_t)(((rows - 1) * ld + n) * size) <= bytes - before;
+  if (!mapped_host(a.p) || !host_range(a.p, &start, &bytes)) return false;
+  const uintptr_t before = reinterpret_cast<uintptr_t>(a.p) - start;
+  return before <= bytes && a.bytes() <= bytes - before;
 }
 
-// Whether every buffer of a call over n tracks is such memory throughout.
-bool mapped_call(const fit_tracks_in* in, const fit_tracks_out* out, const fit_hits* hits,
-                 int64_t n, int nlayer) {
-  return mapped_rows(in->par, 6, in->ld, n, 4) && mapped_rows(in->cov, 21, in->ld, n, 4) &&
-         mapped_rows(in->q, 1, in->ld, n, 4) && mapped_rows(out->par, 6, out->ld, n, 4) &&
-         mapped_rows(out->cov, 21, out->ld, n, 4) && mapped_rows(out->q, 1, out->ld, n, 4) &&
-         mapped_rows(out->chi2, 1, out->ld, n, 4) &&
-         mapped_rows(out->chi2_layer, nlayer, out->ld, n, 4) &&
-         mapped_rows(out->status, 1, out->ld, n, 1) &&
-         mapped_rows(hits->pos, 3 * (int64_t)nlayer, hits->ld, n, 4) &&
-         mapped_rows(hits->cov, 6 * (int64_t)nlayer, hits->ld, n, 4);
+bool overlap(const HostArray& a, const HostArray& b) {
+  const uintptr_t x = reinterpret_cast<uintptr_t>(a.p), y = reinterpret_cast<uintptr_t>(b.p);
+  return a.bytes() && b.bytes() && x < y + b.bytes() && y < x + a.bytes();
+}
+
+// Whether a call over n tracks can run on its buffers in place: every one
+// page-locked throughout, and no output over an input but the same array in
+// the same place (each thread reads its track's column before it writes it;
+// shifted, one thread would overwrite what another has yet to read, while the
+// staged path copies a chunk's inputs before its outputs).
+bool in_place(const fit_tracks_in* in, const fit_tracks_out* out, const fit_hits* hits, int64_t n,
+              int nlayer) {
+  const HostArray ins[] = {{in->par, 6, in->ld, n, 4},
+                           {in->cov, 21, in->ld, n, 4},
+                           {in->q, 1, in->ld, n, 4},
+                           {hits->pos, 3 * (int64_t)nlayer, hits->ld, n, 4},
+                           {hits->cov, 6 * (int64_t)nlayer, hits->ld, n, 4}};
+  const HostArray outs[] = {{out->par, 6, out->ld, n, 4},    {out->cov, 21, out->ld, n, 4},
+                            {out->q, 1, out->ld, n, 4},      {out->chi2, 1, out->ld, n, 4},
+                            {out->chi2_layer, nlayer, out->ld, n, 4},
+                            {out->status, 1, out->ld, n, 1}};
+  for (int o = 0; o < 6; ++o)
+    for (int i = 0; i < 5; ++i) {
+      const bool same = o == i && o < 3 && outs[o].p == ins[i].p &&
+                        (o == 2 || outs[o].ld == ins[i].ld);
+      if (!same && overlap(outs[o], ins[i])) return false;
+    }
+  for (const HostArray& a : ins)
+    if (!mapped_array(a)) return false;
+  for (const HostArray& a : outs)
+    if (!mapped_array(a)) return false;
+  return true;
 }
 
 }  // namespace
@@ -205,8 +232,8 @@ extern "C" int fit_propagate_update_host(fit_handle* h, const fit_tracks_in* in,
   // them in place, which moves only what they touch (5 of a p2z hit's 9
   // floats) at the link's rate and needs no staging: 96000 tracks of both modes
   // 520 -> 334 us, 1.92M 8.1-20.8 -> 6.3 ms.
-  // Pageable buffers go through the staging sets.
-  if (mapped_call(in, out, hits, total, nlayer)) {
+  // Others go through the staging sets.
+  if (in_place(in, out, hits, total, nlayer)) {
     rc = run_fit_streams(h, base_args(in, out, hits, nlayer, h->d_counters),
                          {FIT_LAYOUT_SOA, h->seeded, false, total}, nevt, ntrk, mode, kWho,
                          static_cast<cudaStream_t>(stream));
@@ -289,7 +316,7 @@ extern "C" int fit_probe_host_in_place(const fit_tracks_in* in, const fit_tracks
   g_last_error.clear();
   if (!in || !out || !hits || n < 1 || nlayer < 1)
     return fail(FIT_ERR_ARG, "fit_probe_host_in_place: bad argument");
-  return mapped_call(in, out, hits, n, nlayer) ? 1 : 0;
+  return in_place(in, out, hits, n, nlayer) ? 1 : 0;
 }
 
 extern "C" int fit_propagate_update_mapped(fit_handle* h, const fit_tracks_in* in,

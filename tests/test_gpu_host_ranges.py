@@ -75,3 +75,23 @@ def test_arrays_locked_in_pieces_are_staged(name):
                    [(0, tail)]):
         with _Locked(a, pieces):
             assert not _in_place({**bufs, name: a})
+
+
+def test_outputs_over_other_inputs_are_staged():
+    """In place an output may only be the input it replaces: shifted, narrower
+    or over another array, threads would overwrite what others have yet to
+    read."""
+    bufs = _pinned()
+    own = {k: bufs[k.replace("out", "in")] for k in ("par_out", "cov_out", "q_out")}
+    assert _in_place({**bufs, **own})
+    wide = torch.zeros((30, N + 8)).pin_memory()  # ld of the inputs and the outputs: N + 8
+    par = {"par_in": wide[:6], "cov_in": bufs["cov_in"].new_zeros((21, N + 8)).pin_memory(),
+           "cov_out": torch.zeros((21, N + 8)).pin_memory()}
+    assert _in_place({**bufs, **par, "par_out": wide[:6]})
+    assert _in_place({**bufs, **par, "par_out": wide[6:12]})
+    assert not _in_place({**bufs, **par, "par_out": wide[1:7]})
+    assert not _in_place({**bufs, **par, "par_out": wide.view(-1)[4:].as_strided((6, N + 8), (N + 8, 1))})
+    narrow = {**bufs, "par_out": bufs["par_in"].view(-1)[:6 * (N - 8)].view(6, N - 8)}
+    assert not fit.fit_probe_host_in_place(**narrow, n=N - 8)
+    assert not _in_place({**bufs, "chi2": bufs["hpos"][0, 0]})
+    assert not _in_place({**bufs, "chi2_layer": bufs["hcov"].view(-1)[:NLAYER * N].view(NLAYER, N)})
