@@ -128,8 +128,9 @@ typedef struct {
  * fit_init: creates a handle on CUDA device `device` for the two modes.
  * cfg_r / cfg_z describe the p2r cylinders and the p2z planes; either may be
  * NULL if that mode is never used.  The handle allocates its own small device
- * scratch (status counters) and creates a second CUDA stream with two events
- * (see fit_propagate_update); fit_destroy frees them.
+ * scratch (status counters) and creates a second CUDA stream with two events,
+ * and up to seven more as calls on several streams need them (see
+ * fit_propagate_update); fit_destroy frees them.
  * Errors: FIT_ERR_ARG (bad config), FIT_ERR_CUDA, FIT_ERR_NOMEM.
  */
 int fit_init(fit_handle** h, const fit_config* cfg_r, const fit_config* cfg_z, int device);
@@ -144,10 +145,16 @@ int fit_init(fit_handle** h, const fit_config* cfg_r, const fit_config* cfg_z, i
  * nlayer must equal the configured nlayer of every mode used.
  * The events of a mode run as one kernel launch (one for every 1024 runs of
  * consecutive same-mode events), whatever their order.  A call with events of
- * both modes runs its p2z launch on the handle's second stream, forked from
+ * both modes runs its p2z launch on a second stream of the handle, forked from
  * `stream` before it and joined back after it, so that it overlaps the p2r
- * launch; `stream` follows the whole call as before.  Calls
- * on one handle from several host threads take turns for that stream.
+ * launch; `stream` follows the whole call as before.  The same holds for the
+ * other calls on tracks (layout, host, mapped, plans at the default shape, the
+ * finder, the adjoint, small FP64 calls).  Calls on several streams, from one
+ * host thread or several, do not wait for one another: each caller's stream
+ * has a second stream of its own (with more than eight at work at once, the
+ * launches of a further call follow one another on its `stream`).  Under
+ * stream capture the two launches are branches of the captured graph, and no
+ * stream of the handle joins the capture.
  * Errors: FIT_ERR_ARG (NULL pointer, misaligned pointer or ld, sizes out of
  * range, unconfigured mode), FIT_ERR_CUDA (launch failure).
  */

@@ -242,8 +242,7 @@ struct fit_plan {
   int items_tile = 0;  // tracks per work item of the current table
   int items_tpt = 0;
   unsigned* d_work = nullptr;
-  cudaStream_t cap = nullptr, cap_z = nullptr;  // capture streams
-  cudaEvent_t fork = nullptr, join = nullptr;
+  cudaStream_t cap = nullptr;  // capture stream
   cudaGraphExec_t exec = nullptr;
   const void* key_ptrs[12] = {};
   unsigned long long* d_tune_counters = nullptr;  // counters of the tuning runs
@@ -288,31 +287,6 @@ int build_items(fit_plan* p, int tpb, int tpt) {
   return FIT_OK;
 }
 
-// fit_propagate_update's form on the plan's events, an autotuner candidate:
-// the p2z launch on the plan's second capture stream, a branch of the graph
-// beside the p2r launch.
-int issue_per_mode(fit_plan* p, const FitArgs& base, cudaStream_t s) {
-  // The second capture stream takes launches only once it is forked into the
-  // capture.  A small call is not: it is one launch, or, where its runs exceed
-  // that launch's tables, one launch per mode in order on s.
-  const bool fork = !is_small(p->h, p->total);
-  cudaError_t e = cudaSuccess;
-  if (fork) {
-    e = cudaEventRecord(p->fork, s);
-    if (e == cudaSuccess) e = cudaStreamWaitEvent(p->cap_z, p->fork, 0);
-    if (e != cudaSuccess) return cuda_fail(e, "fit_plan: fork");
-  }
-  const int rc = run_fit(p->h, base, {p->cfg.layout, false, false, p->total},
-                         (int)p->ntrk.size(), p->ntrk.data(), p->mode.data(), "fit_plan", s,
-                         fork ? p->cap_z : s);
-  if (fork) {
-    e = cudaEventRecord(p->join, p->cap_z);
-    if (e == cudaSuccess) e = cudaStreamWaitEvent(s, p->join, 0);
-    if (e != cudaSuccess && rc == FIT_OK) return cuda_fail(e, "fit_plan: join");
-  }
-  return rc;
-}
-
 // Issues the plan's work for one shape on stream s (captured into a graph).
 int issue(fit_plan* p, const FitArgs& base, cudaStream_t s) {
   if (p->total == 0) return FIT_OK;
@@ -335,7 +309,9 @@ int issue(fit_plan* p, const FitArgs& base, cudaStream_t s) {
     if (e != cudaSuccess) return cuda_fail(e, "fit_plan: launch");
     return FIT_OK;
   }
-  return issue_per_mode(p, base, s);
+  // one launch per mode, fit_propagate_update's form: two branches of the graph
+  return run_fit_streams(p->h, base, {p->cfg.layout, false, false, p->total}, (int)p->ntrk.size(),
+                         p->ntrk.data(), p->mode.data(), "fit_plan", s);
 }
 
 void drop_graph(fit_plan* p) {
@@ -466,9 +442,6 @@ int fit_plan_create(fit_handle* h, int nevt, const int64_t* ntrk, const int32_t*
   e = cudaMalloc(&p->d_work, sizeof(unsigned));
   if (e == cudaSuccess) e = cudaMalloc(&p->d_tune_counters, kCounters * sizeof(unsigned long long));
   if (e == cudaSuccess) e = cudaStreamCreateWithFlags(&p->cap, cudaStreamNonBlocking);
-  if (e == cudaSuccess) e = cudaStreamCreateWithFlags(&p->cap_z, cudaStreamNonBlocking);
-  if (e == cudaSuccess) e = cudaEventCreateWithFlags(&p->fork, cudaEventDisableTiming);
-  if (e == cudaSuccess) e = cudaEventCreateWithFlags(&p->join, cudaEventDisableTiming);
   if (e != cudaSuccess) {
     fit_plan_destroy(p);
     return fail(FIT_ERR_NOMEM, std::string("fit_plan_create: ") + cudaGetErrorString(e));
@@ -694,9 +667,6 @@ void fit_plan_destroy(fit_plan* p) {
     if (p->d_items) cudaFree(p->d_items);
     if (p->d_work) cudaFree(p->d_work);
     if (p->d_tune_counters) cudaFree(p->d_tune_counters);
-    if (p->join) cudaEventDestroy(p->join);
-    if (p->fork) cudaEventDestroy(p->fork);
-    if (p->cap_z) cudaStreamDestroy(p->cap_z);
     if (p->cap) cudaStreamDestroy(p->cap);
   }
   delete p;

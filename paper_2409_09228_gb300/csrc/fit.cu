@@ -382,12 +382,11 @@ bool launch_small(const fit_handle* h, const FitArgs& a, bool by_event, int nevt
 bool is_small(int sms, int64_t call_tracks) { return call_tracks <= (int64_t)sms * kBlock; }
 bool is_small(const fit_handle* h, int64_t call_tracks) { return is_small(h->sms, call_tracks); }
 
-// The fused fit of events [0, nevt) on the tracks of a: the p2r events on
-// stream s, the p2z events on sz.
+// The fused fit of events [0, nevt) on the tracks of a.
 int run_fit(const fit_handle* h, const FitArgs& a, const RunOptions& o, int nevt,
-            const int64_t* ntrk, const int32_t* mode, const char* who, cudaStream_t s,
-            cudaStream_t sz) {
+            const int64_t* ntrk, const int32_t* mode, const char* who, ModeStreams& ms) {
   const bool soa = o.layout == FIT_LAYOUT_SOA;
+  const cudaStream_t s = ms.of(FIT_MODE_R);
   if (!o.seeded && is_small(h, o.call_tracks)) {
     const bool done = launch_small(h, a, o.by_event, nevt, ntrk, mode,
                                    [&](const auto& args, unsigned nblk) {
@@ -408,13 +407,85 @@ int run_fit(const fit_handle* h, const FitArgs& a, const RunOptions& o, int nevt
   return launch_runs(h, a, o.by_event, nevt, ntrk, mode, who,
                      [&](const FitArgs& a1, int m, const PairRuns<kMaxRuns>& r) {
                        if (m == FIT_MODE_R && o.seeded) return;
+                       const cudaStream_t sm = ms.of(m);
                        if (soa)
-                         m == FIT_MODE_Z ? launch_fused<FIT_MODE_Z, 0>(a1, r, sz)
-                                         : launch_fused<FIT_MODE_R, 0>(a1, r, s);
+                         m == FIT_MODE_Z ? launch_fused<FIT_MODE_Z, 0>(a1, r, sm)
+                                         : launch_fused<FIT_MODE_R, 0>(a1, r, sm);
                        else
-                         m == FIT_MODE_Z ? launch_fused<FIT_MODE_Z, 1>(a1, r, sz)
-                                         : launch_fused<FIT_MODE_R, 1>(a1, r, s);
+                         m == FIT_MODE_Z ? launch_fused<FIT_MODE_Z, 1>(a1, r, sm)
+                                         : launch_fused<FIT_MODE_R, 1>(a1, r, sm);
                      });
+}
+
+cudaError_t create_side(SideStream& x) {
+  cudaError_t e = cudaStreamCreateWithFlags(&x.st, cudaStreamNonBlocking);
+  if (e == cudaSuccess) e = cudaEventCreateWithFlags(&x.fork, cudaEventDisableTiming);
+  if (e == cudaSuccess) e = cudaEventCreateWithFlags(&x.join, cudaEventDisableTiming);
+  if (e != cudaSuccess) destroy_side(x);
+  return e;
+}
+
+void destroy_side(SideStream& x) {
+  if (x.join) cudaEventDestroy(x.join);
+  if (x.fork) cudaEventDestroy(x.fork);
+  if (x.st) cudaStreamDestroy(x.st);
+  x = SideStream();
+}
+
+namespace {
+
+// A second stream for the caller's stream s, marked busy; NULL if there is
+// none to be had (another thread is queueing on s's, or all are at work).
+SideStream* take_side(fit_handle* h, cudaStream_t s) {
+  unsigned long long id = 0;
+  if (cudaStreamGetId(s, &id) != cudaSuccess) {
+    cudaGetLastError();
+    return nullptr;
+  }
+  std::lock_guard<std::mutex> lock(h->side_mu);
+  SideStream* found = nullptr;
+  for (SideStream& x : h->side)
+    if (x.st && x.caller == id) found = &x;
+  if (found) {
+    if (found->busy) return nullptr;
+  } else {
+    // (queries and creations that another thread's capture must not mind)
+    cudaStreamCaptureMode capture_mode = cudaStreamCaptureModeRelaxed;
+    cudaThreadExchangeStreamCaptureMode(&capture_mode);
+    for (SideStream& x : h->side) {
+      if (x.busy) continue;
+      if (x.st ? cudaStreamQuery(x.st) == cudaSuccess : create_side(x) == cudaSuccess) {
+        found = &x;
+        break;
+      }
+      cudaGetLastError();
+    }
+    cudaThreadExchangeStreamCaptureMode(&capture_mode);
+    if (!found) return nullptr;
+    found->caller = id;
+  }
+  found->busy = true;
+  return found;
+}
+
+}  // namespace
+
+cudaError_t ModeStreams::frontier(Frontier* f, cudaStreamCaptureStatus* status) const {
+  const cudaGraphNode_t* nodes = nullptr;
+  const cudaGraphEdgeData* edges = nullptr;
+  size_t n = 0;
+  const cudaError_t e =
+      cudaStreamGetCaptureInfo(s_, status, nullptr, nullptr, &nodes, &edges, &n);
+  if (e != cudaSuccess || *status != cudaStreamCaptureStatusActive) return e;
+  f->nodes.assign(nodes, nodes + n);
+  f->edges.assign(edges, edges ? edges + n : edges);
+  return e;
+}
+
+cudaError_t ModeStreams::depend(Frontier& f, unsigned how) {
+  return cudaStreamUpdateCaptureDependencies(s_, f.nodes.data(),
+                                             f.edges.empty() ? nullptr : f.edges.data(),
+                                             f.nodes.size(), how);
 }
 
 int ModeStreams::begin(int nevt, const int64_t* ntrk, const int32_t* mode) {
@@ -422,22 +493,53 @@ int ModeStreams::begin(int nevt, const int64_t* ntrk, const int32_t* mode) {
   for (int e = 0; e < nevt; ++e)
     if (ntrk[e] > 0) used[mode[e] == FIT_MODE_Z] = true;
   if (!(used[0] && used[1])) return FIT_OK;
-  lock_ = std::unique_lock<std::mutex>(h_->side_mu);
-  cudaError_t e = cudaEventRecord(h_->fork, s_);
-  if (e == cudaSuccess) e = cudaStreamWaitEvent(h_->side, h_->fork, 0);
+  cudaStreamCaptureStatus status = cudaStreamCaptureStatusNone;
+  if (frontier(&before_, &status) != cudaSuccess) {  // the launches on s_ will say what is wrong
+    cudaGetLastError();
+    return FIT_OK;
+  }
+  if (status != cudaStreamCaptureStatusNone) {
+    captured_ = status == cudaStreamCaptureStatusActive;
+    return FIT_OK;
+  }
+  side_ = take_side(h_, s_);
+  if (!side_) return FIT_OK;
+  cudaError_t e = cudaEventRecord(side_->fork, s_);
+  if (e == cudaSuccess) e = cudaStreamWaitEvent(side_->st, side_->fork, 0);
   if (e != cudaSuccess)
     return cuda_fail(e, (std::string(who_) + ": fork to the second stream").c_str());
-  forked_ = true;
   return FIT_OK;
 }
 
+cudaStream_t ModeStreams::of(int m) {
+  if (m == FIT_MODE_R) return s_;
+  if (side_) return side_->st;
+  if (captured_ && !branched_) {
+    branched_ = true;
+    cudaStreamCaptureStatus status;
+    err_ = frontier(&after_r_, &status);
+    if (err_ == cudaSuccess) err_ = depend(before_, cudaStreamSetCaptureDependencies);
+  }
+  return s_;
+}
+
 int ModeStreams::end(int rc) {
-  if (!forked_) return rc;
-  cudaError_t e = cudaEventRecord(h_->join, h_->side);
-  if (e == cudaSuccess) e = cudaStreamWaitEvent(s_, h_->join, 0);
+  cudaError_t e = err_;
+  if (side_) {
+    e = cudaEventRecord(side_->join, side_->st);
+    if (e == cudaSuccess) e = cudaStreamWaitEvent(s_, side_->join, 0);
+  } else if (branched_ && e == cudaSuccess) {
+    e = depend(after_r_, cudaStreamAddCaptureDependencies);
+  }
   if (e != cudaSuccess && rc == FIT_OK)
     return cuda_fail(e, (std::string(who_) + ": join from the second stream").c_str());
   return rc;
+}
+
+ModeStreams::~ModeStreams() {
+  if (!side_) return;
+  std::lock_guard<std::mutex> lock(h_->side_mu);
+  side_->busy = false;
 }
 
 int run_fit_streams(fit_handle* h, const FitArgs& a, const RunOptions& o, int nevt,
@@ -446,7 +548,7 @@ int run_fit_streams(fit_handle* h, const FitArgs& a, const RunOptions& o, int ne
   const bool one_launch = !o.seeded && is_small(h, o.call_tracks);
   const int rc = one_launch ? FIT_OK : ms.begin(nevt, ntrk, mode);
   if (rc != FIT_OK) return rc;
-  return ms.end(run_fit(h, a, o, nevt, ntrk, mode, who, ms.of(FIT_MODE_R), ms.of(FIT_MODE_Z)));
+  return ms.end(run_fit(h, a, o, nevt, ntrk, mode, who, ms));
 }
 
 // Scratch of fit_propagate_update_noalloc, in the library image instead of
@@ -514,13 +616,8 @@ int fit_init(fit_handle** out, const fit_config* cfg_r, const fit_config* cfg_z,
     return fail(FIT_ERR_NOMEM, std::string("fit_init: cudaMalloc: ") + cudaGetErrorString(e));
   }
   e = cudaMemset(h->d_counters, 0, kCounters * sizeof(unsigned long long));
-  if (e == cudaSuccess) e = cudaStreamCreateWithFlags(&h->side, cudaStreamNonBlocking);
-  if (e == cudaSuccess) e = cudaEventCreateWithFlags(&h->fork, cudaEventDisableTiming);
-  if (e == cudaSuccess) e = cudaEventCreateWithFlags(&h->join, cudaEventDisableTiming);
+  if (e == cudaSuccess) e = create_side(h->side[0]);
   if (e != cudaSuccess) {
-    if (h->join) cudaEventDestroy(h->join);
-    if (h->fork) cudaEventDestroy(h->fork);
-    if (h->side) cudaStreamDestroy(h->side);
     cudaFree(h->d_counters);
     delete h;
     return cuda_fail(e, "fit_init: counters, stream and events");
@@ -698,9 +795,7 @@ void fit_destroy(fit_handle* h) {
     if (h->d_counters || h->d_mlp || h->host_stage) cudaDeviceSynchronize();
     if (h->d_counters) cudaFree(h->d_counters);
     if (h->d_mlp) cudaFree(h->d_mlp);
-    if (h->join) cudaEventDestroy(h->join);
-    if (h->fork) cudaEventDestroy(h->fork);
-    if (h->side) cudaStreamDestroy(h->side);
+    for (SideStream& x : h->side) destroy_side(x);
     destroy_host_stage(h);
   }
   delete h;

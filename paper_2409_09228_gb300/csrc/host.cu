@@ -287,9 +287,10 @@ extern "C" int fit_propagate_update_host(fit_handle* h, const fit_tracks_in* in,
     fit_tracks_out sout{S.par, S.cov, S.q, S.chi2, out->chi2_layer ? S.chi2_layer : nullptr,
                         out->status ? S.status : nullptr, hs->cap};
     fit_hits shit{S.hpos, S.hcov, hs->cap};
+    ModeStreams one(h, s, kWho);  // the chunk's launches in order on its stream
     rc = run_fit(h, base_args(&sin, &sout, &shit, nlayer, h->d_counters),
                  {FIT_LAYOUT_SOA, h->seeded, false, total}, (int)nt_local.size(), nt_local.data(),
-                 md_local.data(), kWho, s, s);
+                 md_local.data(), kWho, one);
     if (rc != FIT_OK) return rc;
     e = copy_rows(out->par + c0, pout, S.par, P, w, 6, cudaMemcpyDeviceToHost, s);
     if (e == cudaSuccess) e = copy_rows(out->cov + c0, pout, S.cov, P, w, 21, cudaMemcpyDeviceToHost, s);

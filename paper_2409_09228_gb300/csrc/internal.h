@@ -7,6 +7,7 @@
 #include <cstdint>
 #include <mutex>
 #include <string>
+#include <vector>
 
 #include "fit.h"
 
@@ -100,6 +101,17 @@ class DeviceGuard {
 };
 
 
+// A second stream of a handle (ModeStreams).
+struct SideStream {
+  cudaStream_t st = nullptr;
+  cudaEvent_t fork = nullptr, join = nullptr;
+  unsigned long long caller = 0;  // id of the stream that it served last
+  bool busy = false;              // a call is queueing on it
+};
+constexpr int kSideStreams = 8;
+cudaError_t create_side(SideStream& x);
+void destroy_side(SideStream& x);
+
 }  // namespace fitimpl
 
 
@@ -115,12 +127,8 @@ struct fit_handle {
   bool seeded = false;    // p2r seeds from d_mlp
   void* host_stage = nullptr;  // staging of fit_propagate_update_host (host.cu)
   float B[2] = {0.f, 0.f};     // field of each mode's configuration
-  // A call with events of both modes runs its p2z launches on `side`, forked
-  // from the caller's stream by `fork` and joined back by `join`; side_mu
-  // keeps concurrent calls from interleaving them (ModeStreams).
-  cudaStream_t side = nullptr;
-  cudaEvent_t fork = nullptr, join = nullptr;
-  std::mutex side_mu;
+  fitimpl::SideStream side[fitimpl::kSideStreams];  // the first from fit_init, others when needed
+  std::mutex side_mu;  // guards the entries' taking and giving back
 };
 
 
@@ -193,36 +201,56 @@ struct RunOptions {
 // Whether a call of that many tracks takes one launch for both modes (fit.cu).
 bool is_small(const fit_handle* h, int64_t call_tracks);
 
-// The fused fit of events [0, nevt) (fit.cu): the p2r events in one launch on
-// stream s (kMaxRuns runs each), the p2z events in one on sz; a small call in
-// one launch on s.
-int run_fit(const fit_handle* h, const FitArgs& a, const RunOptions& o, int nevt,
-            const int64_t* ntrk, const int32_t* mode, const char* who, cudaStream_t s,
-            cudaStream_t sz);
-
 // The two modes' events of a call are independent: with both present, the
-// p2z launches go to the handle's second stream, so that they overlap the p2r
-// launches (their blocks fill the SMs a launch's last wave leaves idle).
-// begin() forks it from the caller's stream s, end(rc) joins it back (even
-// after a failed launch, so that s still follows everything that was queued)
-// and returns rc or the join's error.  A mutex keeps calls from several host
-// threads from interleaving their fork and join.
+// p2z launches go to a second stream, so that they overlap the p2r launches
+// (their blocks fill the SMs a launch's last wave leaves idle).  begin() forks
+// it from the caller's stream s, of(m) is the stream for a launch of mode m
+// (the p2r launches first), and end(rc) joins it back (even after a failed
+// launch, so that s still follows everything that was queued) and returns rc
+// or the first error of its own.  Without begin() every launch goes to s.
+//
+// Calls on different streams must not wait for one another, so each has a
+// second stream of its own: the one that served the same caller's stream
+// before, or one that is idle, or a new one, or, with all kSideStreams at
+// work, none -- the launches then follow one another on s.  Under capture no
+// second stream is used (it would belong to the capture until that ends, and
+// refuse every other call): the p2z launches become a branch of the graph by
+// setting the capture's dependencies back to those of begin().
 class ModeStreams {
  public:
   ModeStreams(fit_handle* h, cudaStream_t s, const char* who) : h_(h), s_(s), who_(who) {}
+  ~ModeStreams();
+  ModeStreams(const ModeStreams&) = delete;
+  ModeStreams& operator=(const ModeStreams&) = delete;
   int begin(int nevt, const int64_t* ntrk, const int32_t* mode);
+  cudaStream_t of(int m);
   int end(int rc);
-  cudaStream_t of(int m) const { return m == FIT_MODE_Z && forked_ ? h_->side : s_; }
 
  private:
+  // What the next captured operation depends on.
+  struct Frontier {
+    std::vector<cudaGraphNode_t> nodes;
+    std::vector<cudaGraphEdgeData> edges;  // empty, or one per node
+  };
+  cudaError_t frontier(Frontier* f, cudaStreamCaptureStatus* status) const;
+  cudaError_t depend(Frontier& f, unsigned how);
+
   fit_handle* h_;
   cudaStream_t s_;
   const char* who_;
-  bool forked_ = false;
-  std::unique_lock<std::mutex> lock_;
+  SideStream* side_ = nullptr;
+  bool captured_ = false, branched_ = false;
+  Frontier before_, after_r_;
+  cudaError_t err_ = cudaSuccess;
 };
 
-// run_fit with the second stream for p2z where both modes are present.
+// The fused fit of events [0, nevt) (fit.cu): the p2r events in one launch
+// (kMaxRuns runs each), the p2z events in one, on ms's streams; a small call
+// in one launch.
+int run_fit(const fit_handle* h, const FitArgs& a, const RunOptions& o, int nevt,
+            const int64_t* ntrk, const int32_t* mode, const char* who, ModeStreams& ms);
+
+// run_fit with a second stream for p2z where both modes are present.
 int run_fit_streams(fit_handle* h, const FitArgs& a, const RunOptions& o, int nevt,
                     const int64_t* ntrk, const int32_t* mode, const char* who, cudaStream_t s);
 
