@@ -261,10 +261,9 @@ class Geometry:
 def _config(g: Optional[Geometry]):
     if g is None:
         return None, None
-    if isinstance(g.surf, (np.ndarray, list, tuple)):
-        surf = np.asarray(g.surf, dtype=np.float32)
-        arr = (ctypes.c_float * surf.size).from_buffer_copy(surf.tobytes())
-    else:
+    if type(g.surf) is np.ndarray and g.surf.ndim == 1 and g.surf.dtype in (np.float32, np.float64):
+        arr = (ctypes.c_float * g.surf.size).from_buffer_copy(g.surf.astype(np.float32).tobytes())
+    else:  # any sequence of numbers, each by float()
         arr = (ctypes.c_float * len(g.surf))(*[float(s) for s in g.surf])
     return fit_config(float(g.B), len(g.surf), arr, int(g.max_iter), float(g.tol),
                       int(g.start)), arr
