@@ -537,10 +537,10 @@ def _chi2_function():
 
         @staticmethod
         def backward(ctx, grad_chi2, _gpar, _gcov):
-            if grad_chi2 is None:
-                return None, None, None, None, None, None, None, None
             hpos, hcov, tape = ctx.saved_tensors
             ld = hpos.shape[-1]
+            if grad_chi2 is None:  # an undefined gradient is zero
+                grad_chi2 = torch.zeros(ld, dtype=torch.float32, device=hpos.device)
             g_hpos = torch.empty_like(hpos)
             g_par0 = torch.empty((6, ld), dtype=torch.float32, device=hpos.device)
             g_cov0 = torch.empty((21, ld), dtype=torch.float32, device=hpos.device)
