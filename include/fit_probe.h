@@ -45,6 +45,19 @@ extern "C" {
 int fit_probe_fp32(int packed, int blocks, int iters, float* out, void* stream, double* flops);
 
 /*
+ * fit_probe_f64: the FP64 fit's arithmetic, out[i] = op(x[i], y[i]) for i < n
+ * (DEVICE arrays of n doubles), asynchronous on `stream`:
+ *   FIT_PROBE_RCP 1 / x, _DIV x / y, _RSQRT 1 / sqrt(x), _SQRT sqrt(x).
+ * Returns FIT_OK, FIT_ERR_ARG or FIT_ERR_CUDA.
+ */
+#define FIT_PROBE_RCP 0
+#define FIT_PROBE_DIV 1
+#define FIT_PROBE_RSQRT 2
+#define FIT_PROBE_SQRT 3
+#define FIT_PROBE_OPS 4
+int fit_probe_f64(int op, const double* x, const double* y, int64_t n, double* out, void* stream);
+
+/*
  * fit_probe_host_in_place: whether fit_propagate_update_host would take these
  * buffers of n tracks in place (1) or stage them (0) on the current device; a
  * question to the driver, nothing runs.  FIT_ERR_ARG on a bad argument.

@@ -149,9 +149,12 @@ __device__ __forceinline__ F2 sel(M2 m, F2 a, F2 b) {
 // (Householder, "The Numerical Treatment of a Single Nonlinear Equation",
 // 1970): with e = 1 - x y, 1/x = y / (1 - e) = y (1 + e + e^2 + ...), and with
 // e = 1 - x y^2, x^(-1/2) = y (1 - e)^(-1/2) = y (1 + e/2 + 3 e^2/8 + ...).
-// What is dropped is below 2^-55, so the results stay within an ulp of the
-// IEEE functions', in 3 and 5 operations.  A zero, subnormal, huge, negative
-// (rsqrt) or non-finite argument goes to those.
+// What is dropped is below 2^-58, so they are good to 0.51 and 1.0 ulp (1 / x
+// and 1 / sqrt(x) of IEEE operations to 0.5 and 1.5), in 3 and 5 operations.
+// Quotient and square root end with Newton's step from the result's residual,
+// which an fma gives without rounding: 0.5 ulp, as the IEEE operations.
+// A zero, subnormal, huge, negative (roots) or non-finite argument goes to
+// those.
 __device__ __forceinline__ double fma(double a, double b, double c) { return ::fma(a, b, c); }
 // 2^-500 <= |x| < 2^500, on the integer pipe; positive: also x > 0
 __device__ __forceinline__ bool mid_range(double x, bool positive) {
@@ -190,7 +193,11 @@ __device__ __forceinline__ double frsqrt(double x) {
 }
 __device__ __forceinline__ double fsqrt(double x) {  // NaN for x < 0, as in FP32
   if (!mid_range(x, true)) return ieee_sqrt(x);
-  return x * frsqrt(x);
+  double y;
+  asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
+  y = ::fma(::fma(-(x * y), y, 1.0), 0.5 * y, y);  // Newton: 2^-38
+  const double r = x * y;
+  return ::fma(::fma(-r, r, x), 0.5 * y, r);
 }
 // |x| < the double whose upper word is hi (a positive one), on the integer pipe
 __device__ __forceinline__ bool below_hi(double x, int hi) {

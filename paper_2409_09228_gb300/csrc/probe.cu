@@ -1,4 +1,5 @@
-// libfit: the FP32 throughput probe of fit_probe.h.  Each thread runs 16
+// libfit: the probes of fit_probe.h: the FP64 operations on arrays, and the
+// FP32 throughput.  In the latter each thread runs 16
 // independent FMA chains, so that one warp alone has enough independent work
 // to cover the FMA latency and the probe measures the pipe's throughput, not
 // its latency; the multiplier and addend are kernel arguments, so nothing
@@ -9,6 +10,7 @@
 
 #include "fit_probe.h"
 #include "internal.h"
+#include "track_math.cuh"
 
 namespace fitimpl {
 namespace {
@@ -49,6 +51,21 @@ __global__ void __launch_bounds__(FIT_PROBE_THREADS)
   out[(int64_t)blockIdx.x * FIT_PROBE_THREADS + threadIdx.x] = s;
 }
 
+__global__ void __launch_bounds__(FIT_PROBE_THREADS)
+    probe_f64(int op, const double* __restrict__ x, const double* __restrict__ y, int64_t n,
+              double* __restrict__ out) {
+  const int64_t i = (int64_t)blockIdx.x * FIT_PROBE_THREADS + threadIdx.x;
+  if (i >= n) return;
+  double r = 0.0;
+  switch (op) {
+    case FIT_PROBE_RCP: r = fitk::frcp(x[i]); break;
+    case FIT_PROBE_DIV: r = fitk::fdiv(x[i], y[i]); break;
+    case FIT_PROBE_RSQRT: r = fitk::frsqrt(x[i]); break;
+    case FIT_PROBE_SQRT: r = fitk::fsqrt(x[i]); break;
+  }
+  out[i] = r;
+}
+
 }  // namespace
 }  // namespace fitimpl
 
@@ -70,4 +87,16 @@ extern "C" int fit_probe_fp32(int packed, int blocks, int iters, float* out, voi
   if (e != cudaSuccess) return cuda_fail(e, "fit_probe_fp32: launch");
   *flops = (double)blocks * FIT_PROBE_THREADS * (double)iters * kChains * 2.0 * (packed ? 2.0 : 1.0);
   return FIT_OK;
+}
+
+extern "C" int fit_probe_f64(int op, const double* x, const double* y, int64_t n, double* out,
+                             void* stream) {
+  g_last_error.clear();
+  const int64_t blocks = (n + FIT_PROBE_THREADS - 1) / FIT_PROBE_THREADS;
+  if (op < 0 || op >= FIT_PROBE_OPS || !x || !y || !out || n < 1 || blocks > 0x7fffffff)
+    return fail(FIT_ERR_ARG, "fit_probe_f64: bad argument");
+  probe_f64<<<(unsigned)blocks, FIT_PROBE_THREADS, 0, static_cast<cudaStream_t>(stream)>>>(
+      op, x, y, n, out);
+  const cudaError_t e = cudaGetLastError();
+  return e == cudaSuccess ? FIT_OK : cuda_fail(e, "fit_probe_f64: launch");
 }

@@ -103,7 +103,8 @@ EXPORTS = ("fit_init", "fit_propagate_update", "fit_sync", "fit_destroy", "fit_l
            "fit_mlp_adam_step", "fit_mlp_train", "fit_mlp_attach", "fit_path_lengths",
            "fit_propagate_update_host", "fit_propagate_update_mapped", "fit_propagate_update_f64",
            "fit_propagate_update_layout", "fit_find_tracks", "fit_find_tracks_f64",
-           "fit_relayout", "fit_probe_fp32", "fit_probe_host_in_place")
+           "fit_relayout", "fit_probe_fp32", "fit_probe_host_in_place",
+           "fit_probe_f64")
 FIT_LAYOUT_SOA = 0
 FIT_LAYOUT_AOSOA32 = 1
 FIT_LAYOUT_TUNE = 2
@@ -202,6 +203,8 @@ def load(build_if_missing: bool = True):
     L.fit_probe_fp32.argtypes = [ctypes.c_int, ctypes.c_int, ctypes.c_int, vp, vp,
                                  ctypes.POINTER(ctypes.c_double)]
     L.fit_probe_fp32.restype = ctypes.c_int
+    L.fit_probe_f64.argtypes = [ci, vp, vp, i64, vp, vp]
+    L.fit_probe_f64.restype = ci
     L.fit_probe_host_in_place.argtypes = [vp, vp, vp, i64, ci]
     L.fit_probe_host_in_place.restype = ci
     L.fit_relayout.argtypes = [vp, i64, ctypes.c_int, vp, i64, ctypes.c_int, ctypes.c_int, i64, vp]
@@ -656,6 +659,13 @@ def fit_last_error() -> str:
 
 
 FIT_PROBE_THREADS = 256
+
+
+def fit_probe_f64(op: int, x, y, out, stream=None) -> None:
+    """out = op(x, y) by the FP64 fit's arithmetic, element by element
+    (include/fit_probe.h): float64 device tensors."""
+    _check(load().fit_probe_f64(int(op), _ptr(x), _ptr(y), out.numel(), _ptr(out),
+                                _stream_handle(stream)))
 
 
 def fit_probe_host_in_place(par_in, cov_in, q_in, hpos, hcov, n: int, par_out, cov_out, q_out,
