@@ -613,6 +613,20 @@ __device__ __forceinline__ void similarity_local_r(T (&c)[15], T ctt, T a02, T a
     }
 }
 
+// s / c and dz / (c c), each rounded as by a division, from one reciprocal:
+// quotients with their remainders folded back.
+__device__ __forceinline__ void tan_slope(double s, double c, double dz, double& tan, double& slope) {
+  const double c2 = c * c;
+  if (!mid_range(c, false)) {
+    tan = ieee_div(s, c);
+    slope = ieee_div(dz, c2);
+    return;
+  }
+  const double i = frcp(c), i2 = i * i, q = s * i, q2 = dz * i2;
+  tan = fma(fma(-c, q, s), i, q);
+  slope = fma(fma(-c2, q2, dz), i2, q2);
+}
+
 // Propagation to the plane z = Z.  Returns the mask of lanes whose plane is
 // behind them; if any lane fails nothing is modified.  ZFREE: the caller
 // guarantees that row and column z of c are zero (true from the first plane
@@ -623,14 +637,11 @@ __device__ __forceinline__ typename Lanes<T>::M prop_z(T (&p)[6], T (&c)[21], Tr
                                                        float Z, const Overlap& ov = Overlap()) {
   ov();  // the caller's independent work, beside the path length's reciprocal
   const T dz = T(Z) - p[2];
-  // double: one reciprocal for tan(theta) and dh/dtheta
-  T icth, tanth;
-  if constexpr (std::is_same_v<T, double>) {
-    icth = frcp(g.cth);
-    tanth = g.sth * icth;
-  } else {
+  T tanth, hth;  // tan(theta) and, in double already, dh/dtheta
+  if constexpr (std::is_same_v<T, double>)
+    tan_slope(g.sth, g.cth, dz, tanth, hth);
+  else
     tanth = fdiv(g.sth, g.cth);
-  }
   const T h = dz * tanth;
   const auto fail = not_(pos(h));
   if (any(fail)) return fail;
@@ -646,11 +657,7 @@ __device__ __forceinline__ typename Lanes<T>::M prop_z(T (&p)[6], T (&c)[21], Tr
   T c1 = cm, s1 = sm;
   turn(c1, s1, cu, su);  // phi + 2u = phi'
   const T hh = T(0.5f) * h * h * dkdw;
-  T hth;  // dh/dtheta
-  if constexpr (std::is_same_v<T, double>)
-    hth = dz * icth * icth;
-  else
-    hth = fdiv(dz, g.cth * g.cth);
+  if constexpr (!std::is_same_v<T, double>) hth = fdiv(dz, g.cth * g.cth);  // dh/dtheta
   // grad h = (0, 0, -tan(theta), 0, 0, dh/dtheta); d p'/d h = (cos phi',
   // sin phi', 0 on the plane, 0, kappa, 0)
   const T gr[6] = {T(0.f), T(0.f), -tanth, T(0.f), T(0.f), hth};

@@ -14,7 +14,7 @@ pytestmark = pytest.mark.gpu
 if not torch.cuda.is_available():  # pragma: no cover - collected on CPU hosts too
     pytest.skip("needs a CUDA device", allow_module_level=True)
 
-RCP, DIV, RSQRT, SQRT = range(4)
+RCP, DIV, RSQRT, SQRT, TAN, SLOPE = range(6)
 getcontext().prec = 60
 N = 20000
 
@@ -66,3 +66,25 @@ def test_special_arguments_are_those_of_ieee(op):
     np.testing.assert_array_equal(np.isnan(got), np.isnan(ref))
     ok = ~np.isnan(ref)
     np.testing.assert_allclose(got[ok], ref[ok], rtol=2.0 ** -52, atol=0.0)
+
+
+# tan(theta) is one IEEE division's (half a unit); dh/dtheta = dz / cos^2 that
+# of a product and a division (2^-53 of the value, one unit at most, and half).
+@pytest.mark.parametrize("op,bound", [(TAN, 0.5001), (SLOPE, 1.5001)], ids=["tan", "slope"])
+def test_plane_propagation_quotients(op, bound):
+    g = np.random.default_rng(151)
+    th = np.concatenate([g.uniform(0.01, np.pi - 0.01, N), np.pi / 2 + 10.0 ** g.uniform(-12, -1, 2000)])
+    c = np.cos(th)
+    x = np.sin(th) if op == TAN else g.uniform(-30.0, 30.0, c.size)
+    exact = [Decimal(float(a)) / (Decimal(float(b)) if op == TAN else Decimal(float(b)) ** 2)
+             for a, b in zip(x, c)]
+    assert _worst(_probe(op, x, c), exact) <= bound
+
+
+@pytest.mark.parametrize("op", [TAN, SLOPE], ids=["tan", "slope"])
+def test_plane_propagation_at_the_ends_of_the_range(op):
+    c = np.array([0.0, -0.0, 5e-324, 1e-200, 1e-160, 1.0, np.inf, np.nan])
+    x = np.full_like(c, 1.5)
+    with np.errstate(all="ignore"):
+        ref = x / c if op == TAN else x / (c * c)
+    np.testing.assert_allclose(_probe(op, x, c), ref, rtol=2.0 ** -50, atol=0.0)
