@@ -48,7 +48,8 @@ int fit_probe_fp32(int packed, int blocks, int iters, float* out, void* stream, 
  * fit_probe_f64: the FP64 fit's arithmetic, out[i] = op(x[i], y[i]) for i < n
  * (DEVICE arrays of n doubles), asynchronous on `stream`:
  *   FIT_PROBE_RCP 1 / x, _DIV x / y, _RSQRT 1 / sqrt(x), _SQRT sqrt(x), _TAN
- *   x / y and _SLOPE x / (y y) as the plane propagation forms them.
+ *   x / y and _SLOPE x / (y y) as the plane propagation forms them, _ATAN
+ *   atan(x) / x for |x| < 1/4.
  * Returns FIT_OK, FIT_ERR_ARG or FIT_ERR_CUDA.
  */
 #define FIT_PROBE_RCP 0
@@ -57,7 +58,8 @@ int fit_probe_fp32(int packed, int blocks, int iters, float* out, void* stream, 
 #define FIT_PROBE_SQRT 3
 #define FIT_PROBE_TAN 4
 #define FIT_PROBE_SLOPE 5
-#define FIT_PROBE_OPS 6
+#define FIT_PROBE_ATAN 6
+#define FIT_PROBE_OPS 7
 int fit_probe_f64(int op, const double* x, const double* y, int64_t n, double* out, void* stream);
 
 /*

@@ -62,6 +62,7 @@ __global__ void __launch_bounds__(FIT_PROBE_THREADS)
     case FIT_PROBE_DIV: r = fitk::fdiv(x[i], y[i]); break;
     case FIT_PROBE_RSQRT: r = fitk::frsqrt(x[i]); break;
     case FIT_PROBE_SQRT: r = fitk::fsqrt(x[i]); break;
+    case FIT_PROBE_ATAN: r = fitk::atan_ratio(x[i]); break;
     case FIT_PROBE_TAN:
     case FIT_PROBE_SLOPE: {
       double tan, slope;

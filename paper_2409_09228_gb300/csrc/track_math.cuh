@@ -682,16 +682,15 @@ __device__ __forceinline__ T atan_ratio(T t) {
                                              T(1.f / 9.f)), T(-1.f / 7.f)), T(1.f / 5.f)),
                       T(-1.f / 3.f)), T(1.f));
 }
-// In double to t^20, or to t^10 for |t| < 1/16 (remainders below 3e-15): where
-// the iteration starts, not what it converges to.
+// In double to t^24, or to t^12 for |t| < 1/16 (the next terms are below 2^-56).
 __device__ __forceinline__ double atan_ratio(double t) {
   const double v = -(t * t);
   if (below_hi(t, 0x3fb00000))
-    return fma(v, fma(v, fma(v, fma(v, fma(v, 1.0 / 11.0, 1.0 / 9.0), 1.0 / 7.0), 1.0 / 5.0),
-                      1.0 / 3.0), 1.0);
-  return fma(v, fma(v, fma(v, fma(v, fma(v, fma(v, fma(v, fma(v, fma(v, fma(v, 1.0 / 21.0, 1.0 / 19.0),
-             1.0 / 17.0), 1.0 / 15.0), 1.0 / 13.0), 1.0 / 11.0), 1.0 / 9.0), 1.0 / 7.0), 1.0 / 5.0),
-             1.0 / 3.0), 1.0);
+    return fma(v, fma(v, fma(v, fma(v, fma(v, fma(v, 1.0 / 13.0, 1.0 / 11.0), 1.0 / 9.0), 1.0 / 7.0),
+                             1.0 / 5.0), 1.0 / 3.0), 1.0);
+  return fma(v, fma(v, fma(v, fma(v, fma(v, fma(v, fma(v, fma(v, fma(v, fma(v, fma(v, fma(v,
+             1.0 / 25.0, 1.0 / 23.0), 1.0 / 21.0), 1.0 / 19.0), 1.0 / 17.0), 1.0 / 15.0), 1.0 / 13.0),
+             1.0 / 11.0), 1.0 / 9.0), 1.0 / 7.0), 1.0 / 5.0), 1.0 / 3.0), 1.0);
 }
 
 // Where the helix of the propagation crosses the cylinder r = R, in closed

@@ -14,7 +14,7 @@ pytestmark = pytest.mark.gpu
 if not torch.cuda.is_available():  # pragma: no cover - collected on CPU hosts too
     pytest.skip("needs a CUDA device", allow_module_level=True)
 
-RCP, DIV, RSQRT, SQRT, TAN, SLOPE = range(6)
+RCP, DIV, RSQRT, SQRT, TAN, SLOPE, ATAN = range(7)
 getcontext().prec = 60
 N = 20000
 
@@ -88,3 +88,23 @@ def test_plane_propagation_at_the_ends_of_the_range(op):
     with np.errstate(all="ignore"):
         ref = x / c if op == TAN else x / (c * c)
     np.testing.assert_allclose(_probe(op, x, c), ref, rtol=2.0 ** -50, atol=0.0)
+
+
+def test_start_of_the_crossing():
+    """atan(t) / t, both ranges of the series and their seam: half a unit for
+    the last sum, an eighth for the terms left out (2^-56 below one), and the
+    inner sums' roundings, at most 1/16 of a unit each way."""
+    g = np.random.default_rng(157)
+    t = np.concatenate([g.uniform(-0.25, 0.25, 4000), g.uniform(-0.0626, 0.0626, 4000),
+                        10.0 ** g.uniform(-300, -2, 200),
+                        [np.nextafter(0.25, 0), 0.0625, np.nextafter(0.0625, 0)]])
+    t = t[np.abs(t) < 0.25]
+
+    def ratio(a):
+        v, term, total, k = -a * a, Decimal(1), Decimal(1), 1
+        while abs(term) > Decimal(10) ** -40:
+            term, k = term * v, k + 2
+            total += term / k
+        return total
+
+    assert _worst(_probe(ATAN, t), [ratio(Decimal(float(a))) for a in t]) <= 0.75
