@@ -47,7 +47,8 @@ extern "C" {
 #define FIT_OK 0
 #define FIT_ERR_ARG (-1)     /* invalid argument (pointer, size, alignment) */
 #define FIT_ERR_CUDA (-2)    /* a CUDA runtime call failed */
-#define FIT_ERR_TIMEOUT (-3) /* fit_sync gave up waiting */
+#define FIT_ERR_TIMEOUT (-3) /* a wait gave up: fit_sync's for its stream, or
+                                fit_mlp_train's for the blocks of its kernel */
 #define FIT_ERR_NOMEM (-4)   /* the library could not allocate its scratch */
 
 /* Per-track status bits. */
@@ -583,9 +584,13 @@ int fit_mlp_adam_step(fit_mlp* m, const float* grad, float lr, void* stream);
  * fit_mlp_train: minimises the mean squared error of the network's output
  * against the targets by Adam over `epochs` passes of batches of cfg->batch
  * consecutive samples (from a per-epoch offset drawn from cfg->seed; n must
- * be >= cfg->batch).  Each step is one forward+backward kernel, one Adam
- * kernel and one kernel that rebuilds the BF16 weights, on `stream`.  loss_per_epoch (HOST [epochs], may be NULL) receives the
- * mean training loss of each epoch; the call then waits for the stream.
+ * be >= cfg->batch).  Up to 512 steps are one cooperative launch on `stream`
+ * (on a device partition too small for its blocks to run together, each step
+ * is two launches).  loss_per_epoch (HOST [epochs], may be NULL) receives the
+ * mean training loss of each epoch; the call waits for the stream.  Errors:
+ * FIT_ERR_ARG, FIT_ERR_NOMEM, FIT_ERR_CUDA, and FIT_ERR_TIMEOUT if a block
+ * of the launch waited seconds for the others; the network (parameters, Adam
+ * state, BF16 weights) is then as before the call.
  */
 int fit_mlp_train(fit_mlp* m, const float* x, const float* target, int64_t n,
                   const fit_mlp_train_config* cfg, float* loss_per_epoch, void* stream);

@@ -70,6 +70,14 @@ int fit_probe_f64(int op, const double* x, const double* y, int64_t n, double* o
 int fit_probe_host_in_place(const fit_tracks_in* in, const fit_tracks_out* out,
                             const fit_hits* hits, int64_t n, int nlayer);
 
+/*
+ * fit_probe_train_limits: for the tests of fit_mlp_train, how often a block of
+ * its kernel looks at the barrier before it gives up (as created: 2^22), and
+ * the most blocks it may count on to run together (0: as many as the device
+ * holds).  FIT_ERR_ARG if m is NULL or blocks < 0.
+ */
+int fit_probe_train_limits(fit_mlp* m, uint32_t looks, int blocks);
+
 #ifdef __cplusplus
 }
 #endif

@@ -8,9 +8,11 @@
 #include <cmath>
 #include <cstdint>
 #include <string>
+#include <utility>
 #include <vector>
 
 #include "fit.h"
+#include "fit_probe.h"
 #include "fused.cuh"
 #include "internal.h"
 #include "mlp.cuh"
@@ -29,7 +31,15 @@ struct fit_mlp {
   int64_t partial_blocks = 0;
   float* d_curve = nullptr;  // loss per epoch
   int curve_cap = 0;
+  // Where a training writes: the parameters and moments above stay as they are
+  // until all of its steps are done, and the two sets then change places.
+  float *d_params_out = nullptr, *d_m_out = nullptr, *d_v_out = nullptr;
   unsigned* d_sync = nullptr;  // the training kernel's grid barrier and error flag
+  // Limits that only the tests change (fit_probe_train_limits): how often a
+  // block looks at the barrier before it gives up (a step takes microseconds,
+  // as many looks seconds), and how many blocks a training takes.
+  unsigned barrier_looks = 1u << 22;
+  int max_blocks = 0;  // 0: as many as fit on the device together
   int64_t step = 0;  // Adam steps taken
   float beta1 = 0.9f, beta2 = 0.999f, eps = 1e-8f;
 };
@@ -494,7 +504,8 @@ __global__ void __launch_bounds__(kAdamThreads)
   if (curve && u == 0) *curve += sum_partials(partials, nblk, kSse) * curve_scale;
 }
 
-// New parameters (already in P): the moments cleared, the image written.
+// New parameters (already in P): the image written, the moments cleared (kept
+// if M is NULL).
 __global__ void __launch_bounds__(kAdamThreads)
     mlp_load_kernel(const float* __restrict__ P, float* __restrict__ M, float* __restrict__ V,
                     TrainImage* img) {
@@ -503,7 +514,7 @@ __global__ void __launch_bounds__(kAdamThreads)
   if (u < mlpk::kParams) {
     const int i = owned_param(u);
     p = P[i];
-    M[i] = V[i] = 0.f;
+    if (M) M[i] = V[i] = 0.f;
   }
   write_image(img, u, p);
 }
@@ -519,24 +530,25 @@ struct TrainSteps {
   int64_t off[kTrainSteps];  // first sample of the step's batch
 };
 
-// How often a block looks at the grid barrier before it gives up (seconds;
-// a step takes microseconds).
-constexpr unsigned kBarrierLooks = 1u << 22;
-
-// Barrier over the grid (cooperative launch): sync[0] counts arrivals, round
-// is the barrier's number from 1.  Returns true if a block gave up waiting,
-// which sync[1] then tells the others and the host.
-__device__ __forceinline__ bool grid_barrier(unsigned* sync, unsigned round) {
+// Barrier over the grid (cooperative launch): sync[0] counts arrivals (modulo
+// 2^32), round is the barrier's number from 1, counted on over a training's
+// launches.  Returns true if a block gave up waiting, after `looks` looks:
+// sync[1] then tells the host, and the others, which read it every 1024 looks.
+// The arrival that is missing keeps every later barrier shut as well, so that
+// launches queued behind leave at their first.
+__device__ __forceinline__ bool grid_barrier(unsigned* sync, unsigned round, unsigned looks) {
   bool gave_up = false;
   __syncthreads();
   if (threadIdx.x == 0) {
+    auto load = [](const unsigned* p) {
+      unsigned v;
+      asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
+      return v;
+    };
     asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(sync) : "memory");
     const unsigned target = round * gridDim.x;
-    for (unsigned looks = 0;; ++looks) {
-      unsigned seen;
-      asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(seen) : "l"(sync) : "memory");
-      if (seen >= target) break;
-      if (looks >= kBarrierLooks) {
+    for (unsigned k = 0; (int)(load(sync) - target) < 0; ++k) {
+      if (k >= looks || ((k & 1023) == 1023 && load(sync + 1))) {
         atomicExch(sync + 1, 1u);
         gave_up = true;
         break;
@@ -559,8 +571,10 @@ __device__ __forceinline__ bool grid_barrier(unsigned* sync, unsigned round) {
 __global__ void __launch_bounds__(kBlock)
     mlp_train_kernel(const __grid_constant__ TrainSteps steps, TrainImage* img,
                      const float* __restrict__ X, const float* __restrict__ T, int64_t n,
-                     int batch, float inv_cnt, float* partials, float* P, float* M, float* V,
-                     AdamBetas betas, float* curve, float curve_scale, unsigned* sync) {
+                     int batch, float inv_cnt, float* partials, const float* P, const float* M,
+                     const float* V, float* P_out, float* M_out, float* V_out, AdamBetas betas,
+                     float* curve, float curve_scale, unsigned* sync, unsigned round,
+                     unsigned looks) {
   __shared__ GradSmem S;
   const int nblk = (batch + kRows - 1) / kRows;
   const int u = blockIdx.x * kBlock + threadIdx.x;
@@ -571,7 +585,6 @@ __global__ void __launch_bounds__(kBlock)
   float loss = u == mlpk::kParams ? curve[epoch] : 0.f;
   Sample smp;
   if ((int)blockIdx.x < nblk) smp = load_sample(X, T, n, steps.off[0], batch, blockIdx.x);
-  unsigned round = 0;
   for (int k = 0; k < steps.count; ++k) {
     if ((int)blockIdx.x < nblk) {
       const uint4* src = reinterpret_cast<const uint4*>(img);
@@ -593,7 +606,7 @@ __global__ void __launch_bounds__(kBlock)
       }
       if (k + 1 < steps.count) smp = load_sample(X, T, n, steps.off[k + 1], batch, blockIdx.x);
     }
-    if (grid_barrier(sync, ++round)) return;
+    if (grid_barrier(sync, ++round, looks)) return;
     if (own >= 0) {
       const float gi = sum_partials(partials, nblk, own);
       if (own != kSse) {
@@ -605,9 +618,9 @@ __global__ void __launch_bounds__(kBlock)
       }
     }
     write_image(img, u, p);
-    if (grid_barrier(sync, ++round)) return;
+    if (grid_barrier(sync, ++round, looks)) return;
   }
-  if (u < mlpk::kParams) P[own] = p, M[own] = m, V[own] = v;
+  if (u < mlpk::kParams) P_out[own] = p, M_out[own] = m, V_out[own] = v;
 }
 
 // ---- the p2r path-length iteration alone ---------------------------------------
@@ -834,7 +847,8 @@ int fit_mlp_create(fit_mlp** out, int device, uint64_t seed) {
   m->device = device;
   const size_t pb = mlpk::kParams * sizeof(float);
   if (cudaMalloc(&m->d_params, pb) != cudaSuccess || cudaMalloc(&m->d_m, pb) != cudaSuccess ||
-      cudaMalloc(&m->d_v, pb) != cudaSuccess ||
+      cudaMalloc(&m->d_v, pb) != cudaSuccess || cudaMalloc(&m->d_params_out, pb) != cudaSuccess ||
+      cudaMalloc(&m->d_m_out, pb) != cudaSuccess || cudaMalloc(&m->d_v_out, pb) != cudaSuccess ||
       cudaMalloc(&m->d_img, sizeof(TrainImage)) != cudaSuccess ||
       cudaMemset(m->d_img, 0, sizeof(TrainImage)) != cudaSuccess ||
       cudaMalloc(&m->d_sync, 2 * sizeof(unsigned)) != cudaSuccess) {
@@ -868,6 +882,9 @@ void fit_mlp_destroy(fit_mlp* m) {
     cudaFree(m->d_params);
     cudaFree(m->d_m);
     cudaFree(m->d_v);
+    cudaFree(m->d_params_out);
+    cudaFree(m->d_m_out);
+    cudaFree(m->d_v_out);
     cudaFree(m->d_img);
     cudaFree(m->d_partials);
     cudaFree(m->d_curve);
@@ -984,6 +1001,8 @@ int fit_mlp_train(fit_mlp* m, const float* x, const float* target, int64_t n,
   cudaError_t e = cudaMemsetAsync(m->d_curve, 0, cfg->epochs * sizeof(float), s);
   if (e == cudaSuccess) e = cudaMemsetAsync(m->d_sync, 0, 2 * sizeof(unsigned), s);
   if (e != cudaSuccess) return cuda_fail(e, "fit_mlp_train: memset");
+  const AdamBetas betas0{m->beta1, m->beta2, m->eps};
+  const int64_t step0 = m->step;
   m->beta1 = cfg->beta1;
   m->beta2 = cfg->beta2;
   m->eps = cfg->eps;
@@ -994,11 +1013,22 @@ int fit_mlp_train(fit_mlp* m, const float* x, const float* target, int64_t n,
   // One cooperative launch for every kTrainSteps steps.  Its blocks must hold
   // a parameter per thread and run together; a device partition too small
   // for that takes the steps as two launches each.
-  const int together = train_blocks(m->device);
+  const int fitting = train_blocks(m->device);
+  const int together = m->max_blocks ? std::min(m->max_blocks, fitting) : fitting;
   const bool one_launch = together > kAdamBlocks;
   const unsigned grid = (unsigned)std::min(std::max(nblk, kAdamBlocks), std::max(together, 1));
   TrainSteps ts;
   ts.count = 0;
+  unsigned round = 0;
+  const float *P = m->d_params, *M = m->d_m, *V = m->d_v;
+  // The network as it was before the call, after a training that did not end.
+  auto undo = [&](int code) {
+    mlp_load_kernel<<<kAdamBlocks, kAdamThreads, 0, s>>>(m->d_params, nullptr, nullptr, m->d_img);
+    cudaStreamSynchronize(s);
+    m->step = step0;
+    m->beta1 = betas0.beta1, m->beta2 = betas0.beta2, m->eps = betas0.eps;
+    return code;
+  };
   int64_t t = 0;
   for (int ep = 0; ep < cfg->epochs; ++ep) {
     const int64_t start = (int64_t)(splitmix64(rs) % (uint64_t)n);
@@ -1023,33 +1053,47 @@ int fit_mlp_train(fit_mlp* m, const float* x, const float* target, int64_t n,
       ts.rate[ts.count] = next_rate(m, lr);
       ts.off[ts.count++] = off;
       if (ts.count < kTrainSteps && t + 1 < total) continue;
-      if (t >= kTrainSteps) e = cudaMemsetAsync(m->d_sync, 0, sizeof(unsigned), s);
       AdamBetas betas{m->beta1, m->beta2, m->eps};
       int batch = cfg->batch;
       int64_t nsamp = n;
       float cnt_inv = inv, cscale = scale;
-      void* args[] = {&ts,      &m->d_img, &x,     &target,     &nsamp,  &batch,    &cnt_inv,
-                      &m->d_partials, &m->d_params, &m->d_m, &m->d_v, &betas, &m->d_curve,
-                      &cscale,  &m->d_sync};
-      if (e == cudaSuccess)
-        e = cudaLaunchCooperativeKernel((const void*)mlp_train_kernel, dim3(grid), dim3(kBlock),
-                                        args, 0, s);
-      if (e != cudaSuccess) return cuda_fail(e, "fit_mlp_train: launch");
+      void* args[] = {&ts, &m->d_img, &x, &target, &nsamp, &batch, &cnt_inv, &m->d_partials,
+                      &P, &M, &V, &m->d_params_out, &m->d_m_out, &m->d_v_out, &betas, &m->d_curve,
+                      &cscale, &m->d_sync, &round, &m->barrier_looks};
+      e = cudaLaunchCooperativeKernel((const void*)mlp_train_kernel, dim3(grid), dim3(kBlock), args,
+                                      0, s);
+      if (e != cudaSuccess) return undo(cuda_fail(e, "fit_mlp_train: launch"));
+      round += 2u * (unsigned)ts.count;
+      P = m->d_params_out, M = m->d_m_out, V = m->d_v_out;
       ts.count = 0;
     }
   }
   unsigned gave_up = 0;
   if (one_launch) {
     e = cudaMemcpyAsync(&gave_up, m->d_sync + 1, sizeof(unsigned), cudaMemcpyDeviceToHost, s);
-    if (e != cudaSuccess) return cuda_fail(e, "fit_mlp_train: barrier status");
+    if (e != cudaSuccess) return undo(cuda_fail(e, "fit_mlp_train: barrier status"));
   }
   e = cudaStreamSynchronize(s);
-  if (e != cudaSuccess) return cuda_fail(e, "fit_mlp_train: synchronize");
-  if (gave_up) return fail(FIT_ERR_TIMEOUT, "fit_mlp_train: the training kernel's barrier timed out");
+  if (e != cudaSuccess) return undo(cuda_fail(e, "fit_mlp_train: synchronize"));
+  if (gave_up)
+    return undo(fail(FIT_ERR_TIMEOUT, "fit_mlp_train: the training kernel's barrier timed out"));
+  if (one_launch) {
+    std::swap(m->d_params, m->d_params_out);
+    std::swap(m->d_m, m->d_m_out);
+    std::swap(m->d_v, m->d_v_out);
+  }
   if (loss_per_epoch) {
     e = cudaMemcpy(loss_per_epoch, m->d_curve, cfg->epochs * sizeof(float), cudaMemcpyDeviceToHost);
     if (e != cudaSuccess) return cuda_fail(e, "fit_mlp_train: copy losses");
   }
+  return FIT_OK;
+}
+
+int fit_probe_train_limits(fit_mlp* m, uint32_t looks, int blocks) {
+  g_last_error.clear();
+  if (!m || blocks < 0) return fail(FIT_ERR_ARG, "fit_probe_train_limits: bad argument");
+  m->barrier_looks = looks;
+  m->max_blocks = blocks;
   return FIT_OK;
 }
 

@@ -104,7 +104,7 @@ EXPORTS = ("fit_init", "fit_propagate_update", "fit_sync", "fit_destroy", "fit_l
            "fit_propagate_update_host", "fit_propagate_update_mapped", "fit_propagate_update_f64",
            "fit_propagate_update_layout", "fit_find_tracks", "fit_find_tracks_f64",
            "fit_relayout", "fit_probe_fp32", "fit_probe_host_in_place",
-           "fit_probe_f64")
+           "fit_probe_f64", "fit_probe_train_limits")
 FIT_LAYOUT_SOA = 0
 FIT_LAYOUT_AOSOA32 = 1
 FIT_LAYOUT_TUNE = 2
@@ -203,6 +203,8 @@ def load(build_if_missing: bool = True):
     L.fit_probe_fp32.argtypes = [ctypes.c_int, ctypes.c_int, ctypes.c_int, vp, vp,
                                  ctypes.POINTER(ctypes.c_double)]
     L.fit_probe_fp32.restype = ctypes.c_int
+    L.fit_probe_train_limits.argtypes = [vp, ctypes.c_uint32, ci]
+    L.fit_probe_train_limits.restype = ci
     L.fit_probe_f64.argtypes = [ci, vp, vp, i64, vp, vp]
     L.fit_probe_f64.restype = ci
     L.fit_probe_host_in_place.argtypes = [vp, vp, vp, i64, ci]
@@ -659,6 +661,11 @@ def fit_last_error() -> str:
 
 
 FIT_PROBE_THREADS = 256
+
+
+def fit_probe_train_limits(m: int, looks: int = 1 << 22, blocks: int = 0) -> None:
+    """Limits of fit_mlp_train's barrier and blocks, for its tests (include/fit_probe.h)."""
+    _check(load().fit_probe_train_limits(m, looks, blocks))
 
 
 def fit_probe_f64(op: int, x, y, out, stream=None) -> None:
