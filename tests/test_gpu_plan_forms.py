@@ -5,6 +5,8 @@ import ctypes
 import numpy as np
 import pytest
 
+import oracle
+import parity
 from paper_2409_09228_gb300 import fit, inputs
 
 torch = pytest.importorskip("torch")
@@ -16,6 +18,7 @@ if not torch.cuda.is_available():  # pragma: no cover - collected on CPU hosts t
 import gpu_util  # noqa: E402
 
 NLAYER = 20
+TABLE = 1024  # pair runs of a launch's table (lone tracks: twice as many)
 SMALL_RUNS = 256  # pair runs of a mode that a small call's one launch holds (lone tracks: twice)
 
 
@@ -155,3 +158,51 @@ def test_info_tells_the_default_form_from_a_persistent_shape():
         fit.fit_plan_destroy(plan)
     f.close()
     assert blocks["default"] == 0 and blocks["given"] == 2 and blocks["most"] > 2
+
+
+# Sizes that fill a launch's tables: three tracks an event give each run a pair
+# and a lone track; events of two from an odd start give two lone tracks each.
+FULL = {"pairs": np.full(2300, 3), "lone": np.concatenate([[1], np.full(2299, 2)])}
+
+
+@pytest.mark.parametrize("fills", FULL)
+@pytest.mark.parametrize("entry", ["fit", "noalloc", "plan", "per_mode"])
+def test_a_full_run_table_takes_another_launch(entry, fills):
+    nt, md = FULL[fills], (np.arange(len(FULL[fills])) % 2).astype(np.int32)
+    for m in (0, 1):
+        pairs, lone = runs(nt, md, m)
+        assert pairs > TABLE if fills == "pairs" else lone > 2 * TABLE
+    ev = inputs.generate_events(nt, md, seed=173, nlayer=NLAYER)
+    ld = gpu_util.pad_ld(ev.n)
+    f = _fitter(ev)
+    d = _device(ev, ld)
+    out = f.outputs(ev.n, ld=ld)
+    for v in out.values():
+        if v is not None:
+            v.fill_(float("nan") if v.is_floating_point() else 77)
+    bufs = dict(par_out=out["par"], cov_out=out["cov"], q_out=out["q"], chi2=out["chi2"],
+                status=out["status"])
+    if entry == "fit":
+        f.run(*d, nt, md, out=out)
+    elif entry == "noalloc":
+        geo = [fit.Geometry(ev.B, s) for s in ev.surf]
+        counts = fit.fit_propagate_update_noalloc(*geo, *d, nt, md, **bufs)
+        for c, n, m in zip(counts, nt, md):
+            assert c["tracks"] == n and n * NLAYER * (m == 0) <= c["iterations"] <= 2 * n * NLAYER * (m == 0)
+    else:
+        plan = fit.fit_plan_create(f.h, nt, md, NLAYER, persistent=entry == "plan")
+        fit.fit_plan_run(plan, *d, **bufs)
+        torch.cuda.synchronize()
+        fit.fit_plan_destroy(plan)
+    if entry != "noalloc":
+        counts = f.sync()
+        assert counts["tracks"] == ev.n
+        assert nt[md == 0].sum() * NLAYER <= counts["iterations"] <= 2 * nt[md == 0].sum() * NLAYER
+    got = {k: out[k][..., :ev.n].cpu().numpy() for k in ("par", "cov", "chi2", "q", "status")}
+    f.close()
+    mode = np.repeat(md, nt)
+    for m in (0, 1):
+        idx = np.nonzero(mode == m)[0]
+        ts = inputs.TrackSet(m, ev.B, ev.surf[m], *(np.ascontiguousarray(a[..., idx]) for a in
+                                                    (ev.par0, ev.cov0, ev.q, ev.hpos, ev.hcov)))
+        parity.check({k: v[..., idx] for k, v in got.items()}, oracle.fit_set(ts), f"{entry} {fills} {m}")
