@@ -54,10 +54,16 @@ struct FindArgs {
 // update takes its candidate from registers.  Loaded one at a time and the
 // chosen one again, the p2r kernel waited on loads 8.2 cycles an instruction
 // (now 0.9): 240k tracks, 4 candidates, 20 layers 217 -> 175 us, and both
-// modes of that size 383 -> 246 us with p2z on the second stream.  Four slots
-// and five blocks of 128 an SM (with addresses formed anew: 4 and 5 blocks
-// 260 us, 4 and 4 271, 5 and 6 268; two slots with 6 and 7 265, three with 5
+// modes of that size 383 -> 246 us with p2z on the second stream.  Four
+// slots (two with 6 and 7 blocks an SM for p2r and p2z 265 us, three with 5
 // and 6 288).  In double, bound by the FP64 pipe, one slot is enough.
+//
+// Five blocks of 128 an SM in float (96 registers; p2r spills 72 bytes in
+// order and 56 with addresses formed anew, p2z none).  Four (no spills) are
+// 3 to 9 % faster up to 200000 tracks of p2r -- 48000 with 4 candidates 47.5
+// us against 50.7, with 9 89.8 against 94.5 -- and up to 10 % slower beyond:
+// 480000 with 4 candidates 311 against 297, with 9 636 against 579, both modes
+// with 4 256 against 250.  The long calls decide.
 template <class T>
 constexpr int kSlots = sizeof(T) == 4 ? 4 : 1;
 // In order: the slots are refilled in the order the candidates lie in memory,

@@ -193,9 +193,12 @@ extern "C" int fit_propagate_update_f64(fit_handle* h, const fit_tracks_in_f64* 
   a.ld_hit = hits->ld;
   a.nlayer = nlayer;
   a.counters = h->d_counters;
-  // Side by side the two modes' blocks spread unevenly over the FP64 pipes
-  // (1354 against 1212 us for 96000 tracks), so only a call that leaves SMs
-  // without a block takes the second stream.
+  // Side by side the two modes' blocks spread unevenly over the FP64 pipes, and
+  // a call of many waves is slower for it (96000 tracks 1354 against 1212 us);
+  // one of a single wave takes the longer mode's time instead of the sum (608
+  // to 9728 tracks 243 us against 411 to 426).  Taken where every block has an
+  // SM to itself; up to twice as many tracks still gain (19456 260 against
+  // 427, with a tenth of them p2r 344 against 444).
   ModeStreams ms(h, static_cast<cudaStream_t>(stream), w.c_str());
   int rc = total <= (int64_t)kBlock64 * h->sms ? ms.begin(nevt, ntrk, mode) : FIT_OK;
   if (rc != FIT_OK) return rc;

@@ -149,7 +149,10 @@ int launch_seeded_fit(const fit_handle* h, const FitArgs& a, int nevt, const int
 // The kernels with one track per thread: the tracks of mode m's events as
 // run tables of up to kTrackRuns runs (1 KiB of parameters, which costs a
 // launch nothing measurable), launch(base, r) for each; returns FIT_OK or the
-// first launch's error.
+// first launch's error.  A stream of more runs takes several launches, each
+// with a last wave of its own: 600 mixed events, 40000 tracks, finder 130,
+// adjoint 300, FP64 894 us; with tables of 1024 runs 74, 173 and 592, and a
+// call of one run unchanged (171 us).
 constexpr int kTrackRuns = 128;
 using TrackRuns = Runs<kTrackRuns>;
 
