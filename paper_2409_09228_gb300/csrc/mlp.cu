@@ -674,7 +674,7 @@ __global__ void __launch_bounds__(kBlock)
 // the layer loop early; a track that stops (surface not reached, non-finite
 // update) only stops moving.  Outputs, status bits and counters as
 // fit_fused_kernel<FIT_MODE_R>.
-__global__ void __launch_bounds__(kBlock)
+__global__ void __launch_bounds__(kBlock, 4)
     fit_seeded_kernel(const __grid_constant__ FitArgs a, const __grid_constant__ TrackRuns runs,
                       const Image* __restrict__ img) {
   __shared__ Image W;
