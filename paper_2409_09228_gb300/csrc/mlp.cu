@@ -673,7 +673,9 @@ __global__ void __launch_bounds__(kBlock)
 // warp evaluate the network together before every layer, so no thread leaves
 // the layer loop early; a track that stops (surface not reached, non-finite
 // update) only stops moving.  Outputs, status bits and counters as
-// fit_fused_kernel<FIT_MODE_R>.
+// fit_fused_kernel<FIT_MODE_R>.  Four blocks an SM fit with or without being
+// asked for; asked for, the compiler keeps 124 registers instead of 125 and
+// 250001 tracks take 230.7 us instead of 233.7.
 __global__ void __launch_bounds__(kBlock, 4)
     fit_seeded_kernel(const __grid_constant__ FitArgs a, const __grid_constant__ TrackRuns runs,
                       const Image* __restrict__ img) {
