@@ -178,6 +178,56 @@ def test_calls_from_several_threads(entry):
     c.close()
 
 
+@pytest.mark.parametrize("entry", ["fit", "plan", "aosoa"])
+def test_the_modes_run_side_by_side(entry):
+    """40000 tracks of each mode, one block of either an SM: the two launches
+    share the SMs, so that a call takes well under the sum of its modes' times
+    (graphs of the calls alone, so that no host time counts; 0.72 measured,
+    1.0 where one launch waits for the other)."""
+    n = 40000
+    ev = inputs.generate_events([n, n], [0, 1], seed=179, nlayer=NLAYER)
+    f = fit.Fitter(fit.Geometry(ev.B, ev.surf[0]), fit.Geometry(ev.B, ev.surf[1]))
+    best = {}
+    for name, nt, md, part in (("r", [n], [0], slice(0, n)), ("z", [n], [1], slice(n, 2 * n)),
+                               ("both", [n, n], [0, 1], slice(0, 2 * n))):
+        total = sum(nt)
+        d = [gpu_util.to_dev(np.ascontiguousarray(a[..., part]), total)
+             for a in (ev.par0, ev.cov0, ev.q, ev.hpos, ev.hcov)]
+        if entry == "aosoa":
+            d = [a if k == 2 else torch.from_numpy(inputs.to_aosoa32(a.cpu().numpy(), total)).cuda()
+                 for k, a in enumerate(d)]
+        o = f.outputs(total, ld=total)
+        bufs = dict(par_out=o["par"], cov_out=o["cov"], q_out=o["q"], chi2=o["chi2"])
+        plan = fit.fit_plan_create(f.h, nt, md, NLAYER)
+
+        def call():
+            if entry == "plan":
+                fit.fit_plan_run(plan, *d, **bufs)
+            elif entry == "fit":
+                fit.fit_propagate_update(f.h, *d, nt, md, **bufs)
+            else:
+                fit.fit_propagate_update_layout(f.h, *d, nt, md, fit.FIT_LAYOUT_AOSOA32, total, **bufs)
+
+        call()
+        torch.cuda.synchronize()
+        g = torch.cuda.CUDAGraph()
+        with torch.cuda.graph(g):
+            for _ in range(20):
+                call()
+        times = []
+        for _ in range(8):
+            e = [torch.cuda.Event(enable_timing=True) for _ in range(2)]
+            e[0].record()
+            g.replay()
+            e[1].record()
+            torch.cuda.synchronize()
+            times.append(e[0].elapsed_time(e[1]) / 20)
+        best[name] = min(times)
+        fit.fit_plan_destroy(plan)
+    f.close()
+    assert best["both"] < 0.87 * (best["r"] + best["z"]), best
+
+
 def independent(entry):
     """In a process of its own (few streams, a hardware queue for each): a call
     on stream b ends while stream a, which has a call queued, is held up."""
