@@ -23,6 +23,7 @@ using mlpk::TrainImage;
 
 struct fit_mlp {
   int device = 0;
+  void* d_block = nullptr;    // holds the fixed arrays: all but d_partials and d_curve
   float* d_params = nullptr;  // [kParams] FP32 master
   float* d_m = nullptr;       // Adam first and second moments
   float* d_v = nullptr;
@@ -847,16 +848,22 @@ int fit_mlp_create(fit_mlp** out, int device, uint64_t seed) {
   DeviceGuard guard(device);
   fit_mlp* m = new fit_mlp();
   m->device = device;
-  const size_t pb = mlpk::kParams * sizeof(float);
-  if (cudaMalloc(&m->d_params, pb) != cudaSuccess || cudaMalloc(&m->d_m, pb) != cudaSuccess ||
-      cudaMalloc(&m->d_v, pb) != cudaSuccess || cudaMalloc(&m->d_params_out, pb) != cudaSuccess ||
-      cudaMalloc(&m->d_m_out, pb) != cudaSuccess || cudaMalloc(&m->d_v_out, pb) != cudaSuccess ||
-      cudaMalloc(&m->d_img, sizeof(TrainImage)) != cudaSuccess ||
-      cudaMemset(m->d_img, 0, sizeof(TrainImage)) != cudaSuccess ||
-      cudaMalloc(&m->d_sync, 2 * sizeof(unsigned)) != cudaSuccess) {
+  // one allocation: six arrays of kParams floats on 256-byte boundaries, the
+  // image and the barrier's two words
+  const size_t pb = (mlpk::kParams * sizeof(float) + 255) & ~size_t(255);
+  const size_t ib = (sizeof(TrainImage) + 255) & ~size_t(255);
+  if (cudaMalloc(&m->d_block, 6 * pb + ib + 2 * sizeof(unsigned)) != cudaSuccess ||
+      cudaMemset(m->d_block, 0, 6 * pb + ib) != cudaSuccess) {
     fit_mlp_destroy(m);
     return fail(FIT_ERR_NOMEM, "fit_mlp_create: cudaMalloc");
   }
+  char* at = static_cast<char*>(m->d_block);
+  for (float** a : {&m->d_params, &m->d_m, &m->d_v, &m->d_params_out, &m->d_m_out, &m->d_v_out}) {
+    *a = reinterpret_cast<float*>(at);
+    at += pb;
+  }
+  m->d_img = reinterpret_cast<TrainImage*>(at);
+  m->d_sync = reinterpret_cast<unsigned*>(at + ib);
   // He-uniform weights (bound sqrt(6 / fan_in)), zero biases
   std::vector<float> P(mlpk::kParams, 0.f);
   uint64_t x = seed;
@@ -881,16 +888,9 @@ void fit_mlp_destroy(fit_mlp* m) {
   {
     DeviceGuard guard(m->device);
     cudaDeviceSynchronize();
-    cudaFree(m->d_params);
-    cudaFree(m->d_m);
-    cudaFree(m->d_v);
-    cudaFree(m->d_params_out);
-    cudaFree(m->d_m_out);
-    cudaFree(m->d_v_out);
-    cudaFree(m->d_img);
+    cudaFree(m->d_block);
     cudaFree(m->d_partials);
     cudaFree(m->d_curve);
-    cudaFree(m->d_sync);
   }
   delete m;
 }
