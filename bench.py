@@ -356,8 +356,8 @@ def config_dict(args):
 def bench_uneven(args, world, rank, local):
     """2000 events, log-normal track counts (median 2000, sigma 1, clipped
     50..20000), p2r or p2z at random per event, 20 layers: one call
-    (fit_propagate_update, one launch per mode) against a plan under a CUDA
-    graph, default and autotuned."""
+    (fit_propagate_update, one launch per mode) against a plan, at its default
+    (one launch per mode, launched directly) and autotuned (a CUDA graph)."""
     import torch
     from paper_2409_09228_gb300 import fit, inputs
 

@@ -1,12 +1,13 @@
 /*
  * fit_probe.h -- measurement and test probes of libfit (C ABI).
  *
- * Not part of the fit.  fit_probe_fp32: the fused kernel's roofline is its FP32 rate against
- * the GPU's FP32 ceiling; the ceiling is derived from unit counts (SMs x 128
- * FP32 lanes x 2 flops x clock), and this probe measures it on the device the
- * fit runs on, with scalar and with packed (two-lane) fused multiply-adds, so
- * that the derived figure is checked rather than assumed.  The paper has no
- * counterpart (it reports throughput, not a roofline).
+ * Not part of the fit.  fit_probe_fp32 measures the FP32 ceiling that the
+ * fused kernel's rate is compared with: it is derived from unit counts (SMs x
+ * 128 FP32 lanes x 2 flops x clock), and the probe checks it on the device the
+ * fit runs on, with scalar and with packed (two-lane) fused multiply-adds.
+ * The others let tests see what no entry point shows: the FP64 arithmetic by
+ * itself, whether host buffers are taken in place, a training whose blocks do
+ * not meet.  The paper has no counterpart.
  */
 #ifndef FIT_PROBE_H
 #define FIT_PROBE_H

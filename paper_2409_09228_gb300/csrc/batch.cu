@@ -1,7 +1,8 @@
 // libfit: plans for many events of uneven size and mixed surface types (p2r /
-// p2z), explicit and tuned shapes replayed from a CUDA graph, with a
-// launch-shape autotuner (fit_plan_* in fit.h).  A plan runs the fused kernels of fit.cu, one launch per mode
-// (the default, launched directly), or one persistent launch:
+// p2z), with a launch-shape autotuner (fit_plan_* in fit.h).  A plan runs the
+// fused kernels of fit.cu, one launch per mode (the default, launched
+// directly), or, with an explicit or tuned shape, replays a CUDA graph of
+// those or of one persistent launch:
 //
 // Work items are tiles of one event: threads_per_block x tracks_per_thread
 // consecutive tracks (two per thread in packed f32x2 instructions, or one),
@@ -34,7 +35,7 @@ struct WorkItem {
 };
 
 struct BatchArgs {
-  FitArgs a;  // buffers, nlayer, counters (a.t0/a.t1/a.geo unused)
+  FitArgs a;  // buffers, nlayer, counters (a.t0 and a.geo unused)
   Geo geo[2];
   const WorkItem* items;
   int nitems;

@@ -1,10 +1,12 @@
-// fit_propagate_update_host: the fused fit on HOST buffers.  The tracks are
-// cut into chunks of at most kChunk; chunk i goes through device staging set
-// i % kSets on internal stream i % kSets -- host-to-device copies, the fused
-// kernels, device-to-host copies -- so the copies of one chunk overlap the fit
-// and copies of the others (paper Sec. 3.1: inputs are copied to the device
-// before the kernel and results back after it).  The caller's stream orders
-// the whole call.
+// fit_propagate_update_host: the fused fit on HOST buffers.  Page-locked ones
+// are read and written by the kernels in place (as by
+// fit_propagate_update_mapped, below); a call with any other is staged: the
+// tracks are cut into chunks of at most kChunk, and chunk i goes through
+// device staging set i % kSets on internal stream i % kSets -- host-to-device
+// copies, the fused kernels, device-to-host copies -- so that the copies of
+// one chunk overlap the fit and copies of the others (paper Sec. 3.1: inputs
+// are copied to the device before the kernel and results back after it).  The
+// caller's stream orders the whole call.
 #include <cuda.h>
 #include <cuda_runtime.h>
 

@@ -367,9 +367,10 @@ def _haddr(a) -> int:
 def fit_propagate_update_host(h: int, par_in, cov_in, q_in, hpos, hcov, ntrk: Sequence[int],
                               mode: Sequence[int], par_out=None, cov_out=None, q_out=None,
                               chi2=None, chi2_layer=None, status=None, stream=None) -> None:
-    """The fused fit on HOST arrays (page-locked torch tensors for overlap, or
-    numpy arrays), copied through the library's device staging in chunks; the
-    arrays must stay alive until the stream passes the call (fit_sync)."""
+    """The fused fit on HOST arrays (torch tensors or numpy arrays): in place
+    where all of them are page-locked (fit.h), otherwise copied through the
+    library's device staging in chunks.  The arrays must stay alive, and the
+    outputs unread, until the stream passes the call (fit_sync)."""
     par_out = par_in if par_out is None else par_out
     cov_out = cov_in if cov_out is None else cov_out
     q_out = q_in if q_out is None else q_out
@@ -440,7 +441,8 @@ def fit_plan_create(h: int, ntrk: Sequence[int], mode: Sequence[int], nlayer: in
                     threads_per_block: int = 128, blocks_per_sm: int = 0,
                     persistent: bool = True, tracks_per_thread: int = 2,
                     layout: int = FIT_LAYOUT_SOA) -> int:
-    """A plan for the batched persistent form (see fit.h)."""
+    """A plan for many events (see fit.h): with the defaults one launch per mode,
+    with blocks_per_sm or another shape one persistent launch under a CUDA graph."""
     nevt, nt, md = _event_bytes(ntrk, mode)
     cfg = fit_launch_config(threads_per_block, blocks_per_sm, int(persistent),
                             int(tracks_per_thread), int(layout))
