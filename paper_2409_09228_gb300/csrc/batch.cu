@@ -233,9 +233,9 @@ struct fit_plan {
   // plan runs the fused kernels on its events (same pairs as the persistent
   // form), one launch per mode.  Each mode then has its own registers (p2z
   // 127 instead of 168 for both) and p2z its staged hits, and no block waits
-  // for the work counter: 2000 uneven mixed events, 4M tracks, 1045 -> 841 us.
+  // for the work counter: 2000 uneven mixed events, 4M tracks, 1045 -> 835 us.
   // Launched directly: two launches cost the host no more than a graph's, and
-  // new buffers no capture (the first pass on them 1132 -> 911 us; 961 captured).
+  // new buffers no capture (the first pass on them 1132 -> 900 us; 50 more captured).
   bool free_form = false;
   int sms = 0;
   WorkItem* d_items = nullptr;

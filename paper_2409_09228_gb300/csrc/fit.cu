@@ -276,7 +276,7 @@ void add_run(PairRuns<kMaxRuns>& r, uint32_t t0, uint32_t t1) {
 // same-mode events gathered in a table, with a new launch where it is full
 // or its tracks span 2^31.  launch(a, m, r) issues the kernel for the
 // runs r of mode m (a.t0: their base; a.geo: the mode's geometry).
-// An uneven mixed batch (500 events, 1M tracks, ~250 runs) takes 0.228 ms in
+// An uneven mixed batch (500 events, 1M tracks, ~250 runs) takes 0.219 ms in
 // two launches; with one launch per run it took 4.11 ms, a run's few blocks
 // leaving most SMs idle for the ~20 us of its layers.
 // by_event: every event is a run of its own.

@@ -233,7 +233,7 @@ extern "C" int fit_propagate_update_host(fit_handle* h, const fit_tracks_in* in,
   // Page-locked buffers that the device reaches: the kernels read and write
   // them in place, which moves only what they touch (5 of a p2z hit's 9
   // floats) at the link's rate and needs no staging: 96000 tracks of both modes
-  // 520 -> 334 us, 1.92M 8.1-20.8 -> 6.3 ms.
+  // 520 -> 323 us, 1.92M 8.1-20.8 -> 6.2 ms.
   // Others go through the staging sets.
   if (in_place(in, out, hits, total, nlayer)) {
     rc = run_fit_streams(h, base_args(in, out, hits, nlayer, h->d_counters),
