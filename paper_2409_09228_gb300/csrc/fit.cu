@@ -390,8 +390,8 @@ bool launch_small(const fit_handle* h, const FitArgs& a, bool by_event, int nevt
 // one warp (a block of 128 per SM, 19456 tracks): 8192 p2r tracks take 14.3 us
 // in the small kernel and 18.5 in pairs.  With two warps per scheduler, at
 // 32768 tracks, pairs are as fast (18.5 us), at 65536 faster (26.6 against 28.3).
-bool is_small(int sms, int64_t call_tracks) { return call_tracks <= (int64_t)sms * kBlock; }
-bool is_small(const fit_handle* h, int64_t call_tracks) { return is_small(h->sms, call_tracks); }
+static bool is_small(int sms, int64_t call_tracks) { return call_tracks <= (int64_t)sms * kBlock; }
+static bool is_small(const fit_handle* h, int64_t call_tracks) { return is_small(h->sms, call_tracks); }
 
 // The fused fit of events [0, nevt) on the tracks of a.
 int run_fit(const fit_handle* h, const FitArgs& a, const RunOptions& o, int nevt,

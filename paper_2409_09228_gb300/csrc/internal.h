@@ -201,9 +201,6 @@ struct RunOptions {
   int64_t call_tracks = 0;  // tracks of the whole call, which may be cut into chunks
 };
 
-// Whether a call of that many tracks takes one launch for both modes (fit.cu).
-bool is_small(const fit_handle* h, int64_t call_tracks);
-
 // The two modes' events of a call are independent: with both present, the
 // p2z launches go to a second stream, so that they overlap the p2r launches
 // (their blocks fill the SMs a launch's last wave leaves idle).  begin() forks
